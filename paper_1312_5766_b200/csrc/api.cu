@@ -6,6 +6,7 @@
 #include <cstring>
 #include <new>
 
+#include "engine.cuh"
 #include "strads_internal.cuh"
 
 using namespace strads;
@@ -58,6 +59,10 @@ struct strads_lasso_s {
   cudaStream_t copy_stream;
   cudaEvent_t copy_fork, copy_done;
   long long ahead_round;     // the round whose early list is in place (-1: none)
+  // one scheduler: whole rounds in one cooperative launch (engine.cu), where the configuration allows it
+  bool engine_ok;
+  Engine engine;
+  alignas(64) unsigned char engine_maps[256];
 };
 
 namespace {
@@ -70,6 +75,9 @@ constexpr int tail_rounds(int kind) { return kGraphRoundsAhead >> (kind + 1); }
 static_assert(tail_rounds(kTailKinds - 1) == 1, "the shortest left-over sequence is one round");
 static_assert(sizeof(strads_lasso_s::tail_exec) / sizeof(cudaGraphExec_t) == kTailKinds, "one slot per left-over sequence");
 constexpr int kEdgeCap = 8192;        // conflicting pairs the Gram kernels can list for the walk (32 KB)
+constexpr int kEngineRounds = 32;     // rounds per launch of the engine: a launch every few hundred microseconds, so that other streams get their turn
+constexpr int kEngineDenseRows = 2048;
+constexpr int kEngineMaxCtas = 192;   // CTAs the engine's scratch provides for
 constexpr int kAheadMaxKeep = 4096;   // sampling ahead: the patch kernel holds 2 P keys in shared memory
 
 Scheduler& on_turn(strads_lasso_s* h) { return h->sch[h->round_host % h->n_sched]; }
@@ -93,7 +101,11 @@ struct Layout {
   size_t off_state, off_n2, off_hist, off_sure, off_boundary, off_cand, off_kept, off_kept_pos, off_dbeta, off_dbeta64,
       off_conflict, off_cand_dbeta64, off_cand_bnew, off_dot_partial, off_dot_ticket, off_margin, off_obj, off_amb, off_xcb, off_walk_blocked, off_walk_ctl, off_walk_cols,
       off_bucket_count, off_bucket_items, off_bucket_vals, off_bucket_cols, off_resid_acc, off_delta_prev, off_edges, off_patch_keys, off_cand_keys, off_survivors, off_bin_off, off_bin_cur, off_ahead_bin_off, off_ahead_bin_cur,
-      off_ahead_state, off_ahead_hist, off_ahead_sure, off_ahead_boundary, off_ahead_keys, off_ahead_idx, total;
+      off_ahead_state, off_ahead_hist, off_ahead_sure, off_ahead_boundary, off_ahead_keys, off_ahead_idx,
+      off_eng_state, off_eng_hist, off_eng_cur, off_eng_win, off_eng_surv, off_eng_xb, off_eng_norm, off_eng_part, off_eng_tickets, total;
+  long long eng_pitch, eng_lo;
+  int eng_list, eng_tiles;
+  bool engine;
   int cap_sure, cap_boundary, mask_words, dot_parts, cap_amb, n_ahead, cap_ahead_boundary, cap_survivors;
   long long ldc, ldcb;
   bool buckets;
@@ -116,13 +128,29 @@ int check_sizes(const strads_lasso_config_t* c) {
   return STRADS_OK;
 }
 
+// Whether the workspace provides for the engine: CSC always; dense X with short columns and the default Gram.
+bool engine_wanted(const strads_lasso_config_t* c) {
+  if (c->flags & (STRADS_FLAG_SIMT_GRAM | STRADS_FLAG_GRAM_3XTF32)) return false;
+  return c->layout == STRADS_CSC || c->n_rows <= kEngineDenseRows;
+}
+// Whether the rounds go through it: one scheduler, and for dense X columns so short that independent ones correlate
+// beyond rho by chance (their correlations scatter with N^-1/2; the line is three of those).  There the launch chain's
+// screen leaves percents of all pairs open and its window fails round after round (463 x 508,999: 888 us per round as
+// launches, 65 here); with longer columns the captured chain of kernels, each with a whole GPU's worth of loads under way,
+// is the faster one (c1 36.3 us against 39.0, c2 42 against 60).
+bool engine_chosen(const strads_lasso_config_t* c) {
+  if (!engine_wanted(c) || n_sched_of(c) > 1) return false;
+  return c->layout == STRADS_CSC || (double)c->n_rows * (double)c->rho * (double)c->rho <= 9.0;
+}
+size_t engine_boundary(size_t winners) { return winners / 2 > 2048 ? winners / 2 : 2048; }
+
 // Slice of the workspace of one scheduler; the first one (`first`) also holds what all share
 // (column norms, the objective's partial sums).
 Layout carve(const strads_lasso_config_t* c, bool first = true) {
   Layout L;
   L.cap_sure = c->n_candidates;
   L.cap_boundary = pow2_ceil(c->n_candidates / 2 > 2048 ? c->n_candidates / 2 : 2048);
-  L.mask_words = (c->n_candidates + 31) / 32;
+  L.mask_words = (c->n_candidates + 127) / 128 * 4;      // (rows of conflict bits start on 16 bytes)
   // CTAs per kept column in the dot kernel: about 1024 CTAs in all, so that every one of them is resident at
   // once (the kernel is a chain of dependent loads per CTA; residency, not depth per thread, hides it)
   long long parts = (1024 + c->n_keep - 1) / c->n_keep;
@@ -143,8 +171,10 @@ Layout carve(const strads_lasso_config_t* c, bool first = true) {
   L.off_dbeta64 = take(sizeof(double) * (size_t)c->n_keep);
   L.off_conflict = take(sizeof(unsigned int) * (size_t)c->n_candidates * L.mask_words);
   const bool dense = c->layout == STRADS_DENSE_COLMAJOR;
-  L.off_cand_dbeta64 = take(dense ? sizeof(double) * (size_t)c->n_candidates : 0);
-  L.off_cand_bnew = take(dense ? sizeof(float) * (size_t)c->n_candidates : 0);
+  L.engine = engine_wanted(c);
+  const bool proposals = dense || L.engine;
+  L.off_cand_dbeta64 = take(proposals ? sizeof(double) * (size_t)c->n_candidates : 0);
+  L.off_cand_bnew = take(proposals ? sizeof(float) * (size_t)c->n_candidates : 0);
   L.off_dot_partial = take(sizeof(double) * (size_t)c->n_keep * L.dot_parts);
   L.off_dot_ticket = take(sizeof(unsigned int) * (size_t)c->n_keep);
   L.off_margin = take(first && (c->flags & STRADS_FLAG_LOGISTIC) ? sizeof(float) * (size_t)c->n_rows : 0);
@@ -168,7 +198,7 @@ Layout carve(const strads_lasso_config_t* c, bool first = true) {
   L.off_delta_prev = take(sizeof(float) * (size_t)c->n_keep);
   L.off_edges = take(sizeof(unsigned int) * kEdgeCap);
   L.off_patch_keys = take(sizeof(unsigned long long) * 2 * (size_t)c->n_keep);
-  L.off_cand_keys = take(dense ? sizeof(unsigned long long) * 2 * (size_t)c->n_candidates : 0);
+  L.off_cand_keys = take(proposals ? sizeof(unsigned long long) * 2 * (size_t)c->n_candidates : 0);
   // keys the sampler's guided first pass saves for its collect pass (many coefficients only): 8 P' of them
   L.cap_survivors = c->n_cols >= (1 << 19) ? 8 * c->n_candidates : 0;
   L.off_survivors = take(sizeof(unsigned long long) * (size_t)L.cap_survivors);
@@ -178,7 +208,8 @@ Layout carve(const strads_lasso_config_t* c, bool first = true) {
   // Dense layouts only: measured on the CSC workloads, a draw running beside the round's many-CTA, latency-bound
   // Gram kernels did not shorten it (c4: 102 -> 106 us per round, c5: 350 -> 384 us; again with the on-demand walk cut
   // to one CTA per SM so that the draw has registers to run in: c4 99 -> 103 us, c5 230 -> 281 us).
-  const bool ahead = first && n_sched_of(c) == 1 && c->n_keep <= kAheadMaxKeep && c->layout == STRADS_DENSE_COLMAJOR;
+  // (the first slice is the same whatever the number of schedulers)
+  const bool ahead = first && c->n_keep <= kAheadMaxKeep && c->layout == STRADS_DENSE_COLMAJOR;
   const long long n_ahead = (long long)c->n_candidates + c->n_keep < c->n_cols ? (long long)c->n_candidates + c->n_keep : c->n_cols;
   L.n_ahead = ahead ? (int)n_ahead : 0;
   L.cap_ahead_boundary = ahead ? pow2_ceil(L.n_ahead / 2 > 2048 ? L.n_ahead / 2 : 2048) : 0;
@@ -190,6 +221,24 @@ Layout carve(const strads_lasso_config_t* c, bool first = true) {
   L.off_ahead_idx = take(sizeof(int) * (size_t)L.n_ahead);
   L.off_ahead_bin_off = take(ahead ? sizeof(int) * (kHistBins + 1) : 0);
   L.off_ahead_bin_cur = take(ahead ? sizeof(unsigned int) * kHistBins : 0);
+  // the round engine: a draw of P' + P winners one round ahead (P' at the round's start when P is too large for that)
+  if (!first) L.engine = false;
+  const bool en = L.engine;
+  L.eng_list = en && c->n_keep <= kAheadMaxKeep ? (int)n_ahead : 0;
+  const size_t most = (size_t)(L.eng_list > c->n_candidates ? L.eng_list : c->n_candidates);
+  L.off_eng_state = take(en ? sizeof(EngineState) : 0);
+  L.off_eng_hist = take(en ? sizeof(unsigned int) * kHistBins : 0);
+  L.off_eng_cur = take(en ? sizeof(unsigned int) * kHistBins : 0);
+  L.off_eng_win = take(en ? sizeof(unsigned long long) * (most + engine_boundary(most)) : 0);
+  L.off_eng_surv = take(en ? sizeof(unsigned long long) * (8 * most + 1024) : 0);
+  L.eng_lo = (c->n_rows + 127) / 128 * 128;
+  L.eng_pitch = 2 * L.eng_lo;
+  const int side = (c->n_candidates + 63) / 64;
+  L.eng_tiles = en && dense ? side * (side + 1) / 2 : 0;
+  L.off_eng_xb = take(en && dense ? sizeof(unsigned short) * (size_t)c->n_candidates * L.eng_pitch : 0);
+  L.off_eng_norm = take(en && dense ? sizeof(double) * (size_t)c->n_candidates : 0);
+  L.off_eng_part = take(en && dense ? sizeof(float) * 128 * 128 * (size_t)kEngineMaxCtas : 0);
+  L.off_eng_tickets = take(sizeof(unsigned int) * (size_t)L.eng_tiles);
   L.total = o;
   return L;
 }
@@ -482,6 +531,46 @@ void fill_ahead(Problem& a, const Problem& p0, const Layout& L, char* ws) {
   a.survivors = nullptr; a.cap_survivors = 0;         // (the early draw is off the round's path: it keeps to the plain passes)
 }
 
+void fill_engine(Engine& en, const Problem& p, const Layout& L, char* ws) {
+  en.es = reinterpret_cast<EngineState*>(ws + L.off_eng_state);
+  en.hist = reinterpret_cast<unsigned int*>(ws + L.off_eng_hist);
+  en.bin_cur = reinterpret_cast<unsigned int*>(ws + L.off_eng_cur);
+  en.win = reinterpret_cast<unsigned long long*>(ws + L.off_eng_win);
+  const size_t most = (size_t)(L.eng_list > p.n_cand ? L.eng_list : p.n_cand);
+  en.cap_boundary = (int)engine_boundary(most);
+  en.cap_win = (int)most + en.cap_boundary;
+  en.surv = reinterpret_cast<unsigned long long*>(ws + L.off_eng_surv);
+  en.cap_surv = (unsigned)(8 * most + 1024);
+  en.n_list = L.eng_list;
+  en.window = window_of(p, p.n_cand);
+  en.xb = reinterpret_cast<unsigned short*>(ws + L.off_eng_xb);
+  en.xb_pitch = L.eng_pitch; en.lo_off = L.eng_lo;
+  en.norm = reinterpret_cast<double*>(ws + L.off_eng_norm);
+  en.part = reinterpret_cast<float*>(ws + L.off_eng_part);
+  en.tile_ticket = reinterpret_cast<unsigned int*>(ws + L.off_eng_tickets);
+}
+
+// What must be zero before a launch of the engine (it leaves it so, unless a wait expired).
+cudaError_t clear_engine(const strads_lasso_s* h) {
+  const Engine& en = h->engine;
+  const Problem& p = h->sch[0].p;
+  cudaError_t e;
+  if ((e = cudaMemsetAsync(en.es, 0, sizeof(EngineState), h->stream)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(en.hist, 0, sizeof(unsigned int) * kHistBins, h->stream)) != cudaSuccess) return e;
+  if (p.layout == STRADS_DENSE_COLMAJOR) {
+    const long long side = (p.n_cand + 63) / 64;
+    return cudaMemsetAsync(en.tile_ticket, 0, sizeof(unsigned int) * (size_t)(side * (side + 1) / 2), h->stream);
+  }
+  if (p.bucket_count != nullptr &&
+      (e = cudaMemsetAsync(p.bucket_count, 0, sizeof(unsigned int) * (size_t)p.N, h->stream)) != cudaSuccess) return e;
+  return cudaMemsetAsync(p.resid_acc, 0, sizeof(long long) * (size_t)p.N, h->stream);
+}
+
+// The engine takes a round unless the steps are timed one by one or the Gram matrix itself is asked for.
+bool engine_runs(const strads_lasso_s* h, const strads_round_out_t* out) {
+  return h->engine_ok && h->prof_events == nullptr && !(out != nullptr && out->gram != nullptr);
+}
+
 void release(strads_lasso_s* h) {
   for (int s = 0; s < STRADS_MAX_SCHEDULERS; ++s) {
     if (h->sch[s].stream != nullptr) cudaStreamDestroy(h->sch[s].stream);
@@ -572,7 +661,17 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
       (e = cudaEventCreateWithFlags(&h->copy_done, cudaEventDisableTiming)) != cudaSuccess)
     return fail(cuda_fail(e, "copy stream"));
   h->ahead_round = -1;
-  h->ahead_ok = L.n_ahead > 0;
+  h->engine_ok = L.engine && engine_chosen(c) && sm_count <= kEngineMaxCtas;
+  if (h->engine_ok) {
+    fill_engine(h->engine, p0, L, ws);
+    if ((e = prepare_engine(p0, h->engine)) != cudaSuccess) return fail(cuda_fail(e, "prepare_engine"));
+    if (p0.layout == STRADS_DENSE_COLMAJOR && (e = encode_engine_maps(p0, h->engine, h->engine_maps)) != cudaSuccess)
+      return fail(cuda_fail(e, "encode_engine_maps"));
+    if (p0.layout == STRADS_DENSE_COLMAJOR &&
+        (e = cudaMemsetAsync(h->engine.xb, 0, sizeof(unsigned short) * (size_t)p0.n_cand * L.eng_pitch, h->stream)) != cudaSuccess)
+      return fail(cuda_fail(e, "cudaMemsetAsync"));
+  }
+  h->ahead_ok = S == 1 && L.n_ahead > 0;
   if (h->ahead_ok) {
     fill_ahead(h->ahead, p0, L, ws);
     if ((e = launch_init_scheduler(h->ahead, p0, h->stream)) != cudaSuccess) return fail(cuda_fail(e, "launch_init_scheduler"));
@@ -612,6 +711,7 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
         return fail(cuda_fail(e, "scheduler stream"));
     }
   }
+  if (h->engine_ok && (e = clear_engine(h)) != cudaSuccess) return fail(cuda_fail(e, "clear_engine"));
   if (S > 1 && (e = cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming)) != cudaSuccess)
     return fail(cuda_fail(e, "cudaEventCreate"));
   *out_handle = h;
@@ -620,6 +720,12 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
 
 int strads_round(strads_handle_t h, const strads_round_out_t* out) {
   if (h == nullptr) return STRADS_ERR_INVALID_ARG;
+  if (engine_runs(h, out)) {
+    h->ahead_round = -1;
+    CK(launch_engine(h->sch[0].p, h->engine, h->engine_maps, 1, false, false, out, h->stream));
+    h->round_host += 1;
+    return STRADS_OK;
+  }
   return one_round(h, out);
 }
 
@@ -671,6 +777,17 @@ static int build_round_graph(strads_lasso_s* h, int tail_kind = -1) {
 
 int strads_run(strads_handle_t h, int64_t n_rounds) {
   if (h == nullptr || n_rounds < 0) return STRADS_ERR_INVALID_ARG;
+  if (engine_runs(h, nullptr)) {
+    while (n_rounds > 0) {
+      const int n = n_rounds < kEngineRounds ? (int)n_rounds : kEngineRounds;
+      const bool ahead = h->engine.n_list > 0;
+      CK(launch_engine(h->sch[0].p, h->engine, h->engine_maps, n, ahead && h->ahead_round == h->round_host, ahead, nullptr, h->stream));
+      h->round_host += n;
+      h->ahead_round = ahead ? h->round_host : -1;
+      n_rounds -= n;
+    }
+    return STRADS_OK;
+  }
   if (h->n_sched > 1) {
     // whole captured sequences where they fit (they start with scheduler 0), the rest enqueued directly
     const long long R = graph_rounds(h);
@@ -746,8 +863,14 @@ int strads_round_host(strads_handle_t h, float* beta_host, float* resid_host, fl
   CK(cudaMemcpyAsync(p.resid, resid_host, sizeof(float) * p.N, cudaMemcpyHostToDevice, h->copy_stream));
   CK(cudaMemcpyAsync(p.beta, beta_host, sizeof(float) * p.J, cudaMemcpyHostToDevice, h->copy_stream));
   CK(cudaEventRecord(h->copy_done, h->copy_stream));
-  const int rc = one_round(h, nullptr, h->copy_done);
-  if (rc) return rc;
+  if (engine_runs(h, nullptr)) {
+    CK(cudaStreamWaitEvent(h->stream, h->copy_done, 0));
+    const int rc = strads_round(h, nullptr);
+    if (rc) return rc;
+  } else {
+    const int rc = one_round(h, nullptr, h->copy_done);
+    if (rc) return rc;
+  }
   CK(cudaMemcpyAsync(beta_host, p.beta, sizeof(float) * p.J, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaMemcpyAsync(resid_host, p.resid, sizeof(float) * p.N, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaMemcpyAsync(delta_host, p.delta, sizeof(float) * p.J, cudaMemcpyDeviceToHost, h->stream));
@@ -871,6 +994,7 @@ int strads_inject_stall(strads_handle_t h, int32_t which) {
     if (sc.p.layout != STRADS_CSC) return STRADS_ERR_INVALID_ARG;
     // an arrival count no barrier of the walk can complete from
     CK(cudaMemsetAsync(&sc.p.walk_ctl->bar_count, 0x40, sizeof(unsigned int), h->stream));
+    if (h->engine_ok) CK(cudaMemsetAsync(&h->engine.es->bar_count, 0x40, sizeof(unsigned int), h->stream));
   } else if (which == STRADS_STALL_GRAM_LOADS) {
     if (sc.p.layout != STRADS_DENSE_COLMAJOR) return STRADS_ERR_INVALID_ARG;
     sc.p.stall = 1;
@@ -892,6 +1016,7 @@ int strads_recover(strads_handle_t h) {
     CK(cudaMemsetAsync(&p.st->status, 0, sizeof(unsigned int), h->stream));
     if (p.layout == STRADS_CSC) CK(cudaMemsetAsync(p.walk_ctl, 0, sizeof(WalkControl), h->stream));
   }
+  if (h->engine_ok) CK(clear_engine(h));
   if (had_stall) drop_round_graph(h);
   h->ahead_round = -1;                                   // (whatever was drawn ahead belongs to the abandoned rounds)
   CK(cudaStreamSynchronize(h->stream));

@@ -1,0 +1,2096 @@
+// Whole rounds of Algorithm 1 in one cooperative launch: one CTA of 512 threads per SM, the steps of a round
+// separated by a grid barrier instead of by kernel boundaries.
+//
+// A round is a chain of short dependent steps over a few MB at most, so what bounds it is the number of times the
+// whole grid has to hand over to itself and what every hand-over costs.  As separate launches a round took 11 to 17
+// kernels, each with its launch, its ramp and the drain of the one before; here it takes four barriers of ~1.5 us, and the
+// draw of the next round runs in the shadow of the steps of this one:
+//
+//   step           dense                                          CSC
+//   1  (all CTAs)  BF16 copies of the candidates' columns,        last round's residual applied; candidates entered
+//                  x_c^T r and would-be changes; scan of the      into the row buckets; scan of the keys of round t + 1
+//                  keys of round t + 1
+//   2  (all CTAs)  Gram tiles on the tensor cores                 inner products from the buckets, x_c^T r and would-be
+//                                                                 changes; keys of round t + 1 below the boundary collected
+//  (2b)            exact products of pairs left open
+//   3              greedy walk (CTA 0); keys of round t + 1       greedy walk (CTA 0); buckets emptied (the others)
+//                  below the boundary collected (the others)
+//  (3b)            all candidates instead of the window           walk over all candidates with conflict rows on demand
+//   4  (all CTAs)  residual, beta, delta; the winners of the draw ranked, corrected for this round's changes
+//
+// Drawing ahead is exact: the draw of round t + 1 collects the P' + P smallest keys by the priorities of round t's
+// start; the update changes at most P priorities, so every candidate of round t + 1 that is not one of those is among
+// them, and its rank follows from its rank in the early list, the old keys of the changed coefficients below it and
+// their new keys below it.
+//
+// The results are those of the kernels used one by one (split-phase calls): same keys, same order of the FP64 sums of
+// CSC columns, same decisions; dense inner products are pairs of floats as in the pack kernel, in another order.
+// No floating-point atomics.  Every barrier wait has an iteration limit (STRADS_STATUS_WAIT_EXPIRED).
+#include <climits>
+
+#include <cuda.h>
+#include <cuda_bf16.h>
+
+#include "engine.cuh"
+#include "walk_pairs.cuh"
+
+namespace strads {
+namespace {
+
+constexpr int kT = 512;                    // threads of a CTA, one CTA per SM
+constexpr int kWarps = kT / 32;
+constexpr unsigned int kFull = 0xffffffffu;
+constexpr unsigned int kSpinLimit = 1u << 22;
+
+// ------------------------------------------------------------------------------------------------
+// Grid barrier: one counter that only grows during a launch.  A CTA may pass when all have arrived target / n times;
+// no CTA can be more than one barrier ahead, so the counter lies within [target, target + n) then -- an arrival count
+// outside that range (strads_inject_stall plants one) never lets anybody pass.
+// ------------------------------------------------------------------------------------------------
+struct Grid {
+  unsigned int* count;
+  unsigned int target, n, limit;
+  unsigned int* status;
+};
+
+// withhold: this CTA does not arrive (an injected stall: everybody's wait runs out).
+__device__ bool grid_sync(Grid& g, bool withhold = false) {
+  __shared__ int s_ok;
+  g.target += g.n;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    if (!withhold) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(g.count) : "memory");
+    unsigned int v, it = 0;
+    bool ok;
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(g.count) : "memory");
+      ok = v - g.target < g.n;
+    } while (!ok && ++it < g.limit);
+    if (!ok) atomicOr(g.status, STRADS_STATUS_WAIT_EXPIRED);
+    s_ok = ok;
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+  return v;
+}
+
+// ------------------------------------------------------------------------------------------------
+// The draw (SAP step 1; the keys and their order are those of sampler.cu).
+//
+// scan     every key below the cutoff carried over from the last draw is binned and saved; the others are recognised
+//          from a few operations (T >= v / w with v = (x + 1/2) 2^-32) and not computed.  Without a cutoff all keys
+//          are computed and binned by their top 12 bits.
+// select   every CTA reads the 4,096 counts, scans them and finds the bin that holds the n_list-th key -- the same in
+//          all of them, so nothing has to be published.
+// collect  the keys up to that bin, saved ones if the scan saved them all, go to `win`, grouped by bin.
+// rank     a key's rank is the start of its group plus the smaller keys inside it.
+//
+// With a cutoff the bins are 64 per octave below it (bits 17 and up of the binary32 time, counted down from the
+// cutoff's): the winners of an exponential race spread over the top octaves, so a group holds P' / 128 keys or fewer
+// where 8 bins per octave (the unguided scan) leave P' / 16.
+// ------------------------------------------------------------------------------------------------
+struct Binning { unsigned int shift, base; };
+__device__ __forceinline__ Binning binning_of(float cut) {
+  Binning b;
+  b.shift = cut > 0.f ? 17u : 32u - kHistBits;
+  const unsigned int top = __float_as_uint(cut) >> 17;
+  b.base = cut > 0.f && top > (unsigned)(kHistBins - 1) ? top - (kHistBins - 1) : 0u;
+  return b;
+}
+__device__ __forceinline__ unsigned int bin_of(const Binning& b, unsigned int bits) {
+  const unsigned int x = bits >> b.shift;
+  return x > b.base ? min(x - b.base, (unsigned)(kHistBins - 1)) : 0u;
+}
+
+constexpr int kQueue = 192;                // survivors of a warp waiting for their keys; a step appends at most 128
+
+// Place of a bin in an array in shared memory: a gap every 32 words, so that threads that own eight consecutive bins
+// each do not meet in the same banks.
+__device__ __forceinline__ int pad(int b) { return b + (b >> 5); }
+
+// What a CTA knows about the draw in progress (shared memory).
+struct DrawShared {
+  unsigned int off[kHistBins + (kHistBins >> 5) + 1];      // winners before each bin, at pad(bin)
+  unsigned int wsum[kWarps];
+  int bnd, refined;                        // the bin of the n_list-th key; whether it had to be cut further
+  unsigned int bnd_count, total;
+  unsigned long long prefix;               // refined: keys of the boundary bin whose top `bits` bits exceed it are no winners
+  int bits;
+  float cut;                               // cutoff of the scan
+};
+
+// w_j = fma(x, y, z) for every importance distribution: (|d|, |d|, eta), (|d|, 1, eta) or (0, 0, 1) -- the same bits as
+// priority_weight, and one sequence of instructions for all three.
+struct WeightForm { bool square, uniform; float one, z; };
+__device__ __forceinline__ WeightForm weight_form(const Problem& p) {
+  const int mode = weight_mode_of(p.flags);
+  WeightForm f;
+  f.square = mode == kWeightSquare; f.uniform = mode == kWeightUniform;
+  f.one = f.uniform ? 0.f : 1.f; f.z = f.uniform ? 1.f : p.eta;
+  return f;
+}
+__device__ __forceinline__ float weight_of(const WeightForm& f, float d) {
+  const float x = f.uniform ? 0.f : fabsf(d);
+  return __fmaf_rn(x, f.square ? x : f.one, f.z);
+}
+__device__ __forceinline__ unsigned long long key_of(const WeightForm& f, float d, uint32_t word, uint32_t j) {
+  return ((unsigned long long)__float_as_uint(__fdiv_rn(unit_exponential_rn(word), weight_of(f, d))) << 32) | j;
+}
+
+// A warp's share of a scan.  f(key, active) is called by whole warps.
+template <typename F>
+__device__ __forceinline__ void scan_keys(const Problem& p, unsigned long long t, float cut, uint2* queue, int warp0, int n_warps, F&& f) {
+  const int lane = threadIdx.x & 31;
+  const long long groups = (p.J + 3) >> 2, whole = p.J >> 2;
+  const WeightForm wf = weight_form(p);
+  // x 2^-32 > 1.02 cut w implies T > cut: the computed E is never below (x + 1/2) 2^-32 up to rounding
+  const float k = cut > 0.f ? __fmul_rn(cut, 1.02f * 4294967296.0f) : __uint_as_float(0x7f800000u);
+  int n = 0;
+  const long long step = (long long)n_warps * 32;
+  // (one trip more than there are steps: the last one only empties the queue)
+  for (long long g0 = (long long)warp0 * 32;; g0 += step) {
+    const bool more = g0 < groups;
+    if (more) {
+      const long long g = g0 + lane;
+      float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (g < whole) {
+        d = __ldcg(reinterpret_cast<const float4*>(p.delta) + g);
+      } else if (g < groups) {
+        const long long j = g << 2;
+        d.x = p.delta[j];
+        if (j + 1 < p.J) d.y = p.delta[j + 1];
+        if (j + 2 < p.J) d.z = p.delta[j + 2];
+      }
+      uint32_t w[4];
+      philox4x32_10((uint32_t)g, (uint32_t)t, (uint32_t)(t >> 32), 0u, (uint32_t)p.seed, (uint32_t)(p.seed >> 32), w);
+      const float dd[4] = {d.x, d.y, d.z, d.w};
+      bool in[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) in[i] = !(__uint2float_rn(w[i]) > __fmul_rn(k, weight_of(wf, dd[i])));
+      if (g >= whole) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) in[i] = in[i] && (g << 2) + i < p.J;
+      }
+      if (!__any_sync(kFull, in[0] | in[1] | in[2] | in[3])) continue;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const unsigned int m = __ballot_sync(kFull, in[i]);
+        if (in[i]) queue[n + __popc(m & ((1u << lane) - 1u))] = make_uint2((uint32_t)(g << 2) + i, w[i]);
+        n += __popc(m);
+      }
+    }
+    if (n > kQueue - 128 || !more) {                     // the keys of the survivors, computed by all lanes together
+      __syncwarp();
+#pragma unroll 1
+      for (int i = 0; i < n; i += 32) {
+        const bool on = i + lane < n;
+        const uint2 e = on ? queue[i + lane] : make_uint2(0u, 0u);
+        f(on ? key_of(wf, p.delta[e.x], e.y, e.x) : ~0ull, on);
+      }
+      __syncwarp();
+      n = 0;
+    }
+    if (!more) break;
+  }
+}
+
+// Shared memory of a scan: the CTA's histogram, then a queue per warp.
+constexpr size_t kScanSmem = sizeof(unsigned int) * kHistBins + sizeof(uint2) * kQueue * kWarps;
+
+// guided: with the cutoff es->t_cut (if there is one).  Also clears the cursors of the groups.
+__device__ __forceinline__ void draw_scan(const Problem& p, const Engine& e, DrawShared& ds, unsigned char* sm, unsigned long long t, bool guided) {
+  unsigned int* sh = reinterpret_cast<unsigned int*>(sm);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint2* queue = reinterpret_cast<uint2*>(sm + sizeof(unsigned int) * kHistBins) + warp * kQueue;
+  const float cut = guided ? e.es->t_cut : 0.f;
+  const Binning bins = binning_of(cut);
+  __syncthreads();
+  for (int b = tid; b < kHistBins; b += kT) sh[b] = 0u;
+  for (int b = (int)blockIdx.x * kT + tid; b < kHistBins; b += (int)gridDim.x * kT) e.bin_cur[b] = 0u;
+  if (tid == 0) ds.cut = cut;
+  __syncthreads();
+  // (a warp takes its steps round-robin over the CTAs: a few thousand coefficients already use every SM)
+  const int w0 = warp * (int)gridDim.x + (int)blockIdx.x, nw = kWarps * (int)gridDim.x;
+  const unsigned int cut_bits = __float_as_uint(cut);
+  scan_keys(p, t, cut, queue, w0, nw, [&](unsigned long long key, bool on) {
+    const unsigned int bits = (unsigned int)(key >> 32);
+    const bool in = on && (cut == 0.f || bits < cut_bits);
+    if (in) atomicAdd(&sh[bin_of(bins, bits)], 1u);
+    if (cut > 0.f) {
+      const unsigned int m = __ballot_sync(kFull, in);
+      if (m == 0u) return;
+      unsigned int at = 0u;
+      if (lane == 0) at = atomicAdd(&e.es->surv_count, (unsigned)__popc(m));
+      at = __shfl_sync(kFull, at, 0) + __popc(m & ((1u << lane) - 1u));
+      if (in && at < e.cap_surv) e.surv[at] = key;
+    }
+  });
+  __syncthreads();
+  for (int b = tid; b < kHistBins; b += kT) {
+    const unsigned int v = sh[b];
+    if (v) atomicAdd(&e.hist[b], v);
+  }
+}
+
+// The bin b with before(b) < k <= before(b) + count(b), and the winners before every bin (ds.total < k: there is none).
+__device__ void draw_select(const Engine& e, DrawShared& ds, unsigned int k) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kPer = kHistBins / kT;
+  static_assert(kPer == 8, "two 16-byte loads per thread");
+  const uint4 a = __ldcg(reinterpret_cast<const uint4*>(e.hist) + 2 * tid), b = __ldcg(reinterpret_cast<const uint4*>(e.hist) + 2 * tid + 1);
+  const unsigned int c[kPer] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+  unsigned int mine = 0u;
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) mine += c[u];
+  unsigned int incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned int v = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += v;
+  }
+  __syncthreads();
+  if (lane == 31) ds.wsum[warp] = incl;
+  if (tid == 0) ds.refined = 0;
+  __syncthreads();
+  unsigned int before = 0u, total = 0u;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) { const unsigned int v = ds.wsum[w]; if (w < warp) before += v; total += v; }
+  unsigned int run = before + incl - mine;
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    ds.off[pad(tid * kPer + u)] = run;
+    if (run < k && k <= run + c[u]) { ds.bnd = tid * kPer + u; ds.bnd_count = c[u]; }
+    run += c[u];
+  }
+  if (tid == 0) { ds.off[pad(kHistBins)] = total; ds.total = total; }
+  __syncthreads();
+}
+
+// Upper edge of the boundary bin, as the bits of a binary32 time.
+__device__ __forceinline__ unsigned int boundary_edge(const DrawShared& ds) {
+  const Binning b = binning_of(ds.cut);
+  const unsigned long long x = (unsigned long long)(b.base + (unsigned)ds.bnd + 1u) << b.shift;
+  return x < 0x7f800000ull ? (unsigned int)x : 0x7f800000u;
+}
+
+__device__ __forceinline__ void take_winner(const Engine& e, const DrawShared& ds, const Binning& bins, unsigned long long key) {
+  const unsigned int bin = bin_of(bins, (unsigned int)(key >> 32)), bnd = (unsigned)ds.bnd;
+  if (bin > bnd || (bin == bnd && ds.refined && (key >> (64 - ds.bits)) > ds.prefix)) return;
+  const unsigned int at = ds.off[pad((int)bin)] + atomicAdd(&e.bin_cur[bin], 1u);
+  if (at < (unsigned)e.cap_win) e.win[at] = key;
+}
+
+// (cold) the winners from all J keys
+__device__ __noinline__ void draw_collect_all(const Problem& p, const Engine& e, const DrawShared& ds, unsigned char* sm, unsigned long long t) {
+  const int warp = (int)threadIdx.x >> 5;
+  const Binning bins = binning_of(ds.cut);
+  const unsigned int edge = boundary_edge(ds);
+  uint2* queue = reinterpret_cast<uint2*>(sm + sizeof(unsigned int) * kHistBins) + warp * kQueue;
+  __syncthreads();
+  scan_keys(p, t, edge < 0x7f800000u ? __uint_as_float(edge) : 0.f, queue, warp * (int)gridDim.x + (int)blockIdx.x, kWarps * (int)gridDim.x,
+            [&](unsigned long long key, bool on) { if (on) take_winner(e, ds, bins, key); });
+}
+
+// ... from the keys the scan saved.
+__device__ __forceinline__ void draw_collect(const Engine& e, const DrawShared& ds, bool spare_last) {
+  const unsigned int n_ctas = gridDim.x - (spare_last && gridDim.x > 1 ? 1u : 0u), n_surv = __ldcg(&e.es->surv_count);
+  const Binning bins = binning_of(ds.cut);
+#pragma unroll 1
+  for (unsigned int i = threadIdx.x * n_ctas + blockIdx.x; i < n_surv; i += n_ctas * kT) take_winner(e, ds, bins, __ldcg(e.surv + i));
+}
+
+// Rare: more keys share the boundary bin than there is room for (thousands of tied times).  The grid cuts the bin
+// further, digit by digit, over all J keys.  False: a barrier gave up.
+__device__ __noinline__ bool draw_refine(const Problem& p, const Engine& e, DrawShared& ds, unsigned char* sm, unsigned long long t, unsigned int k, Grid& g) {
+  const int tid = threadIdx.x, warp = tid >> 5;
+  unsigned int* sh = reinterpret_cast<unsigned int*>(sm);
+  uint2* queue = reinterpret_cast<uint2*>(sm + sizeof(unsigned int) * kHistBins) + warp * kQueue;
+  const Binning bins = binning_of(ds.cut);
+  const unsigned int bnd = (unsigned)ds.bnd;
+  unsigned int sure = ds.off[pad((int)bnd)];                       // winners before the keys still in question
+  unsigned long long prefix = 0ull;
+  int bits = 0;
+  if (blockIdx.x == 0 && tid == 0) atomicOr(&p.st->status, STRADS_STATUS_SAMPLER_REFINED);
+  __shared__ int s_digit;
+  __shared__ unsigned int s_before, s_here, s_w[kWarps];
+  for (unsigned int here = ds.bnd_count; here > (unsigned)e.cap_boundary && bits < 64;) {
+    const int width = min(kHistBits, 64 - bits);
+    if (!grid_sync(g)) return false;                     // everybody has read the counts
+    for (int b = (int)blockIdx.x * kT + tid; b < kHistBins; b += (int)gridDim.x * kT) e.hist[b] = 0u;
+    for (int b = tid; b < kHistBins; b += kT) sh[b] = 0u;
+    if (!grid_sync(g)) return false;
+    const int up = 64 - bits - width;
+    scan_keys(p, t, 0.f, queue, warp * (int)gridDim.x + (int)blockIdx.x, kWarps * (int)gridDim.x, [&](unsigned long long key, bool on) {
+      if (on && bin_of(bins, (unsigned int)(key >> 32)) == bnd && (bits == 0 || (key >> (64 - bits)) == prefix))
+        atomicAdd(&sh[(key >> up) & ((1u << width) - 1u)], 1u);
+    });
+    __syncthreads();
+    for (int b = tid; b < kHistBins; b += kT) if (sh[b]) atomicAdd(&e.hist[b], sh[b]);
+    if (!grid_sync(g)) return false;
+    // the digit that holds the k-th key
+    unsigned int c[kHistBins / kT], mine = 0u;
+#pragma unroll
+    for (int u = 0; u < kHistBins / kT; ++u) { c[u] = __ldcg(e.hist + tid * (kHistBins / kT) + u); mine += c[u]; }
+    unsigned int incl = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned int v = __shfl_up_sync(kFull, incl, o);
+      if ((tid & 31) >= o) incl += v;
+    }
+    if ((tid & 31) == 31) s_w[warp] = incl;
+    __syncthreads();
+    unsigned int run = sure + incl - mine;
+    for (int w = 0; w < warp; ++w) run += s_w[w];
+#pragma unroll
+    for (int u = 0; u < kHistBins / kT; ++u) {
+      if (run < k && k <= run + c[u]) { s_digit = tid * (kHistBins / kT) + u; s_before = run; s_here = c[u]; }
+      run += c[u];
+    }
+    __syncthreads();
+    prefix = (prefix << width) | (unsigned long long)s_digit;
+    bits += width;
+    sure = s_before;
+    here = s_here;
+    __syncthreads();
+  }
+  if (tid == 0) { ds.refined = 1; ds.prefix = prefix; ds.bits = bits; }
+  __syncthreads();
+  return true;
+}
+
+// Selection and collection.  Where the selection needs mending (fewer keys than wanted, or too many that tie) the CTAs
+// that see it say so, and all of them meet in draw_mend behind the next barrier.
+__device__ __forceinline__ void draw_gather(const Problem& p, const Engine& e, DrawShared& ds, unsigned long long t, unsigned int k, bool spare_last) {
+  if (spare_last && gridDim.x > 1 && blockIdx.x == gridDim.x - 1) return;
+  draw_select(e, ds, k);
+  if (ds.total < k || ds.bnd_count > (unsigned)e.cap_boundary || (ds.cut > 0.f ? __ldcg(&e.es->surv_count) > e.cap_surv : true)) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) e.es->mend = 1;
+    return;
+  }
+  draw_collect(e, ds, spare_last);
+}
+
+// (cold) by all CTAs.  False: a barrier gave up.
+__device__ __noinline__ bool draw_mend(const Problem& p, const Engine& e, DrawShared& ds, unsigned char* sm, unsigned long long t, unsigned int k, Grid& g) {
+  draw_select(e, ds, k);
+  if (!grid_sync(g)) return false;                       // everybody has read the counts and the flag
+  if (blockIdx.x == 0 && threadIdx.x == 0) e.es->mend = 0;
+  if (ds.total < k) {
+    // the cutoff was too low (the weights collapsed: the end of the first sweep, say): once more, all keys
+    for (int b = (int)blockIdx.x * kT + (int)threadIdx.x; b < kHistBins; b += (int)gridDim.x * kT) e.hist[b] = 0u;
+    if (!grid_sync(g)) return false;
+    draw_scan(p, e, ds, sm, t, false);
+    if (!grid_sync(g)) return false;
+    draw_select(e, ds, k);
+  }
+  if (ds.bnd_count > (unsigned)e.cap_boundary && !draw_refine(p, e, ds, sm, t, k, g)) return false;
+  draw_collect_all(p, e, ds, sm, t);
+  return grid_sync(g);
+}
+
+// ------------------------------------------------------------------------------------------------
+// This round's changes, as every CTA needs them in step 4.
+// ------------------------------------------------------------------------------------------------
+struct ChangeShared {
+  int n_changed;                           // kept coefficients whose key of the next round changed
+  int wsum[kWarps];
+  unsigned long long dmax;                 // bits of the largest |change|
+};
+
+// Shared memory of step 4: the changed keys (old [n_keep], new [n_keep]), then either the moving columns (dense:
+// residual) or the changed keys indexed by bin (draw_rank).
+constexpr int kStage = 4096;               // moving columns staged at a time
+struct Moving { double d[kStage]; long long off[kStage]; };
+struct ChangedByBin { int before[kHistBins + (kHistBins >> 5)]; int head[kHistBins]; unsigned short next[2 * kStage]; };
+
+// The kept coefficients' changes: how many move, the largest, the keys that change (in any order), and for dense X the
+// moving columns in list order.  Returns the number that move.
+template <bool kDense>
+__device__ int gather_changes(const Problem& p, int nk, bool want_keys, unsigned long long* keys, Moving* mv, ChangeShared& cs) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __syncthreads();
+  if (tid == 0) { cs.n_changed = 0; cs.dmax = 0ull; }
+  __syncthreads();
+  const int per = (nk + kT - 1) / kT, a_lo = min(tid * per, nk), a_hi = min(a_lo + per, nk);
+  unsigned long long dmax = 0ull;
+  double d_first = 0.0;
+  int moving = 0;
+  for (int a = a_lo; a < a_hi; ++a) {
+    const int pos = p.kept_pos[a];
+    const double d = p.cand_dbeta64[pos];
+    unsigned long long o = 0ull, w = 0ull;
+    if (want_keys) { o = p.cand_keys[pos]; w = p.cand_keys[p.n_cand + pos]; }
+    if (a == a_lo) d_first = d;
+    moving += d != 0.0;
+    dmax = max(dmax, (unsigned long long)__double_as_longlong(fabs(d)));
+    if (o != w) {
+      const int at = atomicAdd(&cs.n_changed, 1);
+      keys[at] = o;
+      keys[p.n_keep + at] = w;
+    }
+  }
+  int incl = moving;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (!kDense) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dmax = max(dmax, __shfl_xor_sync(kFull, dmax, o));
+    if (lane == 0 && dmax) atomicMax(&cs.dmax, dmax);
+  }
+  if (lane == 31) cs.wsum[warp] = incl;
+  __syncthreads();
+  int before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) { const int v = cs.wsum[w]; if (w < warp) before += v; total += v; }
+  if (kDense) {
+    int rank = before + incl - moving;
+    for (int a = a_lo; a < a_hi && rank < kStage; ++a) {
+      const double d = a == a_lo ? d_first : p.cand_dbeta64[p.kept_pos[a]];
+      if (d == 0.0) continue;
+      mv->d[rank] = d;
+      mv->off[rank] = (long long)p.kept[a] * p.ld;
+      ++rank;
+    }
+    __syncthreads();
+  }
+  return total;
+}
+
+// Winners ranked; with changes, corrected for the kept coefficients' changed priorities (keys[0 .. n_changed) old,
+// keys[p.n_keep ..) new).  Eight lanes per winner.  A key's place among the changed ones: those in lower bins from
+// a prefix sum over the bins, those in its own bin one by one (a list per bin); a plain count while they are few.
+// Leaves the draw's buffers as the next scan expects them.
+constexpr int kFewChanged = 48;
+template <bool kDense>
+__device__ __forceinline__ void draw_rank(const Problem& p, const Engine& e, const DrawShared& ds, const unsigned long long* keys, ChangedByBin* cb, int n_changed,
+                          int nk, int* wsum, int n_rank, int n_prefetch) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, slice = lane & 7;
+  if ((int)blockIdx.x >= n_rank) return;
+  const Binning bins = binning_of(ds.cut);
+  const unsigned int bnd = (unsigned)ds.bnd;
+  unsigned int total = ds.off[pad((int)bnd)] + (ds.refined ? __ldcg(e.bin_cur + bnd) : ds.bnd_count);
+  total = min(total, (unsigned)e.cap_win);
+  const unsigned long long* old_k = keys;
+  const unsigned long long* new_k = keys + p.n_keep;
+  const bool indexed = n_changed > kFewChanged;
+  if (indexed) {
+    __syncthreads();
+    for (int b = tid; b < kHistBins; b += kT) { cb->before[pad(b)] = 0; cb->head[b] = -1; }
+    __syncthreads();
+    for (int i = tid; i < 2 * n_changed; i += kT) {
+      const unsigned long long key = (i & 1) ? new_k[i >> 1] : old_k[i >> 1];
+      const unsigned int b = bin_of(bins, (unsigned int)(key >> 32));
+      atomicAdd(&cb->before[pad((int)b)], (i & 1) ? 1 : -1);
+      cb->next[i] = (unsigned short)atomicExch(&cb->head[b], i);
+    }
+    __syncthreads();
+    constexpr int kPer = kHistBins / kT;
+    int c[kPer], mine = 0;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) { c[u] = cb->before[pad(tid * kPer + u)]; mine += c[u]; }
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    int run = incl - mine;
+    for (int w = 0; w < warp; ++w) run += wsum[w];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) { cb->before[pad(tid * kPer + u)] = run; run += c[u]; }
+    __syncthreads();
+  }
+  const int items = (int)total + (n_changed > 0 ? nk : 0);   // (new keys by place in the kept list: the order of `keys` is each CTA's own)
+  const int shift = 64 - ds.bits;
+  #pragma unroll 1
+  for (int i0 = (warp * n_rank + (int)blockIdx.x) * 4; i0 < items; i0 += kWarps * n_rank * 4) {
+    const int i = i0 + (lane >> 3);
+    const bool fresh = i >= (int)total;
+    unsigned long long key = 0ull;
+    bool on = i < items;
+    if (on && !fresh) key = __ldcg(e.win + i);
+    if (on && fresh) {
+      const int pos = p.kept_pos[i - (int)total];
+      key = p.cand_keys[p.n_cand + pos];
+      on = key != p.cand_keys[pos];
+    }
+    const int j = (int)(key & 0xffffffffull);
+    long long q0 = 0, q1 = 0;                            // CSC: where the column lies, under way meanwhile
+    double n2 = 0.0;
+    if (!kDense && on && slice == 0) { q0 = p.xptr[j]; q1 = p.xptr[j + 1]; n2 = p.n2[j]; }
+    const unsigned int bin = bin_of(bins, (unsigned int)(key >> 32));
+    // (a new key behind the boundary ranks behind all candidates: the winners before it are more than P')
+    // -- unless the winners are all there are
+    const bool behind = fresh && (bin > bnd || (bin == bnd && ds.refined && (key >> shift) > ds.prefix));
+    if (behind && total < (unsigned long long)p.J) on = false;
+    unsigned int first = 0u, count = 0u;
+    if (on) { first = behind ? total : ds.off[pad((int)bin)]; count = behind ? 0u : (bin < bnd ? ds.off[pad((int)bin + 1)] : total) - first; }
+    int below = 0, struck = 0;
+    for (unsigned int k0 = slice; k0 < count; k0 += 64) {
+      unsigned long long v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = k0 + 8 * u < count ? __ldcg(e.win + first + k0 + 8 * u) : ~0ull;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) below += v[u] < key;
+    }
+    if (!indexed) {
+      for (int a = slice; a < n_changed; a += 8) {
+        const unsigned long long o = old_k[a];
+        below -= o < key;
+        struck |= o == key;
+        below += new_k[a] < key;
+      }
+    } else if (on && slice == 0) {
+      below += cb->before[pad((int)bin)];
+      for (int n = cb->head[bin]; n >= 0 && n != 0xffff; n = cb->next[n]) {
+        if (n & 1) {
+          below += new_k[n >> 1] < key;
+        } else {
+          const unsigned long long o = old_k[n >> 1];
+          below -= o < key;
+          struck |= o == key;
+        }
+      }
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+      below += __shfl_xor_sync(kFull, below, o);
+      struck |= __shfl_xor_sync(kFull, struck, o);
+    }
+    const int rank = (int)first + below;
+    if (on && slice == 0 && (fresh || !struck) && (unsigned)rank < (unsigned)p.n_cand) {
+      p.cand[rank] = j;
+      // the columns of the next round's window start towards L2 while this round's changes are applied
+      if (kDense) {
+        if (rank < n_prefetch)
+          asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p.xv + (long long)j * p.ld), "r"((unsigned)((p.N + 3) >> 2) * 16u) : "memory");
+      } else {
+        WalkColumn col;
+        col.q0 = q0; col.n = (int)(q1 - q0); col.j = j; col.n2 = n2; col.unused = 0.0;
+        p.walk_cols[rank] = col;
+        if (rank < n_prefetch) {
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(p.xrow + q0));
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(p.xv + q0));
+          if (q1 - q0 > 32) {
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p.xrow + q0 + 32));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(p.xv + q0 + 32));
+          }
+        }
+      }
+    }
+  }
+  // the next scan's buffers and cutoff (everybody read them before the last barrier)
+  for (int b = (int)blockIdx.x * kT + tid; b < kHistBins; b += (int)gridDim.x * kT) e.hist[b] = 0u;
+  if (blockIdx.x == 0 && tid == 0) {
+    e.es->surv_count = 0u;
+    // twice the boundary, which changes little from round to round; more where few winners let it scatter
+    const unsigned int edge = boundary_edge(ds);
+    e.es->t_cut = edge < 0x7f800000u ? __fmul_rn(p.n_cand < 64 ? 8.0f : 2.0f, __uint_as_float(edge)) : 0.f;
+  }
+}
+
+// ------------------------------------------------------------------------------------------------
+// Would-be changes (Eq. 2): for the candidate at position `pos` with coefficient j, n = ||x_j||^2 and g = x_j^T r.
+// ------------------------------------------------------------------------------------------------
+__device__ __forceinline__ float exponential_of(const Problem& p, unsigned long long t, uint32_t j) {
+  uint32_t w[4];
+  philox4x32_10(j >> 2, (uint32_t)t, (uint32_t)(t >> 32), 0u, (uint32_t)p.seed, (uint32_t)(p.seed >> 32), w);
+  return unit_exponential_rn((j & 2u) ? ((j & 1u) ? w[3] : w[2]) : ((j & 1u) ? w[1] : w[0]));
+}
+
+__device__ __forceinline__ void propose(const Problem& p, int pos, int j, double n, float b_old, float d_old, double g, float E, bool want_keys) {
+  float b_new = b_old;
+  if (n > 0.0) {
+    const double c = step_scale(p);
+    const double z = (double)b_old + c * g / n;
+    const double m = fabs(z) - c * (double)p.lambda / n;
+    b_new = (float)(m <= 0.0 ? 0.0 : (z > 0.0 ? m : -m));
+  }
+  const double d = isfinite(g) ? (double)b_new - (double)b_old : g - g;        // a non-finite product shows as NaN
+  p.cand_bnew[pos] = b_new;
+  p.cand_dbeta64[pos] = d;
+  if (want_keys) {
+    const int mode = weight_mode_of(p.flags);
+    p.cand_keys[pos] = race_key_from(E, d_old, p.eta, (uint32_t)j, mode);
+    p.cand_keys[p.n_cand + pos] = race_key_from(E, (float)fabs(d), p.eta, (uint32_t)j, mode);
+  }
+}
+
+constexpr int kTurn = 32;                  // candidates a CTA handles per turn of step 1 (dense) / 2 (CSC)
+
+struct RoundOutputs { int* cand; int* kept; float* dbeta; int* counts; };
+
+__device__ void commit_changes(const Problem& p, const Engine& e, int nk, int n_moving, const RoundOutputs& out, bool last) {
+  const int tid = threadIdx.x;
+  DeviceState* st = p.st;
+  for (int a = tid * (int)gridDim.x + (int)blockIdx.x; a < p.n_keep; a += kT * (int)gridDim.x) {
+    float d32 = 0.f;
+    int j = -1;
+    if (a < nk) {
+      const int pos = p.kept_pos[a];
+      const double d = p.cand_dbeta64[pos];
+      j = p.kept[a];
+      p.beta[j] = p.cand_bnew[pos];
+      p.delta[j] = (float)fabs(d);
+      d32 = (float)d;
+      if (!isfinite(d)) atomicOr(&st->status, STRADS_STATUS_NONFINITE);
+    }
+    p.dbeta[a] = d32;
+    if (a >= nk) p.kept[a] = -1;
+    if (last && out.kept != nullptr) out.kept[a] = j;
+    if (last && out.dbeta != nullptr) out.dbeta[a] = d32;
+  }
+  if (last && out.cand != nullptr)                       // (the candidates of this round; the draw ahead would overwrite them)
+    for (int i = tid * (int)gridDim.x + (int)blockIdx.x; i < p.n_cand; i += kT * (int)gridDim.x) out.cand[i] = p.cand[i];
+  if (blockIdx.x == 0 && tid == 0) {
+    const int examined = e.es->n_examined;
+    st->counts[0] = p.n_cand; st->counts[1] = examined; st->counts[2] = nk; st->counts[3] = n_moving;
+    if (last && out.counts != nullptr) { out.counts[0] = p.n_cand; out.counts[1] = examined; out.counts[2] = nk; out.counts[3] = n_moving; }
+    st->totals[0] += 1; st->totals[1] += (unsigned)examined; st->totals[2] += (unsigned)nk; st->totals[3] += (unsigned)n_moving;
+    st->round += (unsigned long long)p.part_count;
+  }
+}
+
+// ------------------------------------------------------------------------------------------------
+// Dense, step 1: BF16 copies of the candidates' columns (operands of the Gram's screen), x_c^T r and the would-be
+// changes.  Candidate lo + cta + k * ctas is the CTA's k-th; `group` warps share a column (a function of N alone, so
+// that a product's bits do not depend on the number of candidates).
+//
+// The candidates are scattered over X (a page each), so what counts is how much is under way per SM: the columns come
+// into shared memory by bulk copies, several whole columns ahead, where a loop of register loads had 41 KB in flight and
+// waited for each trip (384 columns of 40 KB: 13.8 us, 640 of 80 KB: 31 us).  Every thread holds its rows of r in
+// registers for the whole step.
+// ------------------------------------------------------------------------------------------------
+struct TurnShared {
+  double dot[kTurn][kWarps];
+  float E[kTurn];
+};
+struct PackBars { unsigned long long full[kWarps]; unsigned int uses[kWarps]; };
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_t limit) {
+  for (uint32_t it = 0; it < limit; ++it) {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+
+// acc += x * r with acc = hi + lo a pair of floats, product and sum errors kept exactly: ~2^-46 of the summed magnitudes.
+__device__ __forceinline__ void dot_step(float x, float r, float& hi, float& lo) {
+  const float pr = __fmul_rn(x, r);
+  const float pe = __fmaf_rn(x, r, -pr);
+  const float s = __fadd_rn(hi, pr);
+  const float bb = __fsub_rn(s, hi);
+  const float se = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(pr, bb));
+  hi = s;
+  lo = __fadd_rn(lo, __fadd_rn(se, pe));
+}
+
+__device__ __forceinline__ unsigned int bf16x2_bits(float a, float b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const unsigned int*>(&v);
+}
+__device__ __forceinline__ float bf16_residue(float x) { return x - __bfloat162float(__float2bfloat16_rn(x)); }
+__device__ __forceinline__ void store_parts(uint2* bhi, uint2* blo, const float4& x, bool low_parts) {
+  *bhi = make_uint2(bf16x2_bits(x.x, x.y), bf16x2_bits(x.z, x.w));
+  if (low_parts) *blo = make_uint2(bf16x2_bits(bf16_residue(x.x), bf16_residue(x.y)), bf16x2_bits(bf16_residue(x.z), bf16_residue(x.w)));
+}
+
+constexpr int kHeld = 10;                  // groups of four rows of r a thread holds: N <= 4 * 512 * 10
+constexpr size_t kPackSmem = 160 * 1024;
+
+__device__ __forceinline__ int pack_group(int n4) {
+  int group = 1;
+  while (group < kWarps && n4 >= group * 2 * 64) group *= 2;            // (at least two 16-byte groups per lane)
+  return group;
+}
+
+// Four rows of r from group gi on; zero past the end.
+__device__ __forceinline__ float4 resid4(const Problem& p, int gi, int n4, int n4_whole) {
+  float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (gi < n4_whole) {
+    r = reinterpret_cast<const float4*>(p.resid)[gi];
+  } else if (gi < n4) {
+    const long long i = (long long)gi << 2;
+    r.x = p.resid[i];
+    if (i + 1 < p.N) r.y = p.resid[i + 1];
+    if (i + 2 < p.N) r.z = p.resid[i + 2];
+  }
+  return r;
+}
+// Rows past N do not exist (the padding of a column may hold anything).
+__device__ __forceinline__ void mask_rows(const Problem& p, int gi, float4& x) {
+  const long long i = (long long)gi << 2;
+  if (i + 1 >= p.N) x.y = 0.f;
+  if (i + 2 >= p.N) x.z = 0.f;
+  x.w = 0.f;
+}
+
+// products: also x_c^T r and what follows from it (false: the copies alone).
+__device__ void dense_pack(const Problem& p, const Engine& e, unsigned char* sm, TurnShared& ts, PackBars& bars, int lo, int hi,
+                           unsigned long long t_next, bool products, bool want_keys, bool low_parts, uint32_t wait_limit) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int cta = (int)blockIdx.x, n_ctas = (int)gridDim.x;
+  const int n4 = (int)((p.N + 3) >> 2), n4_whole = (int)(p.N >> 2);
+  const int group = pack_group(n4), part = warp & (group - 1), grp = warp / group, groups = kWarps / group;
+  const int mine = hi - lo > cta ? (hi - lo - cta + n_ctas - 1) / n_ctas : 0;
+  // columns of a group under way at once
+  const uint32_t col_bytes = (uint32_t)n4 * 16u;
+  int depth = (int)min((size_t)4, kPackSmem / ((size_t)groups * col_bytes));
+  const bool bulk = depth > 0 && n4 <= kHeld * 32 * group;
+  depth = min(depth, kWarps / groups);                   // (a barrier per column under way)
+  const uint32_t slots = smem_u32(sm) + (uint32_t)(grp * depth) * col_bytes;
+  const int at0 = part * 32 + lane, step = 32 * group;
+  float4 rv[kHeld];
+  if (bulk) {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");         // what this CTA last did with the slots is over
+    __syncthreads();
+    if (part == 0 && lane == 0)
+      for (int i = 0; i < depth && grp + i * groups < mine; ++i) {
+        const uint32_t bar = smem_u32(&bars.full[grp * depth + i]);
+        mbar_expect(bar, col_bytes);
+        bulk_load(slots + (uint32_t)i * col_bytes, p.xv + (long long)p.cand[lo + cta + n_ctas * (grp + i * groups)] * p.ld, col_bytes, bar);
+      }
+    if (products) {
+#pragma unroll
+      for (int u = 0; u < kHeld; ++u) rv[u] = u * step + at0 < n4 ? resid4(p, u * step + at0, n4, n4_whole) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
+  int seen = 0;                                          // columns this group has been through
+  for (int k0 = 0; k0 < mine; k0 += kTurn) {
+    const int turn = min(kTurn, mine - k0);
+    int j_own = 0;
+    double n_own = 0.0;
+    float b_own = 0.f, d_own = 0.f;
+    if (products && tid < turn) {                        // gathers for the end of the turn, under way meanwhile
+      j_own = p.cand[lo + cta + n_ctas * (k0 + tid)];
+      n_own = p.n2[j_own]; b_own = p.beta[j_own]; d_own = p.delta[j_own];
+    }
+    if (products && want_keys && warp == kWarps - 1 && lane < turn)
+      ts.E[lane] = exponential_of(p, t_next, (uint32_t)p.cand[lo + cta + n_ctas * (k0 + lane)]);
+    int k = seen * groups + grp - k0;                    // this group's next column, counted from the turn's first
+    for (; k < turn; k += groups, ++seen) {
+      const int a = lo + cta + n_ctas * (k0 + k);
+      uint2* bhi = reinterpret_cast<uint2*>(e.xb + (long long)a * e.xb_pitch);
+      uint2* blo = reinterpret_cast<uint2*>(e.xb + (long long)a * e.xb_pitch + e.lo_off);
+      float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
+      if (bulk) {
+        const int slot = seen % depth, b = grp * depth + slot;
+        const uint32_t ph = (bars.uses[b] + (unsigned)(seen / depth)) & 1u;
+        if (!mbar_wait(smem_u32(&bars.full[b]), ph, wait_limit) && lane == 0) atomicOr(&p.st->status, STRADS_STATUS_WAIT_EXPIRED);
+        const uint32_t src = slots + (uint32_t)slot * col_bytes;
+#pragma unroll
+        for (int u = 0; u < kHeld; ++u) {
+          const int gi = u * step + at0;
+          if (gi >= n4) break;
+          float4 x;
+          asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(src + (uint32_t)gi * 16u) : "memory");
+          if (gi >= n4_whole) mask_rows(p, gi, x);
+          store_parts(bhi + gi, blo + gi, x, low_parts);
+          if (!products) continue;
+          dot_step(x.x, rv[u].x, h0, l0); dot_step(x.y, rv[u].y, h1, l1);
+          dot_step(x.z, rv[u].z, h0, l0); dot_step(x.w, rv[u].w, h1, l1);
+        }
+        const int nxt = grp + (seen + depth) * groups;   // the column that comes into this slot next
+        if (nxt < mine) {
+          if (group > 1) asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "r"(32 * group) : "memory");
+          else __syncwarp();
+          if (part == 0 && lane == 0) {
+            const uint32_t bar = smem_u32(&bars.full[b]);
+            mbar_expect(bar, col_bytes);
+            bulk_load(src, p.xv + (long long)p.cand[lo + cta + n_ctas * nxt] * p.ld, col_bytes, bar);
+          }
+        }
+      } else {                                           // long columns: straight from global memory
+        const float4* xs = reinterpret_cast<const float4*>(p.xv + (long long)p.cand[a] * p.ld);
+        constexpr int kU = 4;
+        for (int g0 = at0; g0 < n4; g0 += kU * step) {
+          float4 x[kU], r[kU];
+#pragma unroll
+          for (int u = 0; u < kU; ++u) x[u] = g0 + u * step < n4 ? __ldg(xs + g0 + u * step) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int u = 0; u < kU; ++u) r[u] = resid4(p, g0 + u * step, n4, n4_whole);
+#pragma unroll
+          for (int u = 0; u < kU; ++u) {
+            const int gi = g0 + u * step;
+            if (gi >= n4) break;
+            if (gi >= n4_whole) mask_rows(p, gi, x[u]);
+            store_parts(bhi + gi, blo + gi, x[u], low_parts);
+            dot_step(x[u].x, r[u].x, h0, l0); dot_step(x[u].y, r[u].y, h1, l1);
+            dot_step(x[u].z, r[u].z, h0, l0); dot_step(x[u].w, r[u].w, h1, l1);
+          }
+        }
+      }
+      if (products) {
+        const double v = warp_sum(((double)h0 + (double)l0) + ((double)h1 + (double)l1));
+        if (lane == 0) ts.dot[k][part] = v;
+      }
+    }
+    if (!products) continue;
+    __syncthreads();
+    if (tid < turn) {
+      const int a = lo + cta + n_ctas * (k0 + tid);
+      double gsum = 0.0;
+      for (int w = 0; w < group; ++w) gsum += ts.dot[tid][w];
+      const bool dormant = (p.flags & STRADS_FLAG_DYNAMIC_DEPS) && b_own == 0.f && d_own == 0.f;      // (coupling_n2)
+      e.norm[a] = dormant ? 0.0 : sqrt(n_own);
+      propose(p, a, j_own, n_own, b_own, d_own, gsum, want_keys ? ts.E[tid] : 0.f, want_keys);
+    }
+    __syncthreads();
+  }
+  if (bulk) {
+    __syncthreads();
+    if (part == 0 && lane == 0)                          // every slot's barrier has completed this many more phases
+      for (int i = 0; i < depth; ++i) bars.uses[grp * depth + i] += (unsigned)((seen - i + depth - 1) / depth);
+  }
+  // the copies are read by bulk tensor copies (another proxy) behind the next barrier
+  asm volatile("fence.proxy.async;" ::: "memory");
+}
+
+// ------------------------------------------------------------------------------------------------
+// Dense, step 2: conflict bits of all candidate pairs on the tensor cores: tiles of 128 rows x 64 or 128 columns of the
+// upper triangle, BF16 operands by TMA (128-byte swizzle) into a ring in shared memory, tcgen05.mma into tensor memory.
+// As in gram_dense_tc.cu the result is a screen: pairs closer to rho than its error bound go to a list and are decided
+// from exact products.
+//   one term    hi.hi: off by at most 2^-8 relative (operands rounded to 8 bits)
+//   three terms hi.hi + hi.lo + lo.hi: off by at most 3 * 2^-18; for short columns, whose correlations scatter so widely
+//               (standard deviation N^-1/2) that the wider band would leave percents of all pairs open
+// What bounds it is bringing operands from L2 to shared memory (~110 GB/s an SM), so K is split until every CTA has a
+// share; the CTAs of a tile leave their partial sums in global memory, wait for one another (they all run at once) and
+// each adds up and thresholds its share of the rows.  A tile of 128 columns reads fewer operand bytes per product, one
+// of 64 leaves half the partial sums: gram_plan takes the cheaper.
+// ------------------------------------------------------------------------------------------------
+constexpr int kRowsT = kGramRows;                        // rows of a tile
+constexpr int kRingBytes = 192 * 1024;
+constexpr int kMaxStages = 4;
+constexpr size_t kGramSmem = (size_t)kRingBytes + 1024;
+constexpr uint32_t kTmemCols = 128;
+
+// A stage holds two blocks of 64 elements of K for both operands: consecutive ones (one term) or the high and the low
+// parts of one (three terms).  Its size depends on the tile's width alone, so there is a set of barriers per width.
+struct GramShared {
+  unsigned long long full[2][kMaxStages], empty[2][kMaxStages], done;
+  uint32_t tmem;
+  int abort_;
+  double norm_a[kRowsT], norm_b[128];
+  float norm_af[kRowsT], norm_bf[128];
+};
+// Phases of the barriers so far (the same in all threads of a CTA).
+struct GramCount { unsigned int stages[2], units; };
+
+__device__ __forceinline__ double engine_band(long long N, int terms) {
+  return terms == 1 ? 1.0 / 128.0 + (double)N * (1.0 / 33554432.0) : 1.0 / 32768.0 + 3.0 * (double)N * (1.0 / 33554432.0);
+}
+
+__device__ __forceinline__ void tma_box(uint32_t dst, const void* tmap, int x, int y, uint32_t bar) {
+  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+               ::"r"(dst), "l"(tmap), "r"(x), "r"(y), "r"(bar) : "memory");
+}
+// K-major operand, rows of 128 bytes with the 128-byte swizzle, 8-row groups 1024 bytes apart.
+__device__ __forceinline__ uint64_t operand_desc(uint32_t saddr) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+__device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+               ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void mma_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tmem_load16(uint32_t addr, uint32_t (&v)[16]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]),
+                 "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]) : "r"(addr) : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void dense_gram(const Problem& p, const Engine& e, const GramPlan& pl, const void* tmap_rows, const void* tmap_cols,
+                                           unsigned char* sm, GramShared& gs, GramCount& gc, int n, int terms, unsigned int* amb_count,
+                                           uint32_t wait_limit) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int units = pl.tiles * pl.split;
+  if ((int)blockIdx.x >= units) return;
+  const int set = pl.cols == 128 ? 1 : 0;
+  const uint32_t a_bytes = kRowsT * 128, b_bytes = (uint32_t)pl.cols * 128, stage_bytes = 2u * (a_bytes + b_bytes);
+  const unsigned int stages = set ? 3u : 4u;
+  const uint32_t ring = (smem_u32(sm) + 1023u) & ~1023u;
+  float* tile_sm = reinterpret_cast<float*>(sm + (ring - smem_u32(sm)));   // the finished tile (no split), over the ring
+  const double rho = (double)p.rho, band = engine_band(p.N, terms);
+  const float quick = (float)((rho - band) * 0.99999);   // |g| below quick ||a|| ||b||: certainly no conflict
+  const int cols4 = pl.cols >> 2, cols_log = set ? 7 : 6;
+
+  for (int unit = (int)blockIdx.x; unit < units; unit += (int)gridDim.x) {
+    const int tile = unit / pl.split, sp = unit - tile * pl.split;
+    int ri = 0, rem = tile, len = pl.col_blocks;
+    const int per_row = kRowsT >> cols_log;
+    while (rem >= len) { rem -= len; len -= per_row; ++ri; }
+    const int row0 = ri * kRowsT, col0 = (ri * per_row + rem) << cols_log;
+    const int s0 = min(pl.steps, sp * pl.per), count = min(pl.steps, s0 + pl.per) - s0;
+    const unsigned int slot0 = gc.stages[set] % stages, ph0 = (gc.stages[set] / stages) & 1u;
+    if (warp == 0) {
+      // ---- operands (one lane) ----
+      if (lane == 0) {
+        unsigned int slot = slot0, ph = ph0;
+        const int x_step = terms == 1 ? 128 : 64, second = terms == 1 ? 64 : (int)e.lo_off;
+        int x = s0 * x_step;
+#pragma unroll 1
+        for (int st = 0; st < count; ++st, x += x_step) {
+          if (!mbar_wait(smem_u32(&gs.empty[set][slot]), ph ^ 1u, wait_limit)) {
+            gs.abort_ = 1; atomicOr(&p.st->status, STRADS_STATUS_WAIT_EXPIRED);
+            break;
+          }
+          const uint32_t bar = smem_u32(&gs.full[set][slot]), dst = ring + slot * stage_bytes;
+          mbar_expect(bar, stage_bytes);
+          tma_box(dst, tmap_rows, x, row0, bar);
+          tma_box(dst + 2 * a_bytes, set ? tmap_rows : tmap_cols, x, col0, bar);
+          tma_box(dst + a_bytes, tmap_rows, x + second, row0, bar);
+          tma_box(dst + 2 * a_bytes + b_bytes, set ? tmap_rows : tmap_cols, x + second, col0, bar);
+          if (++slot == stages) { slot = 0; ph ^= 1u; }
+        }
+      }
+      __syncwarp();
+    } else if (warp == 1) {
+      // ---- multiplication (one lane): FP32 accumulator, both operands BF16 and K-major, M = 128, N = cols ----
+      if (lane == 0) {
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(pl.cols >> 3) << 17) | ((uint32_t)(kRowsT >> 4) << 24);
+        const uint32_t tmem = gs.tmem;
+        unsigned int slot = slot0, ph = ph0;
+        uint32_t acc = 0u;
+#pragma unroll 1
+        for (int st = 0; st < count; ++st) {
+          if (*(volatile int*)&gs.abort_ || !mbar_wait(smem_u32(&gs.full[set][slot]), ph, wait_limit)) {
+            gs.abort_ = 1; atomicOr(&p.st->status, STRADS_STATUS_WAIT_EXPIRED);
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t sb = ring + slot * stage_bytes;
+          const uint64_t a0 = operand_desc(sb), a1 = operand_desc(sb + a_bytes);
+          const uint64_t b0 = operand_desc(sb + 2 * a_bytes), b1 = operand_desc(sb + 2 * a_bytes + b_bytes);
+#pragma unroll
+          for (uint64_t o = 0; o < 8; o += 2) {          // 16 elements of K per instruction
+            mma_f16(tmem, a0 + o, b0 + o, idesc, acc);
+            acc = 1u;
+            if (terms == 1) {
+              mma_f16(tmem, a1 + o, b1 + o, idesc, 1u);
+            } else {
+              mma_f16(tmem, a0 + o, b1 + o, idesc, 1u);
+              mma_f16(tmem, a1 + o, b0 + o, idesc, 1u);
+            }
+          }
+          mma_commit(smem_u32(&gs.empty[set][slot]));
+          if (++slot == stages) { slot = 0; ph ^= 1u; }
+        }
+        mma_commit(smem_u32(&gs.done));
+      }
+      __syncwarp();
+    } else if (tid >= 256) {                             // the norms of the tile, meanwhile
+      const int i = tid - 256;
+      if (i < kRowsT) {
+        const double v = row0 + i < n ? e.norm[row0 + i] : 0.0;
+        gs.norm_a[i] = v; gs.norm_af[i] = (float)v;
+      } else if (i - kRowsT < pl.cols) {
+        const double v = col0 + i - kRowsT < n ? e.norm[col0 + i - kRowsT] : 0.0;
+        gs.norm_b[i - kRowsT] = v; gs.norm_bf[i - kRowsT] = (float)v;
+      }
+    }
+    const bool ok = mbar_wait(smem_u32(&gs.done), gc.units & 1u, wait_limit);
+    if (!ok && lane == 0) { gs.abort_ = 1; atomicOr(&p.st->status, STRADS_STATUS_WAIT_EXPIRED); }
+    __syncwarp();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    gc.stages[set] += (unsigned)count;
+    gc.units += 1u;
+    {
+      // warp w reads the rows of its quarter of tensor memory, 16 columns at a time
+      const int row = (warp & 3) * 32 + lane;
+#pragma unroll 1
+      for (int c = (warp >> 2) * 16; c < pl.cols; c += 64) {
+        uint32_t v[16];
+        if (count > 0) {
+          tmem_load16(gs.tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c, v);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[i] = 0u;
+        }
+        // the tile's place in global memory, or (no split) where the operands were; group q of four columns of row r lies at
+        // q ^ (r & 15) there: no bank conflicts either way
+        if (pl.split > 1) {
+          uint4* dst = reinterpret_cast<uint4*>(e.part + (size_t)unit * (kRowsT * 128) + (row << cols_log) + c);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) __stcg(dst + i, make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
+        } else {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int q = ((c >> 2) + i) ^ (row & 15);
+            *reinterpret_cast<uint4*>(tile_sm + (row << cols_log) + 4 * q) = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+          }
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    }
+    int r_lo = 0, r_hi = kRowsT;
+    __syncthreads();
+    if (pl.split > 1) {
+      if (tid == 0) {                                    // wait for the other parts of the tile
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(e.tile_ticket + tile) : "memory");
+        unsigned int v = 0u;
+        uint32_t it = 0u;
+        do {
+          asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(e.tile_ticket + tile) : "memory");
+        } while (v < (unsigned)pl.split && ++it < wait_limit);
+        if (v < (unsigned)pl.split) atomicOr(&p.st->status, STRADS_STATUS_WAIT_EXPIRED);
+      }
+      r_lo = sp * kRowsT / pl.split;
+      r_hi = (sp + 1) * kRowsT / pl.split;
+      __syncthreads();
+    }
+    const int total = (r_hi - r_lo) * cols4;
+#pragma unroll 1
+    for (int i0 = 0; i0 < total; i0 += kT) {
+      const int i = i0 + tid;
+      const bool in = i < total;
+      const int r = r_lo + ((in ? i : 0) >> (cols_log - 2)), q = i & (cols4 - 1);
+      float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (pl.split > 1) {
+        const float4* src = reinterpret_cast<const float4*>(e.part + (size_t)tile * pl.split * (kRowsT * 128) + (r << cols_log)) + q;
+        for (int k0 = 0; k0 < pl.split; k0 += 4) {       // in split order
+          float4 u[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) u[k] = in && k0 + k < pl.split ? __ldcg(src + (size_t)(k0 + k) * (kRowsT * 128 / 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) { g4.x += u[k].x; g4.y += u[k].y; g4.z += u[k].z; g4.w += u[k].w; }
+        }
+      } else if (in) {
+        g4 = *reinterpret_cast<const float4*>(tile_sm + (r << cols_log) + 4 * (q ^ (r & 15)));
+      }
+      const int a = row0 + r, b0 = col0 + 4 * q;
+      const float gv[4] = {g4.x, g4.y, g4.z, g4.w};
+      const float lim = quick * gs.norm_af[r];
+      bool near = false;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) near |= fabsf(gv[c]) >= lim * gs.norm_bf[4 * q + c];
+      unsigned int hits = 0u, open = 0u;
+      if (in && near) {
+        const double norm_a = gs.norm_a[r];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const double den = norm_a * gs.norm_b[4 * q + c], gx = fabs((double)gv[c]);
+          const bool live = den > 0.0 && b0 + c > a;
+          if (live && fabs(gx - rho * den) <= band * den) open |= 1u << c;
+          else if (live && gx >= rho * den) hits |= 1u << c;
+        }
+      }
+      unsigned int word = hits << ((lane & 7) * 4);      // eight lanes make one word of the row's bits
+      word |= __shfl_xor_sync(kFull, word, 1);
+      word |= __shfl_xor_sync(kFull, word, 2);
+      word |= __shfl_xor_sync(kFull, word, 4);
+      if (in && (lane & 7) == 0 && a < n && (b0 >> 5) < p.mask_words) p.conflict[(size_t)a * p.mask_words + (b0 >> 5)] = word;
+      if (__any_sync(kFull, open)) {                     // too close to call: listed
+        const int cnt = __popc(open);
+        int incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int u = __shfl_up_sync(kFull, incl, o);
+          if (lane >= o) incl += u;
+        }
+        unsigned int at = 0u;
+        if (lane == 31) at = atomicAdd(amb_count, (unsigned)incl);
+        at = __shfl_sync(kFull, at, 31) + (unsigned)(incl - cnt);
+        for (; open; open &= open - 1u, ++at)
+          if (at < (unsigned)p.cap_amb) p.amb_pairs[at] = ((unsigned)a << 16) | (unsigned)(b0 + __ffs((int)open) - 1);
+      }
+    }
+    if (unit + (int)gridDim.x < units) {                 // (the tile in shared memory, before the next operands)
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      if (__syncthreads_or(*(volatile int*)&gs.abort_)) return;
+    }
+  }
+}
+
+// Exact decision of one pair by a warp.
+__device__ __forceinline__ void decide_exactly(const Problem& p, const Engine& e, int a, int b, bool clear) {
+  const int lane = threadIdx.x & 31;
+  const float* xa = p.xv + (long long)p.cand[a] * p.ld;
+  const float* xb = p.xv + (long long)p.cand[b] * p.ld;
+  const int n4 = (int)(p.N >> 2);
+  double acc = 0.0;
+  for (int g = lane; g < n4; g += 32) {
+    const float4 u = __ldg(reinterpret_cast<const float4*>(xa) + g), w = __ldg(reinterpret_cast<const float4*>(xb) + g);
+    acc += (double)u.x * w.x + (double)u.y * w.y + (double)u.z * w.z + (double)u.w * w.w;
+  }
+  const long long i = ((long long)n4 << 2) + lane;
+  if (i < p.N) acc += (double)xa[i] * xb[i];
+  acc = warp_sum(acc);
+  if (lane == 0) {
+    const double den = e.norm[a] * e.norm[b];
+    unsigned int* word = &p.conflict[(long long)a * p.mask_words + (b >> 5)];
+    if (den > 0.0 && fabs(acc) >= (double)p.rho * den) atomicOr(word, 1u << (b & 31));
+    else if (clear) atomicAnd(word, ~(1u << (b & 31)));
+  }
+}
+
+// ------------------------------------------------------------------------------------------------
+// Dense, step 3: first-fit over the conflict bits, by one CTA.  The rows are brought into shared memory by all its
+// threads (a window's all at once, a long list's in pieces); one warp then takes 32 candidates at a time.  Which of them
+// are blocked is one word of every row kept so far, OR-ed over the lanes; their conflicts among themselves are that word
+// of their own rows, settled one kept member at a time while few are in question, else in passes of warp-wide ORs.  One
+// warp issues an instruction every few cycles, so what counts is their number: keeping a whole mask up to date (a
+// row OR-ed in per kept member) took 1 us per 32 candidates.
+// ------------------------------------------------------------------------------------------------
+constexpr size_t kWalkSmem = 190 * 1024;
+
+__device__ __forceinline__ void dense_walk(const Problem& p, const Engine& e, unsigned char* sm, int n, int n_total) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int words = (n + 31) >> 5, quads = (words + 3) >> 2;
+  const int pitch = quads * 4 + 4;                       // words; rows start four banks apart
+  unsigned int* blocked = reinterpret_cast<unsigned int*>(sm);            // [quads * 4] by the members of earlier pieces
+  unsigned int* rows = blocked + quads * 4;
+  int piece = (int)((kWalkSmem / sizeof(unsigned int) - (size_t)quads * 4) / (size_t)(pitch + 2));
+  piece = min(piece & ~31, words * 32);                  // rows in shared memory at a time (at least 64: 512 words a row)
+  int* s_cand = reinterpret_cast<int*>(rows + (size_t)piece * pitch);     // [piece]
+  int* s_row = s_cand + piece;                           // [piece] where the rows of this piece's kept members start
+  __shared__ int s_nk, s_ex, s_done, s_here;
+  __syncthreads();
+  for (int w = tid; w < quads * 4; w += kT) blocked[w] = 0u;
+  if (tid == 0) { s_nk = 0; s_ex = n; s_done = 0; }
+  for (int r0 = 0; r0 < n; r0 += piece) {
+    const int nr = min(piece, n - r0);
+    const int q0 = (r0 >> 5) >> 2;                       // earlier words are not looked at again
+    const int nq = quads - q0;
+    // sixteen lanes per row, 16 bytes each
+    for (int c = tid & 15; c < nq; c += 16)
+      for (int r = tid >> 4; r < nr; r += 8 * (kT / 16)) {
+        uint4 v[8];
+        const uint4* src = reinterpret_cast<const uint4*>(p.conflict + (size_t)(r0 + r) * p.mask_words) + q0 + c;
+        unsigned int* dst = rows + r * pitch + 4 * (q0 + c);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (r + u * (kT / 16) < nr) v[u] = __ldcg(src + (size_t)u * (kT / 16) * (p.mask_words >> 2));
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (r + u * (kT / 16) < nr) *reinterpret_cast<uint4*>(dst + u * (kT / 16) * pitch) = v[u];
+      }
+    for (int i = tid; i < nr; i += kT) s_cand[i] = p.cand[r0 + i];
+    __syncthreads();
+    if (warp == 0) {
+      int nk = s_nk, here = 0;                           // kept so far; of this piece
+      bool done = false;
+      const int w_end = (r0 + nr + 31) >> 5;
+#pragma unroll 1
+      for (int w = r0 >> 5; w < w_end; ++w) {
+        unsigned int hit = lane == 0 ? blocked[w] : 0u;
+        for (int i = lane; i < here; i += 32) hit |= rows[s_row[i] + w];
+        hit = __reduce_or_sync(kFull, hit);
+        const int m = n - w * 32;
+        unsigned int avail = ~hit & (m >= 32 ? kFull : ((1u << m) - 1u));
+        if (avail == 0u) continue;
+        const int at = w * 32 - r0 + lane, row = at * pitch;
+        unsigned int mine = ((avail >> lane) & 1u) ? (rows[row + w] & (lane == 31 ? 0u : (kFull << (lane + 1)))) : 0u;
+        mine &= avail;
+        unsigned int keep = avail;
+        if (__any_sync(kFull, mine != 0u)) {
+          keep = 0u;
+          if (__popc(avail) <= 10) {
+            while (avail) {
+              const int i = __ffs((int)avail) - 1;
+              keep |= 1u << i;
+              avail &= ~((1u << i) | __shfl_sync(kFull, mine, i));
+            }
+          } else {
+            unsigned int fresh = 0u;
+            while (avail) {
+              avail &= ~__reduce_or_sync(kFull, ((fresh >> lane) & 1u) ? mine : 0u);
+              fresh = avail & ~__reduce_or_sync(kFull, ((avail >> lane) & 1u) ? mine : 0u);
+              keep |= fresh;
+              avail &= ~fresh;
+            }
+          }
+        }
+        const int room = p.n_keep - nk;
+        if (__popc(keep) >= room) {                      // stop exactly at P: drop the surplus from the back
+          while (__popc(keep) > room) keep &= ~(1u << (31 - __clz((int)keep)));
+          done = true;
+          if (lane == 0) s_ex = w * 32 + 32 - __clz((int)keep);
+        }
+        if ((keep >> lane) & 1u) {
+          const int r = __popc(keep & ((1u << lane) - 1u));
+          s_row[here + r] = row;
+          p.kept[nk + r] = s_cand[at];
+          p.kept_pos[nk + r] = w * 32 + lane;
+        }
+        nk += __popc(keep); here += __popc(keep);
+        if (done) break;
+        __syncwarp();
+      }
+      if (lane == 0) { s_nk = nk; s_done = done; s_here = here; }
+    }
+    __syncthreads();
+    if (s_done || r0 + piece >= n) break;
+    // the next pieces' words of this piece's kept members
+    for (int w = ((r0 + nr) >> 5) + tid; w < words; w += kT) {
+      unsigned int acc = blocked[w];
+      for (int i = 0; i < s_here; ++i) acc |= rows[s_row[i] + w];
+      blocked[w] = acc;
+    }
+    __syncthreads();
+  }
+  if (tid == 0) {
+    const int nk = s_nk;
+    EngineState* es = e.es;
+    es->n_kept = nk; es->n_examined = s_ex;
+    es->walk_open = nk < p.n_keep && n < n_total ? 1 : 0;
+    // would the window have done?  (the next round goes straight to the whole list if not)
+    if (n == n_total && e.window < n_total) es->skip_window = nk == p.n_keep && s_ex <= e.window ? 0 : 1;
+  }
+}
+
+// ------------------------------------------------------------------------------------------------
+// Dense, step 4: r <- r - sum_a x_a dbeta_a.  The rows are dealt out evenly, a stretch of 16-byte groups per CTA; a thread
+// takes one group of one column at a time (the moving columns dealt out over kT / groups teams), six loads under way,
+// and the teams' FP64 sums are added in a fixed order.  (Blocks of 32 rows left a CTA three of them in turn at N = 10,000,
+// each with its own reduction: 10.7 us.)
+// ------------------------------------------------------------------------------------------------
+__device__ void dense_apply(const Problem& p, const Moving& mv, double* part, int nk, int n_moving) {
+  const int tid = threadIdx.x;
+  const int n4 = (int)((p.N + 3) >> 2), per = (n4 + (int)gridDim.x - 1) / (int)gridDim.x;
+  const int g_lo = (int)blockIdx.x * per, g_hi = min(n4, g_lo + per);
+  if (g_lo >= n4 || n_moving == 0) return;
+  for (int g0 = g_lo; g0 < g_hi; g0 += kT) {             // (one turn up to 4 * 512 rows per CTA)
+    const int width = min(kT, g_hi - g0), teams = kT / width;
+    const int team = tid / width, q = tid - team * width;
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+    const float* x0 = p.xv + ((long long)(g0 + q) << 2);
+    constexpr int kU = 6;
+    auto add = [&](const float4& x, double d) { s0 += (double)x.x * d; s1 += (double)x.y * d; s2 += (double)x.z * d; s3 += (double)x.w * d; };
+    if (team < teams) {
+      const int here = min(n_moving, kStage);
+      for (int a0 = team; a0 < here; a0 += teams * kU) {
+        float4 x[kU];
+        double d[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          const int a = a0 + u * teams;
+          d[u] = a < here ? mv.d[a] : 0.0;
+          x[u] = a < here ? __ldg(reinterpret_cast<const float4*>(x0 + mv.off[a])) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) add(x[u], d[u]);
+      }
+      if (n_moving > kStage) {                           // beyond what was staged: found again in the kept list
+        int seen = 0;
+        for (int a = 0; a < nk; ++a) {
+          const double d = p.cand_dbeta64[p.kept_pos[a]];
+          if (d == 0.0) continue;
+          if (seen >= kStage && seen % teams == team) add(__ldg(reinterpret_cast<const float4*>(x0 + (long long)p.kept[a] * p.ld)), d);
+          ++seen;
+        }
+      }
+      double* at = part + ((size_t)team * width + q) * 4;
+      at[0] = s0; at[1] = s1; at[2] = s2; at[3] = s3;
+    }
+    __syncthreads();
+    const int rows = width * 4;
+    int tpr = 1;                                         // threads per row
+    while (tpr < 32 && tpr * 2 * rows <= kT) tpr *= 2;
+    for (int r0 = 0; r0 < rows; r0 += kT / tpr) {
+      const int r = r0 + tid / tpr, sub = tid & (tpr - 1);
+      double s = 0.0;
+      if (r < rows)
+        for (int t = sub; t < teams; t += tpr) s += part[(size_t)t * rows + r];
+      for (int o = tpr >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+      const long long row = ((long long)g0 << 2) + r;
+      if (sub == 0 && r < rows && row < p.N && s != 0.0) apply_row(p, row, s);
+    }
+    __syncthreads();
+  }
+}
+
+constexpr unsigned int kFewOpen = 48;                    // open pairs the walking CTA decides itself
+
+// (cold) data whose products cluster at rho: every pair exactly
+__device__ __noinline__ void decide_all(const Problem& p, const Engine& e, int n) {
+  const int warp = (int)threadIdx.x >> 5;
+  for (long long i = (long long)warp * gridDim.x + blockIdx.x; i < (long long)n * n; i += (long long)kWarps * gridDim.x) {
+    const int a = (int)(i / n), b = (int)(i - (long long)a * n);
+    if (b > a) decide_exactly(p, e, a, b, true);
+  }
+}
+
+// ------------------------------------------------------------------------------------------------
+// CSC, steps 1 and 2: the window's pairs that share a row, by row buckets as in gram_csc.cu -- but a warp per candidate
+// (its terms in a list of the warp's own in shared memory: no barrier), no conflict bits (the walk works from the list
+// of conflicting pairs or forms rows on demand), and x_c^T r with the same visit to the column.
+// ------------------------------------------------------------------------------------------------
+constexpr int kTerms = 512;                              // terms a candidate may collect
+struct WarpTerms { unsigned long long key[kTerms]; float fa[kTerms], fb[kTerms]; unsigned short order[kTerms]; };
+constexpr size_t kTermsSmem = sizeof(WarpTerms) * kWarps;
+
+// The entries of candidates [0, n) into the buckets of their rows.  Where the columns lie was noted when the candidates
+// were ranked, but for the dependencies dropped at run time (coupling_n2 follows beta and delta).
+__device__ __forceinline__ void csc_enter(const Problem& p, int n, bool buckets) {
+  const int lane = threadIdx.x & 31;
+  const bool dynamic = (p.flags & STRADS_FLAG_DYNAMIC_DEPS) != 0;
+  if (!buckets && !dynamic) return;
+#pragma unroll 1
+  for (int a = ((int)threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x; a < n; a += kWarps * (int)gridDim.x) {
+    const WalkColumn col = p.walk_cols[a];
+    if (dynamic && lane == 0) p.walk_cols[a].n2 = coupling_n2(p, col.j);
+    if (!buckets) continue;
+    for (int q = lane; q < col.n; q += 32) {
+      const int r = __ldg(p.xrow + col.q0 + q);
+      const float v = __ldg(p.xv + col.q0 + q);
+      const unsigned int slot = atomicAdd(&p.bucket_count[r], 1u);
+      if (slot < (unsigned)kBucketSlots) {
+        p.bucket_items[(size_t)r * kBucketSlots + slot] = a;
+        p.bucket_vals[(size_t)r * kBucketSlots + slot] = v;
+      }
+    }
+  }
+}
+
+// (by all CTAs but the last, which walks meanwhile)
+__device__ void csc_clear_buckets(const Problem& p, int n) {
+  const int cta = (int)blockIdx.x, n_ctas = max(1, (int)gridDim.x - 1), lane = threadIdx.x & 31;
+  if (cta >= n_ctas) return;
+  for (int a = ((int)threadIdx.x >> 5) * n_ctas + cta; a < n; a += kWarps * n_ctas) {
+    const WalkColumn col = p.walk_cols[a];
+    for (int q = lane; q < col.n; q += 32) p.bucket_count[__ldg(p.xrow + col.q0 + q)] = 0u;
+  }
+}
+
+// x_c^T r and the would-be changes of candidates [0, count) (kept: of the kept ones), and with `pairs` their inner
+// products with the later candidates that share a row with them.  The CTA's k-th entry is cta + k * ctas; a warp per entry.
+// What bounds it is the chain of dependent far accesses, so each link's loads go out together: the first two
+// entries of every lane, then the residual, the bucket's count and its first four members at once.
+__device__ __forceinline__ void csc_products(const Problem& p, const Engine& e, TurnShared& ts, unsigned char* sm, int count, bool kept, bool pairs,
+                                             unsigned long long t_next, bool want_keys) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int cta = (int)blockIdx.x, n_ctas = (int)gridDim.x;
+  const double rho = (double)p.rho;
+  WarpTerms& wt = reinterpret_cast<WarpTerms*>(sm)[warp];
+  const int mine = count > cta ? (count - cta + n_ctas - 1) / n_ctas : 0;
+#pragma unroll 1
+  for (int k0 = 0; k0 < mine; k0 += kTurn) {
+    const int turn = min(kTurn, mine - k0);
+    int j_own = 0, pos_own = 0;
+    double n_own = 0.0;
+    float b_own = 0.f, d_own = 0.f;
+    if (tid < turn) {                                    // gathers for the end of the turn, under way meanwhile
+      const int a = cta + n_ctas * (k0 + tid);
+      pos_own = kept ? p.kept_pos[a] : a;
+      j_own = kept ? p.kept[a] : p.cand[a];
+      n_own = p.n2[j_own]; b_own = p.beta[j_own]; d_own = p.delta[j_own];
+    }
+    if (want_keys && warp == kWarps - 1 && lane < turn) {
+      const int a = cta + n_ctas * (k0 + lane);
+      ts.E[lane] = exponential_of(p, t_next, (uint32_t)(kept ? p.kept[a] : p.cand[a]));
+    }
+#pragma unroll 1
+    for (int k = warp; k < turn; k += kWarps) {
+      const int a = cta + n_ctas * (k0 + k);
+      const WalkColumn col = p.walk_cols[kept ? p.kept_pos[a] : a];
+      double acc = 0.0;
+      int n_terms = 0;                                   // (the same in all lanes)
+      bool failed = false;
+#pragma unroll 1
+      for (int q0 = 0; q0 < col.n; q0 += 64) {
+        int r[2];
+        float v[2], x[2];
+        unsigned int cnt[2];
+        int4 it[2];
+        float4 vb[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int q = q0 + 32 * h + lane;
+          r[h] = q < col.n ? __ldg(p.xrow + col.q0 + q) : -1;
+          v[h] = q < col.n ? __ldg(p.xv + col.q0 + q) : 0.f;
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          x[h] = r[h] >= 0 ? p.resid[r[h]] : 0.f;
+          cnt[h] = 0u;
+          it[h] = make_int4(-1, -1, -1, -1); vb[h] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (pairs && r[h] >= 0) {
+            cnt[h] = p.bucket_count[r[h]];
+            it[h] = *reinterpret_cast<const int4*>(p.bucket_items + (size_t)r[h] * kBucketSlots);
+            vb[h] = *reinterpret_cast<const float4*>(p.bucket_vals + (size_t)r[h] * kBucketSlots);
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (r[h] >= 0) acc += (double)v[h] * (double)x[h];
+        if (!pairs) continue;
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+          unsigned int c = h ? cnt[1] : cnt[0];
+          const int rr = h ? r[1] : r[0];
+          const float va = h ? v[1] : v[0];
+          int4 i4 = h ? it[1] : it[0];
+          float4 v4 = h ? vb[1] : vb[0];
+          if (c > (unsigned)kBucketSlots) { failed = true; c = 0u; }
+          for (unsigned int i0 = 0; __any_sync(kFull, i0 < c); i0 += 4) {
+            if (i0 > 0 && i0 < c) {
+              i4 = *reinterpret_cast<const int4*>(p.bucket_items + (size_t)rr * kBucketSlots + i0);
+              v4 = *reinterpret_cast<const float4*>(p.bucket_vals + (size_t)rr * kBucketSlots + i0);
+            }
+            const int b4[4] = {i4.x, i4.y, i4.z, i4.w};
+            const float f4[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const bool on = i0 + u < c && b4[u] > a;
+              const unsigned int m = __ballot_sync(kFull, on);
+              if (on) {
+                const int at = n_terms + __popc(m & ((1u << lane) - 1u));
+                if (at < kTerms) {
+                  wt.key[at] = ((unsigned long long)(unsigned)b4[u] << 32) | (unsigned)(q0 + 32 * h + lane);
+                  wt.fa[at] = va;
+                  wt.fb[at] = f4[u];
+                }
+              }
+              n_terms += __popc(m);
+            }
+          }
+        }
+      }
+      acc = warp_sum(acc);
+      if (lane == 0) ts.dot[k][0] = acc;
+      if (!pairs) continue;
+      if (__any_sync(kFull, failed) || n_terms > kTerms) {
+        if (lane == 0) e.es->bucket_failed = 1;
+        continue;
+      }
+      __syncwarp();
+      // in the order of (b, position in a): every term counts the smaller ones
+#pragma unroll 1
+      for (int at = lane; at < n_terms; at += 32) {
+        const unsigned long long own = wt.key[at];
+        int rank = 0;
+#pragma unroll 4
+        for (int s = 0; s < n_terms; ++s) rank += wt.key[s] < own ? 1 : 0;
+        wt.order[rank] = (unsigned short)at;
+      }
+      __syncwarp();
+#pragma unroll 1
+      for (int at = lane; at < n_terms; at += 32) {
+        const unsigned int b = (unsigned int)(wt.key[wt.order[at]] >> 32);
+        if (at > 0 && (unsigned int)(wt.key[wt.order[at - 1]] >> 32) == b) continue;       // not the first term of its b
+        const double n2b = p.walk_cols[b].n2;
+        float dot = 0.f;
+        for (int s = at; s < n_terms; ++s) {
+          const int o = wt.order[s];
+          if ((unsigned int)(wt.key[o] >> 32) != b) break;
+          dot = fmaf(wt.fa[o], wt.fb[o], dot);
+        }
+        const double den = sqrt(col.n2 * n2b);
+        if (den > 0.0 && fabs((double)dot) >= rho * den) {
+          const unsigned int slot = atomicAdd(&e.es->edge_count, 1u);
+          if (slot < (unsigned)p.cap_edges) p.edges[slot] = ((unsigned int)a << 16) | b;
+        }
+      }
+      __syncwarp();
+    }
+    __syncthreads();
+    if (tid < turn) propose(p, pos_own, j_own, n_own, b_own, d_own, ts.dot[tid][0], want_keys ? ts.E[tid] : 0.f, want_keys);
+    __syncthreads();
+  }
+}
+
+// ------------------------------------------------------------------------------------------------
+// CSC, step 4 and the next step 1: the residual.  Contributions are added as 64-bit fixed-point integers (unit 2^-shift, the
+// same bits in any order) and every row with a non-zero accumulator is updated once behind the next barrier.
+// ------------------------------------------------------------------------------------------------
+__device__ __forceinline__ int csc_shift(const Problem& p, unsigned long long dmax_bits, int nk) {
+  const double m = __longlong_as_double((long long)dmax_bits);
+  if (!(m > 0.0) || !isfinite(m)) return INT_MIN;
+  int x = 0;
+  frexp(m * (double)p.st->x_abs_max * (double)max(nk, 1), &x);
+  return 61 - x;
+}
+
+template <typename F>
+__device__ __forceinline__ void for_moving_entries(const Problem& p, int nk, F&& f) {
+  const int lane = threadIdx.x & 31;
+  for (int a = ((int)threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x; a < nk; a += kWarps * (int)gridDim.x) {
+    const double d = p.cand_dbeta64[p.kept_pos[a]];
+    if (d == 0.0) continue;
+    const int j = p.kept[a];
+    const long long q1 = p.xptr[j + 1];
+    for (long long q = p.xptr[j] + lane; q < q1; q += 32) f(q, d);
+  }
+}
+
+__device__ void csc_scatter(const Problem& p, int nk, int shift) {
+  if (shift == INT_MIN) return;
+  for_moving_entries(p, nk, [&](long long q, double d) {
+    const long long fx = __double2ll_rn(ldexp((double)__ldg(p.xv + q) * d, shift));
+    atomicAdd(reinterpret_cast<unsigned long long*>(p.resid_acc + __ldg(p.xrow + q)), (unsigned long long)fx);
+  });
+}
+
+__device__ void csc_apply(const Problem& p, int nk, int n_moving, int shift) {
+  if (shift == INT_MIN) return;
+  // few moving entries against the rows: visit the entries' rows (the first visitor of a row takes its sum), else all rows
+  if ((double)n_moving * (double)p.nnz * 4.0 < (double)p.N * (double)p.J) {
+    for_moving_entries(p, nk, [&](long long q, double) {
+      const int r = __ldg(p.xrow + q);
+      const long long v = (long long)atomicExch(reinterpret_cast<unsigned long long*>(p.resid_acc + r), 0ull);
+      if (v != 0) apply_row(p, r, ldexp((double)v, -shift));
+    });
+    return;
+  }
+  for (long long r = (long long)blockIdx.x * kT + threadIdx.x; r < p.N; r += (long long)gridDim.x * kT) {
+    const long long v = p.resid_acc[r];
+    if (v != 0) {
+      apply_row(p, r, ldexp((double)v, -shift));
+      p.resid_acc[r] = 0;
+    }
+  }
+}
+
+// ------------------------------------------------------------------------------------------------
+// CSC, step 3b: the walk over all candidates with conflict rows on demand (see walk_csc.cu for the scheme: batches of 32
+// unblocked candidates, picked, merged among themselves and decided by every CTA alike; then the kept members against
+// all later unblocked candidates over the grid; one barrier per batch).  Here candidate a belongs to CTA a mod ctas, which
+// brings its candidates' columns into shared memory once per walk: the grid-wide merges then touch no global memory
+// but the mask, where a lane used to fetch a column (two dependent far accesses) per merge -- 18 us in the first batch.
+// ------------------------------------------------------------------------------------------------
+constexpr int kBatch = 32;
+constexpr int kColCap = 64;                              // entries of a batch member's column in shared memory (longer: global)
+constexpr int kMaxWords = STRADS_MAX_CANDIDATES / 32;
+constexpr int kOwn = 128;                                // candidates a CTA can own (more: their columns stay in global memory)
+constexpr int kOwnEntries = 12288;                       // entries of their columns (96 KB)
+static_assert(kMaxWords <= kT, "a mask word per thread");
+
+struct DemandShared {
+  unsigned int blocked[kMaxWords];
+  int brow[kBatch][kColCap + 1];
+  float bval[kBatch][kColCap + 1];
+  int pos[kBatch], col[kBatch], len[kBatch];
+  long long ptr[kBatch];
+  double n2[kBatch];
+  unsigned int conf[kBatch];
+  int wsum[kWarps];
+  unsigned int keep;
+  int m, cursor, kept, examined, done;
+  int own_at[kOwn + 1], own_free[kOwn], n_free;
+  double own_n2[kOwn];
+  int orow[kOwnEntries];
+  float oval[kOwnEntries];
+};
+
+// x_a^T x_b of two ascending row lists, products added in row order; no branch depends on the data.
+__device__ __forceinline__ float merge_dot(const int* ar, const float* av, int na, const int* br, const float* bv, int nb) {
+  float dot = 0.f;
+  int i = 0, k = 0;
+  while (i < na && k < nb) {
+    const int ra = ar[i], rb = br[k];
+    if (ra == rb) dot = fmaf(av[i], bv[k], dot);
+    i += ra <= rb;
+    k += rb <= ra;
+  }
+  return dot;
+}
+
+// The columns of all candidates lie where p.walk_cols says (written behind the last barrier's far side).  False: a
+// barrier gave up.
+__device__ bool csc_walk_on_demand(const Problem& p, const Engine& e, unsigned char* sm, Grid& g) {
+  DemandShared& s = *reinterpret_cast<DemandShared*>(sm);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int cta = (int)blockIdx.x, n_ctas = (int)gridDim.x, n = p.n_cand, W = (n + 31) >> 5;
+  unsigned int* blocked_g = p.walk_blocked;
+  const double rho = (double)p.rho;
+  __syncthreads();
+  for (int w = tid; w < W; w += kT) s.blocked[w] = 0u;
+  if (cta == 0) for (int w = tid; w < W; w += kT) blocked_g[w] = 0u;
+  if (tid == 0) { s.cursor = 0; s.kept = 0; s.examined = n; s.done = 0; }
+  // this CTA's candidates: cta, cta + n_ctas, ...; own_at: where their entries start in orow / oval
+  const int n_own = n > cta ? (n - cta + n_ctas - 1) / n_ctas : 0;
+  const int n_here = min(n_own, kOwn);
+  for (int k0 = 0; k0 < n_here; k0 += 32) {              // (one warp: at most four trips)
+    if (warp == 0) {
+      const int k = k0 + lane;
+      WalkColumn col;
+      col.n = 0; col.n2 = 0.0;
+      if (k < n_here) col = p.walk_cols[cta + k * n_ctas];
+      int incl = col.n;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += v;
+      }
+      const int base = k0 ? s.own_at[k0] : 0;
+      __syncwarp();
+      if (k0 == 0 && lane == 0) s.own_at[0] = 0;
+      if (k < n_here) { s.own_at[k + 1] = base + incl; s.own_n2[k] = col.n2; }
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+  for (int k = warp; k < n_here; k += kWarps) {
+    const int at = s.own_at[k], cnt = s.own_at[k + 1] - at;
+    if (at + cnt > kOwnEntries) continue;
+    const long long q0 = p.walk_cols[cta + k * n_ctas].q0;
+    for (int q = lane; q < cnt; q += 32) { s.orow[at + q] = __ldg(p.xrow + q0 + q); s.oval[at + q] = __ldg(p.xv + q0 + q); }
+  }
+  if (!grid_sync(g)) return false;                       // the mask in global memory is clear
+
+  while (true) {
+    // ---- A: the next <= 32 unblocked candidates at or after the cursor ----
+    {
+      const int cur = s.cursor, first = tid << 5;
+      unsigned int f = 0u;
+      if (tid < W && first + 32 > cur) {
+        f = ~s.blocked[tid];
+        if (first < cur) f &= kFull << (cur - first);
+        if (first + 32 > n) f &= kFull >> (first + 32 - n);
+      }
+      const int c = __popc(f);
+      int incl = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += v;
+      }
+      if (lane == 31) s.wsum[warp] = incl;
+      __syncthreads();
+      int before = 0, total = 0;
+#pragma unroll
+      for (int k = 0; k < kWarps; ++k) { const int v = s.wsum[k]; if (k < warp) before += v; total += v; }
+      for (int idx = before + incl - c; f != 0u && idx < kBatch; f &= f - 1u, ++idx) s.pos[idx] = first + __ffs((int)f) - 1;
+      if (tid == 0) s.m = min(kBatch, total);
+      if (tid < kBatch) s.conf[tid] = 0u;
+    }
+    __syncthreads();
+    const int m = s.m;
+    if (m == 0) break;                                   // list exhausted (the same in every CTA)
+    // ---- B: the members' columns, sixteen threads each, then the pairs among them, one per thread ----
+    {
+      const int q = tid >> 4, l = tid & 15;
+      if (q < m) {
+        const WalkColumn col = p.walk_cols[s.pos[q]];
+        if (l == 0) { s.col[q] = col.j; s.ptr[q] = col.q0; s.len[q] = col.n; s.n2[q] = col.n2; }
+        if (col.n <= kColCap)
+          for (int i = l; i < col.n; i += 16) { s.brow[q][i] = __ldg(p.xrow + col.q0 + i); s.bval[q][i] = __ldg(p.xv + col.q0 + i); }
+      }
+    }
+    __syncthreads();
+    if (tid < m * (m - 1) / 2) {                         // pair number -> (qa, qb), qa < qb
+      int qb = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)tid)) * 0.5f);
+      while (qb * (qb - 1) / 2 > tid) --qb;
+      while ((qb + 1) * qb / 2 <= tid) ++qb;
+      const int qa = tid - qb * (qb - 1) / 2;
+      const int na = s.len[qa], nb = s.len[qb];
+      float dot;
+      if (na <= kColCap && nb <= kColCap) {
+        dot = merge_dot(s.brow[qa], s.bval[qa], na, s.brow[qb], s.bval[qb], nb);
+      } else {
+        const int* ar = na <= kColCap ? s.brow[qa] : p.xrow + s.ptr[qa];
+        const float* av = na <= kColCap ? s.bval[qa] : p.xv + s.ptr[qa];
+        const int* br = nb <= kColCap ? s.brow[qb] : p.xrow + s.ptr[qb];
+        const float* bv = nb <= kColCap ? s.bval[qb] : p.xv + s.ptr[qb];
+        dot = merge_dot(ar, av, na, br, bv, nb);
+      }
+      const double den = sqrt(s.n2[qa] * s.n2[qb]);
+      if (den > 0.0 && fabs((double)dot) >= rho * den) atomicOr(&s.conf[qa], 1u << qb);
+    }
+    __syncthreads();
+    // ---- C: decide the batch (warp 0, lane = member; the same in every CTA) ----
+    if (warp == 0) {
+      const unsigned int mine = s.conf[lane];            // conflicts with later members only
+      unsigned int und = m >= 32 ? kFull : ((1u << m) - 1u), keep = 0u, fresh = 0u;
+      for (int pass = 0; pass < kBatch && und != 0u; ++pass) {
+        if (pass > 0) und &= ~__reduce_or_sync(kFull, ((fresh >> lane) & 1u) ? mine : 0u);
+        fresh = und & ~__reduce_or_sync(kFull, ((und >> lane) & 1u) ? mine : 0u);
+        keep |= fresh;
+        und &= ~fresh;
+      }
+      const int nk = s.kept, room = p.n_keep - nk;
+      bool done = false;
+      if (__popc(keep) >= room) {                        // stop exactly at P: drop the surplus from the back
+        while (__popc(keep) > room) keep &= ~(1u << (31 - __clz((int)keep)));
+        done = true;
+      }
+      if (cta == 0 && ((keep >> lane) & 1u)) {
+        const int r = nk + __popc(keep & ((1u << lane) - 1u));
+        p.kept[r] = s.col[lane];
+        p.kept_pos[r] = s.pos[lane];
+      }
+      if (lane == 0) {
+        s.keep = keep;
+        s.kept = nk + __popc(keep);
+        s.cursor = s.pos[m - 1] + 1;
+        s.n_free = 0;
+        if (done) { s.examined = s.pos[31 - __clz((int)keep)] + 1; s.done = 1; }
+      }
+    }
+    __syncthreads();
+    if (s.done) break;                                   // P kept: what they block no longer matters
+    // ---- D: the kept members against this CTA's later unblocked candidates ----
+    {
+      const unsigned int keep = s.keep;
+      const int n_new = __popc(keep), first_pos = s.pos[__ffs((int)keep) - 1];
+      for (int k0 = 0; k0 < n_own; k0 += kOwn) {         // (a turn of at most kOwn candidates; one turn as a rule)
+        if (k0 > 0) { __syncthreads(); if (tid == 0) s.n_free = 0; __syncthreads(); }
+        if (tid < kOwn && k0 + tid < n_own) {
+          const int b = cta + (k0 + tid) * n_ctas;
+          if (b > first_pos && !((s.blocked[b >> 5] >> (b & 31)) & 1u)) s.own_free[atomicAdd(&s.n_free, 1)] = k0 + tid;
+        }
+        __syncthreads();
+        const int pairs = s.n_free * n_new;
+        for (int x = tid; x < pairs; x += kT) {
+          const int k = s.own_free[x / n_new];
+          unsigned int rest = keep;
+          for (int y = x - (x / n_new) * n_new; y > 0; --y) rest &= rest - 1u;
+          const int q = __ffs((int)rest) - 1, b = cta + k * n_ctas;
+          if (s.pos[q] >= b) continue;                   // the member comes later in the list: it cannot block b
+          const int na = s.len[q];
+          float dot;
+          double n2b;
+          if (k < n_here && s.own_at[k + 1] <= kOwnEntries && na <= kColCap) {
+            n2b = s.own_n2[k];
+            dot = merge_dot(s.brow[q], s.bval[q], na, s.orow + s.own_at[k], s.oval + s.own_at[k], s.own_at[k + 1] - s.own_at[k]);
+          } else {
+            const WalkColumn cb = p.walk_cols[b];
+            n2b = cb.n2;
+            const int* ar = na <= kColCap ? s.brow[q] : p.xrow + s.ptr[q];
+            const float* av = na <= kColCap ? s.bval[q] : p.xv + s.ptr[q];
+            dot = merge_dot(ar, av, na, p.xrow + cb.q0, p.xv + cb.q0, cb.n);
+          }
+          const double den = sqrt(s.n2[q] * n2b);
+          if (den > 0.0 && fabs((double)dot) >= rho * den) atomicOr(&blocked_g[b >> 5], 1u << (b & 31));
+        }
+      }
+    }
+    if (!grid_sync(g)) return false;
+    for (int w = tid; w < W; w += kT) s.blocked[w] = __ldcg(blocked_g + w);
+    __syncthreads();
+  }
+  if (cta == 0 && tid == 0) {
+    EngineState* es = e.es;
+    es->n_kept = s.kept; es->n_examined = s.examined; es->walk_open = 0;
+    if (e.window < n) es->skip_window = s.kept == p.n_keep && s.examined <= e.window ? 0 : 1;
+  }
+  return true;
+}
+
+// ------------------------------------------------------------------------------------------------
+// The rounds.  Every step is called from one place, so that the loop's code stays within the instruction cache (with each
+// variant of a round written out, 750 KB of it, every step ran from L2 and took two to three times as long).
+// ------------------------------------------------------------------------------------------------
+struct Pending { int nk, n_moving, shift; };             // CSC: the residual's changes of the last round, still in the accumulators
+
+struct EngineMaps { CUtensorMap rows, cols; };           // boxes of 64 elements x 128 and 64 candidates
+
+template <bool kDense>
+__global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Problem p, const __grid_constant__ Engine e,
+                                                  const __grid_constant__ EngineMaps maps, int n_rounds, int have_list, int draw_next,
+                                                  RoundOutputs out) {
+  extern __shared__ __align__(1024) unsigned char sm[];
+  __shared__ DrawShared ds;
+  __shared__ TurnShared ts;
+  __shared__ ChangeShared cs;
+  __shared__ __align__(8) PackBars pb;
+  __shared__ __align__(16) GramShared gs;
+  __shared__ int s_kept, s_examined;
+  // Copies for the functions that are called rarely and not inlined: a reference to the parameters themselves would make
+  // every access to them, in the hot code too, a load from memory.
+  __shared__ Problem sp;
+  __shared__ Engine se;
+  // after a wait that expired nothing runs on this handle until strads_recover (CTAs that disagree on the bit only
+  // meet a barrier that gives up)
+  if (p.st->status & STRADS_STATUS_WAIT_EXPIRED) return;
+  const int tid = threadIdx.x, warp = tid >> 5, cta = (int)blockIdx.x, n_ctas = (int)gridDim.x;
+  if (tid == 0) { sp = p; se = e; }
+  __syncthreads();
+  const bool walker = cta == n_ctas - 1;                 // the CTA that walks
+  const uint32_t limit = p.wait_limit ? p.wait_limit : 1u << 24;
+  GramCount gc = {};
+  if (kDense) {
+    if (tid == 0) {
+      for (int i = 0; i < kWarps; ++i) { mbar_init(smem_u32(&pb.full[i]), 1); pb.uses[i] = 0u; }
+      for (int s = 0; s < 2; ++s)
+        for (int i = 0; i < kMaxStages; ++i) { mbar_init(smem_u32(&gs.full[s][i]), 1); mbar_init(smem_u32(&gs.empty[s][i]), 1); }
+      mbar_init(smem_u32(&gs.done), 1);
+      gs.abort_ = 0;
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (tid < 32) {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&gs.tmem)), "r"(kTmemCols) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    }
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  }
+  Grid g;
+  g.count = &e.es->bar_count; g.target = 0u; g.n = gridDim.x; g.limit = p.wait_limit ? p.wait_limit : kSpinLimit; g.status = &p.st->status;
+  EngineState* es = e.es;
+  unsigned long long t = p.st->round;
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(sm);
+  unsigned char* behind_keys = sm + (e.n_list > 0 ? 2 * sizeof(unsigned long long) * (size_t)p.n_keep : 0);
+  Moving* mv = reinterpret_cast<Moving*>(behind_keys);
+  double* part = reinterpret_cast<double*>(behind_keys + sizeof(Moving));
+  ChangedByBin* cb = reinterpret_cast<ChangedByBin*>(behind_keys + (kDense ? sizeof(Moving) + sizeof(double) * 4 * kT : 0));
+  const bool no_filter = (p.flags & STRADS_FLAG_NO_FILTER) != 0;
+  const int n_total = p.n_cand;
+  Pending last;
+  last.nk = 0; last.n_moving = 0; last.shift = INT_MIN;
+  unsigned int attempts = 0u;                            // dense: Gram passes so far
+  bool have = have_list != 0, ok = true;
+  int left = n_rounds;
+  // One trip per round, and one for a draw that nothing was drawn ahead for (real: false).  CSC ends with a trip that only
+  // applies the last round's changes to the residual.
+  while (true) {
+    if (!kDense) {
+      csc_apply(p, last.nk, last.n_moving, last.shift);
+      last.shift = INT_MIN;
+    }
+    if (left == 0) break;
+    const bool real = have, final_round = real && left == 1;
+    const bool draws = !real || (e.n_list > 0 && (!final_round || draw_next));
+    const unsigned long long td = real ? t + 1 : t;      // the round drawn for
+    const unsigned int k = real ? (unsigned)e.n_list : (unsigned)n_total;
+    bool scanned = !draws, collected = !draws;
+    bool spare = kDense && real && !no_filter;           // the last CTA leaves the draw's winners to the others
+    int n = no_filter ? p.n_keep : e.window, packed = 0, terms = p.N <= 2048 ? 3 : 1;
+    bool window = true, products = true;
+    if (kDense) {
+      if (n < n_total && es->skip_window && !no_filter) n = n_total;
+    } else {
+      window = no_filter || (p.bucket_count != nullptr && !(n < n_total && es->skip_window) && t >= es->avoid_until);
+      if (real) csc_enter(p, window ? n : n_total, window && !no_filter);
+    }
+    // ---- steps 1 to 3, once more over all candidates where a window does not do ----
+    while (true) {
+      GramPlan pl = e.plan[n == n_total ? 1 : 0];
+      if (kDense && real) {
+        if (!no_filter) {
+          if (!products) pl = gram_plan(p.N, n, terms, n_ctas);           // (the screen over again with three terms)
+          for (int i = cta * kT + tid; i < pl.tiles; i += n_ctas * kT) e.tile_ticket[i] = 0u;
+        }
+        dense_pack(p, e, sm, ts, pb, packed, n, t + 1, products, draws, terms == 3, limit);
+      }
+      if (!scanned) { draw_scan(p, e, ds, sm, td, true); scanned = true; }
+      if (kDense) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // (the Gram's operands come in over it)
+      if (!(ok = grid_sync(g))) break;
+      if (kDense && real && !no_filter) {
+        unsigned int* amb = &es->amb_count[attempts & 1u];
+        if (cta == 0 && tid == 0) es->amb_count[(attempts + 1u) & 1u] = 0u;
+        ++attempts;
+        dense_gram(p, e, pl, &maps.rows, &maps.cols, sm, gs, gc, n, terms, amb, limit);
+        if (!(ok = grid_sync(g, p.stall != 0))) break;
+        const unsigned int open = *amb;
+        if (open > (unsigned)p.cap_amb && terms == 1) {
+          // more pairs open than the list holds: again with three terms
+          if (cta == 0 && tid == 0) atomicOr(&p.st->status, STRADS_STATUS_GRAM_FALLBACK);
+          terms = 3; packed = 0; products = false;
+          continue;
+        }
+        const bool listed = open <= (unsigned)p.cap_amb;
+        if (!listed) {
+          if (cta == 0 && tid == 0) atomicOr(&p.st->status, STRADS_STATUS_GRAM_FALLBACK);
+          decide_all(sp, se, n);
+        }
+        if (listed && open > 0u && (open > kFewOpen || walker)) {
+          const unsigned int first = open > kFewOpen ? (unsigned)(warp * n_ctas + cta) : (unsigned)warp;
+          for (unsigned int i = first; i < open; i += open > kFewOpen ? (unsigned)(kWarps * n_ctas) : (unsigned)kWarps) {
+            const unsigned int pr = __ldcg(p.amb_pairs + i);
+            decide_exactly(p, e, (int)(pr >> 16), (int)(pr & 0xffffu), false);
+          }
+          __threadfence();
+        }
+        if (open > kFewOpen && !(ok = grid_sync(g))) break;
+        if (walker) dense_walk(p, e, sm, n, n_total);
+      }
+      if (no_filter && real && walker) {                 // keep the first P
+        for (int i = tid; i < p.n_keep; i += kT) { p.kept[i] = p.cand[i]; p.kept_pos[i] = i; }
+        if (tid == 0) { es->n_kept = p.n_keep; es->n_examined = p.n_keep; es->walk_open = 0; }
+      }
+      // the winners of the draw: by every CTA but the one that walks; CSC in step 3 as well, unless there is none
+      const bool csc_window = !kDense && real && window && !no_filter;
+      if (!collected && !csc_window) { draw_gather(p, e, ds, td, k, spare); collected = true; }
+      if (!kDense && real) {
+        if (!window) {
+          if (!(ok = csc_walk_on_demand(p, e, sm, g))) break;
+          if (!(ok = grid_sync(g))) break;
+        }
+        csc_products(p, e, ts, sm, window ? n : es->n_kept, !window, csc_window, t + 1, draws);
+      }
+      if (!(ok = grid_sync(g))) break;
+      if (!real || no_filter) break;
+      if (!kDense) {
+        if (!window) break;
+        if (walker) {
+          const unsigned int edges = es->edge_count;
+          const int failed = es->bucket_failed;
+          if (tid == 0) { s_kept = 0; s_examined = n; }
+          __syncthreads();
+          bool settled = !failed && edges <= (unsigned)p.cap_edges;
+          if (settled) settled = walk_from_pair_list<kT>(p, p.cand, n, edges, sm, p.kept, &s_kept, &s_examined);
+          __syncthreads();
+          if (tid == 0) {
+            es->n_kept = s_kept; es->n_examined = s_examined;
+            es->walk_open = !settled || (s_kept < p.n_keep && n < n_total) ? 1 : 0;
+            // after an overflow the buckets are left alone: for a round, then twice as long after every further one, to 64
+            if (!settled) es->avoid_until = t + (1ull << es->streak);
+            es->streak = settled ? 0 : min(es->streak + 1, 6);
+            es->bucket_failed = 0; es->edge_count = 0u;
+          }
+        }
+        csc_clear_buckets(p, n);
+        if (!collected) { draw_gather(p, e, ds, td, k, true); collected = true; spare = true; }
+        if (!(ok = grid_sync(g))) break;
+        if (!es->walk_open) break;
+        csc_enter(p, n_total, false);
+        window = false;
+      } else {
+        if (!es->walk_open) break;
+        packed = n; n = n_total; products = true;
+        if (p.N > 2048) terms = 1;
+      }
+    }
+    if (!ok) break;
+    if (draws && es->mend && !(ok = draw_mend(sp, se, ds, sm, td, k, g))) break;
+    // ---- step 4 ----
+    int n_changed = 0, nk = 0;
+    const int n_next = no_filter ? p.n_keep : (e.window < n_total && es->skip_window ? n_total : e.window);   // looked at first
+    if (real) {
+      nk = es->n_kept;
+      const int n_moving = gather_changes<kDense>(p, nk, draws, keys, mv, cs);
+      n_changed = cs.n_changed;
+      commit_changes(p, e, nk, n_moving, out, final_round);
+      last.nk = nk; last.n_moving = n_moving;
+      if (!kDense) {
+        last.shift = csc_shift(p, cs.dmax, nk);
+        csc_scatter(p, nk, last.shift);
+      }
+      --left;
+      ++t;
+    }
+    if (draws) draw_rank<kDense>(p, e, ds, keys, cb, n_changed, nk, cs.wsum, spare ? max(1, n_ctas - 1) : n_ctas, n_next);
+    if (kDense && real) dense_apply(p, *mv, part, nk, last.n_moving);
+    have = draws;
+    if (left == 0 && kDense) break;
+    if (!(ok = grid_sync(g))) break;
+  }
+  if (kDense) {
+    __syncthreads();
+    if (tid < 32) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(gs.tmem), "r"(kTmemCols) : "memory");
+    }
+  }
+  if (!ok) return;
+  if (tid == 0 && atomicInc(&e.es->exit_count, gridDim.x - 1u) == gridDim.x - 1u) {
+    e.es->bar_count = 0u;
+    if (kDense) { e.es->amb_count[0] = 0u; e.es->amb_count[1] = 0u; }
+  }
+}
+
+size_t smem_of(bool dense, int n_keep, bool ahead, int n_cand) {
+  size_t need = kScanSmem;
+  const size_t keys = ahead ? 2 * sizeof(unsigned long long) * (size_t)n_keep : 0;
+  auto at_least = [&](size_t v) { if (need < v) need = v; };
+  at_least(keys);
+  if (dense) {
+    at_least(kPackSmem);
+    at_least(kGramSmem);
+    at_least(kWalkSmem);
+    at_least(keys + sizeof(Moving) + sizeof(double) * 4 * kT + (ahead ? sizeof(ChangedByBin) : 0));
+  } else {
+    at_least(kTermsSmem);
+    at_least(sizeof(DemandShared));
+    at_least(walk_pairs_smem(n_cand, 8192));
+    if (ahead) at_least(keys + sizeof(ChangedByBin));
+  }
+  return need;
+}
+
+}  // namespace
+
+size_t engine_smem(const Problem& p, bool ahead) { return smem_of(p.layout == STRADS_DENSE_COLMAJOR, p.n_keep, ahead, p.n_cand); }
+
+// The grid: one CTA per SM.  (A single thread-block cluster of 16 CTAs for small problems, whose barriers cost a fifth, was
+// slower all the same: c1 41.6 us per round instead of 36.6, every CTA having nine times the candidates to go through.)
+cudaError_t prepare_engine(const Problem& p, Engine& e) {
+  const bool dense = p.layout == STRADS_DENSE_COLMAJOR;
+  const void* fn = dense ? reinterpret_cast<const void*>(k_engine<true>) : reinterpret_cast<const void*>(k_engine<false>);
+  int dev = 0, most = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err != cudaSuccess) return err;
+  if ((err = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return err;
+  cudaFuncAttributes a;
+  if ((err = cudaFuncGetAttributes(&a, fn)) != cudaSuccess) return err;
+  // the largest any handle can need
+  if ((err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes)) != cudaSuccess) return err;
+  e.grid = p.sm_count;
+  if (dense) {
+    const int terms = p.N <= 2048 ? 3 : 1;
+    e.plan[0] = gram_plan(p.N, e.window, terms, e.grid);
+    e.plan[1] = gram_plan(p.N, p.n_cand, terms, e.grid);
+  }
+  return cudaSuccess;
+}
+
+cudaError_t encode_engine_maps(const Problem& p, const Engine& e, void* out) {
+  static_assert(sizeof(EngineMaps) == 256, "two tensor maps");
+  EngineMaps* maps = static_cast<EngineMaps*>(out);
+  void* fn = nullptr;
+  cudaDriverEntryPointQueryResult qres;
+  const cudaError_t err = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
+  if (err != cudaSuccess) return err;
+  if (fn == nullptr || qres != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
+  using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  const cuuint64_t dims[2] = {(cuuint64_t)e.xb_pitch, (cuuint64_t)p.n_cand}, strides[1] = {(cuuint64_t)e.xb_pitch * 2};
+  const cuuint32_t estr[2] = {1, 1};
+  for (int i = 0; i < 2; ++i) {
+    const cuuint32_t box[2] = {64, i ? 64u : (cuuint32_t)kRowsT};
+    const CUresult r = reinterpret_cast<EncodeFn>(fn)(i ? &maps->cols : &maps->rows, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, e.xb, dims, strides, box,
+                                                      estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                                      CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t launch_engine(const Problem& p, const Engine& e, const void* maps, int n_rounds, bool have_list, bool draw_next,
+                          const strads_round_out_t* out, cudaStream_t s) {
+  const bool dense = p.layout == STRADS_DENSE_COLMAJOR;
+  const EngineMaps& tm = *static_cast<const EngineMaps*>(maps);
+  RoundOutputs o = {};
+  if (out != nullptr) { o.cand = out->cand; o.kept = out->kept; o.dbeta = out->dbeta; o.counts = out->counts; }
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)e.grid); cfg.blockDim = dim3(kT); cfg.dynamicSmemBytes = engine_smem(p, e.n_list > 0); cfg.stream = s;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  const int have = have_list ? 1 : 0, next = draw_next ? 1 : 0;
+  return dense ? cudaLaunchKernelEx(&cfg, k_engine<true>, p, e, tm, n_rounds, have, next, o)
+               : cudaLaunchKernelEx(&cfg, k_engine<false>, p, e, tm, n_rounds, have, next, o);
+}
+
+}  // namespace strads

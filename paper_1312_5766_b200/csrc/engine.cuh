@@ -1,0 +1,87 @@
+// Whole rounds in one cooperative launch (engine.cu): what the kernel keeps between rounds, and its launchers.
+#pragma once
+#include "strads_internal.cuh"
+
+namespace strads {
+
+// Device-resident state of the round engine, in the workspace.  Zero before the first launch.
+struct EngineState {
+  unsigned int bar_count;       // grid barrier: arrivals of the launch in flight
+  unsigned int exit_count;      // CTAs of the launch that have left
+  unsigned int surv_count;      // draw: keys the guided scan saved (append cursor)
+  float t_cut;                  // draw: cutoff for the next scan (0: none)
+  unsigned int amb_count[2];    // dense Gram: pairs the screen left open (two counters, in turns)
+  unsigned int edge_count;      // CSC Gram: conflicting pairs listed
+  int bucket_failed;            // CSC Gram: a bucket or a candidate's list of terms overflowed in this round
+  int skip_window;              // the last whole-list walk shows that the window would have been too short again
+  int n_kept, n_examined;       // result of the walk
+  int walk_open;                // the walk could not finish: fewer than P kept inside a window, or chains too long
+  int mend;                     // a draw's selection has to be mended
+  int streak;                   // CSC: attempts with the row buckets in a row that overflowed (or left the walk open)
+  int pad;
+  unsigned long long avoid_until;   // CSC: first round in which they are tried again
+};
+
+// How the pairs of a list are cut into tiles of the dense Gram: kGramRows x cols, K in stages of 128 elements (64 with three
+// terms), `split` CTAs sharing a tile with `per` stages each.
+constexpr int kGramRows = 128;
+struct GramPlan { int cols, col_blocks, tiles, split, steps, per; };
+__host__ __device__ inline GramPlan gram_plan(long long N, int n, int terms, int n_ctas) {
+  GramPlan best = {};
+  float cost = 0.f;
+  const int k = terms == 1 ? 128 : 64;
+  const int row_blocks = (n + kGramRows - 1) / kGramRows, steps = (int)((N + k - 1) / k);
+  for (int cols = 64; cols <= 128; cols += 64) {
+    GramPlan pl;
+    const int per_row = kGramRows / cols;
+    pl.cols = cols;
+    pl.col_blocks = (n + cols - 1) / cols;
+    // row block i meets the column blocks from i * per_row on
+    pl.tiles = row_blocks * pl.col_blocks - per_row * row_blocks * (row_blocks - 1) / 2;
+    pl.steps = steps;
+    pl.split = n_ctas / pl.tiles;
+    if (pl.split > 16) pl.split = 16;
+    if (pl.split > steps) pl.split = steps;
+    if (pl.split < 1) pl.split = 1;
+    pl.per = (steps + pl.split - 1) / pl.split;
+    pl.split = (steps + pl.per - 1) / pl.per;             // (no part without a stage)
+    const int waves = (pl.tiles * pl.split + n_ctas - 1) / n_ctas;
+    // microseconds: 0.35 (64 columns) or 0.45 (128) a stage, and what sharing a tile costs
+    const float c = (float)waves * ((float)pl.per * (cols == 64 ? 0.35f : 0.45f) + (pl.split > 1 ? (cols == 64 ? 2.5f : 3.f) : 0.5f));
+    if (cols == 64 || c < cost) { cost = c; best = pl; }
+  }
+  return best;
+}
+
+// What a launch needs beside the Problem.
+struct Engine {
+  EngineState* es;
+  unsigned int* hist;           // [kHistBins] zero between scans
+  unsigned int* bin_cur;        // [kHistBins] append cursors of the winners' groups
+  unsigned long long* win;      // [cap_win] the winners of a draw, grouped by bin
+  int cap_win, cap_boundary;
+  unsigned long long* surv;     // [cap_surv] keys below the scan's cutoff
+  unsigned int cap_surv;
+  int n_list;                   // winners a draw made one round ahead collects: P' + P (at most J); 0: draws are made at the round's start
+  int window;                   // candidates of the first attempt
+  // dense
+  unsigned short* xb;           // [n_cand][xb_pitch] BF16 high parts of the candidate columns, then (at lo_off) the low parts
+  long long xb_pitch, lo_off;   // elements
+  double* norm;                 // [n_cand] norms of the candidates' columns as the rho test sees them
+  float* part;                  // [ctas][128 * 128] partial Gram tiles
+  unsigned int* tile_ticket;    // [tiles of 64 x 64] zero between rounds
+  GramPlan plan[2];             // for the window and for the whole list
+  int grid;                     // CTAs of the launch
+};
+
+
+cudaError_t prepare_engine(const Problem& p, Engine& e);     // grid and plans (window and n_list are set)
+size_t engine_smem(const Problem& p, bool ahead);
+// n_rounds rounds; have_list: this round's candidates are in p.cand; draw_next: leave the next round's there.
+// out (device pointers or null): the last round's candidates, kept list, changes and counts.
+// Tensor maps over the BF16 copies (dense; two of 128 bytes, 64-byte aligned).
+cudaError_t encode_engine_maps(const Problem& p, const Engine& e, void* out_256_bytes);
+cudaError_t launch_engine(const Problem& p, const Engine& e, const void* maps, int n_rounds, bool have_list, bool draw_next,
+                          const strads_round_out_t* out, cudaStream_t s);
+
+}  // namespace strads

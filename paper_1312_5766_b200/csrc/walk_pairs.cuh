@@ -30,8 +30,8 @@ __host__ __device__ inline size_t walk_pairs_smem(int n_cand, unsigned int n_edg
 // p.kept_pos[0 .. *n_kept) hold the kept coefficients and their positions in the list, and *n_examined the
 // position after the P-th kept one (left alone when fewer than P are kept).  n_kept / n_examined: shared memory.
 template <int kNT>
-__device__ bool walk_from_pair_list(const Problem& p, const int* __restrict__ cand, int n_cand, unsigned int n_edges,
-                                    unsigned char* sm, int* __restrict__ kept_out, int* n_kept, int* n_examined) {
+__device__ bool walk_from_pair_list(const Problem& p, const int* cand, int n_cand, unsigned int n_edges,
+                                    unsigned char* sm, int* kept_out, int* n_kept, int* n_examined) {
   const int tid = threadIdx.x, lane = tid & 31;
   const size_t bytes = ((size_t)n_cand + 15) & ~(size_t)15;
   const int n_words = (n_cand + 31) / 32;

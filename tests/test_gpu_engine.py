@@ -1,0 +1,93 @@
+"""Whole rounds in one launch (csrc/engine.cu) at the sizes where it can go wrong: every round teacher-forced against the
+oracle, then the same rounds through strads_run (candidates drawn one round ahead) against strads_round bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from helpers import oracle_matrix
+from paper_1312_5766_b200 import workloads as wl
+from test_gpu_parity import HALF_ULP32, RTOL_DBETA, _assert_kept_matches
+
+pytestmark = pytest.mark.gpu
+
+CASES = {
+    # dense: one row group and tile; just past a tile of rows, of columns and of K; several pieces of the walk; P' = P = J
+    "one_tile": dict(kind="dense_iid", n_rows=24, n_cols=600, n_true=5, n_candidates=64, n_keep=64, rho=0.5),
+    "tile_edges": dict(kind="dense_iid", n_rows=65, n_cols=900, n_true=5, n_candidates=129, n_keep=40, rho=0.3),
+    "two_windows": dict(kind="dense_iid", n_rows=257, n_cols=3000, n_true=9, n_candidates=1000, n_keep=120, rho=0.15),
+    "walk_in_pieces": dict(kind="dense_grouped", n_rows=401, n_cols=6000, n_true=9, n_candidates=2500, n_keep=300, rho=0.1),
+    "longest_columns": dict(kind="dense_iid", n_rows=2048, n_cols=1500, n_true=9, n_candidates=700, n_keep=100, rho=0.06),
+    "everything": dict(kind="dense_iid", n_rows=100, n_cols=300, n_true=5, n_candidates=300, n_keep=300, rho=0.2),
+    # CSC: buckets that hold; that overflow now and then; columns longer than a warp's two turns; P too large to draw ahead
+    "buckets": dict(kind="csc_uniform", n_rows=3000, n_cols=9000, n_true=50, n_candidates=900, n_keep=130, rho=0.1, nnz_col=33),
+    "full_buckets": dict(kind="csc_uniform", n_rows=1500, n_cols=9000, n_true=50, n_candidates=900, n_keep=130, rho=0.1, nnz_col=40),
+    "long_columns": dict(kind="csc_uniform", n_rows=20000, n_cols=2000, n_true=20, n_candidates=300, n_keep=60, rho=0.1, nnz_col=150),
+    "no_draw_ahead": dict(kind="csc_uniform", n_rows=60000, n_cols=12000, n_true=50, n_candidates=5000, n_keep=4200, rho=0.1, nnz_col=8),
+    "on_demand": dict(kind="csc_zipf", n_rows=20000, n_cols=50000, n_true=50, n_candidates=3000, n_keep=500, rho=0.05, nnz_col=21),
+}
+
+
+@pytest.mark.parametrize("name", list(CASES))
+def test_rounds(name):
+    from paper_1312_5766_b200 import binding as b
+    p = wl.make_problem(dict(CASES[name], lam_frac=0.02, group=20), seed=3)
+    if p.layout == wl.DENSE and p.n_rows % 4:
+        pad = torch.full((p.n_cols, (p.n_rows + 3) // 4 * 4), float("nan"))        # nothing may leak in from the padding
+        pad[:, : p.n_rows] = p.values
+        p.values = pad
+    X = oracle_matrix(p)
+    n2, beta, resid, delta = oracle.init(X, p.y.numpy(), 1e4)
+    lam, eta, rho = float(np.float32(p.lam)), float(np.float32(p.eta)), float(np.float32(p.rho))
+    s, ahead = (b.StradsLasso.from_problem(p, device="cuda") for _ in range(2))
+    n = 14
+    for t in range(n):
+        beta[:] = s.beta.cpu().numpy(); resid[:] = s.resid.cpu().numpy(); delta[:] = s.delta.cpu().numpy()
+        cand, kept, dbeta, counts = (x.cpu().numpy() for x in s.round())
+        nk = int(counts[2])
+        assert np.array_equal(cand, oracle.sample(delta, eta, p.seed, t, p.n_candidates)), t
+        _assert_kept_matches(X, n2, cand, p.n_keep, rho, kept[:nk], int(counts[1]))
+        assert np.all(kept[nk:] == -1)
+        want = oracle.update(X, n2, lam, kept[:nk], beta, resid, delta)
+        assert np.all(np.abs(dbeta[:nk] - want) <= RTOL_DBETA * np.abs(want) + HALF_ULP32 * np.abs(beta[kept[:nk]])), t
+    s.run(40)
+    for k in (1, 33, 20):                                   # launches of different lengths, lists in place and not
+        ahead.run(k)
+    for _ in range(n + 40 - 54):
+        ahead.round()
+    for x, y in ((s.beta, ahead.beta), (s.resid, ahead.resid), (s.delta, ahead.delta)):
+        assert torch.equal(x, y)
+    assert s.totals() == ahead.totals() and s.status()[0] == 0
+
+
+def test_products_that_cluster_at_rho():
+    """Columns of +-1 over a few rows: a third of all pairs correlate at exactly rho, more than any list of open pairs holds."""
+    from paper_1312_5766_b200 import binding as b
+    N, J, P = 20, 2000, 60
+    g = torch.Generator().manual_seed(2)
+    x = (torch.randint(0, 2, (J, N), generator=g) * 2 - 1).float()
+    y = torch.randn(N, generator=g)
+    X = oracle.Matrix.dense(x.numpy())
+    n2 = oracle.colnorm2(X)
+    rho = float(np.float32(0.2))                            # products are even integers: |corr| = 0.2 exactly is |product| = 4
+    s = b.StradsLasso(wl.DENSE, N, J, x.cuda(), y.cuda(), 0.1, 1e-6, rho, J, P, seed=1)
+    for _ in range(3):
+        cand, kept, _, counts = (v.cpu().numpy() for v in s.round())
+        _assert_kept_matches(X, n2, cand, P, rho, kept[: int(counts[2])], int(counts[1]))
+    assert s.status() == (0, 8)                             # informational: pairs decided one by one
+
+
+def test_tied_keys():
+    """Infinite priorities: thousands of race times of exactly 0, far more than the draw's boundary holds."""
+    from paper_1312_5766_b200 import binding as b
+    p = wl.make_problem(dict(kind="csc_uniform", n_rows=3000, n_cols=60000, n_true=20, lam_frac=0.02, n_candidates=700, n_keep=100,
+                             rho=0.1, nnz_col=10), seed=4)
+    s = b.StradsLasso.from_problem(p, device="cuda")
+    s.delta[500:40000] = float("inf")
+    for t in range(3):
+        delta = s.delta.cpu().numpy().astype(np.float64)
+        cand = s.round()[0].cpu().numpy()
+        assert np.array_equal(cand, oracle.sample(delta, float(np.float32(p.eta)), p.seed, t, p.n_candidates))
+    s.run(5)
+    delta = s.delta.cpu().numpy().astype(np.float64)
+    assert np.array_equal(s.round()[0].cpu().numpy(), oracle.sample(delta, float(np.float32(p.eta)), p.seed, 8, p.n_candidates))
