@@ -312,8 +312,9 @@ def measure(workload: str, args, device, rank: int, world: int, dist_ok: bool, p
 
     # ---- device-resident timing: REPEATS regions of K rounds after the warm-up ------------------------------
     s.run(args.warmup)
-    s.run(GRAPH_ROUNDS + 7)                # whatever W is: every captured launch sequence (8 rounds, and 4, 2, 1 for what is
-                                           # left over: 8 + 8 + 4 + 2 + 1 here) has run before the clock starts
+    for _ in range(3):                     # whatever W is: every captured launch sequence (8 rounds, and 4, 2, 1 for what is
+        s.run(GRAPH_ROUNDS + 7)            # left over: 8 + 8 + 4 + 2 + 1 here, captured when they come up for the third
+                                           # time) has run before the clock starts
     tot0 = s.totals()
     evs = [torch.cuda.Event(enable_timing=True) for _ in range(REPEATS + 1)]
     barrier()

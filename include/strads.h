@@ -267,6 +267,11 @@ int strads_profile_end(strads_handle_t h, double* ms_host_out /* [5] */, int64_t
 
 int strads_destroy(strads_handle_t h);
 
+/* The streams, events and captured launch sequences of destroyed handles (driver objects, no device memory of the
+ * caller's) are kept for the next handles, of at most four handles per device: making them costs milliseconds.  This
+ * gives them back.  Any thread, at any time. */
+int strads_release_cached(void);
+
 /* (No counterpart in the paper: a packaging variant of SAP step 1.)
  * The candidate draw of strads_sample for callers that must not allocate device memory -- code that
  * runs inside another component's memory pool, plugins whose host forbids cudaMalloc after start-up,

@@ -33,7 +33,7 @@ EXPORTS = [
     "strads_objective", "strads_sample", "strads_filter", "strads_update", "strads_get_round",
     "strads_set_round", "strads_totals", "strads_status", "strads_colnorm2", "strads_destroy",
     "strads_error_string", "strads_last_cuda_error", "strads_profile_begin", "strads_profile_end",
-    "strads_sample_static", "strads_set_wait_limit", "strads_inject_stall", "strads_recover", "strads_margin",
+    "strads_sample_static", "strads_set_wait_limit", "strads_inject_stall", "strads_recover", "strads_margin", "strads_release_cached",
 ]
 
 

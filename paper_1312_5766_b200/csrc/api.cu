@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include "engine.cuh"
@@ -34,11 +35,10 @@ struct strads_lasso_s {
   // strads_run replays captured launch sequences (fixed for a handle): eight rounds with one scheduler,
   // kGraphTurns turns of every scheduler, pipelined, with several
   cudaStream_t capture_stream;
-  cudaGraph_t round_graph;
-  cudaGraphExec_t round_exec;
   // one scheduler: shorter sequences (4, 2 and 1 rounds; with sampling ahead, from an early list) for what is left over
-  cudaGraph_t tail_graph[3];
-  cudaGraphExec_t tail_exec[3];
+  bool sequence_ready[4];    // kit->exec[0] (the full one) and kit->exec[1 ..] hold this handle's launches
+  long long leftovers[3];    // how often a run has had a left-over of that length
+  struct Kit* kit;           // where the streams, events and executable graphs below come from
   cudaEvent_t fork;          // S > 1: where the schedulers' streams join the caller's stream
   // Sampling ahead (one scheduler; strads_run only): the draw of round t + 1 runs on its own stream beside the Gram
   // and walk of round t, and the round then starts from that list corrected for round t's update.
@@ -65,7 +65,92 @@ struct strads_lasso_s {
   alignas(64) unsigned char engine_maps[256];
 };
 
+// The driver objects of a handle.  Making and destroying them costs far more than many a run (a captured sequence about
+// 10 us per kernel each way: 3.5 ms for c1, 6.8 ms with a candidate window, where 100 rounds take 3 to 4 ms), and a path
+// over lambda makes a handle per point.  So they outlive it: strads_destroy hands them to a pool of at most kKits a
+// device, the next handle on that device takes them from there, and where the problem has the same sizes and options its
+// captured sequences take over the executable graphs by an update of their arguments.  (Not otherwise, although the update
+// succeeds as long as the kernels are the same ones: with other grids a graph replays slower than one made anew, c2 43.2
+// instead of 39.9 us per round.)  strads_release_cached gives them back.
+struct Shape {
+  int layout, n_cand, n_keep, n_sched;
+  unsigned int flags;
+  long long N, J;
+  bool operator==(const Shape& o) const {
+    return layout == o.layout && n_cand == o.n_cand && n_keep == o.n_keep && n_sched == o.n_sched && flags == o.flags && N == o.N && J == o.J;
+  }
+};
+struct Kit {
+  int device;
+  Shape shape;               // of the handle that captured `exec`
+  Kit* next;
+  cudaStream_t capture, ahead, retry, patch, copy, sched[STRADS_MAX_SCHEDULERS];
+  cudaEvent_t ahead_fork, ahead_done, retry_fork, retry_done, patch_fork, patch_done, copy_fork, copy_done, fork;
+  cudaEvent_t ready[STRADS_MAX_SCHEDULERS], updated[STRADS_MAX_SCHEDULERS];
+  cudaGraphExec_t exec[4];
+};
+
 namespace {
+
+constexpr int kKits = 4;
+std::mutex g_kits_mutex;
+Kit* g_kits = nullptr;
+
+Kit* take_kit(int device, const Shape& shape) {
+  Kit* k = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(g_kits_mutex);
+    Kit** best = nullptr;                                // one of the same shape if there is one, else any of the device
+    for (Kit** at = &g_kits; *at != nullptr; at = &(*at)->next)
+      if ((*at)->device == device && (best == nullptr || (*at)->shape == shape)) best = at;
+    if (best != nullptr) { k = *best; *best = k->next; k->next = nullptr; }
+  }
+  if (k == nullptr) {
+    k = new (std::nothrow) Kit();                        // value-initialised: every object null
+    if (k == nullptr) return nullptr;
+    k->device = device;
+  }
+  if (!(k->shape == shape)) {
+    for (cudaGraphExec_t& x : k->exec)
+      if (x != nullptr) { cudaGraphExecDestroy(x); x = nullptr; }
+    k->shape = shape;
+  }
+  return k;
+}
+
+void destroy_kit(Kit* k) {
+  int before = 0;
+  cudaGetDevice(&before);
+  if (before != k->device) cudaSetDevice(k->device);
+  for (cudaStream_t st : {k->capture, k->ahead, k->retry, k->patch, k->copy}) if (st != nullptr) cudaStreamDestroy(st);
+  for (cudaEvent_t ev : {k->ahead_fork, k->ahead_done, k->retry_fork, k->retry_done, k->patch_fork, k->patch_done, k->copy_fork, k->copy_done, k->fork})
+    if (ev != nullptr) cudaEventDestroy(ev);
+  for (int i = 0; i < STRADS_MAX_SCHEDULERS; ++i) {
+    if (k->sched[i] != nullptr) cudaStreamDestroy(k->sched[i]);
+    if (k->ready[i] != nullptr) cudaEventDestroy(k->ready[i]);
+    if (k->updated[i] != nullptr) cudaEventDestroy(k->updated[i]);
+  }
+  for (cudaGraphExec_t x : k->exec) if (x != nullptr) cudaGraphExecDestroy(x);
+  if (before != k->device) cudaSetDevice(before);
+  delete k;
+}
+
+// (nothing of the handle's is in flight any more)
+void give_kit(Kit* k) {
+  {
+    std::lock_guard<std::mutex> lock(g_kits_mutex);
+    int n = 0;
+    for (Kit* q = g_kits; q != nullptr; q = q->next) n += q->device == k->device;
+    if (n < kKits) { k->next = g_kits; g_kits = k; return; }
+  }
+  destroy_kit(k);
+}
+
+// An object of a kit, made when it is first wanted.
+cudaError_t want_stream(cudaStream_t* s, int priority) {
+  return *s != nullptr ? cudaSuccess : cudaStreamCreateWithPriority(s, cudaStreamNonBlocking, priority);
+}
+cudaError_t want_event(cudaEvent_t* ev) { return *ev != nullptr ? cudaSuccess : cudaEventCreateWithFlags(ev, cudaEventDisableTiming); }
 
 constexpr int kProfEvents = 6;   // per round: start, after sample, pack, Gram, walk, update
 constexpr int kGraphTurns = 16;  // S > 1: turns of every scheduler in the captured sequence
@@ -73,7 +158,8 @@ constexpr int kGraphRoundsAhead = 8;  // one scheduler, sampling ahead: rounds i
 constexpr int kTailKinds = 3;         // and in the shorter ones for what is left over: 4, 2, 1 (a run of 20 rounds: 8 + 8 + 4)
 constexpr int tail_rounds(int kind) { return kGraphRoundsAhead >> (kind + 1); }
 static_assert(tail_rounds(kTailKinds - 1) == 1, "the shortest left-over sequence is one round");
-static_assert(sizeof(strads_lasso_s::tail_exec) / sizeof(cudaGraphExec_t) == kTailKinds, "one slot per left-over sequence");
+static_assert(sizeof(Kit::exec) / sizeof(cudaGraphExec_t) == kTailKinds + 1, "one slot per sequence");
+constexpr int kLeftoverUses = 3;      // a left-over sequence is captured when one of its length comes up for the third time
 constexpr int kEdgeCap = 8192;        // conflicting pairs the Gram kernels can list for the walk (32 KB)
 constexpr int kEngineRounds = 32;     // rounds per launch of the engine: a launch every few hundred microseconds, so that other streams get their turn
 constexpr int kEngineDenseRows = 2048;
@@ -572,31 +658,7 @@ bool engine_runs(const strads_lasso_s* h, const strads_round_out_t* out) {
 }
 
 void release(strads_lasso_s* h) {
-  for (int s = 0; s < STRADS_MAX_SCHEDULERS; ++s) {
-    if (h->sch[s].stream != nullptr) cudaStreamDestroy(h->sch[s].stream);
-    if (h->sch[s].block_ready != nullptr) cudaEventDestroy(h->sch[s].block_ready);
-    if (h->sch[s].updated != nullptr) cudaEventDestroy(h->sch[s].updated);
-  }
-  if (h->fork != nullptr) cudaEventDestroy(h->fork);
-  if (h->ahead_stream != nullptr) cudaStreamDestroy(h->ahead_stream);
-  if (h->ahead_fork != nullptr) cudaEventDestroy(h->ahead_fork);
-  if (h->ahead_done != nullptr) cudaEventDestroy(h->ahead_done);
-  if (h->retry_stream != nullptr) cudaStreamDestroy(h->retry_stream);
-  if (h->retry_fork != nullptr) cudaEventDestroy(h->retry_fork);
-  if (h->retry_done != nullptr) cudaEventDestroy(h->retry_done);
-  if (h->patch_stream != nullptr) cudaStreamDestroy(h->patch_stream);
-  if (h->patch_fork != nullptr) cudaEventDestroy(h->patch_fork);
-  if (h->patch_done != nullptr) cudaEventDestroy(h->patch_done);
-  if (h->copy_stream != nullptr) cudaStreamDestroy(h->copy_stream);
-  if (h->copy_fork != nullptr) cudaEventDestroy(h->copy_fork);
-  if (h->copy_done != nullptr) cudaEventDestroy(h->copy_done);
-  if (h->round_exec != nullptr) cudaGraphExecDestroy(h->round_exec);
-  if (h->round_graph != nullptr) cudaGraphDestroy(h->round_graph);
-  for (int k = 0; k < kTailKinds; ++k) {
-    if (h->tail_exec[k] != nullptr) cudaGraphExecDestroy(h->tail_exec[k]);
-    if (h->tail_graph[k] != nullptr) cudaGraphDestroy(h->tail_graph[k]);
-  }
-  if (h->capture_stream != nullptr) cudaStreamDestroy(h->capture_stream);
+  if (h->kit != nullptr) give_kit(h->kit);
   delete h;
 }
 
@@ -639,6 +701,11 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
   auto fail = [&](int code) { release(h); return code; };
   cudaError_t e = cudaGetDevice(&h->device);
   if (e != cudaSuccess) return fail(cuda_fail(e, "cudaGetDevice"));
+  h->kit = take_kit(h->device, Shape{c->layout, c->n_candidates, c->n_keep, S, c->flags, (long long)c->n_rows, (long long)c->n_cols});
+  if (h->kit == nullptr) return fail(STRADS_ERR_INVALID_ARG);
+  Kit& kit = *h->kit;
+  int prio_least = 0, prio_greatest = 0;               // the early draw yields to the round's own kernels
+  if ((e = cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest)) != cudaSuccess) return fail(cuda_fail(e, "priority range"));
   int sm_count = 0;
   e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, h->device);
   if (e != cudaSuccess) return fail(cuda_fail(e, "cudaDeviceGetAttribute"));
@@ -656,10 +723,10 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
   if ((e = prepare_gram_dense_tc()) != cudaSuccess) return fail(cuda_fail(e, "prepare_gram_dense_tc"));
   if ((e = launch_init(p0, h->stream)) != cudaSuccess) return fail(cuda_fail(e, "launch_init"));
   if ((e = launch_resid_from_beta(p0, h->stream)) != cudaSuccess) return fail(cuda_fail(e, "launch_resid_from_beta"));
-  if ((e = cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking)) != cudaSuccess ||
-      (e = cudaEventCreateWithFlags(&h->copy_fork, cudaEventDisableTiming)) != cudaSuccess ||
-      (e = cudaEventCreateWithFlags(&h->copy_done, cudaEventDisableTiming)) != cudaSuccess)
+  if ((e = want_stream(&kit.copy, 0)) != cudaSuccess || (e = want_event(&kit.copy_fork)) != cudaSuccess ||
+      (e = want_event(&kit.copy_done)) != cudaSuccess)
     return fail(cuda_fail(e, "copy stream"));
+  h->copy_stream = kit.copy; h->copy_fork = kit.copy_fork; h->copy_done = kit.copy_done;
   h->ahead_round = -1;
   h->engine_ok = L.engine && engine_chosen(c) && sm_count <= kEngineMaxCtas;
   if (h->engine_ok) {
@@ -675,18 +742,15 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
   if (h->ahead_ok) {
     fill_ahead(h->ahead, p0, L, ws);
     if ((e = launch_init_scheduler(h->ahead, p0, h->stream)) != cudaSuccess) return fail(cuda_fail(e, "launch_init_scheduler"));
-    int prio_least = 0, prio_greatest = 0;             // the early draw yields to the round's own kernels
-    if ((e = cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest)) != cudaSuccess) return fail(cuda_fail(e, "priority range"));
-    if ((e = cudaStreamCreateWithPriority(&h->ahead_stream, cudaStreamNonBlocking, prio_least)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&h->ahead_fork, cudaEventDisableTiming)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&h->ahead_done, cudaEventDisableTiming)) != cudaSuccess ||
-        (e = cudaStreamCreateWithPriority(&h->retry_stream, cudaStreamNonBlocking, prio_least)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&h->retry_fork, cudaEventDisableTiming)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&h->retry_done, cudaEventDisableTiming)) != cudaSuccess ||
-        (e = cudaStreamCreateWithPriority(&h->patch_stream, cudaStreamNonBlocking, prio_greatest)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&h->patch_fork, cudaEventDisableTiming)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&h->patch_done, cudaEventDisableTiming)) != cudaSuccess)
+    if ((e = want_stream(&kit.ahead, prio_least)) != cudaSuccess || (e = want_event(&kit.ahead_fork)) != cudaSuccess ||
+        (e = want_event(&kit.ahead_done)) != cudaSuccess || (e = want_stream(&kit.retry, prio_least)) != cudaSuccess ||
+        (e = want_event(&kit.retry_fork)) != cudaSuccess || (e = want_event(&kit.retry_done)) != cudaSuccess ||
+        (e = want_stream(&kit.patch, prio_greatest)) != cudaSuccess || (e = want_event(&kit.patch_fork)) != cudaSuccess ||
+        (e = want_event(&kit.patch_done)) != cudaSuccess)
       return fail(cuda_fail(e, "sampling-ahead stream"));
+    h->ahead_stream = kit.ahead; h->ahead_fork = kit.ahead_fork; h->ahead_done = kit.ahead_done;
+    h->retry_stream = kit.retry; h->retry_fork = kit.retry_fork; h->retry_done = kit.retry_done;
+    h->patch_stream = kit.patch; h->patch_fork = kit.patch_fork; h->patch_done = kit.patch_done;
   }
   for (int s = 0; s < S; ++s) {
     Scheduler& sc = h->sch[s];
@@ -705,15 +769,15 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
     if (s > 0 && (e = launch_init_scheduler(sc.p, p0, h->stream)) != cudaSuccess)
       return fail(cuda_fail(e, "launch_init_scheduler"));
     if (S > 1) {
-      if ((e = cudaStreamCreateWithFlags(&sc.stream, cudaStreamNonBlocking)) != cudaSuccess ||
-          (e = cudaEventCreateWithFlags(&sc.block_ready, cudaEventDisableTiming)) != cudaSuccess ||
-          (e = cudaEventCreateWithFlags(&sc.updated, cudaEventDisableTiming)) != cudaSuccess)
+      if ((e = want_stream(&kit.sched[s], 0)) != cudaSuccess || (e = want_event(&kit.ready[s])) != cudaSuccess ||
+          (e = want_event(&kit.updated[s])) != cudaSuccess)
         return fail(cuda_fail(e, "scheduler stream"));
+      sc.stream = kit.sched[s]; sc.block_ready = kit.ready[s]; sc.updated = kit.updated[s];
     }
   }
   if (h->engine_ok && (e = clear_engine(h)) != cudaSuccess) return fail(cuda_fail(e, "clear_engine"));
-  if (S > 1 && (e = cudaEventCreateWithFlags(&h->fork, cudaEventDisableTiming)) != cudaSuccess)
-    return fail(cuda_fail(e, "cudaEventCreate"));
+  if (S > 1 && (e = want_event(&kit.fork)) != cudaSuccess) return fail(cuda_fail(e, "cudaEventCreate"));
+  h->fork = kit.fork;
   *out_handle = h;
   return STRADS_OK;
 }
@@ -743,8 +807,10 @@ static int build_round_graph(strads_lasso_s* h, int tail_kind = -1) {
   if (h->capture_stream == nullptr) {
     int prio_least = 0, prio_greatest = 0;
     CK(cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest));
-    CK(cudaStreamCreateWithPriority(&h->capture_stream, cudaStreamNonBlocking, prio_greatest));
+    CK(want_stream(&h->kit->capture, prio_greatest));
+    h->capture_stream = h->kit->capture;
   }
+  cudaGraph_t graph = nullptr;
   cudaStream_t user = h->stream;
   const long long round_before = h->round_host;
   h->stream = h->capture_stream;
@@ -761,17 +827,33 @@ static int build_round_graph(strads_lasso_s* h, int tail_kind = -1) {
       const long long n = tail ? tail_rounds(tail_kind) : graph_rounds(h);
       for (long long i = 0; i < n && rc == STRADS_OK; ++i) rc = one_round(h, nullptr);
     }
-    e = cudaStreamEndCapture(h->capture_stream, tail ? &h->tail_graph[tail_kind] : &h->round_graph);
+    e = cudaStreamEndCapture(h->capture_stream, &graph);
     h->ahead_round = ahead_before;
   }
   h->stream = user;
   h->round_host = round_before;
-  if (rc) return rc;
-  if (e != cudaSuccess) return cuda_fail(e, "stream capture of a round");
+  if (rc != STRADS_OK || e != cudaSuccess) {
+    if (graph != nullptr) cudaGraphDestroy(graph);
+    return rc ? rc : cuda_fail(e, "stream capture of a round");
+  }
+  // an executable graph of the same shape, from this handle or one before it, takes the new arguments over; otherwise
   // instantiated and uploaded now, so that the first launch does not pay for either
-  cudaGraphExec_t* exec = tail ? &h->tail_exec[tail_kind] : &h->round_exec;
-  CK(cudaGraphInstantiate(exec, tail ? h->tail_graph[tail_kind] : h->round_graph, 0));
-  CK(cudaGraphUpload(*exec, user));
+  cudaGraphExec_t& exec = h->kit->exec[tail_kind + 1];
+  if (exec != nullptr) {
+    cudaGraphExecUpdateResultInfo info;
+    if (cudaGraphExecUpdate(exec, graph, &info) != cudaSuccess) {
+      cudaGetLastError();
+      cudaGraphExecDestroy(exec);
+      exec = nullptr;
+    }
+  }
+  if (exec == nullptr) {
+    e = cudaGraphInstantiate(&exec, graph, 0);
+    if (e == cudaSuccess) e = cudaGraphUpload(exec, user);
+  }
+  cudaGraphDestroy(graph);
+  if (e != cudaSuccess) return cuda_fail(e, "instantiation of a round's launches");
+  h->sequence_ready[tail_kind + 1] = true;
   return STRADS_OK;
 }
 
@@ -794,11 +876,11 @@ int strads_run(strads_handle_t h, int64_t n_rounds) {
     long long left = n_rounds;
     while (left > 0) {
       if (h->round_host % h->n_sched == 0 && left >= R) {
-        if (h->round_exec == nullptr) {
+        if (!h->sequence_ready[0]) {
           const int rc = build_round_graph(h);
           if (rc) return rc;
         }
-        CK(cudaGraphLaunch(h->round_exec, h->stream));
+        CK(cudaGraphLaunch(h->kit->exec[0], h->stream));
         h->round_host += R;
         left -= R;
       } else {
@@ -811,40 +893,39 @@ int strads_run(strads_handle_t h, int64_t n_rounds) {
     }
     return STRADS_OK;
   }
+  // Captured sequences: eight rounds where they fit, from the first run on that holds as many; what is left over as shorter
+  // ones, those captured only once they have come up a few times (a fit of 1,000 rounds has one left-over of each
+  // length, which costs 10 us more a round launched kernel by kernel, while capturing the three costs a millisecond or two).
   const bool use_graph = h->prof_events == nullptr && n_rounds > 1;   // step timing needs events between kernels
-  if (use_graph && h->round_exec == nullptr) {
-    const int rc = build_round_graph(h);
-    if (rc) return rc;
-  }
-  for (int k = 0; use_graph && k < kTailKinds; ++k) {
-    if (h->tail_exec[k] != nullptr) continue;
-    const int rc = build_round_graph(h, k);
-    if (rc) return rc;
-  }
   const long long R = graph_rounds(h);
-  for (int64_t i = 0; i < n_rounds; ++i) {
-    if (use_graph) {
-      // (without sampling ahead every round draws its own list: nothing to have in place)
-      const bool have_list = !h->ahead_ok || h->ahead_round == h->round_host;
-      if (have_list && n_rounds - i >= R) {            // the early list of this round is in place: captured rounds
-        CK(cudaGraphLaunch(h->round_exec, h->stream));
-        h->round_host += R;
-        h->ahead_round = h->round_host;
-        i += R - 1;
-      } else if (have_list) {                          // fewer rounds left than a sequence holds: the longest shorter one
-        int k = 0;
-        while (tail_rounds(k) > n_rounds - i) ++k;     // (the last kind is one round)
-        CK(cudaGraphLaunch(h->tail_exec[k], h->stream));
-        h->round_host += tail_rounds(k);
-        h->ahead_round = h->round_host;
-        i += tail_rounds(k) - 1;
-      } else {                                         // first round of a run: draw now, start drawing ahead
-        const int rc = round_sampling_ahead(h, false, h->stream);
+  for (int64_t i = 0; i < n_rounds;) {
+    // (without sampling ahead every round draws its own list: nothing to have in place)
+    const bool have_list = !h->ahead_ok || h->ahead_round == h->round_host;
+    if (use_graph && have_list) {
+      int kind = -1;                                     // the longest sequence that fits
+      while (kind < kTailKinds - 1 && (kind < 0 ? R : tail_rounds(kind)) > n_rounds - i) ++kind;
+      if (kind >= 0 && !h->sequence_ready[kind + 1] && ++h->leftovers[kind] < kLeftoverUses) {
+        for (int k = 0; k < tail_rounds(kind); ++k) {
+          const int rc = h->ahead_ok ? round_sampling_ahead(h, true, h->stream) : one_round(h, nullptr);
+          if (rc) return rc;
+        }
+        i += tail_rounds(kind);
+        continue;
+      }
+      if (!h->sequence_ready[kind + 1]) {
+        const int rc = build_round_graph(h, kind);
         if (rc) return rc;
       }
+      const long long n = kind < 0 ? R : tail_rounds(kind);
+      CK(cudaGraphLaunch(h->kit->exec[kind + 1], h->stream));
+      h->round_host += n;
+      h->ahead_round = h->round_host;
+      i += n;
     } else {
-      const int rc = one_round(h, nullptr);
+      // the first round of a run draws now and starts drawing ahead
+      const int rc = use_graph ? round_sampling_ahead(h, false, h->stream) : one_round(h, nullptr);
       if (rc) return rc;
+      ++i;
     }
   }
   return STRADS_OK;
@@ -966,14 +1047,9 @@ int strads_status(strads_handle_t h, uint32_t* bits_host_out) {
   return STRADS_OK;
 }
 
-// The captured launch sequence holds copies of the kernels' arguments: drop it when one of them changes.
+// The captured launch sequences hold copies of the kernels' arguments: captured again when one of them changes.
 static void drop_round_graph(strads_lasso_s* h) {
-  if (h->round_exec != nullptr) { cudaGraphExecDestroy(h->round_exec); h->round_exec = nullptr; }
-  if (h->round_graph != nullptr) { cudaGraphDestroy(h->round_graph); h->round_graph = nullptr; }
-  for (int k = 0; k < kTailKinds; ++k) {
-    if (h->tail_exec[k] != nullptr) { cudaGraphExecDestroy(h->tail_exec[k]); h->tail_exec[k] = nullptr; }
-    if (h->tail_graph[k] != nullptr) { cudaGraphDestroy(h->tail_graph[k]); h->tail_graph[k] = nullptr; }
-  }
+  for (bool& ready : h->sequence_ready) ready = false;
 }
 
 int strads_set_wait_limit(strads_handle_t h, uint32_t iterations) {
@@ -1083,6 +1159,17 @@ int strads_destroy(strads_handle_t h) {
     delete[] h->prof_events;
   }
   release(h);
+  return STRADS_OK;
+}
+
+int strads_release_cached(void) {
+  Kit* all = nullptr;
+  {
+    std::lock_guard<std::mutex> lock(g_kits_mutex);
+    all = g_kits;
+    g_kits = nullptr;
+  }
+  while (all != nullptr) { Kit* k = all; all = k->next; destroy_kit(k); }
   return STRADS_OK;
 }
 

@@ -26,6 +26,7 @@
 // work, and still frees its tensor memory.  No multicast anywhere.
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <mutex>
 
 #include "strads_internal.cuh"
 #include "walk_pairs.cuh"
@@ -708,14 +709,16 @@ __global__ void __launch_bounds__(256) k_gram_recheck(Problem p, int only_if_sho
 // beside it, measured slower with them (c3: 68.4 us per round with clusters of 9, 65.9 with 8; c2 39.1 / 38.2).
 constexpr int kMaxSplit = 8;
 static int g_max_clusters[kMaxSplit + 1];     // [size]; 0: size not available
+static std::mutex g_clusters_mutex;
+static bool g_clusters_known = false;         // (asked once: the seven queries take 100 us, and every GPU here is alike)
 
 cudaError_t prepare_gram_dense_tc() {
   cudaError_t e = cudaFuncSetAttribute(k_gram_dense_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmem);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_gram_dense_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmem);
   if (e != cudaSuccess) return e;
-  for (int size = 2; size <= kMaxSplit; ++size) {
-    g_max_clusters[size] = 0;
+  std::lock_guard<std::mutex> lock(g_clusters_mutex);
+  for (int size = 2; size <= kMaxSplit && !g_clusters_known; ++size) {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)size; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
@@ -723,9 +726,10 @@ cudaError_t prepare_gram_dense_tc() {
     cfg.gridDim = dim3((unsigned)size * 64); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kDynSmem;
     cfg.attrs = attr; cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_gram_dense_tc<false>, &cfg) == cudaSuccess) g_max_clusters[size] = n;
+    g_max_clusters[size] = cudaOccupancyMaxActiveClusters(&n, k_gram_dense_tc<false>, &cfg) == cudaSuccess ? n : 0;
     cudaGetLastError();                                  // (a size the device refuses is simply not used)
   }
+  g_clusters_known = true;
   return cudaSuccess;
 }
 
