@@ -19,7 +19,7 @@
  *   - every array is allocated, owned and freed by the caller; the handle owns
  *     only host bookkeeping.  X and y are never written and must outlive the
  *     handle, as must beta, resid, delta and the workspace;
- *   - the library allocates no device memory (strads_sample_static keeps about 65 KB of scratch in a
+ *   - the library allocates no device memory (strads_sample_static keeps about 82 KB of scratch in a
  *     fixed device array of its own instead of a workspace);
  *   - arguments are validated on the host before anything is launched; nothing
  *     traps, aborts or waits without a bound;
@@ -276,7 +276,7 @@ int strads_release_cached(void);
  * The candidate draw of strads_sample for callers that must not allocate device memory -- code that
  * runs inside another component's memory pool, plugins whose host forbids cudaMalloc after start-up,
  * latency-critical loops.  It needs no handle and no workspace: the scratch memory of the select
- * passes lives in a fixed array inside the library (about 65 KB on every GPU that loads it, until the
+ * passes lives in a fixed array inside the library (about 82 KB on every GPU that loads it, until the
  * process exits), which limits it to n_candidates <= STRADS_STATIC_MAX_CANDIDATES; larger requests
  * return STRADS_ERR_UNSUPPORTED.  The call allocates nothing (no cudaMalloc / cudaFree, no allocating
  * library routine).

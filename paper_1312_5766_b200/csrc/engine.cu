@@ -2008,6 +2008,78 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
   }
 }
 
+// ------------------------------------------------------------------------------------------------
+// The draw alone (strads_sample_static), all of it in one launch: keys computed once and kept in shared memory, histogram,
+// selection, collection and ranking with two grid barriers between them.  Bound by the launch and the barriers: 22.6 us
+// as six launches (clear, round index, two passes, ordering), each waiting for the one before, at J = 100,000, P' = 2,048;
+// one launch and a clear before it still took 16.4, so the kernel leaves its scratch clear instead (`spare`: another call's
+// barrier, cleared for it in case that call was cut short).
+// A grid of no more CTAs than have keys or winners to go through: the barriers cost less among few.
+// ------------------------------------------------------------------------------------------------
+constexpr size_t kDrawKeys = 144 * 1024;   // keys a CTA keeps in shared memory (more: computed again to collect the winners)
+
+__global__ void __launch_bounds__(kT, 1) k_draw(const __grid_constant__ Problem p, const __grid_constant__ Engine e, unsigned long long t, int kept_groups,
+                                                EngineState* spare) {
+  extern __shared__ __align__(1024) unsigned char sm[];
+  __shared__ DrawShared ds;
+  __shared__ Problem sp;
+  __shared__ Engine se;
+  unsigned int* sh = reinterpret_cast<unsigned int*>(sm);
+  unsigned long long* held = reinterpret_cast<unsigned long long*>(sm + kScanSmem);      // [kept_groups][4][kT]
+  const int tid = threadIdx.x;
+  const long long groups = (p.J + 3) >> 2, whole = p.J >> 2;
+  const WeightForm wf = weight_form(p);
+  const Binning bins = binning_of(0.f);
+  for (int b = tid; b < kHistBins; b += kT) sh[b] = 0u;
+  for (int b = (int)blockIdx.x * kT + tid; b < kHistBins; b += (int)gridDim.x * kT) e.bin_cur[b] = 0u;
+  if (tid == 0) { sp = p; se = e; ds.cut = 0.f; }
+  __syncthreads();
+  Grid g;
+  g.count = &e.es->bar_count; g.target = 0u; g.n = gridDim.x; g.limit = kSpinLimit; g.status = &p.st->status;
+  int turn = 0;
+  for (long long gi = (long long)blockIdx.x * kT + tid; gi < groups; gi += (long long)gridDim.x * kT, ++turn) {
+    float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (gi < whole) {
+      d = __ldg(reinterpret_cast<const float4*>(p.delta) + gi);
+    } else {
+      const long long j = gi << 2;
+      d.x = p.delta[j];
+      if (j + 1 < p.J) d.y = p.delta[j + 1];
+      if (j + 2 < p.J) d.z = p.delta[j + 2];
+    }
+    uint32_t w[4];
+    philox4x32_10((uint32_t)gi, (uint32_t)t, (uint32_t)(t >> 32), 0u, (uint32_t)p.seed, (uint32_t)(p.seed >> 32), w);
+    const float dd[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const long long j = (gi << 2) + i;
+      const unsigned long long key = j < p.J ? key_of(wf, dd[i], w[i], (uint32_t)j) : ~0ull;
+      if (j < p.J) atomicAdd(&sh[bin_of(bins, (unsigned int)(key >> 32))], 1u);
+      if (turn < kept_groups) held[((size_t)turn * 4 + i) * kT + tid] = key;
+    }
+  }
+  __syncthreads();
+  for (int b = tid; b < kHistBins; b += kT)
+    if (sh[b]) atomicAdd(&e.hist[b], sh[b]);
+  if (!grid_sync(g)) return;
+  draw_select(e, ds, (unsigned)p.n_cand);
+  if (ds.bnd_count > (unsigned)e.cap_boundary && !draw_refine(sp, se, ds, sm, t, (unsigned)p.n_cand, g)) return;
+  if (kept_groups > 0) {
+    for (int k = 0; k < turn; ++k)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const unsigned long long key = held[((size_t)k * 4 + i) * kT + tid];
+        if (key != ~0ull) take_winner(e, ds, bins, key);
+      }
+  } else {
+    draw_collect_all(sp, se, ds, sm, t);
+  }
+  if (!grid_sync(g)) return;
+  draw_rank<true>(p, e, ds, nullptr, nullptr, 0, 0, nullptr, (int)gridDim.x, 0);       // (leaves the histogram clear)
+  if (tid == 0 && atomicInc(&e.es->exit_count, gridDim.x - 1u) == gridDim.x - 1u) e.es->bar_count = 0u;
+  if (blockIdx.x == 0 && tid == 0) { spare->bar_count = 0u; spare->exit_count = 0u; }
+}
+
 size_t smem_of(bool dense, int n_keep, bool ahead, int n_cand) {
   size_t need = kScanSmem;
   const size_t keys = ahead ? 2 * sizeof(unsigned long long) * (size_t)n_keep : 0;
@@ -2051,6 +2123,25 @@ cudaError_t prepare_engine(const Problem& p, Engine& e) {
     e.plan[1] = gram_plan(p.N, p.n_cand, terms, e.grid);
   }
   return cudaSuccess;
+}
+
+cudaError_t prepare_draw() { return cudaFuncSetAttribute(k_draw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kScanSmem + kDrawKeys)); }
+
+cudaError_t launch_draw(const Problem& p, const Engine& e, unsigned long long t, EngineState* spare, cudaStream_t s) {
+  const long long groups = (p.J + 3) / 4;
+  const long long need = (groups + kT - 1) / kT, rank = ((long long)e.cap_win * 8 + kT - 1) / kT;
+  long long grid = need > rank ? need : rank;
+  if (grid > p.sm_count) grid = p.sm_count;
+  const long long turns = (groups + grid * kT - 1) / (grid * kT);
+  const bool held = (size_t)turns * 4 * kT * sizeof(unsigned long long) <= kDrawKeys;
+  const size_t smem = kScanSmem + (held ? (size_t)turns * 4 * kT * sizeof(unsigned long long) : 0);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(kT); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_draw, p, e, t, held ? (int)turns : 0, spare);
 }
 
 cudaError_t encode_engine_maps(const Problem& p, const Engine& e, void* out) {

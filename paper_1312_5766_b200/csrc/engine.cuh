@@ -84,4 +84,9 @@ cudaError_t encode_engine_maps(const Problem& p, const Engine& e, void* out_256_
 cudaError_t launch_engine(const Problem& p, const Engine& e, const void* maps, int n_rounds, bool have_list, bool draw_next,
                           const strads_round_out_t* out, cudaStream_t s);
 
+// The draw alone: p.cand[0 .. p.n_cand) for round t from p.delta (e: es, hist, bin_cur and win).  The barrier in es and hist
+// are zero before and after.
+cudaError_t prepare_draw();
+cudaError_t launch_draw(const Problem& p, const Engine& e, unsigned long long t, EngineState* spare, cudaStream_t s);
+
 }  // namespace strads

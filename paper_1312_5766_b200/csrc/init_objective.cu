@@ -77,7 +77,7 @@ __global__ void k_fill_state(Problem p) {
     DeviceState* st = p.st;
     st->round = 0;
     for (int k = 0; k < 4; ++k) { st->totals[k] = 0; st->counts[k] = 0; }
-    st->status = 0; st->hist_ticket = 0; st->sure_count = 0; st->boundary_count = 0;
+    st->status = 0; st->hist_ticket = 0; st->boundary_count = 0;
     st->objective = 0.0;
   }
   for (long long b = i; b < kHistBins; b += stride) p.hist[b] = 0;

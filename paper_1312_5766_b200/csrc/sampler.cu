@@ -16,12 +16,10 @@
 //   k_sample_rank_bins  (the default) orders the winners: bins are in key order already, so every key is
 //                    ranked inside its own group only, and the boundary keys among themselves.
 //   k_sample_patch   corrects a list drawn one round ahead for the coefficients the last update changed.
-//   k_sample_rank_direct (P' <= 2048) / k_sample_sort_chunks + k_sample_rank (larger P'): ordering without
-//                    group arrays (counting over the whole buffer; 1024-key chunk sorts in shared memory,
-//                    then ranks by binary search in the other chunks); used by strads_sample_static.
 #include <cstddef>
 #include <mutex>
 
+#include "engine.cuh"
 #include "strads_internal.cuh"
 
 namespace strads {
@@ -281,15 +279,14 @@ __global__ void __launch_bounds__(kThreads, 4) k_sample_hist(Problem p, int mode
     const unsigned int edge = ((unsigned int)s_bin + 1u) << (32 - kHistBits);
     p.st->t_cut = edge < 0x7f800000u ? __fmul_rn(4.0f, __uint_as_float(edge)) : 0.f;
     p.st->hist_ticket = 0;
-    p.st->sure_count = 0;                             // append cursors of the collect pass that follows
-    p.st->boundary_count = 0;
+    p.st->boundary_count = 0;                         // append cursor of the collect pass that follows
     s_sel.prefix = (unsigned long long)s_bin;
     s_sel.bits = kHistBits;
     s_sel.n_sure = (int)s_before;
     s_sel.n_boundary = (int)sh[s_bin];
   }
   __syncthreads();
-  if (p.bin_off != nullptr) {
+  {
     // Where the sure keys of every bin below the boundary bin start in the `sure` buffer (exclusive prefix of the
     // counts; the boundary bin's own sure keys, if it gets refined, follow at s_before), and the bins' cursors:
     // the collect pass then leaves the winners grouped by their top 12 bits, and ordering them is a matter of
@@ -364,13 +361,8 @@ __global__ void __launch_bounds__(kThreads) k_sample_collect(Problem p) {
   auto take = [&](unsigned long long key) {
     const unsigned long long pfx = key >> shift;
     if (pfx < sel.prefix) {
-      unsigned int i;
-      if (p.bin_off != nullptr) {                      // into the group of its histogram bin
-        const unsigned int bin = min((unsigned int)(key >> (64 - kHistBits)), top_bin);
-        i = (unsigned int)p.bin_off[bin] + atomicAdd(&p.bin_cur[bin], 1u);
-      } else {
-        i = atomicAdd(&p.st->sure_count, 1u);
-      }
+      const unsigned int bin = min((unsigned int)(key >> (64 - kHistBits)), top_bin);      // into the group of its histogram bin
+      const unsigned int i = (unsigned int)p.bin_off[bin] + atomicAdd(&p.bin_cur[bin], 1u);
       if (i < (unsigned)p.cap_sure) p.sure[i] = key;
     } else if (pfx == sel.prefix) {
       const unsigned int i = atomicAdd(&p.st->boundary_count, 1u);
@@ -393,131 +385,6 @@ __global__ void __launch_bounds__(kThreads) k_sample_collect(Problem p) {
   } else {
     for (long long g = (long long)blockIdx.x * kThreads + tid; g < groups; g += (long long)gridDim.x * kThreads)
       for_keys_of_group(p, t, g, 0.f, take);
-  }
-}
-
-// Ascending bitonic sort of n (a power of two) keys in shared memory by the whole CTA.
-__device__ void bitonic_sort(unsigned long long* a, int n) {
-  for (int k = 2; k <= n; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = threadIdx.x; i < (n >> 1); i += blockDim.x) {
-        const int lo = ((i & ~(j - 1)) << 1) | (i & (j - 1));
-        const int hi = lo | j;
-        const unsigned long long x = a[lo], y = a[hi];
-        const bool up = (lo & k) == 0;
-        if ((x > y) == up) { a[lo] = y; a[hi] = x; }
-      }
-      __syncthreads();
-    }
-  }
-}
-
-__device__ int pow2_ceil(int n) { int v = 1; while (v < n) v <<= 1; return v; }
-
-constexpr int kChunk = 1024;             // keys sorted by one CTA
-
-// Which slice of which buffer CTA `c` owns: sure chunks first, then boundary chunks.
-struct ChunkRef { unsigned long long* base; int n; int first; bool is_sure; };
-__device__ __forceinline__ ChunkRef chunk_of(const Problem& p, const SelectState& sel, int c) {
-  const int n_sure = min(sel.n_sure, p.cap_sure), n_bnd = min(sel.n_boundary, p.cap_boundary);
-  const int sure_chunks = (p.cap_sure + kChunk - 1) / kChunk;
-  ChunkRef r;
-  r.is_sure = c < sure_chunks;
-  const int ci = r.is_sure ? c : c - sure_chunks;
-  const int total = r.is_sure ? n_sure : n_bnd;
-  r.first = ci * kChunk;
-  r.n = max(0, min(kChunk, total - r.first));
-  r.base = (r.is_sure ? p.sure : p.boundary) + r.first;
-  return r;
-}
-
-// Step 1 of the final ordering: every CTA sorts one chunk of up to 1024 collected keys in shared memory
-// (bitonic) and writes it back in place.  One CTA sorting all P' keys would be bound by its own shared-memory
-// bandwidth (~100 us for 16,384 keys); chunks run on as many SMs as there are chunks.
-__global__ void __launch_bounds__(512) k_sample_sort_chunks(Problem p) {
-  chain_begin();
-  __shared__ unsigned long long keys[kChunk];
-  const SelectState sel = p.st->sel;
-  const ChunkRef ch = chunk_of(p, sel, blockIdx.x);
-  if (ch.n == 0) return;
-  const int n = pow2_ceil(ch.n);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) keys[i] = i < ch.n ? ch.base[i] : ~0ull;
-  __syncthreads();
-  bitonic_sort(keys, n);
-  for (int i = threadIdx.x; i < ch.n; i += blockDim.x) ch.base[i] = keys[i];
-}
-
-// Number of keys < key in a sorted array (keys are distinct).
-__device__ __forceinline__ int count_less(const unsigned long long* a, int n, unsigned long long key) {
-  int lo = 0, hi = n;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (a[mid] < key) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
-// Step 2: the rank of a key among all collected keys = its index in its own chunk + the number of smaller
-// keys in every other chunk of its buffer (+ n_sure for boundary keys: every sure key is smaller).  The key
-// of rank r < P' is candidate r.  Each other chunk is staged in shared memory and searched there.
-__global__ void __launch_bounds__(512) k_sample_rank(Problem p, int* cand_out) {
-  chain_begin();
-  __shared__ unsigned long long other[kChunk];
-  const SelectState sel = p.st->sel;
-  const ChunkRef ch = chunk_of(p, sel, blockIdx.x);
-  if (blockIdx.x == 0 && threadIdx.x == 0) { p.st->counts[0] = p.n_cand; p.st->surv_count = 0; }
-  if (ch.n == 0) return;
-  const int n_sure = min(sel.n_sure, p.cap_sure), n_bnd = min(sel.n_boundary, p.cap_boundary);
-  const unsigned long long* buf = ch.is_sure ? p.sure : p.boundary;
-  const int total = ch.is_sure ? n_sure : n_bnd;
-  const int i0 = threadIdx.x, i1 = threadIdx.x + 512;           // this thread's (up to) two keys
-  const unsigned long long k0 = i0 < ch.n ? __ldcg(ch.base + i0) : 0ull, k1 = i1 < ch.n ? __ldcg(ch.base + i1) : 0ull;
-  int r0 = i0 + (ch.is_sure ? 0 : n_sure), r1 = i1 + (ch.is_sure ? 0 : n_sure);
-  for (int o = 0; o < total; o += kChunk) {
-    if (o == ch.first) continue;
-    const int n = min(kChunk, total - o);
-    __syncthreads();
-    for (int e = threadIdx.x; e < n; e += 512) other[e] = __ldcg(buf + o + e);
-    __syncthreads();
-    r0 += count_less(other, n, k0);
-    r1 += count_less(other, n, k1);
-  }
-  if (i0 < ch.n && r0 < p.n_cand) { cand_out[r0] = (int)(k0 & 0xffffffffull); if (p.keys_out) p.keys_out[r0] = k0; }
-  if (i1 < ch.n && r1 < p.n_cand) { cand_out[r1] = (int)(k1 & 0xffffffffull); if (p.keys_out) p.keys_out[r1] = k1; }
-}
-
-// Small P': the order of the winners straight from the definition, with no sort.  The rank of a key is the
-// number of smaller keys in its buffer (+ n_sure for boundary keys: every sure key is smaller); the key of
-// rank r < P' is candidate r.  A CTA takes 32 keys of one buffer, stages the whole buffer (<= 2048 keys) in
-// shared memory and counts with eight threads per key, each over an eighth of the buffer.
-constexpr int kDirectMax = 2048;         // P' and the boundary buffer up to this many keys (beyond, sorting is as fast)
-constexpr int kDirectKeys = 32;          // keys per CTA
-__global__ void __launch_bounds__(256) k_sample_rank_direct(Problem p, int* cand_out) {
-  chain_begin();
-  __shared__ unsigned long long all[kDirectMax];
-  const SelectState sel = p.st->sel;
-  if (blockIdx.x == 0 && threadIdx.x == 0) { p.st->counts[0] = p.n_cand; p.st->surv_count = 0; }
-  const int n_sure = min(sel.n_sure, p.cap_sure), n_bnd = min(sel.n_boundary, p.cap_boundary);
-  const int sure_ctas = (p.cap_sure + kDirectKeys - 1) / kDirectKeys;
-  const bool is_sure = (int)blockIdx.x < sure_ctas;
-  const int first = (is_sure ? blockIdx.x : blockIdx.x - sure_ctas) * kDirectKeys;
-  const int total = is_sure ? n_sure : n_bnd;
-  if (first >= total) return;
-  const unsigned long long* buf = is_sure ? p.sure : p.boundary;
-  for (int i = threadIdx.x; i < total; i += 256) all[i] = __ldcg(buf + i);
-  __syncthreads();
-  const int k = first + (threadIdx.x >> 3), slice = threadIdx.x & 7;
-  const unsigned long long key = k < total ? all[k] : 0ull;
-  int below = 0;                                        // thread `slice` looks at keys slice, slice + 8, ...: the eight
-#pragma unroll 8                                        // threads of a key read eight consecutive words (no bank conflict)
-  for (int i = slice; i < total; i += 8) below += all[i] < key;
-  below += __shfl_xor_sync(0xffffffffu, below, 1);
-  below += __shfl_xor_sync(0xffffffffu, below, 2);
-  below += __shfl_xor_sync(0xffffffffu, below, 4);
-  const int rank = below + (is_sure ? 0 : n_sure);
-  if (slice == 0 && k < total && rank < p.n_cand) {
-    cand_out[rank] = (int)(key & 0xffffffffull);
-    if (p.keys_out) p.keys_out[rank] = key;
   }
 }
 
@@ -671,15 +538,7 @@ cudaError_t launch_sample(const Problem& p, int* cand_out, cudaStream_t s) {
   const bool guided = p.J >= (1 << 19);     // (below that the passes are bound by latency, not by arithmetic)
   if ((e = launch_chained(k_sample_hist, (unsigned)blocks, kThreads, 0, s, p, guided ? 1 : 0)) != cudaSuccess) return e;
   if ((e = launch_chained(k_sample_collect, (unsigned)blocks, kThreads, 0, s, p)) != cudaSuccess) return e;
-  if (p.bin_off != nullptr)
-    return launch_chained(k_sample_rank_bins, (unsigned)((p.cap_sure + p.cap_boundary + 31) / 32), 256, 0, s, p, cand_out);
-  if (p.cap_sure <= kDirectMax && p.cap_boundary <= kDirectMax) {
-    const int ctas = (p.cap_sure + kDirectKeys - 1) / kDirectKeys + (p.cap_boundary + kDirectKeys - 1) / kDirectKeys;
-    return launch_chained(k_sample_rank_direct, ctas, 256, 0, s, p, cand_out);
-  }
-  const int chunks = (p.cap_sure + kChunk - 1) / kChunk + (p.cap_boundary + kChunk - 1) / kChunk;
-  if ((e = launch_chained(k_sample_sort_chunks, chunks, 512, 0, s, p)) != cudaSuccess) return e;
-  return launch_chained(k_sample_rank, chunks, 512, 0, s, p, cand_out);
+  return launch_chained(k_sample_rank_bins, (unsigned)((p.cap_sure + p.cap_boundary + 31) / 32), 256, 0, s, p, cand_out);
 }
 
 }  // namespace strads
@@ -687,20 +546,23 @@ cudaError_t launch_sample(const Problem& p, int* cand_out, cudaStream_t s) {
 // ------------------------------------------------------------------------------------------------
 // strads_sample_static: the same candidate draw for callers that cannot allocate device memory.
 //
-// The select passes need scratch memory (a 4096-bin histogram, two key buffers, a few counters).
+// The draw needs scratch memory (a 4096-bin histogram and as many cursors, a buffer of keys, a few counters).
 // The handle-based path carves it out of the caller's workspace; here it lives in one file-scope
 // device array of fixed size, so a caller that may not call cudaMalloc -- code running inside
 // somebody else's memory pool, a plugin whose host forbids allocation after start-up, a real-time
-// loop -- still gets the draw.  Every GPU that loads the library holds these ~65 KB until exit.
+// loop -- still gets the draw.  Every GPU that loads the library holds these ~82 KB until exit.
 // ------------------------------------------------------------------------------------------------
 namespace strads {
 namespace {
 
+constexpr int kStaticTurns = 32;           // barriers that calls take in turn
+constexpr int kStaticBoundary = STRADS_STATIC_MAX_CANDIDATES / 2;
 struct StaticSampleScratch {
   DeviceState st;
-  unsigned int hist[kHistBins];
-  unsigned long long sure[STRADS_STATIC_MAX_CANDIDATES];
-  unsigned long long boundary[STRADS_STATIC_MAX_CANDIDATES / 2];
+  EngineState es[kStaticTurns];
+  __align__(16) unsigned int hist[kHistBins];
+  unsigned int bin_cur[kHistBins];
+  unsigned long long win[STRADS_STATIC_MAX_CANDIDATES + kStaticBoundary];
 };
 
 static __device__ __align__(256) unsigned char g_static_sample_scratch[sizeof(StaticSampleScratch)];
@@ -709,8 +571,7 @@ constexpr int kMaxDevices = 64;
 std::mutex g_static_mutex;
 StaticSampleScratch* g_static_ptr[kMaxDevices] = {};   // device address of the array, per device
 int g_static_sms[kMaxDevices] = {};
-
-__global__ void k_static_set_round(StaticSampleScratch* sc, unsigned long long t) { sc->st.round = t; }
+unsigned int g_static_calls[kMaxDevices] = {};
 
 }  // namespace
 }  // namespace strads
@@ -728,6 +589,7 @@ extern "C" int strads_sample_static(const float* delta_dev, int64_t n_cols, floa
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return STRADS_ERR_CUDA;
   StaticSampleScratch* sc = nullptr;
   int sms = 0;
+  unsigned int call = 0;
   {
     // once per device, with that device current: in host code the array's name is only a stand-in,
     // the address a kernel can use comes from cudaGetSymbolAddress
@@ -737,31 +599,33 @@ extern "C" int strads_sample_static(const float* delta_dev, int64_t n_cols, floa
       if (cudaGetSymbolAddress(&ptr, g_static_sample_scratch) != cudaSuccess || ptr == nullptr) return STRADS_ERR_CUDA;
       if (cudaDeviceGetAttribute(&g_static_sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return STRADS_ERR_CUDA;
+      if (prepare_draw() != cudaSuccess) return STRADS_ERR_CUDA;
       g_static_ptr[dev] = static_cast<StaticSampleScratch*>(ptr);
     }
     sc = g_static_ptr[dev];
     sms = g_static_sms[dev];
+    call = g_static_calls[dev]++;
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // the array keeps whatever the last call left: counters, tickets and histogram must start at zero
-  if (cudaMemsetAsync(sc, 0, offsetof(StaticSampleScratch, sure), s) != cudaSuccess) return STRADS_ERR_CUDA;
-  k_static_set_round<<<1, 1, 0, s>>>(sc, t);
-
+  // The array starts as zeros and a call leaves it so (the histogram, its own barrier; cursors are cleared when they are
+  // wanted).  Should a call be cut short, the next one clears the histogram again and a later one that call's barrier.
   Problem p = {};
+  p.layout = STRADS_DENSE_COLMAJOR;
   p.J = n_cols;
   p.delta = const_cast<float*>(delta_dev);
   p.eta = eta;
   p.seed = seed;
   p.flags = flags;
   p.n_cand = n_candidates;
-  p.n_keep = 1;
   p.st = &sc->st;
-  p.hist = sc->hist;
-  p.sure = sc->sure;
-  p.boundary = sc->boundary;
-  p.cap_sure = n_candidates;
-  p.cap_boundary = STRADS_STATIC_MAX_CANDIDATES / 2;
+  p.cand = cand_dev;
   p.sm_count = sms;
-  p.round_ptr = &sc->st.round;
-  return launch_sample(p, cand_dev, s) == cudaSuccess ? STRADS_OK : STRADS_ERR_CUDA;
+  Engine e = {};
+  e.es = &sc->es[call % kStaticTurns];
+  e.hist = sc->hist;
+  e.bin_cur = sc->bin_cur;
+  e.win = sc->win;
+  e.cap_win = n_candidates + kStaticBoundary;
+  e.cap_boundary = kStaticBoundary;
+  return launch_draw(p, e, t, &sc->es[(call + kStaticTurns / 2) % kStaticTurns], s) == cudaSuccess ? STRADS_OK : STRADS_ERR_CUDA;
 }

@@ -22,8 +22,7 @@ struct DeviceState {
   unsigned long long totals[4]; // rounds, examined, kept, nonzero
   unsigned int status;          // STRADS_STATUS_* bits
   unsigned int hist_ticket;     // "last block done" tickets
-  unsigned int sure_count;      // append cursors of the collect kernel
-  unsigned int boundary_count;
+  unsigned int boundary_count;  // append cursor of the collect kernel
   int counts[4];                // n_cand, n_examined, n_kept, n_nonzero of the current round
   SelectState sel;
   double objective;             // result slot of the objective reduction
@@ -137,7 +136,7 @@ struct Problem {
   const unsigned long long* round_ptr;   // the sampler's round index is *round_ptr + round_ahead
   int round_ahead;
   unsigned long long* keys_out;          // sampler: if set, the winners' keys in rank order go here too
-  int* bin_off;                          // sampler: [kHistBins + 1] where the sure keys of a histogram bin start in `sure` (null: appended in any order)
+  int* bin_off;                          // sampler: [kHistBins + 1] where the sure keys of a histogram bin start in `sure`
   unsigned int* bin_cur;                 // sampler: [kHistBins] append cursor of every bin
   unsigned long long* survivors;         // sampler: [cap_survivors] keys below the guided first pass's cutoff (null: not kept)
   int cap_survivors;
