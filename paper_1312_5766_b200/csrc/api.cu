@@ -188,7 +188,7 @@ struct Layout {
       off_conflict, off_cand_dbeta64, off_cand_bnew, off_dot_partial, off_dot_ticket, off_margin, off_obj, off_amb, off_xcb, off_walk_blocked, off_walk_ctl, off_walk_cols,
       off_bucket_count, off_bucket_items, off_bucket_vals, off_bucket_cols, off_resid_acc, off_delta_prev, off_edges, off_patch_keys, off_cand_keys, off_survivors, off_bin_off, off_bin_cur, off_ahead_bin_off, off_ahead_bin_cur,
       off_ahead_state, off_ahead_hist, off_ahead_sure, off_ahead_boundary, off_ahead_keys, off_ahead_idx,
-      off_eng_state, off_eng_hist, off_eng_cur, off_eng_win, off_eng_surv, off_eng_xb, off_eng_norm, off_eng_part, off_eng_tickets, total;
+      off_eng_state, off_eng_hist, off_eng_cur, off_eng_win, off_eng_surv, off_eng_saved, off_eng_xb, off_eng_norm, off_eng_part, off_eng_tickets, total;
   long long eng_pitch, eng_lo;
   int eng_list, eng_tiles;
   bool engine;
@@ -228,6 +228,8 @@ bool engine_chosen(const strads_lasso_config_t* c) {
   if (!engine_wanted(c) || n_sched_of(c) > 1) return false;
   return c->layout == STRADS_CSC || (double)c->n_rows * (double)c->rho * (double)c->rho <= 9.0;
 }
+// Keys each CTA can save of a scan that finds a few times `winners` of them in all.
+unsigned int engine_saved(size_t winners) { return (unsigned int)(winners / 16 + 64); }
 size_t engine_boundary(size_t winners) { return winners / 2 > 2048 ? winners / 2 : 2048; }
 
 // Slice of the workspace of one scheduler; the first one (`first`) also holds what all share
@@ -278,7 +280,7 @@ Layout carve(const strads_lasso_config_t* c, bool first = true) {
   L.buckets = csc && (size_t)c->n_rows * kBucketSlots * sizeof(int) <= ((size_t)64 << 20);
   L.off_bucket_count = take(L.buckets ? sizeof(unsigned int) * (size_t)c->n_rows : 0);
   L.off_bucket_items = take(L.buckets ? sizeof(int) * (size_t)c->n_rows * kBucketSlots : 0);
-  L.off_bucket_vals = take(L.buckets ? sizeof(float) * (size_t)c->n_rows * kBucketSlots : 0);
+  L.off_bucket_vals = take(L.buckets ? sizeof(float) * (size_t)c->n_rows * kBucketSlots : 0);   // (directly behind: the engine keeps pairs there)
   L.off_bucket_cols = take(L.buckets ? sizeof(BucketColumn) * (size_t)c->n_candidates : 0);
   L.off_resid_acc = take(csc ? sizeof(long long) * (size_t)c->n_rows : 0);
   L.off_delta_prev = take(sizeof(float) * (size_t)c->n_keep);
@@ -316,13 +318,14 @@ Layout carve(const strads_lasso_config_t* c, bool first = true) {
   L.off_eng_hist = take(en ? sizeof(unsigned int) * kHistBins : 0);
   L.off_eng_cur = take(en ? sizeof(unsigned int) * kHistBins : 0);
   L.off_eng_win = take(en ? sizeof(unsigned long long) * (most + engine_boundary(most)) : 0);
-  L.off_eng_surv = take(en ? sizeof(unsigned long long) * (8 * most + 1024) : 0);
+  L.off_eng_surv = take(en ? sizeof(unsigned long long) * kEngineMaxCtas * (size_t)engine_saved(most) : 0);
+  L.off_eng_saved = take(en ? sizeof(unsigned int) * kEngineMaxCtas : 0);
   L.eng_lo = (c->n_rows + 127) / 128 * 128;
   L.eng_pitch = 2 * L.eng_lo;
   const int side = (c->n_candidates + 63) / 64;
   L.eng_tiles = en && dense ? side * (side + 1) / 2 : 0;
   L.off_eng_xb = take(en && dense ? sizeof(unsigned short) * (size_t)c->n_candidates * L.eng_pitch : 0);
-  L.off_eng_norm = take(en && dense ? sizeof(double) * (size_t)c->n_candidates : 0);
+  L.off_eng_norm = take(en ? sizeof(double) * (size_t)c->n_candidates : 0);
   L.off_eng_part = take(en && dense ? sizeof(float) * 128 * 128 * (size_t)kEngineMaxCtas : 0);
   L.off_eng_tickets = take(sizeof(unsigned int) * (size_t)L.eng_tiles);
   L.total = o;
@@ -580,6 +583,7 @@ void fill_problem(Problem& p, const strads_lasso_config_t* c, const Layout& L, c
   p.bucket_count = L.buckets ? reinterpret_cast<unsigned int*>(ws + L.off_bucket_count) : nullptr;
   p.bucket_items = L.buckets ? reinterpret_cast<int*>(ws + L.off_bucket_items) : nullptr;
   p.bucket_vals = L.buckets ? reinterpret_cast<float*>(ws + L.off_bucket_vals) : nullptr;
+  p.bucket_pairs = L.buckets ? reinterpret_cast<int2*>(ws + L.off_bucket_items) : nullptr;
   p.bucket_cols = L.buckets ? reinterpret_cast<BucketColumn*>(ws + L.off_bucket_cols) : nullptr;
   p.part_count = S; p.part_index = s;
   p.sm_count = first ? first->sm_count : 0;
@@ -626,12 +630,14 @@ void fill_engine(Engine& en, const Problem& p, const Layout& L, char* ws) {
   en.cap_boundary = (int)engine_boundary(most);
   en.cap_win = (int)most + en.cap_boundary;
   en.surv = reinterpret_cast<unsigned long long*>(ws + L.off_eng_surv);
-  en.cap_surv = (unsigned)(8 * most + 1024);
+  en.saved = reinterpret_cast<unsigned int*>(ws + L.off_eng_saved);
+  en.cap_surv = engine_saved(most);
   en.n_list = L.eng_list;
   en.window = window_of(p, p.n_cand);
   en.xb = reinterpret_cast<unsigned short*>(ws + L.off_eng_xb);
   en.xb_pitch = L.eng_pitch; en.lo_off = L.eng_lo;
   en.norm = reinterpret_cast<double*>(ws + L.off_eng_norm);
+  en.norm_f = reinterpret_cast<float*>(ws + L.off_eng_norm);
   en.part = reinterpret_cast<float*>(ws + L.off_eng_part);
   en.tile_ticket = reinterpret_cast<unsigned int*>(ws + L.off_eng_tickets);
 }

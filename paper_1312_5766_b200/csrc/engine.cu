@@ -73,6 +73,33 @@ __device__ bool grid_sync(Grid& g, bool withhold = false) {
   return s_ok != 0;
 }
 
+// The same, with work for the other warps while the first one waits: step() until it has nothing left or the wait is over.
+template <typename Step>
+__device__ __forceinline__ bool grid_sync_busy(Grid& g, Step&& step) {
+  __shared__ int s_ok;
+  __shared__ volatile int s_over;
+  g.target += g.n;
+  if (threadIdx.x == 0) s_over = 0;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(g.count) : "memory");
+    unsigned int v, it = 0;
+    bool ok;
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(g.count) : "memory");
+      ok = v - g.target < g.n;
+    } while (!ok && ++it < g.limit);
+    if (!ok) atomicOr(g.status, STRADS_STATUS_WAIT_EXPIRED);
+    s_ok = ok;
+    s_over = 1;
+  } else if (threadIdx.x >= 32) {
+#pragma unroll 1
+    while (!s_over && step()) {}
+  }
+  __syncthreads();
+  return s_ok != 0;
+}
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
@@ -82,7 +109,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 // ------------------------------------------------------------------------------------------------
 // The draw (SAP step 1; the keys and their order are those of sampler.cu).
 //
-// scan     every key below the cutoff carried over from the last draw is binned and saved; the others are recognised
+// scan     every key below the cutoff carried over from the last draw is binned and saved (by each CTA in a stretch of
+//          its own: one counter for all was 2,400 additions to one address, 3.5 us); the others are recognised
 //          from a few operations (T >= v / w with v = (x + 1/2) 2^-32) and not computed.  Without a cutoff all keys
 //          are computed and binned by their top 12 bits.
 // select   every CTA reads the 4,096 counts, scans them and finds the bin that holds the n_list-th key -- the same in
@@ -90,21 +118,26 @@ __device__ __forceinline__ double warp_sum(double v) {
 // collect  the keys up to that bin, saved ones if the scan saved them all, go to `win`, grouped by bin.
 // rank     a key's rank is the start of its group plus the smaller keys inside it.
 //
-// With a cutoff the bins are 64 per octave below it (bits 17 and up of the binary32 time, counted down from the
-// cutoff's): the winners of an exponential race spread over the top octaves, so a group holds P' / 128 keys or fewer
-// where 8 bins per octave (the unguided scan) leave P' / 16.
+// With a cutoff the bins are 128 per octave for the 24 octaves below it and 16 per octave for 64 more, by the distance of
+// the time's bits from the cutoff's: the winners of an exponential race spread over the top octaves, so a group holds
+// P' / 256 keys or fewer where 8 bins per octave (the unguided scan) leave P' / 16; the coarse ones are for rounds in which
+// coefficients never touched (times 10^14 times smaller) and coefficients at rest are drawn together.
 // ------------------------------------------------------------------------------------------------
-struct Binning { unsigned int shift, base; };
+constexpr unsigned int kFineSpan = 24u << 23;            // bits of time: 24 octaves, 3,072 bins
+constexpr int kCoarseBins = kHistBins - 3072;
+struct Binning { unsigned int cut; };                    // bits of the cutoff; 0: none
 __device__ __forceinline__ Binning binning_of(float cut) {
   Binning b;
-  b.shift = cut > 0.f ? 17u : 32u - kHistBits;
-  const unsigned int top = __float_as_uint(cut) >> 17;
-  b.base = cut > 0.f && top > (unsigned)(kHistBins - 1) ? top - (kHistBins - 1) : 0u;
+  b.cut = cut > 0.f ? __float_as_uint(cut) : 0u;
   return b;
 }
 __device__ __forceinline__ unsigned int bin_of(const Binning& b, unsigned int bits) {
-  const unsigned int x = bits >> b.shift;
-  return x > b.base ? min(x - b.base, (unsigned)(kHistBins - 1)) : 0u;
+  if (b.cut == 0u) return min(bits >> (32 - kHistBits), (unsigned)(kHistBins - 1));
+  if (bits >= b.cut) return kHistBins - 1;
+  const unsigned int d = b.cut - bits;
+  if (d < kFineSpan) return kHistBins - 1 - (d >> 16);
+  const unsigned int c = (d - kFineSpan) >> 19;
+  return c < (unsigned)kCoarseBins ? kCoarseBins - 1 - c : 0u;
 }
 
 constexpr int kQueue = 192;                // survivors of a warp waiting for their keys; a step appends at most 128
@@ -122,6 +155,7 @@ struct DrawShared {
   unsigned long long prefix;               // refined: keys of the boundary bin whose top `bits` bits exceed it are no winners
   int bits;
   float cut;                               // cutoff of the scan
+  unsigned int saved;                      // keys below it that this CTA saved
 };
 
 // w_j = fma(x, y, z) for every importance distribution: (|d|, |d|, eta), (|d|, 1, eta) or (0, 0, 1) -- the same bits as
@@ -142,99 +176,122 @@ __device__ __forceinline__ unsigned long long key_of(const WeightForm& f, float 
   return ((unsigned long long)__float_as_uint(__fdiv_rn(unit_exponential_rn(word), weight_of(f, d))) << 32) | j;
 }
 
-// A warp's share of a scan.  f(key, active) is called by whole warps.
+// A warp's share of a scan, step by step: 128 coefficients at a time; those whose keys may lie below the cutoff wait in a
+// queue of the warp's in shared memory until there are enough of them for all lanes.  f(key, active) is called by whole warps.
+struct WarpScan {
+  uint2* queue;
+  long long next, step;                    // Philox block of the warp's next step, and between two
+  int n;                                   // in the queue
+  float k;                                 // x 2^-32 > 1.02 cut w implies T > cut: the computed E is never below (x + 1/2) 2^-32 up to rounding
+};
+__device__ __forceinline__ WarpScan begin_scan(float cut, uint2* queue, int warp0, int n_warps) {
+  WarpScan s;
+  s.queue = queue; s.next = (long long)warp0 * 32; s.step = (long long)n_warps * 32; s.n = 0;
+  s.k = cut > 0.f ? __fmul_rn(cut, 1.02f * 4294967296.0f) : __uint_as_float(0x7f800000u);
+  return s;
+}
+// One step; past the end it only empties the queue.  Whether there was anything to do.
+template <typename F>
+__device__ __forceinline__ bool scan_step(const Problem& p, unsigned long long t, const WeightForm& wf, WarpScan& s, F&& f) {
+  const int lane = threadIdx.x & 31;
+  const long long groups = (p.J + 3) >> 2, whole = p.J >> 2, g = s.next + lane;
+  const bool more = s.next < groups;
+  if (!more && s.n == 0) return false;
+  if (more) {
+    float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (g < whole) {
+      d = __ldcg(reinterpret_cast<const float4*>(p.delta) + g);
+    } else if (g < groups) {
+      const long long j = g << 2;
+      d.x = p.delta[j];
+      if (j + 1 < p.J) d.y = p.delta[j + 1];
+      if (j + 2 < p.J) d.z = p.delta[j + 2];
+    }
+    uint32_t w[4];
+    philox4x32_10((uint32_t)g, (uint32_t)t, (uint32_t)(t >> 32), 0u, (uint32_t)p.seed, (uint32_t)(p.seed >> 32), w);
+    const float dd[4] = {d.x, d.y, d.z, d.w};
+    bool in[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) in[i] = !(__uint2float_rn(w[i]) > __fmul_rn(s.k, weight_of(wf, dd[i])));
+    if (g >= whole) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) in[i] = in[i] && (g << 2) + i < p.J;
+    }
+    s.next += s.step;
+    if (!__any_sync(kFull, in[0] | in[1] | in[2] | in[3])) return true;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const unsigned int m = __ballot_sync(kFull, in[i]);
+      if (in[i]) s.queue[s.n + __popc(m & ((1u << lane) - 1u))] = make_uint2((uint32_t)(g << 2) + i, w[i]);
+      s.n += __popc(m);
+    }
+  }
+  if (s.n > kQueue - 128 || !more) {                     // the keys of the survivors, computed by all lanes together
+    __syncwarp();
+#pragma unroll 1
+    for (int i = 0; i < s.n; i += 32) {
+      const bool on = i + lane < s.n;
+      const uint2 e = on ? s.queue[i + lane] : make_uint2(0u, 0u);
+      f(on ? key_of(wf, p.delta[e.x], e.y, e.x) : ~0ull, on);
+    }
+    __syncwarp();
+    s.n = 0;
+  }
+  return true;
+}
 template <typename F>
 __device__ __forceinline__ void scan_keys(const Problem& p, unsigned long long t, float cut, uint2* queue, int warp0, int n_warps, F&& f) {
-  const int lane = threadIdx.x & 31;
-  const long long groups = (p.J + 3) >> 2, whole = p.J >> 2;
   const WeightForm wf = weight_form(p);
-  // x 2^-32 > 1.02 cut w implies T > cut: the computed E is never below (x + 1/2) 2^-32 up to rounding
-  const float k = cut > 0.f ? __fmul_rn(cut, 1.02f * 4294967296.0f) : __uint_as_float(0x7f800000u);
-  int n = 0;
-  const long long step = (long long)n_warps * 32;
-  // (one trip more than there are steps: the last one only empties the queue)
-  for (long long g0 = (long long)warp0 * 32;; g0 += step) {
-    const bool more = g0 < groups;
-    if (more) {
-      const long long g = g0 + lane;
-      float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (g < whole) {
-        d = __ldcg(reinterpret_cast<const float4*>(p.delta) + g);
-      } else if (g < groups) {
-        const long long j = g << 2;
-        d.x = p.delta[j];
-        if (j + 1 < p.J) d.y = p.delta[j + 1];
-        if (j + 2 < p.J) d.z = p.delta[j + 2];
-      }
-      uint32_t w[4];
-      philox4x32_10((uint32_t)g, (uint32_t)t, (uint32_t)(t >> 32), 0u, (uint32_t)p.seed, (uint32_t)(p.seed >> 32), w);
-      const float dd[4] = {d.x, d.y, d.z, d.w};
-      bool in[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) in[i] = !(__uint2float_rn(w[i]) > __fmul_rn(k, weight_of(wf, dd[i])));
-      if (g >= whole) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) in[i] = in[i] && (g << 2) + i < p.J;
-      }
-      if (!__any_sync(kFull, in[0] | in[1] | in[2] | in[3])) continue;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const unsigned int m = __ballot_sync(kFull, in[i]);
-        if (in[i]) queue[n + __popc(m & ((1u << lane) - 1u))] = make_uint2((uint32_t)(g << 2) + i, w[i]);
-        n += __popc(m);
-      }
-    }
-    if (n > kQueue - 128 || !more) {                     // the keys of the survivors, computed by all lanes together
-      __syncwarp();
+  WarpScan s = begin_scan(cut, queue, warp0, n_warps);
 #pragma unroll 1
-      for (int i = 0; i < n; i += 32) {
-        const bool on = i + lane < n;
-        const uint2 e = on ? queue[i + lane] : make_uint2(0u, 0u);
-        f(on ? key_of(wf, p.delta[e.x], e.y, e.x) : ~0ull, on);
-      }
-      __syncwarp();
-      n = 0;
-    }
-    if (!more) break;
-  }
+  while (scan_step(p, t, wf, s, f)) {}
 }
 
 // Shared memory of a scan: the CTA's histogram, then a queue per warp.
 constexpr size_t kScanSmem = sizeof(unsigned int) * kHistBins + sizeof(uint2) * kQueue * kWarps;
 
-// guided: with the cutoff es->t_cut (if there is one).  Also clears the cursors of the groups.
-__device__ __forceinline__ void draw_scan(const Problem& p, const Engine& e, DrawShared& ds, unsigned char* sm, unsigned long long t, bool guided) {
+// A scan in parts: it can be made in the waits of other work.  guided: with the cutoff es->t_cut (if there is one).
+__device__ __forceinline__ float scan_open(const Engine& e, DrawShared& ds, unsigned char* sm, bool guided) {
   unsigned int* sh = reinterpret_cast<unsigned int*>(sm);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint2* queue = reinterpret_cast<uint2*>(sm + sizeof(unsigned int) * kHistBins) + warp * kQueue;
+  const int tid = threadIdx.x;
   const float cut = guided ? e.es->t_cut : 0.f;
-  const Binning bins = binning_of(cut);
   __syncthreads();
   for (int b = tid; b < kHistBins; b += kT) sh[b] = 0u;
-  for (int b = (int)blockIdx.x * kT + tid; b < kHistBins; b += (int)gridDim.x * kT) e.bin_cur[b] = 0u;
-  if (tid == 0) ds.cut = cut;
+  for (int b = (int)blockIdx.x * kT + tid; b < kHistBins; b += (int)gridDim.x * kT) e.bin_cur[b] = 0u;     // the cursors of the groups
+  if (tid == 0) { ds.cut = cut; ds.saved = 0u; }
   __syncthreads();
-  // (a warp takes its steps round-robin over the CTAs: a few thousand coefficients already use every SM)
-  const int w0 = warp * (int)gridDim.x + (int)blockIdx.x, nw = kWarps * (int)gridDim.x;
-  const unsigned int cut_bits = __float_as_uint(cut);
-  scan_keys(p, t, cut, queue, w0, nw, [&](unsigned long long key, bool on) {
-    const unsigned int bits = (unsigned int)(key >> 32);
-    const bool in = on && (cut == 0.f || bits < cut_bits);
-    if (in) atomicAdd(&sh[bin_of(bins, bits)], 1u);
-    if (cut > 0.f) {
-      const unsigned int m = __ballot_sync(kFull, in);
-      if (m == 0u) return;
-      unsigned int at = 0u;
-      if (lane == 0) at = atomicAdd(&e.es->surv_count, (unsigned)__popc(m));
-      at = __shfl_sync(kFull, at, 0) + __popc(m & ((1u << lane) - 1u));
-      if (in && at < e.cap_surv) e.surv[at] = key;
-    }
-  });
+  return cut;
+}
+__device__ __forceinline__ void scan_found(const Engine& e, DrawShared& ds, unsigned int* sh, const Binning& bins, unsigned long long key, bool on) {
+  const unsigned int bits = (unsigned int)(key >> 32);
+  if (!on || (bins.cut != 0u && bits >= bins.cut)) return;
+  atomicAdd(&sh[bin_of(bins, bits)], 1u);
+  if (bins.cut != 0u) {
+    const unsigned int at = atomicAdd(&ds.saved, 1u);
+    if (at < e.cap_surv) e.surv[(size_t)blockIdx.x * e.cap_surv + at] = key;
+  }
+}
+__device__ __forceinline__ void scan_close(const Engine& e, const DrawShared& ds, unsigned char* sm) {
+  const unsigned int* sh = reinterpret_cast<const unsigned int*>(sm);
   __syncthreads();
-  for (int b = tid; b < kHistBins; b += kT) {
+  if (threadIdx.x == 0) e.saved[blockIdx.x] = ds.saved;
+  for (int b = threadIdx.x; b < kHistBins; b += kT) {
     const unsigned int v = sh[b];
     if (v) atomicAdd(&e.hist[b], v);
   }
+}
+__device__ __forceinline__ uint2* scan_queue(unsigned char* sm) {
+  return reinterpret_cast<uint2*>(sm + sizeof(unsigned int) * kHistBins) + (threadIdx.x >> 5) * kQueue;
+}
+
+// (a warp takes its steps round-robin over the CTAs: a few thousand coefficients already use every SM)
+__device__ __forceinline__ void draw_scan(const Problem& p, const Engine& e, DrawShared& ds, unsigned char* sm, unsigned long long t, bool guided) {
+  unsigned int* sh = reinterpret_cast<unsigned int*>(sm);
+  const float cut = scan_open(e, ds, sm, guided);
+  const Binning bins = binning_of(cut);
+  scan_keys(p, t, cut, scan_queue(sm), (int)(threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x, kWarps * (int)gridDim.x,
+            [&](unsigned long long key, bool on) { scan_found(e, ds, sh, bins, key, on); });
+  scan_close(e, ds, sm);
 }
 
 // The bin b with before(b) < k <= before(b) + count(b), and the winners before every bin (ds.total < k: there is none).
@@ -274,7 +331,11 @@ __device__ void draw_select(const Engine& e, DrawShared& ds, unsigned int k) {
 // Upper edge of the boundary bin, as the bits of a binary32 time.
 __device__ __forceinline__ unsigned int boundary_edge(const DrawShared& ds) {
   const Binning b = binning_of(ds.cut);
-  const unsigned long long x = (unsigned long long)(b.base + (unsigned)ds.bnd + 1u) << b.shift;
+  const unsigned int bin = (unsigned)ds.bnd;
+  unsigned long long x;
+  if (b.cut == 0u) x = (unsigned long long)(bin + 1u) << (32 - kHistBits);
+  else if (bin >= (unsigned)kCoarseBins) x = b.cut - ((kHistBins - 1u - bin) << 16) + 1u;
+  else x = b.cut - kFineSpan - ((kCoarseBins - 1u - bin) << 19) + 1u;
   return x < 0x7f800000ull ? (unsigned int)x : 0x7f800000u;
 }
 
@@ -296,12 +357,16 @@ __device__ __noinline__ void draw_collect_all(const Problem& p, const Engine& e,
             [&](unsigned long long key, bool on) { if (on) take_winner(e, ds, bins, key); });
 }
 
-// ... from the keys the scan saved.
+// ... from the keys the scan saved: every CTA its own, and a share of the last one's where that has other work.
 __device__ __forceinline__ void draw_collect(const Engine& e, const DrawShared& ds, bool spare_last) {
-  const unsigned int n_ctas = gridDim.x - (spare_last && gridDim.x > 1 ? 1u : 0u), n_surv = __ldcg(&e.es->surv_count);
   const Binning bins = binning_of(ds.cut);
+  const unsigned int own = ds.saved, more = spare_last ? __ldcg(e.saved + gridDim.x - 1u) : 0u;
+  const unsigned long long* mine = e.surv + (size_t)blockIdx.x * e.cap_surv;
+  const unsigned long long* its = e.surv + (size_t)(gridDim.x - 1u) * e.cap_surv;
 #pragma unroll 1
-  for (unsigned int i = threadIdx.x * n_ctas + blockIdx.x; i < n_surv; i += n_ctas * kT) take_winner(e, ds, bins, __ldcg(e.surv + i));
+  for (unsigned int i = threadIdx.x; i < own; i += kT) take_winner(e, ds, bins, __ldcg(mine + i));
+#pragma unroll 1
+  for (unsigned int i = threadIdx.x * (gridDim.x - 1u) + blockIdx.x; i < more; i += kT * (gridDim.x - 1u)) take_winner(e, ds, bins, __ldcg(its + i));
 }
 
 // Rare: more keys share the boundary bin than there is room for (thousands of tied times).  The grid cuts the bin
@@ -367,8 +432,10 @@ __device__ __noinline__ bool draw_refine(const Problem& p, const Engine& e, Draw
 __device__ __forceinline__ void draw_gather(const Problem& p, const Engine& e, DrawShared& ds, unsigned long long t, unsigned int k, bool spare_last) {
   if (spare_last && gridDim.x > 1 && blockIdx.x == gridDim.x - 1) return;
   draw_select(e, ds, k);
-  if (ds.total < k || ds.bnd_count > (unsigned)e.cap_boundary || (ds.cut > 0.f ? __ldcg(&e.es->surv_count) > e.cap_surv : true)) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) e.es->mend = 1;
+  // (a stretch that overflowed is seen by its owner alone: the others' winners are collected all the same, and again)
+  const bool too_many = ds.saved > e.cap_surv || (spare_last && blockIdx.x == 0 && __ldcg(e.saved + gridDim.x - 1u) > e.cap_surv);
+  if (ds.total < k || ds.bnd_count > (unsigned)e.cap_boundary || ds.cut == 0.f || too_many) {
+    if (threadIdx.x == 0 && (blockIdx.x == 0 || too_many)) e.es->mend = 1;
     return;
   }
   draw_collect(e, ds, spare_last);
@@ -388,6 +455,8 @@ __device__ __noinline__ bool draw_mend(const Problem& p, const Engine& e, DrawSh
     draw_select(e, ds, k);
   }
   if (ds.bnd_count > (unsigned)e.cap_boundary && !draw_refine(p, e, ds, sm, t, k, g)) return false;
+  for (int b = (int)blockIdx.x * kT + (int)threadIdx.x; b < kHistBins; b += (int)gridDim.x * kT) e.bin_cur[b] = 0u;
+  if (!grid_sync(g)) return false;
   draw_collect_all(p, e, ds, sm, t);
   return grid_sync(g);
 }
@@ -464,14 +533,14 @@ __device__ int gather_changes(const Problem& p, int nk, bool want_keys, unsigned
 }
 
 // Winners ranked; with changes, corrected for the kept coefficients' changed priorities (keys[0 .. n_changed) old,
-// keys[p.n_keep ..) new).  Eight lanes per winner.  A key's place among the changed ones: those in lower bins from
-// a prefix sum over the bins, those in its own bin one by one (a list per bin); a plain count while they are few.
+// keys[p.n_keep ..) new).  A key's place among the changed ones: those in lower bins from a prefix sum over the bins, those
+// in its own bin one by one (a list per bin); a plain count while they are few.
 // Leaves the draw's buffers as the next scan expects them.
 constexpr int kFewChanged = 48;
 template <bool kDense>
 __device__ __forceinline__ void draw_rank(const Problem& p, const Engine& e, const DrawShared& ds, const unsigned long long* keys, ChangedByBin* cb, int n_changed,
                           int nk, int* wsum, int n_rank, int n_prefetch) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, slice = lane & 7;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if ((int)blockIdx.x >= n_rank) return;
   const Binning bins = binning_of(ds.cut);
   const unsigned int bnd = (unsigned)ds.bnd;
@@ -511,9 +580,12 @@ __device__ __forceinline__ void draw_rank(const Problem& p, const Engine& e, con
   }
   const int items = (int)total + (n_changed > 0 ? nk : 0);   // (new keys by place in the kept list: the order of `keys` is each CTA's own)
   const int shift = 64 - ds.bits;
-  #pragma unroll 1
-  for (int i0 = (warp * n_rank + (int)blockIdx.x) * 4; i0 < items; i0 += kWarps * n_rank * 4) {
-    const int i = i0 + (lane >> 3);
+  // lanes per winner: two where there are too many, eight for the larger groups of an unguided draw
+  const int share = items * 4 > n_rank * kT ? 1 : (bins.cut == 0u && items * 8 <= n_rank * kT ? 3 : 2);
+  const int lanes = 1 << share, slice = lane & (lanes - 1), per_warp = 32 >> share;
+#pragma unroll 1
+  for (int i0 = (warp * n_rank + (int)blockIdx.x) * per_warp; i0 < items; i0 += kWarps * n_rank * per_warp) {
+    const int i = i0 + (lane >> share);
     const bool fresh = i >= (int)total;
     unsigned long long key = 0ull;
     bool on = i < items;
@@ -535,15 +607,17 @@ __device__ __forceinline__ void draw_rank(const Problem& p, const Engine& e, con
     unsigned int first = 0u, count = 0u;
     if (on) { first = behind ? total : ds.off[pad((int)bin)]; count = behind ? 0u : (bin < bnd ? ds.off[pad((int)bin + 1)] : total) - first; }
     int below = 0, struck = 0;
-    for (unsigned int k0 = slice; k0 < count; k0 += 64) {
+#pragma unroll 1
+    for (unsigned int k0 = slice; k0 < count; k0 += 8 * lanes) {
       unsigned long long v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = k0 + 8 * u < count ? __ldcg(e.win + first + k0 + 8 * u) : ~0ull;
+      for (int u = 0; u < 8; ++u) v[u] = k0 + lanes * u < count ? __ldcg(e.win + first + k0 + lanes * u) : ~0ull;
 #pragma unroll
       for (int u = 0; u < 8; ++u) below += v[u] < key;
     }
     if (!indexed) {
-      for (int a = slice; a < n_changed; a += 8) {
+#pragma unroll 1
+      for (int a = slice; a < n_changed; a += lanes) {
         const unsigned long long o = old_k[a];
         below -= o < key;
         struck |= o == key;
@@ -561,8 +635,8 @@ __device__ __forceinline__ void draw_rank(const Problem& p, const Engine& e, con
         }
       }
     }
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {
+#pragma unroll 1
+    for (int o = 1; o < lanes; o <<= 1) {
       below += __shfl_xor_sync(kFull, below, o);
       struck |= __shfl_xor_sync(kFull, struck, o);
     }
@@ -577,6 +651,7 @@ __device__ __forceinline__ void draw_rank(const Problem& p, const Engine& e, con
         WalkColumn col;
         col.q0 = q0; col.n = (int)(q1 - q0); col.j = j; col.n2 = n2; col.unused = 0.0;
         p.walk_cols[rank] = col;
+        e.norm_f[rank] = (float)n2;
         if (rank < n_prefetch) {
           asm volatile("prefetch.global.L2 [%0];" ::"l"(p.xrow + q0));
           asm volatile("prefetch.global.L2 [%0];" ::"l"(p.xv + q0));
@@ -591,7 +666,6 @@ __device__ __forceinline__ void draw_rank(const Problem& p, const Engine& e, con
   // the next scan's buffers and cutoff (everybody read them before the last barrier)
   for (int b = (int)blockIdx.x * kT + tid; b < kHistBins; b += (int)gridDim.x * kT) e.hist[b] = 0u;
   if (blockIdx.x == 0 && tid == 0) {
-    e.es->surv_count = 0u;
     // twice the boundary, which changes little from round to round; more where few winners let it scatter
     const unsigned int edge = boundary_edge(ds);
     e.es->t_cut = edge < 0x7f800000u ? __fmul_rn(p.n_cand < 64 ? 8.0f : 2.0f, __uint_as_float(edge)) : 0.f;
@@ -607,21 +681,28 @@ __device__ __forceinline__ float exponential_of(const Problem& p, unsigned long 
   return unit_exponential_rn((j & 2u) ? ((j & 1u) ? w[3] : w[2]) : ((j & 1u) ? w[1] : w[0]));
 }
 
-__device__ __forceinline__ void propose(const Problem& p, int pos, int j, double n, float b_old, float d_old, double g, float E, bool want_keys) {
-  float b_new = b_old;
-  if (n > 0.0) {
-    const double c = step_scale(p);
-    const double z = (double)b_old + c * g / n;
-    const double m = fabs(z) - c * (double)p.lambda / n;
+// In two parts: what does not depend on g is made while the products are under way.
+struct Proposal { double n, threshold; float b_old; unsigned long long old_key; };
+__device__ __forceinline__ Proposal propose_begin(const Problem& p, int j, double n, float b_old, float d_old, float E, bool want_keys) {
+  Proposal q;
+  q.n = n; q.b_old = b_old;
+  q.threshold = n > 0.0 ? step_scale(p) * (double)p.lambda / n : 0.0;
+  q.old_key = want_keys ? race_key_from(E, d_old, p.eta, (uint32_t)j, weight_mode_of(p.flags)) : 0ull;
+  return q;
+}
+__device__ __forceinline__ void propose_end(const Problem& p, const Proposal& q, int pos, int j, double g, float E, bool want_keys) {
+  float b_new = q.b_old;
+  if (q.n > 0.0) {
+    const double z = (double)q.b_old + step_scale(p) * g / q.n;
+    const double m = fabs(z) - q.threshold;
     b_new = (float)(m <= 0.0 ? 0.0 : (z > 0.0 ? m : -m));
   }
-  const double d = isfinite(g) ? (double)b_new - (double)b_old : g - g;        // a non-finite product shows as NaN
+  const double d = isfinite(g) ? (double)b_new - (double)q.b_old : g - g;      // a non-finite product shows as NaN
   p.cand_bnew[pos] = b_new;
   p.cand_dbeta64[pos] = d;
   if (want_keys) {
-    const int mode = weight_mode_of(p.flags);
-    p.cand_keys[pos] = race_key_from(E, d_old, p.eta, (uint32_t)j, mode);
-    p.cand_keys[p.n_cand + pos] = race_key_from(E, (float)fabs(d), p.eta, (uint32_t)j, mode);
+    p.cand_keys[pos] = q.old_key;
+    p.cand_keys[p.n_cand + pos] = race_key_from(E, (float)fabs(d), p.eta, (uint32_t)j, weight_mode_of(p.flags));
   }
 }
 
@@ -670,10 +751,7 @@ __device__ void commit_changes(const Problem& p, const Engine& e, int nk, int n_
 // waited for each trip (384 columns of 40 KB: 13.8 us, 640 of 80 KB: 31 us).  Every thread holds its rows of r in
 // registers for the whole step.
 // ------------------------------------------------------------------------------------------------
-struct TurnShared {
-  double dot[kTurn][kWarps];
-  float E[kTurn];
-};
+struct TurnShared { double dot[kTurn][kWarps]; };
 struct PackBars { unsigned long long full[kWarps]; unsigned int uses[kWarps]; };
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -781,15 +859,19 @@ __device__ void dense_pack(const Problem& p, const Engine& e, unsigned char* sm,
   int seen = 0;                                          // columns this group has been through
   for (int k0 = 0; k0 < mine; k0 += kTurn) {
     const int turn = min(kTurn, mine - k0);
+    // what the end of the turn needs of a candidate, by the lanes of the last warp
     int j_own = 0;
-    double n_own = 0.0;
-    float b_own = 0.f, d_own = 0.f;
-    if (products && tid < turn) {                        // gathers for the end of the turn, under way meanwhile
-      j_own = p.cand[lo + cta + n_ctas * (k0 + tid)];
-      n_own = p.n2[j_own]; b_own = p.beta[j_own]; d_own = p.delta[j_own];
+    float E = 0.f;
+    Proposal prop = {};
+    bool dormant = false;
+    if (products && warp == kWarps - 1 && lane < turn) {
+      j_own = p.cand[lo + cta + n_ctas * (k0 + lane)];
+      const double n_own = p.n2[j_own];
+      const float b_own = p.beta[j_own], d_own = p.delta[j_own];
+      if (want_keys) E = exponential_of(p, t_next, (uint32_t)j_own);
+      prop = propose_begin(p, j_own, n_own, b_own, d_own, E, want_keys);
+      dormant = (p.flags & STRADS_FLAG_DYNAMIC_DEPS) && b_own == 0.f && d_own == 0.f;      // (coupling_n2)
     }
-    if (products && want_keys && warp == kWarps - 1 && lane < turn)
-      ts.E[lane] = exponential_of(p, t_next, (uint32_t)p.cand[lo + cta + n_ctas * (k0 + lane)]);
     int k = seen * groups + grp - k0;                    // this group's next column, counted from the turn's first
     for (; k < turn; k += groups, ++seen) {
       const int a = lo + cta + n_ctas * (k0 + k);
@@ -850,13 +932,12 @@ __device__ void dense_pack(const Problem& p, const Engine& e, unsigned char* sm,
     }
     if (!products) continue;
     __syncthreads();
-    if (tid < turn) {
-      const int a = lo + cta + n_ctas * (k0 + tid);
+    if (warp == kWarps - 1 && lane < turn) {
+      const int a = lo + cta + n_ctas * (k0 + lane);
       double gsum = 0.0;
-      for (int w = 0; w < group; ++w) gsum += ts.dot[tid][w];
-      const bool dormant = (p.flags & STRADS_FLAG_DYNAMIC_DEPS) && b_own == 0.f && d_own == 0.f;      // (coupling_n2)
-      e.norm[a] = dormant ? 0.0 : sqrt(n_own);
-      propose(p, a, j_own, n_own, b_own, d_own, gsum, want_keys ? ts.E[tid] : 0.f, want_keys);
+      for (int w = 0; w < group; ++w) gsum += ts.dot[lane][w];
+      e.norm[a] = dormant ? 0.0 : sqrt(prop.n);
+      propose_end(p, prop, a, j_own, gsum, E, want_keys);
     }
     __syncthreads();
   }
@@ -1342,29 +1423,42 @@ __device__ __noinline__ void decide_all(const Problem& p, const Engine& e, int n
 // (its terms in a list of the warp's own in shared memory: no barrier), no conflict bits (the walk works from the list
 // of conflicting pairs or forms rows on demand), and x_c^T r with the same visit to the column.
 // ------------------------------------------------------------------------------------------------
-constexpr int kTerms = 512;                              // terms a candidate may collect
-struct WarpTerms { unsigned long long key[kTerms]; float fa[kTerms], fb[kTerms]; unsigned short order[kTerms]; };
-constexpr size_t kTermsSmem = sizeof(WarpTerms) * kWarps;
+constexpr int kMaxWords = STRADS_MAX_CANDIDATES / 32;
+constexpr int kMet = 512;                                // candidates one candidate may meet
+constexpr int kMetSlots = 1024;                          // of the table they are looked up in
+constexpr int kPart = 64;                                // positions of a column at a time
+constexpr unsigned short kFree = 0xffff;
+struct __align__(16) MetTable {
+  int4 entry[kPart];                     // of a position of the column: row, terms before it, value
+  float dot[kMetSlots];
+  unsigned short key[kMetSlots];         // the candidate met (kFree between candidates)
+  unsigned short slot[kMet];             // the slots in use
+  unsigned char pos[kPart * kBucketSlots];   // position of a term
+};
+constexpr int kNear = 8192;                              // candidates whose norms a CTA keeps in shared memory
+constexpr size_t kTermsSmem = sizeof(MetTable) * kWarps + sizeof(float) * kNear;
+static_assert(STRADS_MAX_CANDIDATES < kFree && kPart <= 256, "16 bits per candidate, 8 per position");
 
 // The entries of candidates [0, n) into the buckets of their rows.  Where the columns lie was noted when the candidates
 // were ranked, but for the dependencies dropped at run time (coupling_n2 follows beta and delta).
-__device__ __forceinline__ void csc_enter(const Problem& p, int n, bool buckets) {
+__device__ __forceinline__ void csc_enter(const Problem& p, const Engine& e, int n, bool buckets) {
   const int lane = threadIdx.x & 31;
   const bool dynamic = (p.flags & STRADS_FLAG_DYNAMIC_DEPS) != 0;
   if (!buckets && !dynamic) return;
 #pragma unroll 1
   for (int a = ((int)threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x; a < n; a += kWarps * (int)gridDim.x) {
     const WalkColumn col = p.walk_cols[a];
-    if (dynamic && lane == 0) p.walk_cols[a].n2 = coupling_n2(p, col.j);
+    if (dynamic && lane == 0) {
+      const double n2 = coupling_n2(p, col.j);
+      p.walk_cols[a].n2 = n2;
+      e.norm_f[a] = (float)n2;
+    }
     if (!buckets) continue;
     for (int q = lane; q < col.n; q += 32) {
       const int r = __ldg(p.xrow + col.q0 + q);
       const float v = __ldg(p.xv + col.q0 + q);
       const unsigned int slot = atomicAdd(&p.bucket_count[r], 1u);
-      if (slot < (unsigned)kBucketSlots) {
-        p.bucket_items[(size_t)r * kBucketSlots + slot] = a;
-        p.bucket_vals[(size_t)r * kBucketSlots + slot] = v;
-      }
+      if (slot < (unsigned)kBucketSlots) p.bucket_pairs[(size_t)r * kBucketSlots + slot] = make_int2(a, __float_as_int(v));
     }
   }
 }
@@ -1381,45 +1475,53 @@ __device__ void csc_clear_buckets(const Problem& p, int n) {
 
 // x_c^T r and the would-be changes of candidates [0, count) (kept: of the kept ones), and with `pairs` their inner
 // products with the later candidates that share a row with them.  The CTA's k-th entry is cta + k * ctas; a warp per entry.
-// What bounds it is the chain of dependent far accesses, so each link's loads go out together: the first two
-// entries of every lane, then the residual, the bucket's count and its first four members at once.
+// What bounds it is the chain of dependent far accesses -- column, row, bucket -- so each link's loads go out together,
+// and then the number of instructions per term.  The terms of 64 positions are laid out in the order of positions and dealt to
+// the lanes, however unevenly the buckets are filled; a term is added to its candidate's product in a table of the
+// warp's, terms of one candidate within a warp's step one after the other.  (Collecting the terms first and gathering those of one
+// candidate afterwards is quadratic in their number: 36 us for columns of 50 entries in 5,000 rows, 384 candidates; 10 now.)
 __device__ __forceinline__ void csc_products(const Problem& p, const Engine& e, TurnShared& ts, unsigned char* sm, int count, bool kept, bool pairs,
                                              unsigned long long t_next, bool want_keys) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int cta = (int)blockIdx.x, n_ctas = (int)gridDim.x;
   const double rho = (double)p.rho;
-  WarpTerms& wt = reinterpret_cast<WarpTerms*>(sm)[warp];
+  MetTable& wt = reinterpret_cast<MetTable*>(sm)[warp];
+  float* norm_f = reinterpret_cast<float*>(sm + sizeof(MetTable) * kWarps);
   const int mine = count > cta ? (count - cta + n_ctas - 1) / n_ctas : 0;
+  if (mine == 0) return;
+  if (pairs) {
+    for (int i = lane; i < kMetSlots / 8; i += 32) reinterpret_cast<uint4*>(wt.key)[i] = make_uint4(kFull, kFull, kFull, kFull);
+    for (int i = tid; i < min(count, kNear); i += kT) norm_f[i] = __ldcg(e.norm_f + i);
+    __syncthreads();
+  }
 #pragma unroll 1
   for (int k0 = 0; k0 < mine; k0 += kTurn) {
     const int turn = min(kTurn, mine - k0);
+    // what the end of the turn needs of a candidate, by the lanes of the last warp
     int j_own = 0, pos_own = 0;
-    double n_own = 0.0;
-    float b_own = 0.f, d_own = 0.f;
-    if (tid < turn) {                                    // gathers for the end of the turn, under way meanwhile
-      const int a = cta + n_ctas * (k0 + tid);
+    float E = 0.f;
+    Proposal prop = {};
+    if (warp == kWarps - 1 && lane < turn) {
+      const int a = cta + n_ctas * (k0 + lane);
       pos_own = kept ? p.kept_pos[a] : a;
       j_own = kept ? p.kept[a] : p.cand[a];
-      n_own = p.n2[j_own]; b_own = p.beta[j_own]; d_own = p.delta[j_own];
-    }
-    if (want_keys && warp == kWarps - 1 && lane < turn) {
-      const int a = cta + n_ctas * (k0 + lane);
-      ts.E[lane] = exponential_of(p, t_next, (uint32_t)(kept ? p.kept[a] : p.cand[a]));
+      const double n_own = p.n2[j_own];
+      const float b_own = p.beta[j_own], d_own = p.delta[j_own];
+      if (want_keys) E = exponential_of(p, t_next, (uint32_t)j_own);
+      prop = propose_begin(p, j_own, n_own, b_own, d_own, E, want_keys);
     }
 #pragma unroll 1
     for (int k = warp; k < turn; k += kWarps) {
       const int a = cta + n_ctas * (k0 + k);
       const WalkColumn col = p.walk_cols[kept ? p.kept_pos[a] : a];
       double acc = 0.0;
-      int n_terms = 0;                                   // (the same in all lanes)
+      int n_met = 0;                                     // (the same in all lanes)
       bool failed = false;
 #pragma unroll 1
-      for (int q0 = 0; q0 < col.n; q0 += 64) {
+      for (int q0 = 0; q0 < col.n; q0 += kPart) {
         int r[2];
         float v[2], x[2];
         unsigned int cnt[2];
-        int4 it[2];
-        float4 vb[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int q = q0 + 32 * h + lane;
@@ -1430,88 +1532,103 @@ __device__ __forceinline__ void csc_products(const Problem& p, const Engine& e, 
         for (int h = 0; h < 2; ++h) {
           x[h] = r[h] >= 0 ? p.resid[r[h]] : 0.f;
           cnt[h] = 0u;
-          it[h] = make_int4(-1, -1, -1, -1); vb[h] = make_float4(0.f, 0.f, 0.f, 0.f);
           if (pairs && r[h] >= 0) {
             cnt[h] = p.bucket_count[r[h]];
-            it[h] = *reinterpret_cast<const int4*>(p.bucket_items + (size_t)r[h] * kBucketSlots);
-            vb[h] = *reinterpret_cast<const float4*>(p.bucket_vals + (size_t)r[h] * kBucketSlots);
+            // the bucket's first members towards L1 at the same time
+            asm volatile("{ .reg .u32 t; ld.global.u32 t, [%0]; }" ::"l"(p.bucket_pairs + (size_t)r[h] * kBucketSlots) : "memory");
           }
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h)
           if (r[h] >= 0) acc += (double)v[h] * (double)x[h];
         if (!pairs) continue;
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-          unsigned int c = h ? cnt[1] : cnt[0];
-          const int rr = h ? r[1] : r[0];
-          const float va = h ? v[1] : v[0];
-          int4 i4 = h ? it[1] : it[0];
-          float4 v4 = h ? vb[1] : vb[0];
-          if (c > (unsigned)kBucketSlots) { failed = true; c = 0u; }
-          for (unsigned int i0 = 0; __any_sync(kFull, i0 < c); i0 += 4) {
-            if (i0 > 0 && i0 < c) {
-              i4 = *reinterpret_cast<const int4*>(p.bucket_items + (size_t)rr * kBucketSlots + i0);
-              v4 = *reinterpret_cast<const float4*>(p.bucket_vals + (size_t)rr * kBucketSlots + i0);
-            }
-            const int b4[4] = {i4.x, i4.y, i4.z, i4.w};
-            const float f4[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const bool on = i0 + u < c && b4[u] > a;
-              const unsigned int m = __ballot_sync(kFull, on);
-              if (on) {
-                const int at = n_terms + __popc(m & ((1u << lane) - 1u));
-                if (at < kTerms) {
-                  wt.key[at] = ((unsigned long long)(unsigned)b4[u] << 32) | (unsigned)(q0 + 32 * h + lane);
-                  wt.fa[at] = va;
-                  wt.fb[at] = f4[u];
-                }
-              }
-              n_terms += __popc(m);
-            }
-          }
+        for (int h = 0; h < 2; ++h)
+          if (cnt[h] > (unsigned)kBucketSlots) { failed = true; cnt[h] = 0u; }
+        const unsigned int both = cnt[0] | (cnt[1] << 16);
+        unsigned int incl = both;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const unsigned int u = __shfl_up_sync(kFull, incl, o);
+          if (lane >= o) incl += u;
         }
+        const unsigned int all = __shfl_sync(kFull, incl, 31);
+        const int n0 = (int)(all & 0xffffu), n_terms = n0 + (int)(all >> 16);
+        const int off[2] = {(int)((incl - both) & 0xffffu), n0 + (int)((incl - both) >> 16)};
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          wt.entry[32 * h + lane] = make_int4(r[h], off[h], __float_as_int(v[h]), 0);
+          for (unsigned int i = 0; i < cnt[h]; ++i) wt.pos[off[h] + i] = (unsigned char)(32 * h + lane);
+        }
+        __syncwarp();
+        auto load = [&](int at, float& fa) {
+          if (at >= n_terms) return make_int2(-1, 0);
+          const int4 en = wt.entry[wt.pos[at]];
+          fa = __int_as_float(en.z);
+          return p.bucket_pairs[(size_t)en.x * kBucketSlots + (at - en.y)];
+        };
+        float fa_next = 0.f;
+        int2 next = load(lane, fa_next);
+#pragma unroll 1
+        for (int at = 0; at < n_terms; at += 32) {
+          const int b = next.x;
+          const float fa = fa_next, fb = __int_as_float(next.y);
+          next = load(at + 32 + lane, fa_next);
+          const bool on = b > a;
+          const unsigned int peers = __match_any_sync(kFull, on ? b : ~lane);
+          const unsigned int before = peers & ((1u << lane) - 1u);
+          bool added = false;
+          int slot = b & (kMetSlots - 1);
+          if (on && before == 0u) {
+            unsigned short seen;
+            while ((seen = atomicCAS(&wt.key[slot], kFree, (unsigned short)b)) != kFree && seen != (unsigned short)b) slot = (slot + 1) & (kMetSlots - 1);
+            added = seen == kFree;
+            wt.dot[slot] = fmaf(fa, fb, added ? 0.f : wt.dot[slot]);
+          }
+          const unsigned int m = __ballot_sync(kFull, added);
+          if (added) {
+            const int i = n_met + __popc(m & ((1u << lane) - 1u));
+            if (i < kMet) wt.slot[i] = (unsigned short)slot; else wt.key[slot] = kFree;
+          }
+          n_met += __popc(m);
+          // the other terms of a candidate within these 32, in their order
+          slot = __shfl_sync(kFull, slot, __ffs((int)peers) - 1);
+          unsigned int turn_of = on ? (unsigned)__popc(before) : 0u;
+#pragma unroll 1
+          for (unsigned int i = 1; __any_sync(kFull, turn_of >= i); ++i) {
+            if (turn_of == i) wt.dot[slot] = fmaf(fa, fb, wt.dot[slot]);
+            __syncwarp();
+          }
+          __syncwarp();
+          if (n_met > kMet) break;
+        }
+        if (n_met > kMet) break;
       }
       acc = warp_sum(acc);
       if (lane == 0) ts.dot[k][0] = acc;
       if (!pairs) continue;
-      if (__any_sync(kFull, failed) || n_terms > kTerms) {
-        if (lane == 0) e.es->bucket_failed = 1;
-        continue;
-      }
-      __syncwarp();
-      // in the order of (b, position in a): every term counts the smaller ones
+      const bool overflow = __any_sync(kFull, failed) || n_met > kMet;
+      if (overflow && lane == 0) e.es->bucket_failed = 1;
+      const float bound = 0.9999f * (float)(rho * rho * col.n2);
 #pragma unroll 1
-      for (int at = lane; at < n_terms; at += 32) {
-        const unsigned long long own = wt.key[at];
-        int rank = 0;
-#pragma unroll 4
-        for (int s = 0; s < n_terms; ++s) rank += wt.key[s] < own ? 1 : 0;
-        wt.order[rank] = (unsigned short)at;
-      }
-      __syncwarp();
-#pragma unroll 1
-      for (int at = lane; at < n_terms; at += 32) {
-        const unsigned int b = (unsigned int)(wt.key[wt.order[at]] >> 32);
-        if (at > 0 && (unsigned int)(wt.key[wt.order[at - 1]] >> 32) == b) continue;       // not the first term of its b
-        const double n2b = p.walk_cols[b].n2;
-        float dot = 0.f;
-        for (int s = at; s < n_terms; ++s) {
-          const int o = wt.order[s];
-          if ((unsigned int)(wt.key[o] >> 32) != b) break;
-          dot = fmaf(wt.fa[o], wt.fb[o], dot);
-        }
-        const double den = sqrt(col.n2 * n2b);
+      for (int i = lane; i < min(n_met, kMet); i += 32) {
+        const int slot = wt.slot[i], b = wt.key[slot];
+        const float dot = wt.dot[slot];
+        wt.key[slot] = kFree;
+        // (FP64 only where the product is near the threshold, or where binary32 does not reach)
+        const float limit = bound * (b < kNear ? norm_f[b] : __ldcg(e.norm_f + b));
+        if (limit > 1e-30f && limit < 1e38f && dot * dot < limit) continue;
+        const double den = sqrt(col.n2 * p.walk_cols[b].n2);
         if (den > 0.0 && fabs((double)dot) >= rho * den) {
-          const unsigned int slot = atomicAdd(&e.es->edge_count, 1u);
-          if (slot < (unsigned)p.cap_edges) p.edges[slot] = ((unsigned int)a << 16) | b;
+          const unsigned int slot_e = atomicAdd(&e.es->edge_count, 1u);
+          if (slot_e < (unsigned)p.cap_edges) p.edges[slot_e] = ((unsigned int)a << 16) | (unsigned)b;
         }
       }
       __syncwarp();
     }
     __syncthreads();
-    if (tid < turn) propose(p, pos_own, j_own, n_own, b_own, d_own, ts.dot[tid][0], want_keys ? ts.E[tid] : 0.f, want_keys);
+    if (warp == kWarps - 1 && lane < turn) propose_end(p, prop, pos_own, j_own, ts.dot[lane][0], E, want_keys);
     __syncthreads();
   }
 }
@@ -1577,10 +1694,10 @@ __device__ void csc_apply(const Problem& p, int nk, int n_moving, int shift) {
 // ------------------------------------------------------------------------------------------------
 constexpr int kBatch = 32;
 constexpr int kColCap = 64;                              // entries of a batch member's column in shared memory (longer: global)
-constexpr int kMaxWords = STRADS_MAX_CANDIDATES / 32;
 constexpr int kOwn = 128;                                // candidates a CTA can own (more: their columns stay in global memory)
+constexpr int kHeldEntries = 24;                         // entries of a candidate's column held in registers (longer: merged)
 constexpr int kOwnEntries = 12288;                       // entries of their columns (96 KB)
-static_assert(kMaxWords <= kT, "a mask word per thread");
+static_assert(kMaxWords <= kT && kOwn * 4 <= kT, "a mask word per thread, four threads per own candidate");
 
 struct DemandShared {
   unsigned int blocked[kMaxWords];
@@ -1595,6 +1712,7 @@ struct DemandShared {
   int m, cursor, kept, examined, done;
   int own_at[kOwn + 1], own_free[kOwn], n_free;
   double own_n2[kOwn];
+  long long own_q0[kOwn];
   int orow[kOwnEntries];
   float oval[kOwnEntries];
 };
@@ -1612,9 +1730,10 @@ __device__ __forceinline__ float merge_dot(const int* ar, const float* av, int n
   return dot;
 }
 
-// The columns of all candidates lie where p.walk_cols says (written behind the last barrier's far side).  False: a
-// barrier gave up.
-__device__ bool csc_walk_on_demand(const Problem& p, const Engine& e, unsigned char* sm, Grid& g) {
+// The columns of all candidates lie where p.walk_cols says (written behind the last barrier's far side).  step(): work for
+// the warps that wait at its barriers.  False: a barrier gave up.
+template <typename Step>
+__device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, const Engine& e, unsigned char* sm, Grid& g, Step&& step) {
   DemandShared& s = *reinterpret_cast<DemandShared*>(sm);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int cta = (int)blockIdx.x, n_ctas = (int)gridDim.x, n = p.n_cand, W = (n + 31) >> 5;
@@ -1627,33 +1746,38 @@ __device__ bool csc_walk_on_demand(const Problem& p, const Engine& e, unsigned c
   // this CTA's candidates: cta, cta + n_ctas, ...; own_at: where their entries start in orow / oval
   const int n_own = n > cta ? (n - cta + n_ctas - 1) / n_ctas : 0;
   const int n_here = min(n_own, kOwn);
-  for (int k0 = 0; k0 < n_here; k0 += 32) {              // (one warp: at most four trips)
-    if (warp == 0) {
-      const int k = k0 + lane;
-      WalkColumn col;
-      col.n = 0; col.n2 = 0.0;
-      if (k < n_here) col = p.walk_cols[cta + k * n_ctas];
-      int incl = col.n;
+  // (kOwn threads find the columns, then four threads per candidate bring the entries: two far accesses in all)
+  {
+    long long q0 = 0;
+    int cnt = 0;
+    if (tid < n_here) {
+      const WalkColumn col = p.walk_cols[cta + tid * n_ctas];
+      q0 = col.q0; cnt = col.n;
+      s.own_n2[tid] = col.n2;
+    }
+    int incl = cnt;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += v;
-      }
-      const int base = k0 ? s.own_at[k0] : 0;
-      __syncwarp();
-      if (k0 == 0 && lane == 0) s.own_at[0] = 0;
-      if (k < n_here) { s.own_at[k + 1] = base + incl; s.own_n2[k] = col.n2; }
-      __syncwarp();
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (lane == 31) s.wsum[warp] = incl;
+    __syncthreads();
+    int before = 0;
+    for (int k = 0; k < warp; ++k) before += s.wsum[k];
+    if (tid == 0) s.own_at[0] = 0;
+    if (tid < n_here) { s.own_at[tid + 1] = before + incl; s.own_q0[tid] = q0; }
+    __syncthreads();
+    const int k = tid >> 2;
+    if (k < n_here) {
+      const int at = s.own_at[k], m = s.own_at[k + 1] - at;
+      const long long from = s.own_q0[k];
+      if (at + m <= kOwnEntries)
+#pragma unroll 4
+        for (int q = tid & 3; q < m; q += 4) { s.orow[at + q] = __ldg(p.xrow + from + q); s.oval[at + q] = __ldg(p.xv + from + q); }
     }
   }
-  __syncthreads();
-  for (int k = warp; k < n_here; k += kWarps) {
-    const int at = s.own_at[k], cnt = s.own_at[k + 1] - at;
-    if (at + cnt > kOwnEntries) continue;
-    const long long q0 = p.walk_cols[cta + k * n_ctas].q0;
-    for (int q = lane; q < cnt; q += 32) { s.orow[at + q] = __ldg(p.xrow + q0 + q); s.oval[at + q] = __ldg(p.xv + q0 + q); }
-  }
-  if (!grid_sync(g)) return false;                       // the mask in global memory is clear
+  if (!grid_sync_busy(g, step)) return false;            // the mask in global memory is clear
 
   while (true) {
     // ---- A: the next <= 32 unblocked candidates at or after the cursor ----
@@ -1757,32 +1881,56 @@ __device__ bool csc_walk_on_demand(const Problem& p, const Engine& e, unsigned c
           if (b > first_pos && !((s.blocked[b >> 5] >> (b & 31)) & 1u)) s.own_free[atomicAdd(&s.n_free, 1)] = k0 + tid;
         }
         __syncthreads();
-        const int pairs = s.n_free * n_new;
-        for (int x = tid; x < pairs; x += kT) {
-          const int k = s.own_free[x / n_new];
-          unsigned int rest = keep;
-          for (int y = x - (x / n_new) * n_new; y > 0; --y) rest &= rest - 1u;
-          const int q = __ffs((int)rest) - 1, b = cta + k * n_ctas;
-          if (s.pos[q] >= b) continue;                   // the member comes later in the list: it cannot block b
-          const int na = s.len[q];
-          float dot;
-          double n2b;
-          if (k < n_here && s.own_at[k + 1] <= kOwnEntries && na <= kColCap) {
-            n2b = s.own_n2[k];
-            dot = merge_dot(s.brow[q], s.bval[q], na, s.orow + s.own_at[k], s.oval + s.own_at[k], s.own_at[k + 1] - s.own_at[k]);
-          } else {
-            const WalkColumn cb = p.walk_cols[b];
-            n2b = cb.n2;
-            const int* ar = na <= kColCap ? s.brow[q] : p.xrow + s.ptr[q];
-            const float* av = na <= kColCap ? s.bval[q] : p.xv + s.ptr[q];
-            dot = merge_dot(ar, av, na, p.xrow + cb.q0, p.xv + cb.q0, cb.n);
+        // A team of threads per candidate, each with a share of the members.  A thread holds its candidate's column in
+        // registers and compares every entry of a member's with all of it: no step waits for the one before, where a merge
+        // of two sorted lists is 2 nnz dependent steps.
+        const int n_free = s.n_free, teams = n_free > 0 ? max(1, min(n_new, kT / n_free)) : 1;
+        const int c = tid / teams;
+        if (c < n_free) {
+          const int k = s.own_free[c], b = cta + k * n_ctas;
+          const bool here = k < n_here && s.own_at[k + 1] <= kOwnEntries;
+          const int at = here ? s.own_at[k] : 0, nb = here ? s.own_at[k + 1] - at : 0;
+          const bool held = here && nb <= kHeldEntries;
+          int rb[kHeldEntries];
+          float vb[kHeldEntries];
+          if (held) {
+#pragma unroll
+            for (int i = 0; i < kHeldEntries; ++i) { rb[i] = i < nb ? s.orow[at + i] : 0x7fffffff; vb[i] = i < nb ? s.oval[at + i] : 0.f; }
           }
-          const double den = sqrt(s.n2[q] * n2b);
-          if (den > 0.0 && fabs((double)dot) >= rho * den) atomicOr(&blocked_g[b >> 5], 1u << (b & 31));
+          for (int y = tid - c * teams; y < n_new; y += teams) {
+            unsigned int rest = keep;
+            for (int z = y; z > 0; --z) rest &= rest - 1u;
+            const int q = __ffs((int)rest) - 1;
+            if (s.pos[q] >= b) continue;                 // the member comes later in the list: it cannot block b
+            const int na = s.len[q];
+            float dot = 0.f;
+            double n2b;
+            if (held && na <= kColCap) {
+              n2b = s.own_n2[k];
+#pragma unroll 1
+              for (int i = 0; i < na; ++i) {
+                const int ra = s.brow[q][i];
+                const float va = s.bval[q][i];
+#pragma unroll
+                for (int j = 0; j < kHeldEntries; ++j) dot = rb[j] == ra ? fmaf(va, vb[j], dot) : dot;
+              }
+            } else if (here && na <= kColCap) {
+              n2b = s.own_n2[k];
+              dot = merge_dot(s.brow[q], s.bval[q], na, s.orow + at, s.oval + at, nb);
+            } else {
+              const WalkColumn cb = p.walk_cols[b];
+              n2b = cb.n2;
+              const int* ar = na <= kColCap ? s.brow[q] : p.xrow + s.ptr[q];
+              const float* av = na <= kColCap ? s.bval[q] : p.xv + s.ptr[q];
+              dot = merge_dot(ar, av, na, p.xrow + cb.q0, p.xv + cb.q0, cb.n);
+            }
+            const double den = sqrt(s.n2[q] * n2b);
+            if (den > 0.0 && fabs((double)dot) >= rho * den) { atomicOr(&blocked_g[b >> 5], 1u << (b & 31)); break; }
+          }
         }
       }
     }
-    if (!grid_sync(g)) return false;
+    if (!grid_sync_busy(g, step)) return false;
     for (int w = tid; w < W; w += kT) s.blocked[w] = __ldcg(blocked_g + w);
     __syncthreads();
   }
@@ -1879,7 +2027,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
       if (n < n_total && es->skip_window && !no_filter) n = n_total;
     } else {
       window = no_filter || (p.bucket_count != nullptr && !(n < n_total && es->skip_window) && t >= es->avoid_until);
-      if (real) csc_enter(p, window ? n : n_total, window && !no_filter);
+      if (real) csc_enter(p, e, window ? n : n_total, window && !no_filter);
     }
     // ---- steps 1 to 3, once more over all candidates where a window does not do ----
     while (true) {
@@ -1891,9 +2039,11 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
         }
         dense_pack(p, e, sm, ts, pb, packed, n, t + 1, products, draws, terms == 3, limit);
       }
-      if (!scanned) { draw_scan(p, e, ds, sm, td, true); scanned = true; }
+      // a walk on demand leaves the SMs mostly idle, at its barriers above all: the scan is made there
+      const bool during_walk = !kDense && real && !window && !scanned;
+      if (!scanned && !during_walk) { draw_scan(p, e, ds, sm, td, true); scanned = true; }
       if (kDense) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // (the Gram's operands come in over it)
-      if (!(ok = grid_sync(g))) break;
+      if (!(during_walk && !(p.flags & STRADS_FLAG_DYNAMIC_DEPS)) && !(ok = grid_sync(g))) break;      // (the walk begins with a barrier)
       if (kDense && real && !no_filter) {
         unsigned int* amb = &es->amb_count[attempts & 1u];
         if (cta == 0 && tid == 0) es->amb_count[(attempts + 1u) & 1u] = 0u;
@@ -1929,11 +2079,26 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
       }
       // the winners of the draw: by every CTA but the one that walks; CSC in step 3 as well, unless there is none
       const bool csc_window = !kDense && real && window && !no_filter;
-      if (!collected && !csc_window) { draw_gather(p, e, ds, td, k, spare); collected = true; }
+      if (!collected && !csc_window && !during_walk) { draw_gather(p, e, ds, td, k, spare); collected = true; }
       if (!kDense && real) {
         if (!window) {
-          if (!(ok = csc_walk_on_demand(p, e, sm, g))) break;
+          unsigned char* sm_scan = sm + sizeof(DemandShared);
+          unsigned int* sh = reinterpret_cast<unsigned int*>(sm_scan);
+          const float cut = during_walk ? scan_open(e, ds, sm_scan, true) : 0.f;
+          const Binning bins = binning_of(cut);
+          const WeightForm wf = weight_form(p);
+          WarpScan scan = begin_scan(cut, scan_queue(sm_scan), warp * n_ctas + cta, kWarps * n_ctas);
+          auto step = [&]() {
+            return during_walk && scan_step(p, td, wf, scan, [&](unsigned long long key, bool on) { scan_found(e, ds, sh, bins, key, on); });
+          };
+          if (!(ok = csc_walk_on_demand(p, e, sm, g, step))) break;
+          if (during_walk) {
+#pragma unroll 1
+            while (step()) {}
+            scan_close(e, ds, sm_scan);
+          }
           if (!(ok = grid_sync(g))) break;
+          if (during_walk) { draw_gather(p, e, ds, td, k, false); scanned = collected = true; }
         }
         csc_products(p, e, ts, sm, window ? n : es->n_kept, !window, csc_window, t + 1, draws);
       }
@@ -1962,7 +2127,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
         if (!collected) { draw_gather(p, e, ds, td, k, true); collected = true; spare = true; }
         if (!(ok = grid_sync(g))) break;
         if (!es->walk_open) break;
-        csc_enter(p, n_total, false);
+        csc_enter(p, e, n_total, false);
         window = false;
       } else {
         if (!es->walk_open) break;
@@ -2092,7 +2257,7 @@ size_t smem_of(bool dense, int n_keep, bool ahead, int n_cand) {
     at_least(keys + sizeof(Moving) + sizeof(double) * 4 * kT + (ahead ? sizeof(ChangedByBin) : 0));
   } else {
     at_least(kTermsSmem);
-    at_least(sizeof(DemandShared));
+    at_least(sizeof(DemandShared) + kScanSmem);
     at_least(walk_pairs_smem(n_cand, 8192));
     if (ahead) at_least(keys + sizeof(ChangedByBin));
   }

@@ -8,7 +8,6 @@ namespace strads {
 struct EngineState {
   unsigned int bar_count;       // grid barrier: arrivals of the launch in flight
   unsigned int exit_count;      // CTAs of the launch that have left
-  unsigned int surv_count;      // draw: keys the guided scan saved (append cursor)
   float t_cut;                  // draw: cutoff for the next scan (0: none)
   unsigned int amb_count[2];    // dense Gram: pairs the screen left open (two counters, in turns)
   unsigned int edge_count;      // CSC Gram: conflicting pairs listed
@@ -60,14 +59,16 @@ struct Engine {
   unsigned int* bin_cur;        // [kHistBins] append cursors of the winners' groups
   unsigned long long* win;      // [cap_win] the winners of a draw, grouped by bin
   int cap_win, cap_boundary;
-  unsigned long long* surv;     // [cap_surv] keys below the scan's cutoff
+  unsigned long long* surv;     // [ctas][cap_surv] keys below the scan's cutoff, and how many each CTA saved
+  unsigned int* saved;          // [ctas]
   unsigned int cap_surv;
   int n_list;                   // winners a draw made one round ahead collects: P' + P (at most J); 0: draws are made at the round's start
   int window;                   // candidates of the first attempt
   // dense
   unsigned short* xb;           // [n_cand][xb_pitch] BF16 high parts of the candidate columns, then (at lo_off) the low parts
   long long xb_pitch, lo_off;   // elements
-  double* norm;                 // [n_cand] norms of the candidates' columns as the rho test sees them
+  double* norm;                 // [n_cand] dense: norms of the candidates' columns as the rho test sees them
+  float* norm_f;                // [n_cand] CSC: their squares, rounded
   float* part;                  // [ctas][128 * 128] partial Gram tiles
   unsigned int* tile_ticket;    // [tiles of 64 x 64] zero between rounds
   GramPlan plan[2];             // for the window and for the whole list

@@ -129,6 +129,7 @@ struct Problem {
   unsigned int* bucket_count;   // [N] candidates of this round's list with an entry in row i (zero between rounds)
   int* bucket_items;            // [N][kBucketSlots] their positions in the list
   float* bucket_vals;           // [N][kBucketSlots] their values in row i
+  int2* bucket_pairs;           // [N][kBucketSlots] position and value side by side (the round engine; same memory as the two above)
   BucketColumn* bucket_cols;    // [P'] where each candidate's column lies, as the bucket kernels need it
   int sm_count;
   // sampling ahead (one scheduler): the draw of round t + 1 is made during round t from the priorities of its start
