@@ -337,7 +337,8 @@ bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) &
 // Conflict bits of all candidate pairs.  Dense: tensor-core kernel unless the FP32 Gram itself is wanted
 // (debug output) or the SIMT kernel is asked for.
 // n_total: length of the whole list (n_cand < n_total: a window).  *walked: the Gram kernel's last CTA also settles the
-// walk (dense tensor-core window), so that the walk kernel behind it only runs if that CTA leaves it the job.
+// walk (tensor-core screen), so that what is behind it only runs if that CTA leaves it the job: the walk kernel, and before
+// it launch_gram_rest where the launch covers the whole list.
 cudaError_t launch_gram(const Scheduler& sc, cudaStream_t s, const int* cand, int n_cand, int n_total, float* gram_dbg,
                         bool only_if_short, cudaEvent_t after_pack = nullptr, bool* walked = nullptr) {
   const Problem& p = sc.p;
@@ -350,7 +351,9 @@ cudaError_t launch_gram(const Scheduler& sc, cudaStream_t s, const int* cand, in
   }
   if (p.layout == STRADS_CSC) return launch_gram_csc(p, cand, n_cand, gram_dbg, only_if_short, window, s);
   if (gram_dbg != nullptr || (p.flags & STRADS_FLAG_SIMT_GRAM)) return launch_gram_dense_simt(p, cand, n_cand, gram_dbg, s);
-  return launch_gram_dense_tc(p, sc.gram_tmap, cand, n_cand, n_total, only_if_short, window, after_pack, s, walked);
+  const bool tail = walked != nullptr && !only_if_short && !(p.flags & STRADS_FLAG_GRAM_3XTF32);
+  if (tail) *walked = true;
+  return launch_gram_dense_tc(p, sc.gram_tmap, cand, n_cand, n_total, only_if_short, tail, after_pack, s);
 }
 
 // The greedy walk stops at P kept, so it normally looks at little more than the first P candidates: form the
@@ -382,6 +385,7 @@ int gram_and_filter(const Scheduler& sc, cudaStream_t s, const int* cand, int n_
   CK(launch_gram(sc, s, cand, window, n_cand, gram_dbg, false, after_pack, &walked));
   if (after_gram) CK(cudaEventRecord(after_gram, s));
   cudaStream_t rs = s;
+  if (walked && window == n_cand) CK(launch_gram_rest(p, sc.gram_tmap, cand, n_cand, s));
   CK(launch_filter(p, cand, window, n_cand, false, p.kept, rs, walked));
   if (window < n_cand) {
     if (p.layout == STRADS_CSC) {
@@ -428,14 +432,17 @@ int one_round(strads_lasso_s* h, const strads_round_out_t* out, cudaEvent_t befo
   return STRADS_OK;
 }
 
-// What follows a window whose Gram kernel could not finish the job (its last CTA left the walk to the walk kernel,
-// or fewer than P were kept inside the window): the walk kernel on the window if asked for, the whole-list Gram and
-// walk if the window was short, then the gated copies of the correction of the early list and of the update.
+// What follows a screen that could not finish the job (its last CTA left the walk to the walk kernel, or fewer than P
+// were kept inside the window): the walk kernel if asked for, the whole-list Gram and walk if the window was short, then
+// the gated copies of the correction of the early list and of the update.
 int retry_sequence(strads_lasso_s* h, const Scheduler& sc, int window, bool early_patch, cudaStream_t rs) {
   const Problem& p = sc.p;
+  if (window == p.n_cand) CK(launch_gram_rest(p, sc.gram_tmap, p.cand, p.n_cand, rs));
   CK(launch_filter(p, p.cand, window, p.n_cand, false, p.kept, rs, true));
-  CK(launch_gram(sc, rs, p.cand, p.n_cand, p.n_cand, nullptr, true));
-  CK(launch_filter(p, p.cand, p.n_cand, p.n_cand, true, p.kept, rs));
+  if (window < p.n_cand) {
+    CK(launch_gram(sc, rs, p.cand, p.n_cand, p.n_cand, nullptr, true));
+    CK(launch_filter(p, p.cand, p.n_cand, p.n_cand, true, p.kept, rs));
+  }
   if (early_patch) CK(launch_sample_patch(p, h->ahead, p.cand, rs, true, 2));
   CK(launch_update(p, p.kept, 1, true, rs, 2));
   return STRADS_OK;
@@ -470,8 +477,8 @@ int round_sampling_ahead(strads_lasso_s* h, bool have_list, cudaStream_t main) {
   CK(launch_sample(h->ahead, h->ahead.cand, h->ahead_stream));
   CK(cudaEventRecord(h->ahead_done, h->ahead_stream));
   const int window = window_of(p, p.n_cand);
-  if (!early_patch || window >= p.n_cand || (p.flags & STRADS_FLAG_GRAM_3XTF32)) {
-    // no window, or a Gram that does not walk: everything in a row
+  if (!early_patch || (p.flags & STRADS_FLAG_GRAM_3XTF32)) {
+    // a Gram that does not walk: everything in a row
     const int rc = gram_and_filter(sc, main, p.cand, p.n_cand, nullptr);
     if (rc) return rc;
     CK(cudaStreamWaitEvent(main, h->ahead_done, 0));

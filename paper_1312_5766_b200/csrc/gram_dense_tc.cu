@@ -140,27 +140,57 @@ __device__ __forceinline__ float tf32_lo(float x) {
   return __uint_as_float(__float_as_uint(x - hi) & 0xffffe000u);
 }
 
+// Pairs the screen left open.  A CTA keeps the first few of its own (four per warp: a dozen microseconds of exact products
+// at most) and decides them itself before it leaves, the grid's CTAs side by side; the others go to the list in
+// global memory.
+constexpr unsigned int kOwnOpen = 24;
+struct OwnOpen { unsigned int n, pair[kOwnOpen]; };
+// A row's conflicts (bit j: with b0 + j; those above the diagonal are listed for the walk) and the pairs left open.  Few rows
+// have any, and the code runs from a cold instruction cache once per launch, so it is a loop of its own: as part of the
+// unrolled tests it made the kernel 84 KB long.
+// (Single arguments: a reference to the kernel's parameters would copy them to the stack.)
+__device__ __noinline__ void report_pairs(unsigned int* edges, unsigned int* edge_count, unsigned int cap_edges, unsigned int* amb, unsigned int* amb_count,
+                                          unsigned int cap_amb, OwnOpen* own, int a, int b0, uint32_t listed, uint32_t open) {
+#pragma unroll 1
+  for (uint32_t m = listed | open; m; m &= m - 1u) {
+    const int j = __ffs((int)m) - 1;
+    const unsigned int pr = ((unsigned int)a << 16) | (unsigned int)(b0 + j);
+    if ((listed >> j) & 1u) {
+      const unsigned int slot = atomicAdd(edge_count, 1u);
+      if (slot < cap_edges) edges[slot] = pr;
+      continue;
+    }
+    if (own != nullptr) {
+      const unsigned int i = atomicAdd(&own->n, 1u);
+      if (i < kOwnOpen) { own->pair[i] = pr; continue; }
+    }
+    const unsigned int slot = atomicAdd(amb_count, 1u);
+    if (slot < cap_amb) amb[slot] = pr;
+  }
+}
+__device__ __forceinline__ void report(const Problem& p, OwnOpen* own, int a, int b0, uint32_t word, uint32_t open) {
+  const uint32_t above = a < b0 ? 0xffffffffu : (a - b0 >= 31 ? 0u : 0xffffffffu << (a - b0 + 1));
+  if ((word & above) | open)
+    report_pairs(p.edges, &p.st->edge_count, (unsigned)p.cap_edges, p.amb_pairs, &p.st->amb_count, (unsigned)p.cap_amb, own, a, b0, word & above, open);
+}
+
 // 32 Gram values of row a against columns b0 .. b0 + 31 -> conflict bits.  Screen mode leaves the pairs
-// inside the band undecided (bit clear) and appends them to the list k_gram_recheck works through.
+// inside the band undecided (bit clear).
 template <bool kScreen>
 __device__ __forceinline__ uint32_t decide_word(const Problem& p, const uint32_t (&v)[32], int a, int b0, int n_cand,
-                                                double norm_a, const double* norm_b, double rho, double band) {
-  uint32_t word = 0u;
+                                                double norm_a, const double* norm_b, double rho, double band, OwnOpen* own) {
+  uint32_t word = 0u, open = 0u;
 #pragma unroll
   for (int j = 0; j < 32; ++j) {
     const int b = b0 + j;
     const double den = norm_a * norm_b[j];
     const double g = fabs((double)__uint_as_float(v[j]));
     const bool live = a < n_cand && b < n_cand && a != b && den > 0.0;
-    bool hit = live && g >= rho * den;
-    if (kScreen && live && b > a && fabs(g - rho * den) <= band * den) {
-      hit = false;
-      const unsigned int slot = atomicAdd(&p.st->amb_count, 1u);
-      if (slot < (unsigned)p.cap_amb) p.amb_pairs[slot] = ((unsigned int)a << 16) | (unsigned int)b;
-    }
-    if (hit && b > a) list_conflict(p, a, b);
-    word |= (uint32_t)hit << j;
+    const bool close = kScreen && live && b > a && fabs(g - rho * den) <= band * den;
+    open |= (uint32_t)close << j;
+    word |= (uint32_t)(live && !close && g >= rho * den) << j;
   }
+  report(p, own, a, b0, word, open);
   return word;
 }
 
@@ -294,23 +324,28 @@ __global__ void __launch_bounds__(kPackThreads) k_pack_candidates(Problem p, con
   }
 }
 
-// Exact decision for one pair the screen could not call, by a whole warp: FP64 dot product of the two columns of X.  Setting a bit is idempotent and order-independent, so the result is deterministic.
-__device__ __forceinline__ void recheck_pair(const Problem& p, unsigned int pr, int lane) {
-  const long long n4 = (p.N + 3) >> 2;
-  const int a = (int)(pr >> 16), b = (int)(pr & 0xffffu);
-  const float4* xa = reinterpret_cast<const float4*>(p.xv + (long long)p.cand_cur[a] * p.ld);
-  const float4* xb = reinterpret_cast<const float4*>(p.xv + (long long)p.cand_cur[b] * p.ld);
+// x_a^T x_b in FP64 by a warp.
+__device__ __noinline__ double exact_product(const float* xa, const float* xb, long long N) {
+  const int lane = threadIdx.x & 31;
   double acc = 0.0;
-  for (long long g = lane; g < n4; g += 32) {
-    const float4 u = xa[g], w = xb[g];
+#pragma unroll 2
+  for (long long g = lane; g < (N + 3) >> 2; g += 32) {
+    const float4 u = reinterpret_cast<const float4*>(xa)[g], w = reinterpret_cast<const float4*>(xb)[g];
     const long long i = g << 2;
     acc += (double)u.x * w.x;
-    if (i + 1 < p.N) acc += (double)u.y * w.y;
-    if (i + 2 < p.N) acc += (double)u.z * w.z;
-    if (i + 3 < p.N) acc += (double)u.w * w.w;
+    if (i + 1 < N) acc += (double)u.y * w.y;
+    if (i + 2 < N) acc += (double)u.z * w.z;
+    if (i + 3 < N) acc += (double)u.w * w.w;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  return acc;
+}
+// Exact decision for one pair the screen could not call, by a whole warp.  Setting a bit is idempotent and
+// order-independent, so the result is deterministic.
+__device__ __forceinline__ void recheck_pair(const Problem& p, unsigned int pr, int lane) {
+  const int a = (int)(pr >> 16), b = (int)(pr & 0xffffu);
+  const double acc = exact_product(p.xv + (long long)p.cand_cur[a] * p.ld, p.xv + (long long)p.cand_cur[b] * p.ld, p.N);
   if (lane == 0) {
     const double den = sqrt(coupling_n2(p, p.cand_cur[a])) * sqrt(coupling_n2(p, p.cand_cur[b]));
     if (den > 0.0 && fabs(acc) >= (double)p.rho * den) {
@@ -325,7 +360,8 @@ __device__ __forceinline__ void recheck_pair(const Problem& p, unsigned int pr, 
 //   - the pairs the screen left open, normally a handful or none, are decided exactly.  "Few" is a budget of
 //     multiply-adds for this one CTA (2^21, some tens of microseconds at worst): short columns leave many pairs
 //     open (their correlations scatter widely around rho) but each is cheap, long columns hardly any.  Beyond the
-//     budget the window is handed to the whole-list retry, whose Gram has a recheck kernel of its own;
+//     budget a window is handed to the whole-list retry, whose Gram has a recheck kernel of its own, and a whole list
+//     to the kernels of launch_gram_rest;
 //   - the greedy first-fit walk is settled from the list of conflicting pairs; if that list is incomplete or the
 //     chains of dependent decisions are too long, the walk kernel behind this one does it from the bit rows
 //     (walk_pending), otherwise that kernel returns at once.
@@ -345,7 +381,9 @@ __device__ void window_tail(const Problem& p, const int* __restrict__ cand, int 
   __threadfence();
   const unsigned int n_amb = __ldcg(&st->amb_count);
   if (n_amb > (unsigned)p.cap_amb || n_amb > kInlineRecheck || (long long)n_amb * p.N > kInlineRecheckWork) {
-    if (tid == 0) {                                      // the whole-list retry takes over (it has the 3xTF32 fallback)
+    if (tid == 0 && n_cand == n_total) {                 // left as it is to the recheck and 3xTF32 kernels and the walk behind them
+      st->gram_ticket = 0u; st->walk_pending = 1; st->route = 1;
+    } else if (tid == 0) {                               // the whole-list retry takes over (it has the 3xTF32 fallback)
       st->gram_ticket = 0u; st->window_short = 1; st->route = 1; st->walk_pending = 0;
       st->amb_count = 0; st->edge_count = 0; st->edges_off = 0;
     }
@@ -361,6 +399,7 @@ __device__ void window_tail(const Problem& p, const int* __restrict__ cand, int 
   if (!settled) {
     if (tid == 0) {
       st->gram_ticket = 0u; st->walk_pending = 1; st->route = 1;
+      st->amb_count = 0;                                 // (all decided)
     }
     return;
   }
@@ -396,6 +435,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_dense_tc(Problem p, const 
   __shared__ uint32_t s_tmem_base;
   __shared__ volatile int s_abort;
   __shared__ double normA[kTile], normB[kTile];                        // ||x|| of the tile's rows / columns
+  __shared__ OwnOpen s_own;
+  OwnOpen* own = tail ? &s_own : nullptr;
 
   if (only_if_short && !p.st->window_short) return;
   // as a fallback the 3xTF32 variant runs only when the screen's list overflowed
@@ -418,6 +459,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_dense_tc(Problem p, const 
   const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[kStages]), done_bar = smem_u32(&bars[2 * kStages]);
 
   if (tid == 0) {
+    s_own.n = 0u;
     for (int s = 0; s < kStages; ++s) { mbar_init(full0 + 8 * s, kFullCount); mbar_init(empty0 + 8 * s, 1); }
     mbar_init(done_bar, 1);
     s_abort = 0;
@@ -597,7 +639,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_dense_tc(Problem p, const 
         for (int c = 0; c < kTile / 32; ++c) {
           uint32_t v[32];
           tmem_load32(tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c * 32), v);
-          const uint32_t word = decide_word<!k3x>(p, v, a, tj * kTile + c * 32, n_cand, norm_a, normB + c * 32, rho, band);
+          const uint32_t word = decide_word<!k3x>(p, v, a, tj * kTile + c * 32, n_cand, norm_a, normB + c * 32, rho, band, own);
           const int widx = tj * (kTile / 32) + c;
           if (a < n_cand && widx < p.mask_words) p.conflict[(long long)a * p.mask_words + widx] = word;
         }
@@ -651,22 +693,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_dense_tc(Problem p, const 
         const int a = ti * kTile + la;
         const double norm_a = normA[la];
         const float g4[4] = {acc.x, acc.y, acc.z, acc.w};
-        unsigned int nib = 0u;
+        unsigned int nib = 0u, open = 0u;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const int b = tj * kTile + lane * 4 + k;
           const double den = norm_a * normB[lane * 4 + k];
           const double g = fabs((double)g4[k]);
           const bool live = a < n_cand && b < n_cand && a != b && den > 0.0;
-          bool hit = live && g >= rho * den;
-          if (live && b > a && fabs(g - rho * den) <= band * den) {
-            hit = false;                                   // too close to call: decided exactly by the recheck
-            const unsigned int slot = atomicAdd(&p.st->amb_count, 1u);
-            if (slot < (unsigned)p.cap_amb) p.amb_pairs[slot] = ((unsigned int)a << 16) | (unsigned int)b;
-          }
-          if (hit && b > a) list_conflict(p, a, b);
-          nib |= (unsigned int)hit << k;
+          const bool close = live && b > a && fabs(g - rho * den) <= band * den;      // decided exactly later
+          open |= (unsigned int)close << k;
+          nib |= (unsigned int)(live && !close && g >= rho * den) << k;
         }
+        report(p, own, a, tj * kTile + lane * 4, nib, open);
         unsigned int word = nib << ((lane & 7) * 4);       // 8 lanes make one 32-column mask word
         word |= __shfl_xor_sync(0xffffffffu, word, 1);
         word |= __shfl_xor_sync(0xffffffffu, word, 2);
@@ -685,13 +723,17 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_dense_tc(Problem p, const 
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
   }
-  if (tail) window_tail(p, p.cand_cur, n_cand, n_total, tiles_ptr);
+  if (!k3x && tail) {
+    for (unsigned int e = warp; e < min(s_own.n, kOwnOpen); e += kThreads / 32) recheck_pair(p, s_own.pair[e], lane);
+    window_tail(p, p.cand_cur, n_cand, n_total, tiles_ptr);
+  }
 }
 
 // All pairs the screen left open: one warp per pair.
-__global__ void __launch_bounds__(256) k_gram_recheck(Problem p, int only_if_short) {
+__global__ void __launch_bounds__(256) k_gram_recheck(Problem p, int only_if_short, int only_if_pending) {
   chain_begin();
   if (only_if_short && !p.st->window_short) return;
+  if (only_if_pending && !p.st->walk_pending) return;
   const unsigned int n = p.st->amb_count;
   if (n > (unsigned)p.cap_amb) return;                 // overflow: the 3xTF32 kernel redoes every bit instead
   const int lane = threadIdx.x & 31;
@@ -758,12 +800,11 @@ cudaError_t encode_gram_tensor_map(const Problem& p, void* out) {
 
 // pack -> screen (K split inside clusters when the tiles are few) -> exact recheck of the borderline pairs -> (only
 // if their list overflowed) 3xTF32 over everything.
-// `fallback_elsewhere`: the launch covers a window (n_cand of n_total candidates) and a whole-list retry follows; an
-// overflow of the borderline list is then handled by that retry, not by a 3xTF32 launch here, and the last CTA of
-// the screen rechecks and walks (*walked = true: the caller's walk kernel need only run if walk_pending is raised).
+// `tail`: the last CTA of the screen rechecks and walks, so that the caller's walk kernel need only run if walk_pending is
+// raised, and nothing follows the screen here: where it covers a window (n_cand of n_total candidates), a whole-list retry
+// behind it also handles an overflow of the borderline list; where it covers the whole list, launch_gram_rest does.
 cudaError_t launch_gram_dense_tc(const Problem& p, const void* tmap, const int* cand, int n_cand, int n_total, bool only_if_short,
-                                 bool fallback_elsewhere, cudaEvent_t after_pack, cudaStream_t s, bool* walked) {
-  if (walked != nullptr) *walked = false;
+                                 bool tail, cudaEvent_t after_pack, cudaStream_t s) {
   const int n_tiles = (n_cand + kTile - 1) / kTile;
   const int tiles = n_tiles * (n_tiles + 1) / 2;
   const int ois = only_if_short ? 1 : 0;
@@ -782,19 +823,29 @@ cudaError_t launch_gram_dense_tc(const Problem& p, const void* tmap, const int* 
   const int pack_ctas = only_if_short ? (n_cand < 4 * p.sm_count ? n_cand : 4 * p.sm_count) : n_cand;
   if ((e = launch_chained(k_pack_candidates, pack_ctas, kPackThreads, 0, s, q, cand, n_cand, ois)) != cudaSuccess) return e;
   if (after_pack != nullptr && (e = cudaEventRecord(after_pack, s)) != cudaSuccess) return e;   // optional step timing
-  if (!(p.flags & STRADS_FLAG_GRAM_3XTF32)) {
-    const int tail = (fallback_elsewhere && !only_if_short) ? 1 : 0;
+  const bool screen = !(p.flags & STRADS_FLAG_GRAM_3XTF32);
+  if (screen) {
     const int ctas = n_split > 1 ? tiles * n_split : (tiles < p.sm_count ? tiles : p.sm_count);
     if ((e = launch_chained_cluster(k_gram_dense_tc<false>, ctas, kThreads, kDynSmem, s, n_split, q, tm, n_cand, n_total,
-                                    n_tiles, n_split, ois, tail)) != cudaSuccess)
+                                    n_tiles, n_split, ois, tail ? 1 : 0)) != cudaSuccess)
       return e;
-    if (tail && walked != nullptr) *walked = true;
-    if (!tail && (e = launch_chained(k_gram_recheck, p.sm_count * 2, 256, 0, s, q, ois)) != cudaSuccess) return e;
+    if (tail) return cudaSuccess;
+    if ((e = launch_chained(k_gram_recheck, p.sm_count * 2, 256, 0, s, q, ois, 0)) != cudaSuccess) return e;
   }
-  if (!fallback_elsewhere || (p.flags & STRADS_FLAG_GRAM_3XTF32))
-    return launch_chained(k_gram_dense_tc<true>, tiles < p.sm_count ? tiles : p.sm_count, kThreads, kDynSmem, s, q, tm, n_cand, n_total,
-                          n_tiles, 1, ois, 0);
-  return cudaSuccess;
+  return launch_chained(k_gram_dense_tc<true>, tiles < p.sm_count ? tiles : p.sm_count, kThreads, kDynSmem, s, q, tm, n_cand, n_total,
+                        n_tiles, 1, ois, 0);
+}
+
+// What a screen of the whole list with a tail leaves undone when more pairs are open than its CTAs decide themselves (data
+// that cluster at rho): launches that return at once otherwise.
+cudaError_t launch_gram_rest(const Problem& p, const void* tmap, const int* cand, int n_cand, cudaStream_t s) {
+  const int n_tiles = (n_cand + kTile - 1) / kTile, tiles = n_tiles * (n_tiles + 1) / 2;
+  Problem q = p;
+  q.cand_cur = cand;
+  const cudaError_t e = launch_chained(k_gram_recheck, p.sm_count * 2, 256, 0, s, q, 0, 1);
+  if (e != cudaSuccess) return e;
+  return launch_chained(k_gram_dense_tc<true>, tiles < p.sm_count ? tiles : p.sm_count, kThreads, kDynSmem, s, q,
+                        *static_cast<const CUtensorMap*>(tmap), n_cand, n_cand, n_tiles, 1, 0, 0);
 }
 
 }  // namespace strads

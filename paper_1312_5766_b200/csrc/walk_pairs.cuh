@@ -12,7 +12,8 @@
 // The CTA that runs this has the rest of the grid idle behind it, and with so few warps every instruction waits
 // for the one before it (time stamps: ~1 us per pass and per scan when each was a loop over all candidates with
 // its own barriers), so the work is cut to short chains: only the second members of listed pairs are ever
-// undecided, the passes touch nothing but the pairs, and the kept sequence is numbered from warp ballots.
+// undecided, the passes touch nothing but the pairs, and the kept sequence is numbered from warp ballots.  The loops are
+// not unrolled: most make a trip or two, and the code comes from a cold instruction cache (19 KB of it otherwise).
 #pragma once
 #include "strads_internal.cuh"
 
@@ -46,18 +47,23 @@ __device__ bool walk_from_pair_list(const Problem& p, const int* cand, int n_can
   int cv[kAhead];
 #pragma unroll
   for (int u = 0; u < kAhead; ++u) cv[u] = tid + u * kNT < n_cand ? cand[tid + u * kNT] : 0;
+#pragma unroll 1
   for (int i = tid; i < n_cand; i += kNT) state[i] = 1;                    // kept unless a listed pair says otherwise
+#pragma unroll 1
   for (unsigned int k = tid; k < n_edges; k += kNT) e[k] = __ldcg(p.edges + k);
   __syncthreads();
   if (n_edges > 0) {
+#pragma unroll 1
     for (unsigned int k = tid; k < n_edges; k += kNT) {                   // (several threads may store the same values: benign)
       const int b = (int)(e[k] & 0xffffu);
       state[b] = 0; hit[b] = 0; pend[b] = 0;
     }
     __syncthreads();
     bool settled = false;
+#pragma unroll 1
     for (int pass = 0; pass < kSparsePasses && !settled; ++pass) {
       const unsigned char mark = (unsigned char)(pass + 1);
+#pragma unroll 1
       for (unsigned int k = tid; k < n_edges; k += kNT) {
         const int a = (int)(e[k] >> 16), b = (int)(e[k] & 0xffffu);
         if (state[b] == 0) {
@@ -68,6 +74,7 @@ __device__ bool walk_from_pair_list(const Problem& p, const int* cand, int n_can
       }
       __syncthreads();
       int open = 0;
+#pragma unroll 1
       for (unsigned int k = tid; k < n_edges; k += kNT) {                 // every thread that shares b reads the same and stores the same
         const int b = (int)(e[k] & 0xffffu);
         if (state[b] == 0) {
@@ -82,6 +89,7 @@ __device__ bool walk_from_pair_list(const Problem& p, const int* cand, int n_can
   }
   // kept members in order: a ballot per 32 consecutive candidates, one warp numbers the words, and every thread
   // writes the kept candidates it looked at, at their ranks, up to P
+#pragma unroll 1
   for (int i0 = tid - lane; i0 < n_cand; i0 += kNT) {
     const int i = i0 + lane;
     const unsigned int word = __ballot_sync(0xffffffffu, i < n_cand && state[i] == 1);
@@ -90,6 +98,7 @@ __device__ bool walk_from_pair_list(const Problem& p, const int* cand, int n_can
   __syncthreads();
   if (tid < 32) {
     unsigned int carry = 0u;
+#pragma unroll 1
     for (int w0 = 0; w0 < n_words; w0 += 32) {
       const int w = w0 + lane;
       const unsigned int c = w < n_words ? (unsigned int)__popc(wbits[w]) : 0u;
@@ -106,6 +115,7 @@ __device__ bool walk_from_pair_list(const Problem& p, const int* cand, int n_can
   }
   __syncthreads();
   int u = 0;
+#pragma unroll 1
   for (int i = tid; i < n_cand; i += kNT, ++u) {
     const unsigned int word = wbits[i >> 5];
     if ((word >> lane) & 1u) {                             // (i and tid have the same lane: kNT is a multiple of 32)
