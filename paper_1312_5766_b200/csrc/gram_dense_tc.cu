@@ -230,6 +230,7 @@ __device__ __forceinline__ void pack_candidate(const Problem& p, const int* __re
   const long long n4 = p.ldc >> 2;                      // ldc = N rounded up to 4 <= ld
   unsigned short* dstb = p.xcb + (long long)a * p.ldcb;   // (ldcb >= ldc: every group of four has its place)
   if (!p.proposals) {
+#pragma unroll 2
     for (long long g = threadIdx.x; g < n4; g += blockDim.x) {
       store_bf16x4(dstb, g, __ldg(src + g));
     }
@@ -251,6 +252,7 @@ __device__ __forceinline__ void pack_candidate(const Problem& p, const int* __re
   float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
   constexpr int kU = 4;                                 // column loads in flight per thread
   const long long first = threadIdx.x < kPackStream ? (long long)threadIdx.x : n4;      // (the extra warp: no trips)
+#pragma unroll 1
   for (long long g0 = first; g0 < n4; g0 += (long long)kU * kPackStream) {
     float4 xv[kU], rv[kU];
 #pragma unroll

@@ -38,50 +38,31 @@ __device__ __forceinline__ bool key_surely_above(float cut, float d, float eta, 
   return v > __fmul_rn(__fmul_rn(cut, w), 1.01f);
 }
 
-// Calls f(key) for each of the (up to) four coefficients of Philox block g, leaving out those whose key is
-// certainly above `cut` (cut <= 0: none is left out).
+// Calls f(key) for each of the (up to) four coefficients of Philox block g that this scheduler owns.
 template <typename F>
-__device__ __forceinline__ void for_keys_of_group(const Problem& p, unsigned long long t, long long g, float cut, F&& f) {
+__device__ __forceinline__ void for_keys_of_group(const Problem& p, unsigned long long t, long long g, F&& f) {
   uint32_t w[4];
   philox4x32_10((uint32_t)g, (uint32_t)t, (uint32_t)(t >> 32), 0u, (uint32_t)p.seed, (uint32_t)(p.seed >> 32), w);
   const long long j0 = g * 4;
   const int mode = weight_mode_of(p.flags);
-  if (cut > 0.f && p.part_count <= 1 && j0 + 3 < p.J) {
-    const float4 d = __ldg(reinterpret_cast<const float4*>(p.delta + j0));
-    if (!key_surely_above(cut, d.x, p.eta, w[0], mode)) f(race_key64(d.x, p.eta, w[0], (uint32_t)j0, mode));
-    if (!key_surely_above(cut, d.y, p.eta, w[1], mode)) f(race_key64(d.y, p.eta, w[1], (uint32_t)j0 + 1, mode));
-    if (!key_surely_above(cut, d.z, p.eta, w[2], mode)) f(race_key64(d.z, p.eta, w[2], (uint32_t)j0 + 2, mode));
-    if (!key_surely_above(cut, d.w, p.eta, w[3], mode)) f(race_key64(d.w, p.eta, w[3], (uint32_t)j0 + 3, mode));
-    return;
-  }
-  if (p.part_count > 1) {                              // only the coefficients this scheduler owns take part
-    const unsigned int S = (unsigned)p.part_count, r0 = (unsigned int)j0 % S;
-#pragma unroll
-    for (unsigned int i = 0; i < 4; ++i)
-      if (j0 + i < p.J && (r0 + i) % S == (unsigned)p.part_index) {
-        const float d = __ldg(p.delta + j0 + i);
-        if (cut > 0.f && key_surely_above(cut, d, p.eta, w[i], mode)) continue;
-        f(race_key64(d, p.eta, w[i], (uint32_t)(j0 + i), mode));
-      }
-    return;
-  }
+  const unsigned int S = (unsigned)max(p.part_count, 1), r0 = S > 1u ? (unsigned int)j0 % S : 0u;
+  float d[4] = {0.f, 0.f, 0.f, 0.f};
   if (j0 + 3 < p.J) {
-    const float4 d = __ldg(reinterpret_cast<const float4*>(p.delta + j0));
-    f(race_key64(d.x, p.eta, w[0], (uint32_t)j0, mode));
-    f(race_key64(d.y, p.eta, w[1], (uint32_t)j0 + 1, mode));
-    f(race_key64(d.z, p.eta, w[2], (uint32_t)j0 + 2, mode));
-    f(race_key64(d.w, p.eta, w[3], (uint32_t)j0 + 3, mode));
+    const float4 v = __ldg(reinterpret_cast<const float4*>(p.delta + j0));
+    d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
   } else {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (j0 + i < p.J) f(race_key64(p.delta[j0 + i], p.eta, w[i], (uint32_t)(j0 + i), mode));
+    for (int i = 0; i < 4; ++i) if (j0 + i < p.J) d[i] = p.delta[j0 + i];
   }
+#pragma unroll
+  for (unsigned int i = 0; i < 4; ++i)
+    if (j0 + i < p.J && (S == 1u || (r0 + i) % S == (unsigned)p.part_index)) f(race_key64(d[i], p.eta, w[i], (uint32_t)(j0 + i), mode));
 }
 
 // The same with a cutoff, for a whole warp: lane l looks at Philox block g0 + l.  Few coefficients survive the
 // cheap test, so computing their keys on the spot would leave most lanes idle while one works; the survivors
 // (index, Philox word) go to a queue of the warp in shared memory instead and the keys of a full queue are
-// computed by all lanes together.  drain_keys() must follow the last call.
+// computed by all lanes together (drain_keys).
 constexpr int kQueue = 256;              // entries per warp; a call appends at most 128
 struct KeyQueue { uint2* slots; int n; };
 
@@ -89,6 +70,7 @@ template <typename F>
 __device__ __forceinline__ void drain_keys(const Problem& p, KeyQueue& q, F&& f) {
   const int mode = weight_mode_of(p.flags);
   __syncwarp();
+#pragma unroll 1
   for (int i = (int)(threadIdx.x & 31); i < q.n; i += 32) {
     const uint2 e = q.slots[i];
     f(race_key64(__ldg(p.delta + e.x), p.eta, e.y, e.x, mode));
@@ -97,9 +79,8 @@ __device__ __forceinline__ void drain_keys(const Problem& p, KeyQueue& q, F&& f)
   q.n = 0;
 }
 
-template <typename F>
 __device__ __forceinline__ void queue_keys_of_groups(const Problem& p, unsigned long long t, long long g0, long long groups,
-                                                     float cut, KeyQueue& q, F&& f) {
+                                                     float cut, KeyQueue& q) {
   const int lane = threadIdx.x & 31;
   const long long g = g0 + lane;
   const int mode = weight_mode_of(p.flags);
@@ -123,7 +104,6 @@ __device__ __forceinline__ void queue_keys_of_groups(const Problem& p, unsigned 
       if (in[i]) q.slots[q.n + __popc(mask & ((1u << lane) - 1u))] = make_uint2(j0 + i, w[i]);
       q.n += __popc(mask);
     }
-    if (q.n > kQueue - 128) drain_keys(p, q, f);
     return;
   }
   uint32_t w[4] = {0u, 0u, 0u, 0u};
@@ -148,7 +128,35 @@ __device__ __forceinline__ void queue_keys_of_groups(const Problem& p, unsigned 
     if (in) q.slots[q.n + __popc(mask & ((1u << lane) - 1u))] = make_uint2((uint32_t)(j0 + i), w[i]);
     q.n += __popc(mask);
   }
-  if (q.n > kQueue - 128) drain_keys(p, q, f);
+}
+
+// f(key) for every coefficient of the grid-stride share of this warp whose key may lie below the cutoff.  The queue is
+// drained in one place: a key's hundred instructions written out wherever a queue may be full made the kernels 110 and 54
+// KB long, and they come from a cold instruction cache every round.
+template <typename F>
+__device__ __forceinline__ void for_keys_below(const Problem& p, unsigned long long t, float cut, uint2* slots, F&& f) {
+  const long long groups = (p.J + 3) >> 2;
+  KeyQueue q = {slots, 0};
+#pragma unroll 1
+  for (long long g0 = (long long)blockIdx.x * kThreads + (threadIdx.x & ~31);; g0 += (long long)gridDim.x * kThreads) {
+    if (g0 < groups) queue_keys_of_groups(p, t, g0, groups, cut, q);
+    if (q.n > kQueue - 128 || g0 >= groups) drain_keys(p, q, f);
+    if (g0 >= groups) break;
+  }
+}
+
+// (rare, so out of the way: no cutoff yet, a cutoff that was too low, thousands of keys in one bin)  All keys whose top
+// `bits` bits are `prefix`, counted by their next `width` bits.
+__device__ __noinline__ void count_all_keys(const float* delta, long long J, float eta, unsigned int flags, unsigned long long seed, int part_count,
+                                            int part_index, unsigned long long t, long long first, long long step, int bits,
+                                            unsigned long long prefix, int width, unsigned int* sh) {
+  Problem q;                                             // what the keys depend on
+  q.delta = const_cast<float*>(delta); q.J = J; q.eta = eta; q.flags = flags; q.seed = seed; q.part_count = part_count; q.part_index = part_index;
+#pragma unroll 1
+  for (long long g = first; g < (J + 3) >> 2; g += step)
+    for_keys_of_group(q, t, g, [&](unsigned long long key) {
+      if (bits == 0 || (key >> (64 - bits)) == prefix) atomicAdd(&sh[(key >> (64 - bits - width)) & ((1u << width) - 1u)], 1u);
+    });
 }
 
 // Whole CTA (kThreads threads): the bin b with before(b) < k_rem <= before(b) + h[b], where before(b)
@@ -194,10 +202,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_sample_hist(Problem p, int mode
   __shared__ int s_last;
   __shared__ SelectState s_sel;
   const int tid = threadIdx.x;
+#pragma unroll 4
   for (int b = tid; b < kHistBins; b += kThreads) sh[b] = 0;
   __syncthreads();
   const unsigned long long t = *p.round_ptr + (unsigned long long)p.round_ahead;
-  const long long groups = (p.J + 3) >> 2;
   const float cut = mode == 1 ? p.st->t_cut : 0.f;
   const unsigned int cut_bin = cut > 0.f ? (__float_as_uint(cut) >> (32 - kHistBits)) : (unsigned)kHistBins;   // bins below it are complete
   // Guided pass: the keys below the cutoff (a few times P' of them) are also saved, so that the collect pass can
@@ -215,15 +223,13 @@ __global__ void __launch_bounds__(kThreads, 4) k_sample_hist(Problem p, int mode
   };
   if (cut > 0.f) {
     __shared__ uint2 s_queue[kThreads / 32][kQueue];
-    KeyQueue q = {s_queue[tid >> 5], 0};
-    for (long long g0 = (long long)blockIdx.x * kThreads + (tid & ~31); g0 < groups; g0 += (long long)gridDim.x * kThreads)
-      queue_keys_of_groups(p, t, g0, groups, cut, q, count);
-    drain_keys(p, q, count);
+    for_keys_below(p, t, cut, s_queue[tid >> 5], count);
   } else {
-    for (long long g = (long long)blockIdx.x * kThreads + tid; g < groups; g += (long long)gridDim.x * kThreads)
-      for_keys_of_group(p, t, g, 0.f, count);
+    count_all_keys(p.delta, p.J, p.eta, p.flags, p.seed, p.part_count, p.part_index, t, (long long)blockIdx.x * kThreads + tid,
+                   (long long)gridDim.x * kThreads, 0, 0ull, kHistBits, sh);
   }
   __syncthreads();
+#pragma unroll 4
   for (int b = tid; b < kHistBins; b += kThreads)
     if (sh[b]) atomicAdd(&p.hist[b], sh[b]);
   __threadfence();
@@ -265,8 +271,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_sample_hist(Problem p, int mode
       __syncthreads();
       for (int b = tid; b < kHistBins; b += kThreads) sh[b] = 0;
       __syncthreads();
-      for (long long g = tid; g < groups; g += kThreads)
-        for_keys_of_group(p, t, g, 0.f, [&](unsigned long long key) { atomicAdd(&sh[(unsigned int)(key >> (64 - kHistBits))], 1u); });
+      count_all_keys(p.delta, p.J, p.eta, p.flags, p.seed, p.part_count, p.part_index, t, tid, kThreads, 0, 0ull, kHistBits, sh);
       __syncthreads();
     }
   }
@@ -329,11 +334,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_sample_hist(Problem p, int mode
     __syncthreads();
     for (int b = tid; b < kHistBins; b += kThreads) sh[b] = 0;
     __syncthreads();
-    for (long long g = tid; g < groups; g += kThreads)
-      for_keys_of_group(p, t, g, 0.f, [&](unsigned long long key) {
-        if ((key >> (64 - bits)) == prefix)
-          atomicAdd(&sh[(key >> (64 - bits - width)) & ((1u << width) - 1u)], 1u);
-      });
+    count_all_keys(p.delta, p.J, p.eta, p.flags, p.seed, p.part_count, p.part_index, t, tid, kThreads, bits, prefix, width, sh);
     __syncthreads();
     find_bin(sh, 1 << width, (long long)p.n_cand - s_sel.n_sure, &s_bin, &s_before);
     if (tid == 0) {
@@ -352,7 +353,6 @@ __global__ void __launch_bounds__(kThreads) k_sample_collect(Problem p) {
   chain_begin();
   const SelectState sel = p.st->sel;
   const unsigned long long t = *p.round_ptr + (unsigned long long)p.round_ahead;
-  const long long groups = (p.J + 3) >> 2;
   const int shift = 64 - sel.bits;
   // keys certainly above the boundary's upper edge are not computed
   unsigned long long edge = sel.bits <= 32 ? ((sel.prefix + 1ull) << (32 - sel.bits)) : (sel.prefix >> (sel.bits - 32));
@@ -372,19 +372,18 @@ __global__ void __launch_bounds__(kThreads) k_sample_collect(Problem p) {
   const int tid = threadIdx.x;
   if (p.st->surv_valid) {                              // every key below the first pass's cutoff is at hand
     const unsigned int n = p.st->surv_count;
+#pragma unroll 1
     for (unsigned int i = blockIdx.x * (unsigned)kThreads + tid; i < n; i += gridDim.x * (unsigned)kThreads)
       take(__ldcg(p.survivors + i));
     return;
   }
   if (cut > 0.f) {
     __shared__ uint2 s_queue[kThreads / 32][kQueue];
-    KeyQueue q = {s_queue[tid >> 5], 0};
-    for (long long g0 = (long long)blockIdx.x * kThreads + (tid & ~31); g0 < groups; g0 += (long long)gridDim.x * kThreads)
-      queue_keys_of_groups(p, t, g0, groups, cut, q, take);
-    drain_keys(p, q, take);
+    for_keys_below(p, t, cut, s_queue[tid >> 5], take);
   } else {
-    for (long long g = (long long)blockIdx.x * kThreads + tid; g < groups; g += (long long)gridDim.x * kThreads)
-      for_keys_of_group(p, t, g, 0.f, take);
+#pragma unroll 1
+    for (long long g = (long long)blockIdx.x * kThreads + tid; g < (p.J + 3) >> 2; g += (long long)gridDim.x * kThreads)
+      for_keys_of_group(p, t, g, take);
   }
 }
 

@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(kThreads) k_apply_dense(Problem p, const int* 
 #pragma unroll
   for (int k = 0; k < 4; ++k)
     if (a_lo + k < a_hi) { d_first[k] = change_of(a_lo + k); mine += d_first[k] != 0.0; }
+#pragma unroll 1
   for (int a = a_lo + 4; a < a_hi; ++a) mine += change_of(a) != 0.0;
   int incl = mine;
 #pragma unroll
@@ -166,6 +167,7 @@ __global__ void __launch_bounds__(kThreads) k_apply_dense(Problem p, const int* 
   const int rank0 = before + incl - mine;                 // rank of this thread's first moving entry
 
   double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+#pragma unroll 1
   for (int base = 0; base < n_moving; base += kStageCols) {
     const int n_here = min(kStageCols, n_moving - base);
     if (base > 0) __syncthreads();
@@ -180,10 +182,12 @@ __global__ void __launch_bounds__(kThreads) k_apply_dense(Problem p, const int* 
 #pragma unroll
       for (int k = 0; k < 4; ++k)
         if (a_lo + k < a_hi) place(a_lo + k, d_first[k]);
+#pragma unroll 1
       for (int a = a_lo + 4; a < a_hi; ++a) place(a, change_of(a));
     }
     __syncthreads();
     if (i < p.N) {
+#pragma unroll 1
       for (int a0 = slot; a0 < n_here; a0 += kColSlots * 8) {
         float4 xv[8];
         double d[8];
@@ -216,6 +220,7 @@ __global__ void __launch_bounds__(kThreads) k_apply_dense(Problem p, const int* 
   DeviceState* st = p.st;
   const int cta = blockIdx.x, n_ctas = gridDim.x;
   if (proposals) {
+#pragma unroll 1
     for (int a = cta * kThreads + tid; a < p.n_keep; a += n_ctas * kThreads) {
       if (a >= n_kept) { p.dbeta[a] = 0.f; continue; }
       const int pos = p.kept_pos[a], j = kept[a];
