@@ -397,7 +397,7 @@ def measure(workload: str, args, device, rank: int, world: int, dist_ok: bool, p
     e2e_kept_all, e2e_ms = aggregate(e2e_kept, (time.perf_counter() - t0) * 1e3, dist_ok, device)
     h2d = 4 * (2 * p.n_cols + p.n_rows)
     rec["e2e"] = {"value": e2e_kept_all / (e2e_ms * 1e-3), "unit": UNIT, "h2d_bytes_per_step": h2d,
-                  "d2h_bytes_per_step": h2d + 4 * (2 * p.n_keep + 4), "steps": e2e_steps}
+                  "d2h_bytes_per_step": 4 * p.n_rows + 16 * p.n_keep + 16, "steps": e2e_steps}   # resid; kept, dbeta, beta, delta of the kept; counts
 
     # ---- CPU baseline: the oracle on a bounded sample of the same workload (rank 0, N = 1 only) ----
     rec["cpu_baseline"] = None

@@ -177,9 +177,11 @@ int strads_round(strads_handle_t h, const strads_round_out_t* out);
 int strads_run(strads_handle_t h, int64_t n_rounds);
 
 /* The same round as strads_round for callers whose state lives in HOST memory: copies
- * beta[J], resid[N], delta[J] host->device, runs one round, copies them back together with
- * the optional host outputs (kept [P], dbeta [P], counts [4]; NULL = not wanted), and waits
- * for the stream.  Host buffers should be pinned for the copies to be asynchronous. */
+ * beta[J], resid[N], delta[J] host->device, runs one round, brings back what it changed (resid, and beta and
+ * delta of the kept coefficients) together with the optional host outputs (kept [P], dbeta [P], counts [4];
+ * NULL = not wanted), and waits for the stream.  Host buffers should be pinned for the copies to be
+ * asynchronous.  The first call allocates 16 P + 16 bytes of pinned host memory, which outlives the handle as
+ * its streams do (strads_release_cached). */
 int strads_round_host(strads_handle_t h, float* beta_host, float* resid_host, float* delta_host,
                       int32_t* kept_host, float* dbeta_host, int32_t* counts_host);
 

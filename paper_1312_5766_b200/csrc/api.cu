@@ -88,6 +88,8 @@ struct Kit {
   cudaEvent_t ahead_fork, ahead_done, retry_fork, retry_done, patch_fork, patch_done, copy_fork, copy_done, fork;
   cudaEvent_t ready[STRADS_MAX_SCHEDULERS], updated[STRADS_MAX_SCHEDULERS];
   cudaGraphExec_t exec[4];
+  unsigned char* results;    // strads_round_host: pinned, 16 P + 16 bytes (at most 256 KB)
+  size_t results_bytes;
 };
 
 namespace {
@@ -131,6 +133,7 @@ void destroy_kit(Kit* k) {
     if (k->updated[i] != nullptr) cudaEventDestroy(k->updated[i]);
   }
   for (cudaGraphExec_t x : k->exec) if (x != nullptr) cudaGraphExecDestroy(x);
+  if (k->results != nullptr) cudaFreeHost(k->results);
   if (before != k->device) cudaSetDevice(before);
   delete k;
 }
@@ -426,8 +429,8 @@ int one_round(strads_lasso_s* h, const strads_round_out_t* out, cudaEvent_t befo
   if (ev) { CK(cudaEventRecord(ev[5], h->stream)); h->prof_rounds += 1; }
   h->round_host += 1;
   if (out != nullptr) {
-    if (out->cand) CK(cudaMemcpyAsync(out->cand, p.cand, sizeof(int) * p.n_cand, cudaMemcpyDeviceToDevice, h->stream));
-    if (out->kept || out->dbeta || out->counts) CK(launch_export(p, p.kept, out->kept, out->dbeta, out->counts, h->stream));
+    if (out->cand || out->kept || out->dbeta || out->counts)
+      CK(launch_export(p, p.kept, {out->cand, out->kept, out->dbeta, out->counts, nullptr, nullptr}, h->stream));
   }
   return STRADS_OK;
 }
@@ -949,6 +952,20 @@ int strads_round_host(strads_handle_t h, float* beta_host, float* resid_host, fl
   if (h == nullptr || !beta_host || !resid_host || !delta_host) return STRADS_ERR_INVALID_ARG;
   const Problem& p = on_turn(h).p;
   if (p.flags & STRADS_FLAG_LOGISTIC) return STRADS_ERR_UNSUPPORTED;      // (the margin lives on the device)
+  // A round changes beta and delta of the kept coefficients only; the host's copies of the others are the ones that were sent.
+  // So the residual comes back and the kept coefficients' values, which the last kernel writes to pinned memory itself
+  // (10,000 x 100,000: two copies of 400 KB and four small ones cost 27 us of a 127 us round behind its update).
+  const size_t P = (size_t)p.n_keep, need = 16 * P + 16;
+  if (h->kit->results_bytes < need) {
+    if (h->kit->results != nullptr) CK(cudaFreeHost(h->kit->results));
+    h->kit->results = nullptr; h->kit->results_bytes = 0;
+    CK(cudaHostAlloc(reinterpret_cast<void**>(&h->kit->results), need, cudaHostAllocPortable));
+    h->kit->results_bytes = need;
+  }
+  Export to = {};
+  to.counts = reinterpret_cast<int*>(h->kit->results);
+  to.kept = to.counts + 4;
+  to.dbeta = reinterpret_cast<float*>(to.kept + P); to.beta = to.dbeta + P; to.delta = to.beta + P;
   // delta first, on the handle's stream: the draw can start as soon as it is there; beta and the residual follow on
   // a second stream (behind whatever the handle's stream still has in flight) and are awaited before the Gram
   CK(cudaEventRecord(h->copy_fork, h->stream));
@@ -965,13 +982,19 @@ int strads_round_host(strads_handle_t h, float* beta_host, float* resid_host, fl
     const int rc = one_round(h, nullptr, h->copy_done);
     if (rc) return rc;
   }
-  CK(cudaMemcpyAsync(beta_host, p.beta, sizeof(float) * p.J, cudaMemcpyDeviceToHost, h->stream));
+  CK(launch_export(p, p.kept, to, h->stream));
   CK(cudaMemcpyAsync(resid_host, p.resid, sizeof(float) * p.N, cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaMemcpyAsync(delta_host, p.delta, sizeof(float) * p.J, cudaMemcpyDeviceToHost, h->stream));
-  if (kept_host) CK(cudaMemcpyAsync(kept_host, p.kept, sizeof(int) * p.n_keep, cudaMemcpyDeviceToHost, h->stream));
-  if (dbeta_host) CK(cudaMemcpyAsync(dbeta_host, p.dbeta, sizeof(float) * p.n_keep, cudaMemcpyDeviceToHost, h->stream));
-  if (counts_host) CK(cudaMemcpyAsync(counts_host, p.st->counts, sizeof(int) * 4, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
+  const int n_kept = to.counts[2] < p.n_keep ? to.counts[2] : p.n_keep;
+  for (int a = 0; a < n_kept; ++a) {
+    const int j = to.kept[a];
+    if (j < 0 || j >= p.J) continue;                     // (never, unless a wait expired)
+    beta_host[j] = to.beta[a];
+    delta_host[j] = to.delta[a];
+  }
+  if (kept_host) memcpy(kept_host, to.kept, sizeof(int) * P);
+  if (dbeta_host) memcpy(dbeta_host, to.dbeta, sizeof(float) * P);
+  if (counts_host) memcpy(counts_host, to.counts, sizeof(int) * 4);
   return STRADS_OK;
 }
 
@@ -998,7 +1021,7 @@ int strads_filter(strads_handle_t h, const int32_t* cand_dev, int32_t n_cand, in
   CK(launch_set_counts(sc.p, n_cand, 0, 0, h->stream));
   const int rc = gram_and_filter(sc, h->stream, cand_dev, n_cand, gram_dev_or_null);
   if (rc) return rc;
-  CK(launch_export(sc.p, sc.p.kept, kept_dev, nullptr, counts_dev, h->stream));
+  CK(launch_export(sc.p, sc.p.kept, {nullptr, kept_dev, nullptr, counts_dev, nullptr, nullptr}, h->stream));
   return STRADS_OK;
 }
 
@@ -1011,7 +1034,7 @@ int strads_update(strads_handle_t h, const int32_t* kept_dev, int32_t n_kept, fl
   if (n_kept > 0)
     CK(cudaMemcpyAsync(p.kept, kept_dev, sizeof(int) * n_kept, cudaMemcpyDeviceToDevice, h->stream));
   CK(launch_update(p, p.kept, 0, false, h->stream));
-  if (dbeta_dev) CK(launch_export(p, p.kept, nullptr, dbeta_dev, nullptr, h->stream));
+  if (dbeta_dev) CK(launch_export(p, p.kept, {nullptr, nullptr, dbeta_dev, nullptr, nullptr, nullptr}, h->stream));
   return STRADS_OK;
 }
 

@@ -482,7 +482,9 @@ cudaError_t launch_filter(const Problem& p, const int* cand, int n_cand, int n_t
                           cudaStream_t s, bool only_if_pending = false);
 cudaError_t launch_update(const Problem& p, const int* kept, int advance, bool after_pack, cudaStream_t s, int gate = 0);
 cudaError_t launch_set_counts(const Problem& p, int n_cand, int n_examined, int n_kept, cudaStream_t s);
-cudaError_t launch_export(const Problem& p, const int* kept, int* kept_out, float* dbeta_out, int* counts_out,
-                          cudaStream_t s);
+// Copies of a round's results (null: not wanted): the candidates, the kept list filled up with -1, the changes filled up with
+// 0, the four counts; beta and delta of the kept coefficients as they are now (both or neither).
+struct Export { int* cand; int* kept; float* dbeta; int* counts; float* beta; float* delta; };
+cudaError_t launch_export(const Problem& p, const int* kept, const Export& to, cudaStream_t s);
 
 }  // namespace strads

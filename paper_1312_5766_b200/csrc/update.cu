@@ -331,14 +331,21 @@ __global__ void k_set_counts(Problem p, int n_cand, int n_examined, int n_kept) 
   p.st->counts[0] = n_cand; p.st->counts[1] = n_examined; p.st->counts[2] = n_kept; p.st->counts[3] = 0;
 }
 
-__global__ void k_export(Problem p, const int* kept, int* kept_out, float* dbeta_out, int* counts_out) {
+// What a round leaves for its caller, in one launch (the candidates as a copy of their own cost the chain 4 us: a copy waits
+// for the kernel before it and the next kernel for the copy).  The destinations may be host memory the device can write.
+__global__ void k_export(Problem p, const int* kept, Export to) {
   chain_begin();
-  const int n_kept = p.st->counts[2];
-  for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < p.n_keep; a += gridDim.x * blockDim.x) {
-    if (kept_out != nullptr) kept_out[a] = a < n_kept ? kept[a] : -1;
-    if (dbeta_out != nullptr) dbeta_out[a] = a < n_kept ? p.dbeta[a] : 0.f;
+  const int n_kept = p.st->counts[2], first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+  for (int a = first; a < p.n_keep; a += step) {
+    const bool on = a < n_kept;
+    const int j = on ? kept[a] : -1;
+    if (to.kept != nullptr) to.kept[a] = j;
+    if (to.dbeta != nullptr) to.dbeta[a] = on ? p.dbeta[a] : 0.f;
+    if (to.beta != nullptr && on) { to.beta[a] = p.beta[j]; to.delta[a] = p.delta[j]; }
   }
-  if (counts_out != nullptr && blockIdx.x == 0 && threadIdx.x < 4) counts_out[threadIdx.x] = p.st->counts[threadIdx.x];
+  if (to.cand != nullptr)
+    for (int i = first; i < p.n_cand; i += step) to.cand[i] = p.cand[i];
+  if (to.counts != nullptr && first < 4) to.counts[first] = p.st->counts[first];
 }
 
 }  // namespace
@@ -370,9 +377,9 @@ cudaError_t launch_set_counts(const Problem& p, int n_cand, int n_examined, int 
   return launch_chained(k_set_counts, 1, 1, 0, s, p, n_cand, n_examined, n_kept);
 }
 
-cudaError_t launch_export(const Problem& p, const int* kept, int* kept_out, float* dbeta_out, int* counts_out,
-                          cudaStream_t s) {
-  return launch_chained(k_export, (p.n_keep + 255) / 256, 256, 0, s, p, kept, kept_out, dbeta_out, counts_out);
+cudaError_t launch_export(const Problem& p, const int* kept, const Export& to, cudaStream_t s) {
+  const int n = to.cand != nullptr && p.n_cand > p.n_keep ? p.n_cand : p.n_keep;
+  return launch_chained(k_export, (n + 255) / 256, 256, 0, s, p, kept, to);
 }
 
 }  // namespace strads
