@@ -1937,6 +1937,7 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, const Engin
   if (cta == 0 && tid == 0) {
     EngineState* es = e.es;
     es->n_kept = s.kept; es->n_examined = s.examined; es->walk_open = 0;
+    if (es->avoid > 0) es->avoid -= 1;
     if (e.window < n) es->skip_window = s.kept == p.n_keep && s.examined <= e.window ? 0 : 1;
   }
   return true;
@@ -2026,7 +2027,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
     if (kDense) {
       if (n < n_total && es->skip_window && !no_filter) n = n_total;
     } else {
-      window = no_filter || (p.bucket_count != nullptr && !(n < n_total && es->skip_window) && t >= es->avoid_until);
+      window = no_filter || (p.bucket_count != nullptr && !(n < n_total && es->skip_window) && es->avoid == 0);
       if (real) csc_enter(p, e, window ? n : n_total, window && !no_filter);
     }
     // ---- steps 1 to 3, once more over all candidates where a window does not do ----
@@ -2118,7 +2119,8 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
             es->n_kept = s_kept; es->n_examined = s_examined;
             es->walk_open = !settled || (s_kept < p.n_keep && n < n_total) ? 1 : 0;
             // after an overflow the buckets are left alone: for a round, then twice as long after every further one, to 64
-            if (!settled) es->avoid_until = t + (1ull << es->streak);
+            // (a count of rounds, not the round to wait for: strads_set_round may go back); this round's walk counts too
+            if (!settled) es->avoid = 1 + (1 << es->streak);
             es->streak = settled ? 0 : min(es->streak + 1, 6);
             es->bucket_failed = 0; es->edge_count = 0u;
           }

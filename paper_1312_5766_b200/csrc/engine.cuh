@@ -17,8 +17,7 @@ struct EngineState {
   int walk_open;                // the walk could not finish: fewer than P kept inside a window, or chains too long
   int mend;                     // a draw's selection has to be mended
   int streak;                   // CSC: attempts with the row buckets in a row that overflowed (or left the walk open)
-  int pad;
-  unsigned long long avoid_until;   // CSC: first round in which they are tried again
+  int avoid;                    // CSC: rounds until they are tried again
 };
 
 // How the pairs of a list are cut into tiles of the dense Gram: kGramRows x cols, K in stages of 128 elements (64 with three
