@@ -248,7 +248,8 @@ def rooflines(p: wl.LassoProblem, workload: str, step_ms: dict, kept_per_round: 
             "algorithmic_ops_per_launch": ops,
             "peak_source": "148 SMs x 128 lanes x max SM clock: one merge step (compare + advance) per lane per cycle",
             "note": "inner products of sparse columns counted as sorted-list merge steps, over a few MB of columns: bound by "
-                    "dependent loads and barriers, not by HBM"}
+                    "dependent loads and barriers, not by HBM; the timed regions make this step inside whole rounds in one "
+                    "launch, launch_ms is the kernel that makes it where the steps are launched one by one"}
         upd_bytes = 8.0 * nnz_col * kept_per_round + 8.0 * p.n_rows
         pack_bytes = 0.0
         ns_bytes = 8.0 * nnz_col * (p.n_candidates + kept_per_round) + 8.0 * p.n_rows
@@ -270,26 +271,22 @@ def rooflines(p: wl.LassoProblem, workload: str, step_ms: dict, kept_per_round: 
     return out
 
 
-def launches_per_round(p: wl.LassoProblem) -> int:
-    """Kernels of the library launched per round of strads_run (its fixed sequence; launches of the whole-list retry
-    return at once when the window sufficed)."""
-    window = window_of(p)
-    if p.layout == wl.DENSE:
-        n = 3              # the early draw of the next round: histogram pass, collect pass, ordering
-        n += 1             # correction of the early list
-        n += 2             # pack, window Gram (screen + cluster split-K + recheck + walk)
-        n += 1             # update
-        if window < p.n_candidates:
-            # retry branch: walk kernel on the window (if the Gram's last CTA left it the job), pack, screen, recheck, 3xTF32,
-            # walk of the whole list, gated correction of the early list, gated update
-            n += 8
-        else:
-            n += 3         # no window: recheck, 3xTF32 fallback, walk kernel
-        return n
-    n = 3 + 3 + 1 + 3      # draw; bucket fill, bucket dots, all-pairs fallback; walk; dot, scatter, apply
-    if window < p.n_candidates:
-        n += 1             # cooperative on-demand walk
-    return n
+def launches_of_run(p: wl.LassoProblem, steps: int) -> int:
+    """Kernels of the library launched by a strads_run of `steps` rounds (dense: a fixed sequence per round; launches of the
+    retry branch return at once when the screen's last CTA settled the round)."""
+    if p.layout != wl.DENSE:
+        return (steps + 31) // 32          # whole rounds in one launch, 32 of them at most
+    n = 3                  # the early draw of the next round: histogram pass, collect pass, ordering
+    n += 1                 # correction of the early list
+    n += 2                 # pack, Gram (screen + cluster split-K + recheck + walk)
+    n += 1                 # update
+    if window_of(p) < p.n_candidates:
+        # retry branch: walk kernel on the window (if the Gram's last CTA left it the job), pack, screen, recheck, 3xTF32,
+        # walk of the whole list, gated correction of the early list, gated update
+        n += 8
+    else:
+        n += 5             # no window: recheck, 3xTF32 fallback, walk kernel, gated correction and update
+    return n * steps
 
 
 def measure(workload: str, args, device, rank: int, world: int, dist_ok: bool, peaks: dict, with_cpu: float,
@@ -415,7 +412,7 @@ def measure(workload: str, args, device, rank: int, world: int, dist_ok: bool, p
         else:
             rec["cpu_baseline"] = {"value": None, "unit": UNIT, "cores": 1, "kind": "oracle",
                                    "sample": "not run: the host has too little free memory for a copy of the design matrix"}
-    rec["gpu_launches"] = launches_per_round(p) * args.steps * REPEATS
+    rec["gpu_launches"] = launches_of_run(p, args.steps) * REPEATS
     s.close()
     del s, p
     torch.cuda.empty_cache()
