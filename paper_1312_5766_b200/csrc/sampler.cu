@@ -518,7 +518,7 @@ cudaError_t prepare_sample(const Problem&) {
 cudaError_t launch_sample_patch(const Problem& p, const Problem& ahead, int* cand_out, cudaStream_t s, bool from_cand,
                                 int gate) {
   const int ctas = (ahead.n_cand + 31) / 32 + (p.n_keep + 7) / 8;        // list elements by eight threads, new keys by warp
-  return launch_chained(k_sample_patch, ctas, 256, 2 * sizeof(unsigned long long) * (size_t)p.n_keep, s, p,
+  return launch_chained_split(p.layout == STRADS_DENSE_COLMAJOR, k_sample_patch, ctas, 256, 2 * sizeof(unsigned long long) * (size_t)p.n_keep, s, p,
                         (const unsigned long long*)ahead.keys_out, ahead.n_cand, cand_out, from_cand ? 1 : 0, gate);
 }
 
