@@ -791,12 +791,12 @@ __device__ __forceinline__ unsigned int bf16x2_bits(float a, float b) {
   return *reinterpret_cast<const unsigned int*>(&v);
 }
 __device__ __forceinline__ float bf16_residue(float x) { return x - __bfloat162float(__float2bfloat16_rn(x)); }
-__device__ __forceinline__ void store_parts(uint2* bhi, uint2* blo, const float4& x, bool low_parts) {
+__device__ __forceinline__ void store_parts(uint2* bhi, uint2* blo, const float4& x) {
   *bhi = make_uint2(bf16x2_bits(x.x, x.y), bf16x2_bits(x.z, x.w));
-  if (low_parts) *blo = make_uint2(bf16x2_bits(bf16_residue(x.x), bf16_residue(x.y)), bf16x2_bits(bf16_residue(x.z), bf16_residue(x.w)));
+  *blo = make_uint2(bf16x2_bits(bf16_residue(x.x), bf16_residue(x.y)), bf16x2_bits(bf16_residue(x.z), bf16_residue(x.w)));
 }
 
-constexpr int kHeld = 10;                  // groups of four rows of r a thread holds: N <= 4 * 512 * 10
+constexpr int kHeld = 4;                   // groups of four rows of r a thread holds: a group has a lane per 16 rows or more (pack_group)
 constexpr size_t kPackSmem = 160 * 1024;
 
 __device__ __forceinline__ int pack_group(int n4) {
@@ -826,9 +826,8 @@ __device__ __forceinline__ void mask_rows(const Problem& p, int gi, float4& x) {
   x.w = 0.f;
 }
 
-// products: also x_c^T r and what follows from it (false: the copies alone).
 __device__ void dense_pack(const Problem& p, const Engine& e, unsigned char* sm, TurnShared& ts, PackBars& bars, int lo, int hi,
-                           unsigned long long t_next, bool products, bool want_keys, bool low_parts, uint32_t wait_limit) {
+                           unsigned long long t_next, bool want_keys, uint32_t wait_limit) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int cta = (int)blockIdx.x, n_ctas = (int)gridDim.x;
   const int n4 = (int)((p.N + 3) >> 2), n4_whole = (int)(p.N >> 2);
@@ -837,25 +836,20 @@ __device__ void dense_pack(const Problem& p, const Engine& e, unsigned char* sm,
   // columns of a group under way at once
   const uint32_t col_bytes = (uint32_t)n4 * 16u;
   int depth = (int)min((size_t)4, kPackSmem / ((size_t)groups * col_bytes));
-  const bool bulk = depth > 0 && n4 <= kHeld * 32 * group;
   depth = min(depth, kWarps / groups);                   // (a barrier per column under way)
   const uint32_t slots = smem_u32(sm) + (uint32_t)(grp * depth) * col_bytes;
   const int at0 = part * 32 + lane, step = 32 * group;
   float4 rv[kHeld];
-  if (bulk) {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");         // what this CTA last did with the slots is over
-    __syncthreads();
-    if (part == 0 && lane == 0)
-      for (int i = 0; i < depth && grp + i * groups < mine; ++i) {
-        const uint32_t bar = smem_u32(&bars.full[grp * depth + i]);
-        mbar_expect(bar, col_bytes);
-        bulk_load(slots + (uint32_t)i * col_bytes, p.xv + (long long)p.cand[lo + cta + n_ctas * (grp + i * groups)] * p.ld, col_bytes, bar);
-      }
-    if (products) {
-#pragma unroll
-      for (int u = 0; u < kHeld; ++u) rv[u] = u * step + at0 < n4 ? resid4(p, u * step + at0, n4, n4_whole) : make_float4(0.f, 0.f, 0.f, 0.f);
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");           // what this CTA last did with the slots is over
+  __syncthreads();
+  if (part == 0 && lane == 0)
+    for (int i = 0; i < depth && grp + i * groups < mine; ++i) {
+      const uint32_t bar = smem_u32(&bars.full[grp * depth + i]);
+      mbar_expect(bar, col_bytes);
+      bulk_load(slots + (uint32_t)i * col_bytes, p.xv + (long long)p.cand[lo + cta + n_ctas * (grp + i * groups)] * p.ld, col_bytes, bar);
     }
-  }
+#pragma unroll
+  for (int u = 0; u < kHeld; ++u) rv[u] = u * step + at0 < n4 ? resid4(p, u * step + at0, n4, n4_whole) : make_float4(0.f, 0.f, 0.f, 0.f);
   int seen = 0;                                          // columns this group has been through
   for (int k0 = 0; k0 < mine; k0 += kTurn) {
     const int turn = min(kTurn, mine - k0);
@@ -864,7 +858,7 @@ __device__ void dense_pack(const Problem& p, const Engine& e, unsigned char* sm,
     float E = 0.f;
     Proposal prop = {};
     bool dormant = false;
-    if (products && warp == kWarps - 1 && lane < turn) {
+    if (warp == kWarps - 1 && lane < turn) {
       j_own = p.cand[lo + cta + n_ctas * (k0 + lane)];
       const double n_own = p.n2[j_own];
       const float b_own = p.beta[j_own], d_own = p.delta[j_own];
@@ -878,59 +872,34 @@ __device__ void dense_pack(const Problem& p, const Engine& e, unsigned char* sm,
       uint2* bhi = reinterpret_cast<uint2*>(e.xb + (long long)a * e.xb_pitch);
       uint2* blo = reinterpret_cast<uint2*>(e.xb + (long long)a * e.xb_pitch + e.lo_off);
       float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
-      if (bulk) {
-        const int slot = seen % depth, b = grp * depth + slot;
-        const uint32_t ph = (bars.uses[b] + (unsigned)(seen / depth)) & 1u;
-        if (!mbar_wait(smem_u32(&bars.full[b]), ph, wait_limit) && lane == 0) atomicOr(&p.st->status, STRADS_STATUS_WAIT_EXPIRED);
-        const uint32_t src = slots + (uint32_t)slot * col_bytes;
+      const int slot = seen % depth, b = grp * depth + slot;
+      const uint32_t ph = (bars.uses[b] + (unsigned)(seen / depth)) & 1u;
+      if (!mbar_wait(smem_u32(&bars.full[b]), ph, wait_limit) && lane == 0) atomicOr(&p.st->status, STRADS_STATUS_WAIT_EXPIRED);
+      const uint32_t src = slots + (uint32_t)slot * col_bytes;
 #pragma unroll
-        for (int u = 0; u < kHeld; ++u) {
-          const int gi = u * step + at0;
-          if (gi >= n4) break;
-          float4 x;
-          asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(src + (uint32_t)gi * 16u) : "memory");
-          if (gi >= n4_whole) mask_rows(p, gi, x);
-          store_parts(bhi + gi, blo + gi, x, low_parts);
-          if (!products) continue;
-          dot_step(x.x, rv[u].x, h0, l0); dot_step(x.y, rv[u].y, h1, l1);
-          dot_step(x.z, rv[u].z, h0, l0); dot_step(x.w, rv[u].w, h1, l1);
-        }
-        const int nxt = grp + (seen + depth) * groups;   // the column that comes into this slot next
-        if (nxt < mine) {
-          if (group > 1) asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "r"(32 * group) : "memory");
-          else __syncwarp();
-          if (part == 0 && lane == 0) {
-            const uint32_t bar = smem_u32(&bars.full[b]);
-            mbar_expect(bar, col_bytes);
-            bulk_load(src, p.xv + (long long)p.cand[lo + cta + n_ctas * nxt] * p.ld, col_bytes, bar);
-          }
-        }
-      } else {                                           // long columns: straight from global memory
-        const float4* xs = reinterpret_cast<const float4*>(p.xv + (long long)p.cand[a] * p.ld);
-        constexpr int kU = 4;
-        for (int g0 = at0; g0 < n4; g0 += kU * step) {
-          float4 x[kU], r[kU];
-#pragma unroll
-          for (int u = 0; u < kU; ++u) x[u] = g0 + u * step < n4 ? __ldg(xs + g0 + u * step) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-          for (int u = 0; u < kU; ++u) r[u] = resid4(p, g0 + u * step, n4, n4_whole);
-#pragma unroll
-          for (int u = 0; u < kU; ++u) {
-            const int gi = g0 + u * step;
-            if (gi >= n4) break;
-            if (gi >= n4_whole) mask_rows(p, gi, x[u]);
-            store_parts(bhi + gi, blo + gi, x[u], low_parts);
-            dot_step(x[u].x, r[u].x, h0, l0); dot_step(x[u].y, r[u].y, h1, l1);
-            dot_step(x[u].z, r[u].z, h0, l0); dot_step(x[u].w, r[u].w, h1, l1);
-          }
+      for (int u = 0; u < kHeld; ++u) {
+        const int gi = u * step + at0;
+        if (gi >= n4) break;
+        float4 x;
+        asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(src + (uint32_t)gi * 16u) : "memory");
+        if (gi >= n4_whole) mask_rows(p, gi, x);
+        store_parts(bhi + gi, blo + gi, x);
+        dot_step(x.x, rv[u].x, h0, l0); dot_step(x.y, rv[u].y, h1, l1);
+        dot_step(x.z, rv[u].z, h0, l0); dot_step(x.w, rv[u].w, h1, l1);
+      }
+      const int nxt = grp + (seen + depth) * groups;   // the column that comes into this slot next
+      if (nxt < mine) {
+        if (group > 1) asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "r"(32 * group) : "memory");
+        else __syncwarp();
+        if (part == 0 && lane == 0) {
+          const uint32_t bar = smem_u32(&bars.full[b]);
+          mbar_expect(bar, col_bytes);
+          bulk_load(src, p.xv + (long long)p.cand[lo + cta + n_ctas * nxt] * p.ld, col_bytes, bar);
         }
       }
-      if (products) {
-        const double v = warp_sum(((double)h0 + (double)l0) + ((double)h1 + (double)l1));
-        if (lane == 0) ts.dot[k][part] = v;
-      }
+      const double v = warp_sum(((double)h0 + (double)l0) + ((double)h1 + (double)l1));
+      if (lane == 0) ts.dot[k][part] = v;
     }
-    if (!products) continue;
     __syncthreads();
     if (warp == kWarps - 1 && lane < turn) {
       const int a = lo + cta + n_ctas * (k0 + lane);
@@ -941,11 +910,9 @@ __device__ void dense_pack(const Problem& p, const Engine& e, unsigned char* sm,
     }
     __syncthreads();
   }
-  if (bulk) {
-    __syncthreads();
-    if (part == 0 && lane == 0)                          // every slot's barrier has completed this many more phases
-      for (int i = 0; i < depth; ++i) bars.uses[grp * depth + i] += (unsigned)((seen - i + depth - 1) / depth);
-  }
+  __syncthreads();
+  if (part == 0 && lane == 0)                            // every slot's barrier has completed this many more phases
+    for (int i = 0; i < depth; ++i) bars.uses[grp * depth + i] += (unsigned)((seen - i + depth - 1) / depth);
   // the copies are read by bulk tensor copies (another proxy) behind the next barrier
   asm volatile("fence.proxy.async;" ::: "memory");
 }
@@ -954,10 +921,9 @@ __device__ void dense_pack(const Problem& p, const Engine& e, unsigned char* sm,
 // Dense, step 2: conflict bits of all candidate pairs on the tensor cores: tiles of 128 rows x 64 or 128 columns of the
 // upper triangle, BF16 operands by TMA (128-byte swizzle) into a ring in shared memory, tcgen05.mma into tensor memory.
 // As in gram_dense_tc.cu the result is a screen: pairs closer to rho than its error bound go to a list and are decided
-// from exact products.
-//   one term    hi.hi: off by at most 2^-8 relative (operands rounded to 8 bits)
-//   three terms hi.hi + hi.lo + lo.hi: off by at most 3 * 2^-18; for short columns, whose correlations scatter so widely
-//               (standard deviation N^-1/2) that the wider band would leave percents of all pairs open
+// from exact products.  The columns are short, so their correlations scatter widely (standard deviation N^-1/2) and the
+// error band of a product of BF16 roundings (2^-8) would leave percents of all pairs open: three products, hi.hi + hi.lo
+// + lo.hi, off by at most 3 * 2^-18.
 // What bounds it is bringing operands from L2 to shared memory (~110 GB/s an SM), so K is split until every CTA has a
 // share; the CTAs of a tile leave their partial sums in global memory, wait for one another (they all run at once) and
 // each adds up and thresholds its share of the rows.  A tile of 128 columns reads fewer operand bytes per product, one
@@ -969,8 +935,7 @@ constexpr int kMaxStages = 4;
 constexpr size_t kGramSmem = (size_t)kRingBytes + 1024;
 constexpr uint32_t kTmemCols = 128;
 
-// A stage holds two blocks of 64 elements of K for both operands: consecutive ones (one term) or the high and the low
-// parts of one (three terms).  Its size depends on the tile's width alone, so there is a set of barriers per width.
+// A stage holds the high and the low parts of 64 elements of K for both operands.  Its size depends on the tile's width alone, so there is a set of barriers per width.
 struct GramShared {
   unsigned long long full[2][kMaxStages], empty[2][kMaxStages], done;
   uint32_t tmem;
@@ -981,9 +946,7 @@ struct GramShared {
 // Phases of the barriers so far (the same in all threads of a CTA).
 struct GramCount { unsigned int stages[2], units; };
 
-__device__ __forceinline__ double engine_band(long long N, int terms) {
-  return terms == 1 ? 1.0 / 128.0 + (double)N * (1.0 / 33554432.0) : 1.0 / 32768.0 + 3.0 * (double)N * (1.0 / 33554432.0);
-}
+__device__ __forceinline__ double engine_band(long long N) { return 1.0 / 32768.0 + 3.0 * (double)N * (1.0 / 33554432.0); }
 
 __device__ __forceinline__ void tma_box(uint32_t dst, const void* tmap, int x, int y, uint32_t bar) {
   asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
@@ -1008,7 +971,7 @@ __device__ __forceinline__ void tmem_load16(uint32_t addr, uint32_t (&v)[16]) {
 }
 
 __device__ __forceinline__ void dense_gram(const Problem& p, const Engine& e, const GramPlan& pl, const void* tmap_rows, const void* tmap_cols,
-                                           unsigned char* sm, GramShared& gs, GramCount& gc, int n, int terms, unsigned int* amb_count,
+                                           unsigned char* sm, GramShared& gs, GramCount& gc, int n, unsigned int* amb_count,
                                            uint32_t wait_limit) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int units = pl.tiles * pl.split;
@@ -1018,7 +981,7 @@ __device__ __forceinline__ void dense_gram(const Problem& p, const Engine& e, co
   const unsigned int stages = set ? 3u : 4u;
   const uint32_t ring = (smem_u32(sm) + 1023u) & ~1023u;
   float* tile_sm = reinterpret_cast<float*>(sm + (ring - smem_u32(sm)));   // the finished tile (no split), over the ring
-  const double rho = (double)p.rho, band = engine_band(p.N, terms);
+  const double rho = (double)p.rho, band = engine_band(p.N);
   const float quick = (float)((rho - band) * 0.99999);   // |g| below quick ||a|| ||b||: certainly no conflict
   const int cols4 = pl.cols >> 2, cols_log = set ? 7 : 6;
 
@@ -1034,7 +997,7 @@ __device__ __forceinline__ void dense_gram(const Problem& p, const Engine& e, co
       // ---- operands (one lane) ----
       if (lane == 0) {
         unsigned int slot = slot0, ph = ph0;
-        const int x_step = terms == 1 ? 128 : 64, second = terms == 1 ? 64 : (int)e.lo_off;
+        const int x_step = 64, second = (int)e.lo_off;
         int x = s0 * x_step;
 #pragma unroll 1
         for (int st = 0; st < count; ++st, x += x_step) {
@@ -1073,12 +1036,8 @@ __device__ __forceinline__ void dense_gram(const Problem& p, const Engine& e, co
           for (uint64_t o = 0; o < 8; o += 2) {          // 16 elements of K per instruction
             mma_f16(tmem, a0 + o, b0 + o, idesc, acc);
             acc = 1u;
-            if (terms == 1) {
-              mma_f16(tmem, a1 + o, b1 + o, idesc, 1u);
-            } else {
-              mma_f16(tmem, a0 + o, b1 + o, idesc, 1u);
-              mma_f16(tmem, a1 + o, b0 + o, idesc, 1u);
-            }
+            mma_f16(tmem, a0 + o, b1 + o, idesc, 1u);
+            mma_f16(tmem, a1 + o, b0 + o, idesc, 1u);
           }
           mma_commit(smem_u32(&gs.empty[set][slot]));
           if (++slot == stages) { slot = 0; ph ^= 1u; }
@@ -2022,8 +1981,8 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
     const unsigned int k = real ? (unsigned)e.n_list : (unsigned)n_total;
     bool scanned = !draws, collected = !draws;
     bool spare = kDense && real && !no_filter;           // the last CTA leaves the draw's winners to the others
-    int n = no_filter ? p.n_keep : e.window, packed = 0, terms = p.N <= 2048 ? 3 : 1;
-    bool window = true, products = true;
+    int n = no_filter ? p.n_keep : e.window, packed = 0;
+    bool window = true;
     if (kDense) {
       if (n < n_total && es->skip_window && !no_filter) n = n_total;
     } else {
@@ -2032,13 +1991,11 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
     }
     // ---- steps 1 to 3, once more over all candidates where a window does not do ----
     while (true) {
-      GramPlan pl = e.plan[n == n_total ? 1 : 0];
+      const GramPlan& pl = e.plan[n == n_total ? 1 : 0];
       if (kDense && real) {
-        if (!no_filter) {
-          if (!products) pl = gram_plan(p.N, n, terms, n_ctas);           // (the screen over again with three terms)
+        if (!no_filter)
           for (int i = cta * kT + tid; i < pl.tiles; i += n_ctas * kT) e.tile_ticket[i] = 0u;
-        }
-        dense_pack(p, e, sm, ts, pb, packed, n, t + 1, products, draws, terms == 3, limit);
+        dense_pack(p, e, sm, ts, pb, packed, n, t + 1, draws, limit);
       }
       // a walk on demand leaves the SMs mostly idle, at its barriers above all: the scan is made there
       const bool during_walk = !kDense && real && !window && !scanned;
@@ -2049,15 +2006,9 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
         unsigned int* amb = &es->amb_count[attempts & 1u];
         if (cta == 0 && tid == 0) es->amb_count[(attempts + 1u) & 1u] = 0u;
         ++attempts;
-        dense_gram(p, e, pl, &maps.rows, &maps.cols, sm, gs, gc, n, terms, amb, limit);
+        dense_gram(p, e, pl, &maps.rows, &maps.cols, sm, gs, gc, n, amb, limit);
         if (!(ok = grid_sync(g, p.stall != 0))) break;
         const unsigned int open = *amb;
-        if (open > (unsigned)p.cap_amb && terms == 1) {
-          // more pairs open than the list holds: again with three terms
-          if (cta == 0 && tid == 0) atomicOr(&p.st->status, STRADS_STATUS_GRAM_FALLBACK);
-          terms = 3; packed = 0; products = false;
-          continue;
-        }
         const bool listed = open <= (unsigned)p.cap_amb;
         if (!listed) {
           if (cta == 0 && tid == 0) atomicOr(&p.st->status, STRADS_STATUS_GRAM_FALLBACK);
@@ -2136,8 +2087,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
         window = false;
       } else {
         if (!es->walk_open) break;
-        packed = n; n = n_total; products = true;
-        if (p.N > 2048) terms = 1;
+        packed = n; n = n_total;
       }
     }
     if (!ok) break;
@@ -2288,9 +2238,8 @@ cudaError_t prepare_engine(const Problem& p, Engine& e) {
   if ((err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)a.sharedSizeBytes)) != cudaSuccess) return err;
   e.grid = p.sm_count;
   if (dense) {
-    const int terms = p.N <= 2048 ? 3 : 1;
-    e.plan[0] = gram_plan(p.N, e.window, terms, e.grid);
-    e.plan[1] = gram_plan(p.N, p.n_cand, terms, e.grid);
+    e.plan[0] = gram_plan(p.N, e.window, e.grid);
+    e.plan[1] = gram_plan(p.N, p.n_cand, e.grid);
   }
   return cudaSuccess;
 }

@@ -20,14 +20,13 @@ struct EngineState {
   int avoid;                    // CSC: rounds until they are tried again
 };
 
-// How the pairs of a list are cut into tiles of the dense Gram: kGramRows x cols, K in stages of 128 elements (64 with three
-// terms), `split` CTAs sharing a tile with `per` stages each.
+// How the pairs of a list are cut into tiles of the dense Gram: kGramRows x cols, K in stages of 64 elements, `split` CTAs sharing a tile with `per` stages each.
 constexpr int kGramRows = 128;
 struct GramPlan { int cols, col_blocks, tiles, split, steps, per; };
-__host__ __device__ inline GramPlan gram_plan(long long N, int n, int terms, int n_ctas) {
+__host__ __device__ inline GramPlan gram_plan(long long N, int n, int n_ctas) {
   GramPlan best = {};
   float cost = 0.f;
-  const int k = terms == 1 ? 128 : 64;
+  const int k = 64;
   const int row_blocks = (n + kGramRows - 1) / kGramRows, steps = (int)((N + k - 1) / k);
   for (int cols = 64; cols <= 128; cols += 64) {
     GramPlan pl;
