@@ -276,7 +276,7 @@ Layout carve(const strads_lasso_config_t* c, bool first = true) {
   L.ldcb = (c->n_rows + 7) / 8 * 8;
   L.off_xcb = take(c->layout == STRADS_DENSE_COLMAJOR ? sizeof(unsigned short) * (size_t)c->n_candidates * L.ldcb : 0);
   const bool csc = c->layout == STRADS_CSC;                            // on-demand walk (CSC)
-  L.off_walk_blocked = take(csc ? sizeof(unsigned int) * (size_t)L.mask_words : 0);
+  L.off_walk_blocked = take(csc ? sizeof(unsigned int) * kWalkMasks * (size_t)L.mask_words : 0);
   L.off_walk_ctl = take(csc ? sizeof(WalkControl) : 0);
   L.off_walk_cols = take(csc ? sizeof(WalkColumn) * (size_t)c->n_candidates : 0);
   // CSC Gram by row buckets: provided for while the buckets' candidate lists stay below 64 MB (N <= 2^20; their values take as much)

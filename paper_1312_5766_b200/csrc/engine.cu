@@ -1696,11 +1696,10 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, const Engin
   DemandShared& s = *reinterpret_cast<DemandShared*>(sm);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int cta = (int)blockIdx.x, n_ctas = (int)gridDim.x, n = p.n_cand, W = (n + 31) >> 5;
-  unsigned int* blocked_g = p.walk_blocked;
   const double rho = (double)p.rho;
   __syncthreads();
   for (int w = tid; w < W; w += kT) s.blocked[w] = 0u;
-  if (cta == 0) for (int w = tid; w < W; w += kT) blocked_g[w] = 0u;
+  if (cta == 0) for (int w = tid; w < kWalkMasks * p.mask_words; w += kT) p.walk_blocked[w] = 0u;
   if (tid == 0) { s.cursor = 0; s.kept = 0; s.examined = n; s.done = 0; }
   // this CTA's candidates: cta, cta + n_ctas, ...; own_at: where their entries start in orow / oval
   const int n_own = n > cta ? (n - cta + n_ctas - 1) / n_ctas : 0;
@@ -1738,7 +1737,8 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, const Engin
   }
   if (!grid_sync_busy(g, step)) return false;            // the mask in global memory is clear
 
-  while (true) {
+  for (unsigned int batch = 0u;; ++batch) {
+    unsigned int* blocked_g = p.walk_blocked + walk_mask_at(batch, p.mask_words);      // this batch's conflicts
     // ---- A: the next <= 32 unblocked candidates at or after the cursor ----
     {
       const int cur = s.cursor, first = tid << 5;
@@ -1890,7 +1890,7 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, const Engin
       }
     }
     if (!grid_sync_busy(g, step)) return false;
-    for (int w = tid; w < W; w += kT) s.blocked[w] = __ldcg(blocked_g + w);
+    for (int w = tid; w < W; w += kT) s.blocked[w] |= __ldcg(blocked_g + w);
     __syncthreads();
   }
   if (cta == 0 && tid == 0) {

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include "strads.h"
+#include "walk_mask.cuh"
 
 namespace strads {
 
@@ -121,7 +122,7 @@ struct Problem {
   double* cand_dbeta64;         // [n_cand] proposed change of candidate position a
   float* cand_bnew;             // [n_cand] proposed new beta
   const int* cand_cur;          // candidate list of the Gram in flight (set per launch)
-  unsigned int* walk_blocked;   // CSC on-demand walk: running mask [mask_words], OR-ed into by the whole grid
+  unsigned int* walk_blocked;   // CSC on-demand walk: masks of blocked candidates [kWalkMasks][mask_words] (walk_mask.cuh)
   WalkControl* walk_ctl;
   WalkColumn* walk_cols;        // ... [P'] where each candidate's column lies, gathered when the walk starts
   long long* resid_acc;         // CSC: [N] fixed-point accumulators of the residual update (zero between rounds)

@@ -12,9 +12,9 @@
 //   C  decide the batch (who is kept) from those in-batch conflicts;
 // then the expensive part is shared out over the grid:
 //   D  for every candidate just kept, merge its column against all later unblocked candidates (a warp per
-//      32 of them, a lane per pair) and OR the resulting conflict words into the mask in global memory
-//      (integer OR: any order gives the same mask);
-// one grid-wide barrier, and every CTA reloads the mask.  The barrier is a counter + generation word in
+//      32 of them, a lane per pair) and OR the resulting conflict words into a mask in global memory
+//      (integer OR: any order gives the same mask; two masks in turns, walk_mask.cuh);
+// one grid-wide barrier, and every CTA ORs that mask into its own.  The barrier is a counter + generation word in
 // global memory; every spin has an iteration limit, after which the CTA raises STRADS_STATUS_WAIT_EXPIRED
 // and leaves (the launch is cooperative, so all CTAs are resident and the limit is never met in practice).
 // The kept list equals that of the full-Gram walk: same correlations (same order of the same products),
@@ -99,13 +99,12 @@ __global__ void __launch_bounds__(kThreads) k_walk_csc(Problem p, const int* __r
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned int n_ctas = gridDim.x;
   const unsigned int full = 0xffffffffu;
-  unsigned int* blocked_g = p.walk_blocked;
   const double rho = (double)p.rho;
   const bool rows_aligned = (reinterpret_cast<unsigned long long>(p.xrow) & 15ull) == 0ull;   // (xv always is)
 
   for (int w = tid; w < W; w += kThreads) blocked[w] = 0u;
   if (blockIdx.x == 0)
-    for (int w = tid; w < W; w += kThreads) blocked_g[w] = 0u;
+    for (int w = tid; w < kWalkMasks * p.mask_words; w += kThreads) p.walk_blocked[w] = 0u;
   // where every candidate's column lies, gathered by the whole grid once (the first barrier publishes it): a merge
   // of step D then finds its column in one access instead of three dependent ones
   for (int a = (int)(blockIdx.x * kThreads) + tid; a < n_cand; a += (int)(n_ctas * kThreads)) {
@@ -118,9 +117,10 @@ __global__ void __launch_bounds__(kThreads) k_walk_csc(Problem p, const int* __r
     p.walk_cols[a] = col;
   }
   if (tid == 0) { s_cursor = 0; s_kept = 0; s_examined = n_cand; s_done = 0; }
-  bool ok = grid_barrier(c, n_ctas, &p.st->status, spin_limit);       // nobody ORs into the global mask before it is cleared
+  bool ok = grid_barrier(c, n_ctas, &p.st->status, spin_limit);       // nobody ORs into the global masks before they are cleared
 
-  while (ok) {
+  for (unsigned int batch = 0u; ok; ++batch) {
+    unsigned int* blocked_g = p.walk_blocked + walk_mask_at(batch, p.mask_words);       // this batch's conflicts
     // ---- A: the next <= 32 candidates at or after the cursor that are not blocked: every thread counts the free
     //      positions of two mask words, a scan over the CTA numbers them, and the first 32 are the batch (late batches
     //      find theirs thousands of positions further on: one warp scanning 1,024 positions per trip took 4 us) ----
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(kThreads) k_walk_csc(Problem p, const int* __r
     }
     ok = grid_barrier(c, n_ctas, &p.st->status, spin_limit);
     if (!ok) break;
-    for (int w = tid; w < W; w += kThreads) blocked[w] = __ldcg(&blocked_g[w]);
+    for (int w = tid; w < W; w += kThreads) blocked[w] |= __ldcg(&blocked_g[w]);
     __syncthreads();
   }
 
