@@ -86,6 +86,9 @@ typedef enum { STRADS_DENSE_COLMAJOR = 0, STRADS_CSC = 1 } strads_layout_t;
                                           beta_j' = S(beta_j + 4 x_j^T resid / n_j, 4 lambda / n_j).  The margin is kept
                                           in the workspace (strads_margin); strads_round_host is not available.     */
 
+#define STRADS_FLAG_STALL        256u   /* strads_sample_static only, to exercise its error contract: the call's device-side
+                                          wait runs out after milliseconds                        */
+
 /* limits */
 #define STRADS_MAX_CANDIDATES 16384     /* P' <= 16384 (positions in the candidate list are packed into 16 bits
                                            in the lists of pairs; the walk holds P' / 32 mask words per CTA) */
@@ -288,7 +291,9 @@ int strads_release_cached(void);
  * that device current); make that first call before any stream capture begins.  All calls on one
  * device share the array and it keeps the previous call's contents (the call clears what must start
  * at zero), so two calls that overlap on the GPU -- different streams, or different threads -- race:
- * serialise them. */
+ * serialise them.
+ * Should the call's bounded wait run out, places of cand_dev that it did not come to hold -1 (an index
+ * otherwise), and the next call starts from a clean array. */
 #define STRADS_STATIC_MAX_CANDIDATES 4096
 int strads_sample_static(const float* delta_dev, int64_t n_cols, float eta, uint64_t seed, uint64_t t,
                          int32_t n_candidates, uint32_t flags, int32_t* cand_dev, void* stream);

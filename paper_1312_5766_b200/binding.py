@@ -25,6 +25,7 @@ FLAG_FULL_GRAM = 16
 FLAG_ABS_WEIGHT = 32
 FLAG_DYNAMIC_DEPS = 64
 FLAG_LOGISTIC = 128
+FLAG_STALL = 256                          # sample_static only
 MAX_CANDIDATES = 16384
 STALL_WALK_BARRIER, STALL_GRAM_LOADS = 1, 2
 

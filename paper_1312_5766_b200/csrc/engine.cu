@@ -1735,7 +1735,7 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, const Engin
         for (int q = tid & 3; q < m; q += 4) { s.orow[at + q] = __ldg(p.xrow + from + q); s.oval[at + q] = __ldg(p.xv + from + q); }
     }
   }
-  if (!grid_sync_busy(g, step)) return false;            // the mask in global memory is clear
+  if (!grid_sync_busy(g, step)) return false;            // the masks in global memory are clear
 
   for (unsigned int batch = 0u;; ++batch) {
     unsigned int* blocked_g = p.walk_blocked + walk_mask_at(batch, p.mask_words);      // this batch's conflicts
@@ -2132,18 +2132,23 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
 // The draw alone (strads_sample_static), all of it in one launch: keys computed once and kept in shared memory, histogram,
 // selection, collection and ranking with two grid barriers between them.  Bound by the launch and the barriers: 22.6 us
 // as six launches (clear, round index, two passes, ordering), each waiting for the one before, at J = 100,000, P' = 2,048;
-// one launch and a clear before it still took 16.4, so the kernel leaves its scratch clear instead (`spare`: another call's
-// barrier, cleared for it in case that call was cut short).
+// one launch and a clear before it still took 16.4, so the kernel leaves its scratch clear instead.
+// A call whose wait runs out leaves -1 in the places of the list that it did not come to, and says so to the next one
+// (EngineState::dirty), which then clears the histogram behind a barrier of its own: every CTA leaves through the same few
+// lines, and the one that leaves last sets the barrier back and knows from their count whether any of them gave up.
 // A grid of no more CTAs than have keys or winners to go through: the barriers cost less among few.
 // ------------------------------------------------------------------------------------------------
 constexpr size_t kDrawKeys = 144 * 1024;   // keys a CTA keeps in shared memory (more: computed again to collect the winners)
 
-__global__ void __launch_bounds__(kT, 1) k_draw(const __grid_constant__ Problem p, const __grid_constant__ Engine e, unsigned long long t, int kept_groups,
-                                                EngineState* spare) {
-  extern __shared__ __align__(1024) unsigned char sm[];
-  __shared__ DrawShared ds;
-  __shared__ Problem sp;
-  __shared__ Engine se;
+// (cold; out of line, as the kernel runs from a cold instruction cache)  False: a wait gave up.
+__device__ __noinline__ bool clear_histogram(const Engine& e, Grid& g) {
+  for (int b = (int)blockIdx.x * kT + (int)threadIdx.x; b < kHistBins; b += (int)gridDim.x * kT) e.hist[b] = 0u;
+  return grid_sync(g);
+}
+
+// False: a wait gave up.
+__device__ __forceinline__ bool draw_alone(const Problem& p, const Engine& e, DrawShared& ds, Problem& sp, Engine& se, unsigned char* sm, unsigned long long t,
+                                           int kept_groups, int stall) {
   unsigned int* sh = reinterpret_cast<unsigned int*>(sm);
   unsigned long long* held = reinterpret_cast<unsigned long long*>(sm + kScanSmem);      // [kept_groups][4][kT]
   const int tid = threadIdx.x;
@@ -2151,11 +2156,16 @@ __global__ void __launch_bounds__(kT, 1) k_draw(const __grid_constant__ Problem 
   const WeightForm wf = weight_form(p);
   const Binning bins = binning_of(0.f);
   for (int b = tid; b < kHistBins; b += kT) sh[b] = 0u;
-  for (int b = (int)blockIdx.x * kT + tid; b < kHistBins; b += (int)gridDim.x * kT) e.bin_cur[b] = 0u;
+  static_assert(STRADS_STATIC_MAX_CANDIDATES <= kHistBins, "a place of the list per bin");
+  for (int b = (int)blockIdx.x * kT + tid; b < kHistBins; b += (int)gridDim.x * kT) {
+    e.bin_cur[b] = 0u;
+    if (b < p.n_cand) p.cand[b] = -1;
+  }
+  const int dirty = e.es->dirty;
   if (tid == 0) { sp = p; se = e; ds.cut = 0.f; }
   __syncthreads();
   Grid g;
-  g.count = &e.es->bar_count; g.target = 0u; g.n = gridDim.x; g.limit = kSpinLimit; g.status = &p.st->status;
+  g.count = &e.es->bar_count; g.target = 0u; g.n = gridDim.x; g.limit = p.wait_limit ? p.wait_limit : kSpinLimit; g.status = &p.st->status;
   int turn = 0;
   for (long long gi = (long long)blockIdx.x * kT + tid; gi < groups; gi += (long long)gridDim.x * kT, ++turn) {
     float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -2179,11 +2189,12 @@ __global__ void __launch_bounds__(kT, 1) k_draw(const __grid_constant__ Problem 
     }
   }
   __syncthreads();
+  if (dirty && !clear_histogram(se, g)) return false;    // (the same in every CTA: it changes when the last one leaves)
   for (int b = tid; b < kHistBins; b += kT)
     if (sh[b]) atomicAdd(&e.hist[b], sh[b]);
-  if (!grid_sync(g)) return;
+  if (!grid_sync(g, stall != 0 && blockIdx.x == 0)) return false;
   draw_select(e, ds, (unsigned)p.n_cand);
-  if (ds.bnd_count > (unsigned)e.cap_boundary && !draw_refine(sp, se, ds, sm, t, (unsigned)p.n_cand, g)) return;
+  if (ds.bnd_count > (unsigned)e.cap_boundary && !draw_refine(sp, se, ds, sm, t, (unsigned)p.n_cand, g)) return false;
   if (kept_groups > 0) {
     for (int k = 0; k < turn; ++k)
 #pragma unroll
@@ -2194,10 +2205,25 @@ __global__ void __launch_bounds__(kT, 1) k_draw(const __grid_constant__ Problem 
   } else {
     draw_collect_all(sp, se, ds, sm, t);
   }
-  if (!grid_sync(g)) return;
+  if (!grid_sync(g)) return false;
   draw_rank<true>(p, e, ds, nullptr, nullptr, 0, 0, nullptr, (int)gridDim.x, 0);       // (leaves the histogram clear)
-  if (tid == 0 && atomicInc(&e.es->exit_count, gridDim.x - 1u) == gridDim.x - 1u) e.es->bar_count = 0u;
-  if (blockIdx.x == 0 && tid == 0) { spare->bar_count = 0u; spare->exit_count = 0u; }
+  return true;
+}
+
+__global__ void __launch_bounds__(kT, 1) k_draw(const __grid_constant__ Problem p, const __grid_constant__ Engine e, unsigned long long t, int kept_groups,
+                                                int stall) {
+  extern __shared__ __align__(1024) unsigned char sm[];
+  __shared__ DrawShared ds;
+  __shared__ Problem sp;
+  __shared__ Engine se;
+  const bool ok = draw_alone(p, e, ds, sp, se, sm, t, kept_groups, stall);
+  if (threadIdx.x != 0) return;
+  constexpr unsigned int kGaveUp = 1u << 16;             // (fewer CTAs than that)
+  const unsigned int left = atomicAdd(&e.es->exit_count, ok ? 1u : 1u + kGaveUp);
+  if ((left & (kGaveUp - 1u)) != gridDim.x - 1u) return;
+  e.es->exit_count = 0u;
+  e.es->bar_count = 0u;
+  e.es->dirty = !ok || left >= kGaveUp ? 1 : 0;
 }
 
 size_t smem_of(bool dense, int n_keep, bool ahead, int n_cand) {
@@ -2246,7 +2272,7 @@ cudaError_t prepare_engine(const Problem& p, Engine& e) {
 
 cudaError_t prepare_draw() { return cudaFuncSetAttribute(k_draw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kScanSmem + kDrawKeys)); }
 
-cudaError_t launch_draw(const Problem& p, const Engine& e, unsigned long long t, EngineState* spare, cudaStream_t s) {
+cudaError_t launch_draw(const Problem& p, const Engine& e, unsigned long long t, cudaStream_t s) {
   const long long groups = (p.J + 3) / 4;
   const long long need = (groups + kT - 1) / kT, rank = ((long long)e.cap_win * 8 + kT - 1) / kT;
   long long grid = need > rank ? need : rank;
@@ -2260,7 +2286,7 @@ cudaError_t launch_draw(const Problem& p, const Engine& e, unsigned long long t,
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(kT); cfg.dynamicSmemBytes = smem; cfg.stream = s;
   cfg.attrs = attr; cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_draw, p, e, t, held ? (int)turns : 0, spare);
+  return cudaLaunchKernelEx(&cfg, k_draw, p, e, t, held ? (int)turns : 0, p.stall);
 }
 
 cudaError_t encode_engine_maps(const Problem& p, const Engine& e, void* out) {

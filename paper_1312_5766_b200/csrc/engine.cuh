@@ -18,6 +18,7 @@ struct EngineState {
   int mend;                     // a draw's selection has to be mended
   int streak;                   // CSC: attempts with the row buckets in a row that overflowed (or left the walk open)
   int avoid;                    // CSC: rounds until they are tried again
+  int dirty;                    // strads_sample_static: the last call gave up and left the histogram as it was
 };
 
 // How the pairs of a list are cut into tiles of the dense Gram: kGramRows x cols, K in stages of 64 elements, `split` CTAs sharing a tile with `per` stages each.
@@ -83,9 +84,9 @@ cudaError_t encode_engine_maps(const Problem& p, const Engine& e, void* out_256_
 cudaError_t launch_engine(const Problem& p, const Engine& e, const void* maps, int n_rounds, bool have_list, bool draw_next,
                           const strads_round_out_t* out, cudaStream_t s);
 
-// The draw alone: p.cand[0 .. p.n_cand) for round t from p.delta (e: es, hist, bin_cur and win).  The barrier in es and hist
-// are zero before and after.
+// The draw alone: p.cand[0 .. p.n_cand) for round t from p.delta (e: es, hist, bin_cur and win).  The barrier in es is zero before
+// and after, and hist unless es->dirty says otherwise.
 cudaError_t prepare_draw();
-cudaError_t launch_draw(const Problem& p, const Engine& e, unsigned long long t, EngineState* spare, cudaStream_t s);
+cudaError_t launch_draw(const Problem& p, const Engine& e, unsigned long long t, cudaStream_t s);
 
 }  // namespace strads

@@ -554,11 +554,10 @@ cudaError_t launch_sample(const Problem& p, int* cand_out, cudaStream_t s) {
 namespace strads {
 namespace {
 
-constexpr int kStaticTurns = 32;           // barriers that calls take in turn
 constexpr int kStaticBoundary = STRADS_STATIC_MAX_CANDIDATES / 2;
 struct StaticSampleScratch {
   DeviceState st;
-  EngineState es[kStaticTurns];
+  EngineState es;
   __align__(16) unsigned int hist[kHistBins];
   unsigned int bin_cur[kHistBins];
   unsigned long long win[STRADS_STATIC_MAX_CANDIDATES + kStaticBoundary];
@@ -570,7 +569,6 @@ constexpr int kMaxDevices = 64;
 std::mutex g_static_mutex;
 StaticSampleScratch* g_static_ptr[kMaxDevices] = {};   // device address of the array, per device
 int g_static_sms[kMaxDevices] = {};
-unsigned int g_static_calls[kMaxDevices] = {};
 
 }  // namespace
 }  // namespace strads
@@ -588,7 +586,6 @@ extern "C" int strads_sample_static(const float* delta_dev, int64_t n_cols, floa
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return STRADS_ERR_CUDA;
   StaticSampleScratch* sc = nullptr;
   int sms = 0;
-  unsigned int call = 0;
   {
     // once per device, with that device current: in host code the array's name is only a stand-in,
     // the address a kernel can use comes from cudaGetSymbolAddress
@@ -603,11 +600,10 @@ extern "C" int strads_sample_static(const float* delta_dev, int64_t n_cols, floa
     }
     sc = g_static_ptr[dev];
     sms = g_static_sms[dev];
-    call = g_static_calls[dev]++;
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // The array starts as zeros and a call leaves it so (the histogram, its own barrier; cursors are cleared when they are
-  // wanted).  Should a call be cut short, the next one clears the histogram again and a later one that call's barrier.
+  // The array starts as zeros and a call leaves it so (the histogram, the barrier; cursors are cleared when they are wanted).
+  // A call whose wait ran out leaves a note, by which the next one clears the histogram before it uses it.
   Problem p = {};
   p.layout = STRADS_DENSE_COLMAJOR;
   p.J = n_cols;
@@ -620,11 +616,12 @@ extern "C" int strads_sample_static(const float* delta_dev, int64_t n_cols, floa
   p.cand = cand_dev;
   p.sm_count = sms;
   Engine e = {};
-  e.es = &sc->es[call % kStaticTurns];
+  e.es = &sc->es;
   e.hist = sc->hist;
   e.bin_cur = sc->bin_cur;
   e.win = sc->win;
   e.cap_win = n_candidates + kStaticBoundary;
   e.cap_boundary = kStaticBoundary;
-  return launch_draw(p, e, t, &sc->es[(call + kStaticTurns / 2) % kStaticTurns], s) == cudaSuccess ? STRADS_OK : STRADS_ERR_CUDA;
+  if (flags & STRADS_FLAG_STALL) { p.stall = 1; p.wait_limit = 4096; }
+  return launch_draw(p, e, t, s) == cudaSuccess ? STRADS_OK : STRADS_ERR_CUDA;
 }

@@ -99,3 +99,30 @@ def test_dense_gram_pipeline_gives_up_and_the_handle_recovers():
     for x, y in ((s.beta, ref.beta), (s.resid, ref.resid), (s.delta, ref.delta)):
         assert torch.equal(x, y)
     assert s.status()[0] == 0 and s.get_round() == 20
+
+
+def test_static_draw_gives_up_and_the_next_call_is_whole_again():
+    """Also several such calls in a row, and a captured call replayed after one (its arguments are fixed at capture)."""
+    import oracle
+    b = _binding()
+    J, n_cand, eta = 60_003, 700, 1e-6
+    g = torch.Generator(device="cuda").manual_seed(4)
+    delta = torch.rand(J, generator=g, device="cuda") * 1e-2
+    want = torch.from_numpy(oracle.sample(delta.cpu().numpy().astype(np.float64), float(np.float32(eta)), 5, 2, n_cand).astype(np.int32)).cuda()
+    out = torch.empty(n_cand, dtype=torch.int32, device="cuda")
+    assert torch.equal(b.sample_static(delta, eta, 5, 2, n_cand, out=out), want)
+    graph, out_g = torch.cuda.CUDAGraph(), torch.empty(n_cand, dtype=torch.int32, device="cuda")
+    stream = torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=stream):
+        b.sample_static(delta, eta, 5, 2, n_cand, out=out_g)
+    for stalls in (1, 3):
+        for after in ("call", "replay"):
+            for _ in range(stalls):
+                got = b.sample_static(delta, eta, 5, 2, n_cand, flags=b.FLAG_STALL, out=out)
+                assert bool((got < 0).any())                # nothing that could be taken for a list
+            if after == "replay":
+                graph.replay()
+                assert torch.equal(out_g, want)
+                out_g.zero_()
+            assert torch.equal(b.sample_static(delta, eta, 5, 2, n_cand, out=out), want)
+            assert torch.equal(b.sample_static(delta, eta, 5, 2, n_cand, out=out), want)
