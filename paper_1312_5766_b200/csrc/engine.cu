@@ -1669,6 +1669,7 @@ struct DemandShared {
   int wsum[kWarps];
   unsigned int keep;
   int m, cursor, kept, examined, done;
+  int batch, mask_at;                                    // batches decided; where the conflicts of the last one go in walk_blocked
   int own_at[kOwn + 1], own_free[kOwn], n_free;
   double own_n2[kOwn];
   long long own_q0[kOwn];
@@ -1700,7 +1701,7 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, const Engin
   __syncthreads();
   for (int w = tid; w < W; w += kT) s.blocked[w] = 0u;
   if (cta == 0) for (int w = tid; w < kWalkMasks * p.mask_words; w += kT) p.walk_blocked[w] = 0u;
-  if (tid == 0) { s.cursor = 0; s.kept = 0; s.examined = n; s.done = 0; }
+  if (tid == 0) { s.cursor = 0; s.kept = 0; s.examined = n; s.done = 0; s.batch = 0; }
   // this CTA's candidates: cta, cta + n_ctas, ...; own_at: where their entries start in orow / oval
   const int n_own = n > cta ? (n - cta + n_ctas - 1) / n_ctas : 0;
   const int n_here = min(n_own, kOwn);
@@ -1737,8 +1738,7 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, const Engin
   }
   if (!grid_sync_busy(g, step)) return false;            // the masks in global memory are clear
 
-  for (unsigned int batch = 0u;; ++batch) {
-    unsigned int* blocked_g = p.walk_blocked + walk_mask_at(batch, p.mask_words);      // this batch's conflicts
+  while (true) {
     // ---- A: the next <= 32 unblocked candidates at or after the cursor ----
     {
       const int cur = s.cursor, first = tid << 5;
@@ -1823,6 +1823,8 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, const Engin
         s.keep = keep;
         s.kept = nk + __popc(keep);
         s.cursor = s.pos[m - 1] + 1;
+        s.mask_at = walk_mask_at((unsigned)s.batch, p.mask_words);
+        s.batch += 1;
         s.n_free = 0;
         if (done) { s.examined = s.pos[31 - __clz((int)keep)] + 1; s.done = 1; }
       }
@@ -1884,13 +1886,13 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, const Engin
               dot = merge_dot(ar, av, na, p.xrow + cb.q0, p.xv + cb.q0, cb.n);
             }
             const double den = sqrt(s.n2[q] * n2b);
-            if (den > 0.0 && fabs((double)dot) >= rho * den) { atomicOr(&blocked_g[b >> 5], 1u << (b & 31)); break; }
+            if (den > 0.0 && fabs((double)dot) >= rho * den) { atomicOr(p.walk_blocked + s.mask_at + (b >> 5), 1u << (b & 31)); break; }
           }
         }
       }
     }
     if (!grid_sync_busy(g, step)) return false;
-    for (int w = tid; w < W; w += kT) s.blocked[w] |= __ldcg(blocked_g + w);
+    for (int w = tid; w < W; w += kT) s.blocked[w] |= __ldcg(p.walk_blocked + s.mask_at + w);
     __syncthreads();
   }
   if (cta == 0 && tid == 0) {

@@ -94,6 +94,7 @@ __global__ void __launch_bounds__(kThreads) k_walk_csc(Problem p, const int* __r
   __shared__ unsigned int s_conf[kBatch];
   __shared__ unsigned int s_keep;
   __shared__ int s_m, s_cursor, s_kept, s_examined, s_done;
+  __shared__ int s_batch, s_mask_at;                     // batches decided; where the conflicts of the last one go in walk_blocked
   WalkControl* c = p.walk_ctl;
   const int W = (n_cand + 31) >> 5;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -116,11 +117,10 @@ __global__ void __launch_bounds__(kThreads) k_walk_csc(Problem p, const int* __r
     col.unused = 0.0;
     p.walk_cols[a] = col;
   }
-  if (tid == 0) { s_cursor = 0; s_kept = 0; s_examined = n_cand; s_done = 0; }
+  if (tid == 0) { s_cursor = 0; s_kept = 0; s_examined = n_cand; s_done = 0; s_batch = 0; }
   bool ok = grid_barrier(c, n_ctas, &p.st->status, spin_limit);       // nobody ORs into the global masks before they are cleared
 
-  for (unsigned int batch = 0u; ok; ++batch) {
-    unsigned int* blocked_g = p.walk_blocked + walk_mask_at(batch, p.mask_words);       // this batch's conflicts
+  while (ok) {
     // ---- A: the next <= 32 candidates at or after the cursor that are not blocked: every thread counts the free
     //      positions of two mask words, a scan over the CTA numbers them, and the first 32 are the batch (late batches
     //      find theirs thousands of positions further on: one warp scanning 1,024 positions per trip took 4 us) ----
@@ -253,6 +253,8 @@ __global__ void __launch_bounds__(kThreads) k_walk_csc(Problem p, const int* __r
       if (lane == 0) {
         s_keep = keep;
         s_kept = nk + __popc(keep);
+        s_mask_at = walk_mask_at((unsigned)s_batch, p.mask_words);
+        s_batch += 1;
         if (done) { s_examined = s_pos[31 - __clz(keep)] + 1; s_done = 1; }
         else s_cursor = s_pos[m - 1] + 1;
       }
@@ -323,12 +325,12 @@ __global__ void __launch_bounds__(kThreads) k_walk_csc(Problem p, const int* __r
         else if (need <= 28) dot = sparse_dot_fetched4<7>(ar, av, na, p, q0, nb);
         else if (need <= 36) dot = sparse_dot_fetched4<9>(ar, av, na, p, q0, nb);
         else dot = sparse_dot_arrays(ar, av, na, p.xrow + q0, p.xv + q0, nb);
-        if (den > 0.0 && fabs((double)dot) >= rho * den) atomicOr(&blocked_g[b >> 5], 1u << (b & 31));
+        if (den > 0.0 && fabs((double)dot) >= rho * den) atomicOr(p.walk_blocked + s_mask_at + (b >> 5), 1u << (b & 31));
       }
     }
     ok = grid_barrier(c, n_ctas, &p.st->status, spin_limit);
     if (!ok) break;
-    for (int w = tid; w < W; w += kThreads) blocked[w] |= __ldcg(&blocked_g[w]);
+    for (int w = tid; w < W; w += kThreads) blocked[w] |= __ldcg(p.walk_blocked + s_mask_at + w);
     __syncthreads();
   }
 
