@@ -1169,7 +1169,7 @@ __device__ __forceinline__ void dense_gram(const Problem& p, const Engine& e, co
 }
 
 // Exact decision of one pair by a warp.
-__device__ __forceinline__ void decide_exactly(const Problem& p, const Engine& e, int a, int b, bool clear) {
+__device__ __forceinline__ void decide_exactly(const Problem& p, const Engine& e, int a, int b) {
   const int lane = threadIdx.x & 31;
   const float* xa = p.xv + (long long)p.cand[a] * p.ld;
   const float* xb = p.xv + (long long)p.cand[b] * p.ld;
@@ -1184,9 +1184,7 @@ __device__ __forceinline__ void decide_exactly(const Problem& p, const Engine& e
   acc = warp_sum(acc);
   if (lane == 0) {
     const double den = e.norm[a] * e.norm[b];
-    unsigned int* word = &p.conflict[(long long)a * p.mask_words + (b >> 5)];
-    if (den > 0.0 && fabs(acc) >= (double)p.rho * den) atomicOr(word, 1u << (b & 31));
-    else if (clear) atomicAnd(word, ~(1u << (b & 31)));
+    if (den > 0.0 && fabs(acc) >= (double)p.rho * den) atomicOr(&p.conflict[(long long)a * p.mask_words + (b >> 5)], 1u << (b & 31));
   }
 }
 
@@ -1368,12 +1366,77 @@ __device__ void dense_apply(const Problem& p, const Moving& mv, double* part, in
 
 constexpr unsigned int kFewOpen = 48;                    // open pairs the walking CTA decides itself
 
-// (cold) data whose products cluster at rho: every pair exactly
+// (cold) Data whose products cluster at rho leave more pairs open than the list holds: all pairs of the first n candidates
+// exactly, tiles of 32 x 128 of the upper triangle.  32 rows of the tile's columns at a time lie in shared memory as
+// binary64, and a thread adds up 2 x 4 products: bound by reading the operands there (a warp's step takes 9 cycles of shared
+// memory and 4 of the FP64 pipe).  A warp per pair, both columns read again for every pair and the lower triangle stepped
+// through as well, took 9.7 ms per round at 4,096 candidates of 900 rows, this takes 2.2 (the launch chain's 3xTF32 pass, list
+// included, 4.2 to 4.8).  4 x 4 products take 1.5, but need registers that the rest of the kernel then spills: rounds
+// that never come here 2 % slower.
+constexpr int kExactRows = 32, kExactCols = 128, kExactK = 32;
+struct ExactTile { double a[kExactK][kExactRows], b[kExactK][kExactCols], norm[kExactRows + kExactCols]; const float* col[kExactRows + kExactCols]; };
+
 __device__ __noinline__ void decide_all(const Problem& p, const Engine& e, int n) {
-  const int warp = (int)threadIdx.x >> 5;
-  for (long long i = (long long)warp * gridDim.x + blockIdx.x; i < (long long)n * n; i += (long long)kWarps * gridDim.x) {
-    const int a = (int)(i / n), b = (int)(i - (long long)a * n);
-    if (b > a) decide_exactly(p, e, a, b, true);
+  extern __shared__ __align__(1024) unsigned char sm[];
+  ExactTile& s = *reinterpret_cast<ExactTile*>(sm);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  static_assert(kWarps * 2 == kExactRows && 32 * 4 == kExactCols, "2 x 4 products a thread");
+  constexpr int kBoth = kExactRows + kExactCols, kStaged = (kBoth * (kExactK / 4) + kT - 1) / kT;         // columns; groups of four rows a thread brings in
+  const int n4 = (int)((p.N + 3) >> 2), row_tiles = (n + kExactRows - 1) / kExactRows, col_tiles = (n + kExactCols - 1) / kExactCols;
+  unsigned int tile = 0u;
+  for (int r = 0; r < row_tiles; ++r) {
+    for (int c = r * kExactRows / kExactCols; c < col_tiles; ++c) {
+      if (tile++ % gridDim.x != blockIdx.x) continue;
+      const int row0 = r * kExactRows, col0 = c * kExactCols;
+      __syncthreads();                                   // (the tile before)
+      if (tid < kBoth) {
+        const int i = tid < kExactRows ? row0 + tid : col0 + tid - kExactRows;
+        s.norm[tid] = i < n ? e.norm[i] : 0.0;
+        s.col[tid] = i < n ? p.xv + (long long)p.cand[i] * p.ld : nullptr;
+      }
+      __syncthreads();
+      double acc[2][4] = {};
+      for (int g0 = 0; g0 < n4; g0 += kExactK / 4) {
+        float4 v[kStaged];
+#pragma unroll
+        for (int u = 0; u < kStaged; ++u) {
+          const int g = g0 + (tid + u * kT) / kBoth;
+          const float4* src = reinterpret_cast<const float4*>(s.col[(tid + u * kT) % kBoth]);
+          v[u] = src != nullptr && g < n4 && g < g0 + kExactK / 4 ? __ldg(src + g) : make_float4(0.f, 0.f, 0.f, 0.f);
+          if (4ll * g + 3 >= p.N && g < n4) mask_rows(p, g, v[u]);
+        }
+        __syncthreads();                                 // (the rows before)
+#pragma unroll
+        for (int u = 0; u < kStaged; ++u) {
+          const int i = (tid + u * kT) % kBoth, k = (tid + u * kT) / kBoth * 4;
+          if (k >= kExactK) continue;
+          double* dst = i < kExactRows ? &s.a[k][i] : &s.b[k][i - kExactRows];
+          const int pitch = i < kExactRows ? kExactRows : kExactCols;
+          dst[0] = v[u].x; dst[pitch] = v[u].y; dst[2 * pitch] = v[u].z; dst[3 * pitch] = v[u].w;
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int k = 0; k < kExactK; ++k) {
+          const double2 a = *reinterpret_cast<const double2*>(&s.a[k][warp * 2]);
+#pragma unroll
+          for (int y = 0; y < 4; ++y) {
+            const double b = s.b[k][lane + 32 * y];
+#pragma unroll
+            for (int x = 0; x < 2; ++x) acc[x][y] = fma(x ? a.y : a.x, b, acc[x][y]);
+          }
+        }
+      }
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const int a = row0 + warp * 2 + x;
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+          const double den = s.norm[warp * 2 + x] * s.norm[kExactRows + lane + 32 * y];
+          const unsigned int word = __ballot_sync(kFull, col0 + lane + 32 * y > a && den > 0.0 && fabs(acc[x][y]) >= (double)p.rho * den);
+          if (lane == 0 && a < n && (col0 >> 5) + y < p.mask_words) p.conflict[(size_t)a * p.mask_words + (col0 >> 5) + y] = word;
+        }
+      }
+    }
   }
 }
 
@@ -2020,7 +2083,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
           const unsigned int first = open > kFewOpen ? (unsigned)(warp * n_ctas + cta) : (unsigned)warp;
           for (unsigned int i = first; i < open; i += open > kFewOpen ? (unsigned)(kWarps * n_ctas) : (unsigned)kWarps) {
             const unsigned int pr = __ldcg(p.amb_pairs + i);
-            decide_exactly(p, e, (int)(pr >> 16), (int)(pr & 0xffffu), false);
+            decide_exactly(p, e, (int)(pr >> 16), (int)(pr & 0xffffu));
           }
           __threadfence();
         }

@@ -77,6 +77,26 @@ def test_products_that_cluster_at_rho():
     assert s.status() == (0, 8)                             # informational: pairs decided one by one
 
 
+# one tile of all pairs and more; rows that end inside a group of four and of 32, with columns padded by NaN
+@pytest.mark.parametrize("N,J,product", [(70, 1900, 4), (33, 1601, 3), (97, 2177, 5)])
+def test_all_pairs_exactly(N, J, product):
+    """Columns of +-1 over a few rows: more pairs correlate at exactly rho than any list of open pairs holds."""
+    from paper_1312_5766_b200 import binding as b
+    P = 60
+    g = torch.Generator().manual_seed(2)
+    x = torch.full((J, (N + 3) // 4 * 4), float("nan"))
+    x[:, :N] = (torch.randint(0, 2, (J, N), generator=g) * 2 - 1).float()
+    y = torch.randn(N, generator=g)
+    X = oracle.Matrix.dense(x.numpy(), n_rows=N)
+    n2 = oracle.colnorm2(X)
+    rho = float(np.float32(product / N))                    # products are whole numbers of N's parity
+    s = b.StradsLasso(wl.DENSE, N, J, x.cuda(), y.cuda(), 0.1, 1e-6, rho, J, P, seed=1)
+    for _ in range(3):
+        cand, kept, _, counts = (v.cpu().numpy() for v in s.round())
+        _assert_kept_matches(X, n2, cand, P, rho, kept[: int(counts[2])], int(counts[1]))
+    assert s.status() == (0, 8)                             # informational: pairs decided one by one
+
+
 def test_tied_keys():
     """Infinite priorities: thousands of race times of exactly 0, far more than the draw's boundary holds."""
     from paper_1312_5766_b200 import binding as b
