@@ -133,7 +133,8 @@ typedef struct {
                          SIMT Gram kernel, which is the one that can export its values)      */
 } strads_round_out_t;
 
-/* Bytes of device workspace that `cfg` needs (pointer fields of cfg are not read). */
+/* Bytes of device workspace that `cfg` needs (pointer fields of cfg are not read).  Whether whole rounds go in one
+ * launch depends on rho, and with it the size; with rho left at 0 the answer covers any. */
 int strads_workspace_bytes(const strads_lasso_config_t* cfg, size_t* out_bytes);
 
 /* Algorithm 1's initialisation: n_j = ||x_j||^2 for all j, resid = y - X beta, delta_j = C,

@@ -217,8 +217,8 @@ int check_sizes(const strads_lasso_config_t* c) {
   return STRADS_OK;
 }
 
-// Whether the workspace provides for the engine: CSC always; dense X with short columns and the default Gram.
-bool engine_wanted(const strads_lasso_config_t* c) {
+// Whether the engine can take the rounds of one scheduler: CSC always; dense X with short columns and the default Gram.
+bool engine_possible(const strads_lasso_config_t* c) {
   if (c->flags & (STRADS_FLAG_SIMT_GRAM | STRADS_FLAG_GRAM_3XTF32)) return false;
   return c->layout == STRADS_CSC || c->n_rows <= kEngineDenseRows;
 }
@@ -228,16 +228,19 @@ bool engine_wanted(const strads_lasso_config_t* c) {
 // launches, 65 here); with longer columns the captured chain of kernels, each with a whole GPU's worth of loads under way,
 // is the faster one (c1 36.3 us against 39.0, c2 42 against 60).
 bool engine_chosen(const strads_lasso_config_t* c) {
-  if (!engine_wanted(c) || n_sched_of(c) > 1) return false;
+  if (!engine_possible(c) || n_sched_of(c) > 1) return false;
   return c->layout == STRADS_CSC || (double)c->n_rows * (double)c->rho * (double)c->rho <= 9.0;
 }
+// Whether the workspace provides for it (1,000 x 10,000, P' = 200: 13.6 of 15.3 MB): where it is chosen.  A query of the size need not have
+// set rho; it is then answered for any.
+bool engine_provided(const strads_lasso_config_t* c) { return c->rho > 0.f ? engine_chosen(c) : engine_possible(c); }
 // Keys each CTA can save of a scan that finds a few times `winners` of them in all.
 unsigned int engine_saved(size_t winners) { return (unsigned int)(winners / 16 + 64); }
 size_t engine_boundary(size_t winners) { return winners / 2 > 2048 ? winners / 2 : 2048; }
 
 // Slice of the workspace of one scheduler; the first one (`first`) also holds what all share
-// (column norms, the objective's partial sums).
-Layout carve(const strads_lasso_config_t* c, bool first = true) {
+// (column norms, the objective's partial sums) and, with `engine`, the round engine's buffers.
+Layout carve(const strads_lasso_config_t* c, bool first, bool engine) {
   Layout L;
   L.cap_sure = c->n_candidates;
   L.cap_boundary = pow2_ceil(c->n_candidates / 2 > 2048 ? c->n_candidates / 2 : 2048);
@@ -262,7 +265,7 @@ Layout carve(const strads_lasso_config_t* c, bool first = true) {
   L.off_dbeta64 = take(sizeof(double) * (size_t)c->n_keep);
   L.off_conflict = take(sizeof(unsigned int) * (size_t)c->n_candidates * L.mask_words);
   const bool dense = c->layout == STRADS_DENSE_COLMAJOR;
-  L.engine = engine_wanted(c);
+  L.engine = first && engine;
   const bool proposals = dense || L.engine;
   L.off_cand_dbeta64 = take(proposals ? sizeof(double) * (size_t)c->n_candidates : 0);
   L.off_cand_bnew = take(proposals ? sizeof(float) * (size_t)c->n_candidates : 0);
@@ -313,7 +316,6 @@ Layout carve(const strads_lasso_config_t* c, bool first = true) {
   L.off_ahead_bin_off = take(ahead ? sizeof(int) * (kHistBins + 1) : 0);
   L.off_ahead_bin_cur = take(ahead ? sizeof(unsigned int) * kHistBins : 0);
   // the round engine: a draw of P' + P winners one round ahead (P' at the round's start when P is too large for that)
-  if (!first) L.engine = false;
   const bool en = L.engine;
   L.eng_list = en && c->n_keep <= kAheadMaxKeep ? (int)n_ahead : 0;
   const size_t most = (size_t)(L.eng_list > c->n_candidates ? L.eng_list : c->n_candidates);
@@ -686,7 +688,7 @@ int strads_workspace_bytes(const strads_lasso_config_t* cfg, size_t* out_bytes) 
   if (out_bytes == nullptr) return STRADS_ERR_INVALID_ARG;
   const int rc = check_sizes(cfg);
   if (rc) return rc;
-  *out_bytes = carve(cfg).total + (size_t)(n_sched_of(cfg) - 1) * carve(cfg, false).total;
+  *out_bytes = carve(cfg, true, engine_provided(cfg)).total + (size_t)(n_sched_of(cfg) - 1) * carve(cfg, false, false).total;
   return STRADS_OK;
 }
 
@@ -706,8 +708,12 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
   // first phase turns from a randomised sweep into one in index order
   if (c->c_init > STRADS_MAX_C_INIT) return STRADS_ERR_INVALID_ARG;
   const int S = n_sched_of(c);
-  const Layout L = carve(c), Lrest = carve(c, false);
-  if (c->workspace_bytes < L.total + (size_t)(S - 1) * Lrest.total) return STRADS_ERR_WORKSPACE_TOO_SMALL;
+  const Layout Lrest = carve(c, false, false);
+  const size_t rest = (size_t)(S - 1) * Lrest.total;
+  Layout L = carve(c, true, engine_provided(c));
+  // (a workspace sized for a larger rho, with which the engine would not be chosen, still does: without the engine)
+  if (L.engine && c->workspace_bytes < L.total + rest) L = carve(c, true, false);
+  if (c->workspace_bytes < L.total + rest) return STRADS_ERR_WORKSPACE_TOO_SMALL;
 
   strads_lasso_s* h = new (std::nothrow) strads_lasso_s();     // value-initialised: every pointer null
   if (h == nullptr) return STRADS_ERR_INVALID_ARG;
@@ -744,7 +750,7 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
     return fail(cuda_fail(e, "copy stream"));
   h->copy_stream = kit.copy; h->copy_fork = kit.copy_fork; h->copy_done = kit.copy_done;
   h->ahead_round = -1;
-  h->engine_ok = L.engine && engine_chosen(c) && sm_count <= kEngineMaxCtas;
+  h->engine_ok = L.engine && sm_count <= kEngineMaxCtas;
   if (h->engine_ok) {
     fill_engine(h->engine, p0, L, ws);
     if ((e = prepare_engine(p0, h->engine)) != cudaSuccess) return fail(cuda_fail(e, "prepare_engine"));

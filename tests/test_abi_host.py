@@ -76,6 +76,33 @@ def test_workspace_query_and_size_checks(lib):
         assert lib.strads_workspace_bytes(C.byref(cfg), C.byref(out)) == -1, (S, n_cand)
 
 
+def test_workspace_provides_for_one_launch_rounds_only_where_they_are_made(lib):
+    """Their buffers (partial tiles alone 12 MB with dense X): one scheduler, and dense X only up to N rho^2 = 9."""
+    from paper_1312_5766_b200 import binding as b
+
+    def need(rho, **kw):
+        cfg = b.Config()
+        cfg.layout, cfg.n_rows, cfg.n_cols, cfg.ld, cfg.n_candidates, cfg.n_keep = 0, 1000, 10_000, 4096, 512, 32
+        cfg.rho = rho
+        for k, v in kw.items():
+            setattr(cfg, k, v)
+        out = C.c_size_t(0)
+        assert lib.strads_workspace_bytes(C.byref(cfg), C.byref(out)) == 0
+        return out.value
+
+    tiles = 192 * 128 * 128 * 4
+    assert need(0.1) + tiles < need(0.05)                    # 1,000 rows: N rho^2 = 10 and 2.5
+    assert need(0.1, n_rows=880) + 4 * 512 * 120 > need(0.1) + tiles
+    assert need(0.1, n_rows=880, n_schedulers=2) < need(0.1, n_rows=880)
+    csc = dict(layout=1, nnz=500_000, n_rows=50_000, n_candidates=2048, n_keep=256)
+    assert need(0.1, **csc) == need(0.0, **csc)
+    one, two, four = (need(0.1, n_schedulers=s, **csc) for s in (1, 2, 4))
+    assert (four - two) // 2 > two - one                     # the first of several has no such buffers either
+    # rho not known yet: enough for any
+    for kw in (dict(), dict(n_rows=2048), dict(n_rows=3000), dict(n_schedulers=4), csc, dict(csc, n_schedulers=3)):
+        assert all(need(0.0, **kw) >= need(rho, **kw) for rho in (0.01, 0.1, 0.5)), kw
+
+
 def test_init_rejects_bad_pointers_and_parameters_without_touching_the_gpu(lib):
     from paper_1312_5766_b200 import binding as b
 

@@ -63,3 +63,38 @@ def test_handles_in_turn_and_side_by_side(kw):
             for x, y in zip(out, want[i % 4]):
                 assert torch.equal(x, y), i
     assert b.load().strads_release_cached() == 0
+
+
+def test_a_workspace_sized_for_another_rho():
+    """Sized with rho = 0.1 (no buffers for rounds in one launch), used with rho = 0.05, which would have them: other kernels, same rounds."""
+    import ctypes as C
+    from paper_1312_5766_b200 import binding as b
+    p = wl.make_problem(dict(SHAPES["no_window"], rho=0.05), seed=6, device="cuda")
+    s = b.StradsLasso.from_problem(p, device="cuda")
+    lib, cfg = b.load(), b.Config()
+    C.memmove(C.byref(cfg), C.byref(s._cfg), C.sizeof(cfg))
+    need = C.c_size_t(0)
+    cfg.rho = 0.1
+    assert lib.strads_workspace_bytes(C.byref(cfg), C.byref(need)) == 0 and need.value < s.workspace.numel()
+    cfg.rho = p.rho
+    ws = torch.empty(need.value, dtype=torch.uint8, device="cuda")
+    beta, resid, delta = torch.zeros_like(s.beta), torch.empty_like(s.resid), torch.empty_like(s.delta)
+    cfg.workspace, cfg.workspace_bytes = ws.data_ptr(), need.value
+    cfg.beta, cfg.resid, cfg.delta = beta.data_ptr(), resid.data_ptr(), delta.data_ptr()
+    h = C.c_void_p(None)
+    assert lib.strads_lasso_init(C.byref(cfg), C.byref(h)) == 0
+    kept = torch.empty(2, p.n_keep, dtype=torch.int32, device="cuda")
+    for _ in range(6):
+        out = b.RoundOut()
+        out.kept = kept[1].data_ptr()
+        assert lib.strads_round(h, C.byref(out)) == 0
+        kept[0].copy_(s.round()[1])
+        assert torch.equal(kept[0], kept[1])
+    assert lib.strads_run(h, 20) == 0
+    s.run(20)
+    torch.cuda.synchronize()
+    for x, y in ((s.beta, beta), (s.resid, resid), (s.delta, delta)):
+        assert float((x - y).norm()) <= 1e-5 * float(x.norm())          # dense products in another order
+    assert lib.strads_destroy(h) == 0
+    cfg.workspace_bytes = need.value - 256
+    assert lib.strads_lasso_init(C.byref(cfg), C.byref(h)) == -3
