@@ -752,17 +752,22 @@ __global__ void __launch_bounds__(256) k_gram_recheck(Problem p, int only_if_sho
 // when it runs alone (c2's window 22 -> 19 us), but the round as replayed, with the draw of the next round on a stream
 // beside it, measured slower with them (c3: 68.4 us per round with clusters of 9, 65.9 with 8; c2 39.1 / 38.2).
 constexpr int kMaxSplit = 8;
-static int g_max_clusters[kMaxSplit + 1];     // [size]; 0: size not available
+constexpr int kMaxDevices = 64;
+struct Clusters { bool known; int most[kMaxSplit + 1]; };      // [size]; 0: size not available
+static Clusters g_clusters[kMaxDevices];      // asked once per device: the seven queries take 100 us
 static std::mutex g_clusters_mutex;
-static bool g_clusters_known = false;         // (asked once: the seven queries take 100 us, and every GPU here is alike)
 
 cudaError_t prepare_gram_dense_tc() {
   cudaError_t e = cudaFuncSetAttribute(k_gram_dense_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmem);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_gram_dense_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmem);
   if (e != cudaSuccess) return e;
+  int dev = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaSuccess;         // (no clusters there)
   std::lock_guard<std::mutex> lock(g_clusters_mutex);
-  for (int size = 2; size <= kMaxSplit && !g_clusters_known; ++size) {
+  Clusters& c = g_clusters[dev];
+  for (int size = 2; size <= kMaxSplit && !c.known; ++size) {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)size; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
@@ -770,10 +775,10 @@ cudaError_t prepare_gram_dense_tc() {
     cfg.gridDim = dim3((unsigned)size * 64); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kDynSmem;
     cfg.attrs = attr; cfg.numAttrs = 1;
     int n = 0;
-    g_max_clusters[size] = cudaOccupancyMaxActiveClusters(&n, k_gram_dense_tc<false>, &cfg) == cudaSuccess ? n : 0;
+    c.most[size] = cudaOccupancyMaxActiveClusters(&n, k_gram_dense_tc<false>, &cfg) == cudaSuccess ? n : 0;
     cudaGetLastError();                                  // (a size the device refuses is simply not used)
   }
-  g_clusters_known = true;
+  c.known = true;
   return cudaSuccess;
 }
 
@@ -813,10 +818,11 @@ cudaError_t launch_gram_dense_tc(const Problem& p, const void* tmap, const int* 
   // few tiles (a candidate window): share each tile's K range among the CTAs of a cluster so that all SMs work; the
   // largest cluster size of which the device holds `tiles` at once (one wave), and at least two stages of K each
   int n_split = 1;
-  if (tiles * 2 <= p.sm_count) {
+  int dev = 0;
+  if (tiles * 2 <= p.sm_count && cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices) {
     const int n_st = (int)((p.N + 2 * kScreenK - 1) / (2 * kScreenK));
     for (int size = kMaxSplit; size >= 2; --size)
-      if (g_max_clusters[size] >= tiles && size * 2 <= n_st) { n_split = size; break; }
+      if (g_clusters[dev].most[size] >= tiles && size * 2 <= n_st) { n_split = size; break; }
   }
   Problem q = p;
   q.cand_cur = cand;
