@@ -111,3 +111,66 @@ def test_tied_keys():
     s.run(5)
     delta = s.delta.cpu().numpy().astype(np.float64)
     assert np.array_equal(s.round()[0].cpu().numpy(), oracle.sample(delta, float(np.float32(p.eta)), p.seed, 8, p.n_candidates))
+
+
+# rows in the buckets on average 6.4 of 16 (every other round overflows one) and 10 (every attempt does)
+@pytest.mark.parametrize("nnz_col", [25, 40])
+def test_round_index_set_back_while_the_buckets_rest(nnz_col):
+    """After an overflow the row buckets rest for a number of rounds; going back to an earlier round in that time changes nothing."""
+    from paper_1312_5766_b200 import binding as b
+    p = wl.make_problem(dict(CASES["full_buckets"], lam_frac=0.02, nnz_col=nnz_col), seed=5)
+    s, fresh = (b.StradsLasso.from_problem(p, device="cuda") for _ in range(2))
+    s.run(3)
+    start = [t.clone() for t in (s.beta, s.resid, s.delta)]
+    want = [[t.clone() for t in s.round()] for _ in range(12)]
+    end = [t.clone() for t in (s.beta, s.resid, s.delta)]
+    for first in (1, 2, 5, 12):                             # rounds gone before the next return
+        for t, c in zip((s.beta, s.resid, s.delta), start):
+            t.copy_(c)
+        s.set_round(3)
+        for i in range(first):
+            for x, y in zip(s.round(), want[i]):
+                assert torch.equal(x, y), (first, i)
+    for x, y in zip((s.beta, s.resid, s.delta), end):
+        assert torch.equal(x, y)
+    fresh.run(15)
+    for x, y in zip((fresh.beta, fresh.resid, fresh.delta), end):
+        assert torch.equal(x, y)
+
+
+MENDED = {
+    # the untouched coefficients run out: the cutoff carried over is far too low for the draw of the next round
+    "dense": dict(kind="dense_iid", n_rows=64, n_cols=1201, n_true=9, n_candidates=300, n_keep=90, rho=0.37),
+    "csc": dict(kind="csc_uniform", n_rows=5000, n_cols=3003, n_true=9, n_candidates=500, n_keep=130, rho=0.1, nnz_col=20),
+    "few": dict(kind="csc_uniform", n_rows=5000, n_cols=603, n_true=9, n_candidates=40, n_keep=30, rho=0.1, nnz_col=20),
+}
+
+
+@pytest.mark.parametrize("tied", [False, True])
+@pytest.mark.parametrize("name", list(MENDED))
+def test_launches_that_end_in_a_mended_draw(name, tied):
+    """The draw for the round behind a launch's last one selected anew (too few keys below the cutoff, or -- tied -- more equal
+    keys than there is room for): the next launch finds histogram and cursors as it expects them."""
+    from paper_1312_5766_b200 import binding as b
+    cfg = dict(MENDED[name], lam_frac=0.02)
+    if tied:
+        cfg.update(n_cols=30_000)
+    p = wl.make_problem(cfg, seed=6)
+    s, ahead = (b.StradsLasso.from_problem(p, device="cuda") for _ in range(2))
+    eta, n = float(np.float32(p.eta)), 24
+    if tied:
+        for h in (s, ahead):
+            h.delta[2_000:25_000] = float("inf")
+            h.set_round(0)
+    for t in range(n):
+        delta = s.delta.cpu().numpy().astype(np.float64)
+        assert np.array_equal(s.round()[0].cpu().numpy(), oracle.sample(delta, eta, p.seed, t, p.n_candidates)), t
+        ahead.run(1)                                        # a launch per round, each with the draw of the next
+        for x, y in ((s.beta, ahead.beta), (s.resid, ahead.resid), (s.delta, ahead.delta)):
+            assert torch.equal(x, y), t
+    ahead.run(7)
+    for _ in range(7):
+        s.round()
+    for x, y in ((s.beta, ahead.beta), (s.resid, ahead.resid), (s.delta, ahead.delta)):
+        assert torch.equal(x, y)
+    assert (s.status()[1] & 1) == (1 if tied else 0)        # ties: the boundary was cut further
