@@ -140,9 +140,12 @@ __device__ __forceinline__ float tf32_lo(float x) {
   return __uint_as_float(__float_as_uint(x - hi) & 0xffffe000u);
 }
 
-// Pairs the screen left open.  A CTA keeps the first few of its own (four per warp: a dozen microseconds of exact products
-// at most) and decides them itself before it leaves, the grid's CTAs side by side; the others go to the list in
-// global memory.
+// Pairs the screen left open.  A CTA keeps the first few of its own (four per warp) and decides them itself before it
+// leaves, the grid's CTAs side by side; the others go to the list in global memory.  A turn -- a pair per warp -- takes 4 us
+// at 5,000 rows and 15 at 20,000, where 80 CTAs then bring in 5 TB/s.  What overflows costs a whole list some 75 us more at
+// 20,000 rows (the kernels behind the screen), a window a round of the whole list (400 to 700 us).  With 36 or 48 instead of
+// 24 a whole list of 512 candidates of 20,000 rows with some 25 open pairs a CTA takes 162 and 153 instead of 190 us per
+// round, with more open pairs 218 and 209 instead of 198 or 267 and 291 instead of 267.
 constexpr unsigned int kOwnOpen = 24;
 struct OwnOpen { unsigned int n, pair[kOwnOpen]; };
 // A row's conflicts (bit j: with b0 + j; those above the diagonal are listed for the walk) and the pairs left open.  Few rows
@@ -343,11 +346,50 @@ __device__ __noinline__ double exact_product(const float* xa, const float* xb, l
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   return acc;
 }
+// The same sums for long columns.  Bound by the latency of the loads, so those of eight groups of four rows are under way
+// together: with two, six warps of a CTA took 35 us for a pair each of 20,000 rows, with eight 15 (512 candidates, some 15
+// open pairs a CTA: 183 -> 117 us per round; 5,000 rows 45 -> 41).  In kernels of its own: columns of 1,000 rows meet open
+// pairs every round, and as instructions come from a cold cache a round paid 0.5 % for the longer code beside them.
+constexpr long long kLongColumn = 4096;
+__device__ __noinline__ double exact_product_long(const float* xa, const float* xb, long long N) {
+  const int lane = threadIdx.x & 31;
+  double acc = 0.0;
+  constexpr int kU = 8;
+  const float4 *a4 = reinterpret_cast<const float4*>(xa), *b4 = reinterpret_cast<const float4*>(xb);
+  long long g = lane;
+#pragma unroll 1
+  for (; (g + 32 * kU) * 4 <= N; g += 32 * kU) {         // (whole groups only)
+    float4 u[kU], w[kU];
+#pragma unroll
+    for (int i = 0; i < kU; ++i) { u[i] = a4[g + 32 * i]; w[i] = b4[g + 32 * i]; }
+#pragma unroll
+    for (int i = 0; i < kU; ++i) {
+      acc += (double)u[i].x * w[i].x;
+      acc += (double)u[i].y * w[i].y;
+      acc += (double)u[i].z * w[i].z;
+      acc += (double)u[i].w * w[i].w;
+    }
+  }
+#pragma unroll 1
+  for (; g < (N + 3) >> 2; g += 32) {
+    const float4 u = a4[g], w = b4[g];
+    const long long i = g << 2;
+    acc += (double)u.x * w.x;
+    if (i + 1 < N) acc += (double)u.y * w.y;
+    if (i + 2 < N) acc += (double)u.z * w.z;
+    if (i + 3 < N) acc += (double)u.w * w.w;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  return acc;
+}
 // Exact decision for one pair the screen could not call, by a whole warp.  Setting a bit is idempotent and
 // order-independent, so the result is deterministic.
+template <bool kLong>
 __device__ __forceinline__ void recheck_pair(const Problem& p, unsigned int pr, int lane) {
   const int a = (int)(pr >> 16), b = (int)(pr & 0xffffu);
-  const double acc = exact_product(p.xv + (long long)p.cand_cur[a] * p.ld, p.xv + (long long)p.cand_cur[b] * p.ld, p.N);
+  const float *xa = p.xv + (long long)p.cand_cur[a] * p.ld, *xb = p.xv + (long long)p.cand_cur[b] * p.ld;
+  const double acc = kLong ? exact_product_long(xa, xb, p.N) : exact_product(xa, xb, p.N);
   if (lane == 0) {
     const double den = sqrt(coupling_n2(p, p.cand_cur[a])) * sqrt(coupling_n2(p, p.cand_cur[b]));
     if (den > 0.0 && fabs(acc) >= (double)p.rho * den) {
@@ -359,11 +401,10 @@ __device__ __forceinline__ void recheck_pair(const Problem& p, unsigned int pr, 
 
 // What follows the window's Gram on the round's path, done by the CTA of the Gram kernel that finishes last
 // instead of by launches of their own:
-//   - the pairs the screen left open, normally a handful or none, are decided exactly.  "Few" is a budget of
-//     multiply-adds for this one CTA (2^21, some tens of microseconds at worst): short columns leave many pairs
-//     open (their correlations scatter widely around rho) but each is cheap, long columns hardly any.  Beyond the
-//     budget a window is handed to the whole-list retry, whose Gram has a recheck kernel of its own, and a whole list
-//     to the kernels of launch_gram_rest;
+//   - the pairs listed as open, normally a handful or none, are decided exactly.  "Few" is a budget of
+//     multiply-adds for this one CTA (2^21): short columns leave many pairs open (their correlations scatter widely around
+//     rho) but each is cheap, long columns hardly any.  Beyond the budget a window is handed to the whole-list retry, whose
+//     Gram has a recheck kernel of its own, and a whole list to the kernels of launch_gram_rest;
 //   - the greedy first-fit walk is settled from the list of conflicting pairs; if that list is incomplete or the
 //     chains of dependent decisions are too long, the walk kernel behind this one does it from the bit rows
 //     (walk_pending), otherwise that kernel returns at once.
@@ -371,6 +412,7 @@ __device__ __forceinline__ void recheck_pair(const Problem& p, unsigned int pr, 
 // at the end of the branch that holds the walk kernel and the whole-list retry.
 constexpr unsigned int kInlineRecheck = 4096;
 constexpr long long kInlineRecheckWork = 1ll << 21;
+template <bool kLong>
 __device__ void window_tail(const Problem& p, const int* __restrict__ cand, int n_cand, int n_total, unsigned char* sm) {
   __shared__ int s_last, s_kept, s_examined;
   DeviceState* st = p.st;
@@ -391,7 +433,7 @@ __device__ void window_tail(const Problem& p, const int* __restrict__ cand, int 
     }
     return;
   }
-  for (unsigned int e = tid >> 5; e < n_amb; e += blockDim.x >> 5) recheck_pair(p, __ldcg(p.amb_pairs + e), tid & 31);
+  for (unsigned int e = tid >> 5; e < n_amb; e += blockDim.x >> 5) recheck_pair<kLong>(p, __ldcg(p.amb_pairs + e), tid & 31);
   if (tid == 0) { s_kept = 0; s_examined = n_cand; }
   __syncthreads();
   const unsigned int n_edges = __ldcg(&st->edge_count);
@@ -420,7 +462,8 @@ __device__ void window_tail(const Problem& p, const int* __restrict__ cand, int 
 // a slice of K (a window of few tiles would otherwise use few SMs); the partial tiles are combined through
 // distributed shared memory, in split order.  tail: 0 none; 1 the CTA of the grid that finishes last rechecks the
 // pairs the screen left open and settles the greedy walk from the list of conflicting pairs (window_tail).
-template <bool k3x>
+// kLong: columns of kLongColumn rows or more.
+template <bool k3x, bool kLong>
 __global__ void __launch_bounds__(kThreads, 1) k_gram_dense_tc(Problem p, const __grid_constant__ CUtensorMap tmap,
                                                                 int n_cand, int n_total, int n_tiles, int n_split, int only_if_short,
                                                                 int tail) {
@@ -726,8 +769,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_dense_tc(Problem p, const 
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
   }
   if (!k3x && tail) {
-    for (unsigned int e = warp; e < min(s_own.n, kOwnOpen); e += kThreads / 32) recheck_pair(p, s_own.pair[e], lane);
-    window_tail(p, p.cand_cur, n_cand, n_total, tiles_ptr);
+    for (unsigned int e = warp; e < min(s_own.n, kOwnOpen); e += kThreads / 32) recheck_pair<kLong>(p, s_own.pair[e], lane);
+    window_tail<kLong>(p, p.cand_cur, n_cand, n_total, tiles_ptr);
   }
 }
 
@@ -741,7 +784,7 @@ __global__ void __launch_bounds__(256) k_gram_recheck(Problem p, int only_if_sho
   const int lane = threadIdx.x & 31;
   const unsigned int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const unsigned int n_warps = (gridDim.x * blockDim.x) >> 5;
-  for (unsigned int e = warp; e < n; e += n_warps) recheck_pair(p, p.amb_pairs[e], lane);
+  for (unsigned int e = warp; e < n; e += n_warps) recheck_pair<false>(p, p.amb_pairs[e], lane);
 }
 
 }  // namespace
@@ -758,10 +801,9 @@ static Clusters g_clusters[kMaxDevices];      // asked once per device: the seve
 static std::mutex g_clusters_mutex;
 
 cudaError_t prepare_gram_dense_tc() {
-  cudaError_t e = cudaFuncSetAttribute(k_gram_dense_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmem);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_gram_dense_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmem);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
+  for (auto fn : {k_gram_dense_tc<false, false>, k_gram_dense_tc<false, true>, k_gram_dense_tc<true, false>})
+    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmem)) != cudaSuccess) return e;
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxDevices) return cudaSuccess;         // (no clusters there)
@@ -775,7 +817,7 @@ cudaError_t prepare_gram_dense_tc() {
     cfg.gridDim = dim3((unsigned)size * 64); cfg.blockDim = dim3(kThreads); cfg.dynamicSmemBytes = kDynSmem;
     cfg.attrs = attr; cfg.numAttrs = 1;
     int n = 0;
-    c.most[size] = cudaOccupancyMaxActiveClusters(&n, k_gram_dense_tc<false>, &cfg) == cudaSuccess ? n : 0;
+    c.most[size] = cudaOccupancyMaxActiveClusters(&n, k_gram_dense_tc<false, false>, &cfg) == cudaSuccess ? n : 0;
     cudaGetLastError();                                  // (a size the device refuses is simply not used)
   }
   c.known = true;
@@ -837,13 +879,13 @@ cudaError_t launch_gram_dense_tc(const Problem& p, const void* tmap, const int* 
   const bool screen = !(p.flags & STRADS_FLAG_GRAM_3XTF32);
   if (screen) {
     const int ctas = n_split > 1 ? tiles * n_split : (tiles < p.sm_count ? tiles : p.sm_count);
-    if ((e = launch_chained_cluster(k_gram_dense_tc<false>, ctas, kThreads, kDynSmem, s, n_split, q, tm, n_cand, n_total,
+    if ((e = launch_chained_cluster(p.N < kLongColumn ? k_gram_dense_tc<false, false> : k_gram_dense_tc<false, true>, ctas, kThreads, kDynSmem, s, n_split, q, tm, n_cand, n_total,
                                     n_tiles, n_split, ois, tail ? 1 : 0)) != cudaSuccess)
       return e;
     if (tail) return cudaSuccess;
     if ((e = launch_chained_split(true, k_gram_recheck, p.sm_count * 2, 256, 0, s, q, ois, 0)) != cudaSuccess) return e;
   }
-  return launch_chained(k_gram_dense_tc<true>, tiles < p.sm_count ? tiles : p.sm_count, kThreads, kDynSmem, s, q, tm, n_cand, n_total,
+  return launch_chained(k_gram_dense_tc<true, false>, tiles < p.sm_count ? tiles : p.sm_count, kThreads, kDynSmem, s, q, tm, n_cand, n_total,
                         n_tiles, 1, ois, 0);
 }
 
@@ -855,7 +897,7 @@ cudaError_t launch_gram_rest(const Problem& p, const void* tmap, const int* cand
   q.cand_cur = cand;
   const cudaError_t e = launch_chained_split(true, k_gram_recheck, p.sm_count * 2, 256, 0, s, q, 0, 1);
   if (e != cudaSuccess) return e;
-  return launch_chained(k_gram_dense_tc<true>, tiles < p.sm_count ? tiles : p.sm_count, kThreads, kDynSmem, s, q,
+  return launch_chained(k_gram_dense_tc<true, false>, tiles < p.sm_count ? tiles : p.sm_count, kThreads, kDynSmem, s, q,
                         *static_cast<const CUtensorMap*>(tmap), n_cand, n_cand, n_tiles, 1, 0, 0);
 }
 

@@ -29,6 +29,28 @@ def test_open_pairs(n_rows, n_candidates, n_keep, rho):
     assert s.status()[0] == 0
 
 
+# long columns: a few turns of every CTA; more pairs than the CTAs decide themselves; the shortest; rows that end inside a
+# group of four, just behind and just before whole trips
+@pytest.mark.parametrize("n_rows,rho", [(20_004, 0.024), (20_004, 0.012), (4096, 0.05), (4097, 0.05), (5119, 0.045), (5123, 0.045)])
+def test_open_pairs_of_long_columns(n_rows, rho):
+    from paper_1312_5766_b200 import binding as b
+    p = wl.make_problem(dict(kind="dense_iid", n_rows=n_rows, n_cols=700, n_true=20, lam_frac=0.02, n_candidates=161, n_keep=90, rho=rho), seed=9)
+    if n_rows % 4:
+        pad = torch.full((p.n_cols, (n_rows + 3) // 4 * 4), float("nan"))          # nothing may leak in from the padding
+        pad[:, :n_rows] = p.values
+        p.values = pad
+    X = oracle_matrix(p)
+    n2 = oracle.colnorm2(X)
+    s, ahead = (b.StradsLasso.from_problem(p, device="cuda") for _ in range(2))
+    for _ in range(4):
+        cand, kept, _, counts = (v.cpu().numpy() for v in s.round())
+        _assert_kept_matches(X, n2, cand, 90, float(np.float32(rho)), kept[: int(counts[2])], int(counts[1]))
+    ahead.run(4)
+    for x, y in ((s.beta, ahead.beta), (s.resid, ahead.resid), (s.delta, ahead.delta)):
+        assert torch.equal(x, y)
+    assert s.status()[0] == 0
+
+
 @pytest.mark.parametrize("n_candidates,bits", [(300, 0), (1600, 8)])
 def test_products_that_cluster_at_rho(n_candidates, bits):
     """Columns of +-1 over a few rows: a third of all pairs correlate at exactly rho.  Two schedulers: not whole rounds in one launch."""
