@@ -43,10 +43,11 @@ NCU_TRAFFIC = {
     # profiles/ncu_k_gram_dense_tc_window_c3_J20000.md: 25.75 MB read + 0 written per launch (captured with J cut to 20,000;
     # the kernel reads the window's BF16 copies only, so its traffic does not depend on J) = the algorithmic 2 N W
     ("c3", "k_gram_dense_tc<screen>"): 25.75e6,
-    # profiles/ncu_full_round_kernels_c4.md: 6.82 MB read per launch (the buckets of the window candidates' rows)
-    ("c4", "k_csc_bucket_dots"): 6.82e6,
-    # k_walk_csc spins on a grid barrier: no multi-pass capture of it is made (one-pass launch list only)
+    # profiles/k_engine.md: one-pass captures of whole launches (32 rounds)
+    ("c4", "k_engine<csc>"): 66.3e6,
+    ("c5", "k_engine<csc>"): 402.9e6,
 }
+ENGINE_ROUNDS = 32                         # CSC: whole rounds in one launch, that many at most
 
 
 def measured_peaks():
@@ -230,16 +231,16 @@ def rooflines(p: wl.LassoProblem, workload: str, step_ms: dict, kept_per_round: 
     else:
         nnz_col = p.nnz / p.n_cols
         if step_ms["walk_ms"] >= step_ms["gram_ms"]:
-            # dominant: the cooperative on-demand walk; every kept candidate's column is merged with every later
-            # candidate not yet blocked (at most all examined ones): <= 2 nnz_col - 1 compare steps per merge
-            kernel = "k_walk_csc"
+            # its longest step is the walk on demand: every kept candidate's column is merged with every later candidate
+            # not yet blocked (at most all examined ones): <= 2 nnz_col - 1 compare steps per merge
             ops = kept_per_round * examined_per_round * (2.0 * nnz_col - 1.0)
-            ms = step_ms["walk_ms"]
         else:
-            # dominant: the inner products of the window's pairs that share a row
-            kernel = "k_csc_bucket_dots"
+            # its longest step is the inner products of the window's pairs that share a row
             ops = 0.5 * window * (window - 1) * (nnz_col * nnz_col / p.n_rows) * (2.0 * nnz_col - 1.0)
-            ms = step_ms["gram_ms"]
+        # whole rounds in one launch: the kernel of the timed regions, all its steps in its time
+        kernel = "k_engine<csc>"
+        ms = ENGINE_ROUNDS * ms_per_step
+        ops *= ENGINE_ROUNDS
         peak = 148 * 128 * peaks["sm_max_mhz"] * 1e6 / 1e12        # integer / FP32 lanes x clock, T op/s
         achieved = ops / (ms * 1e-3) / 1e12
         out["roofline"] = {
@@ -247,9 +248,9 @@ def rooflines(p: wl.LassoProblem, workload: str, step_ms: dict, kept_per_round: 
             "frac": achieved / peak, "traffic": NCU_TRAFFIC.get((workload, kernel)), "window": window, "launch_ms": ms,
             "algorithmic_ops_per_launch": ops,
             "peak_source": "148 SMs x 128 lanes x max SM clock: one merge step (compare + advance) per lane per cycle",
-            "note": "inner products of sparse columns counted as sorted-list merge steps, over a few MB of columns: bound by "
-                    "dependent loads and barriers, not by HBM; the timed regions make this step inside whole rounds in one "
-                    "launch, launch_ms is the kernel that makes it where the steps are launched one by one"}
+            "note": f"a launch is {ENGINE_ROUNDS} whole rounds; of their steps only the inner products of sparse columns are "
+                    "counted, as sorted-list merge steps, over a few MB of columns: bound by dependent loads and barriers, "
+                    "not by HBM"}
         upd_bytes = 8.0 * nnz_col * kept_per_round + 8.0 * p.n_rows
         pack_bytes = 0.0
         ns_bytes = 8.0 * nnz_col * (p.n_candidates + kept_per_round) + 8.0 * p.n_rows
@@ -275,7 +276,7 @@ def launches_of_run(p: wl.LassoProblem, steps: int) -> int:
     """Kernels of the library launched by a strads_run of `steps` rounds (dense: a fixed sequence per round; launches of the
     retry branch return at once when the screen's last CTA settled the round)."""
     if p.layout != wl.DENSE:
-        return (steps + 31) // 32          # whole rounds in one launch, 32 of them at most
+        return (steps + ENGINE_ROUNDS - 1) // ENGINE_ROUNDS
     n = 3                  # the early draw of the next round: histogram pass, collect pass, ordering
     n += 1                 # correction of the early list
     n += 2                 # pack, Gram (screen + cluster split-K + recheck + walk)
@@ -348,8 +349,9 @@ def measure(workload: str, args, device, rank: int, world: int, dist_ok: bool, p
         "step_ms": step_ms, "step_ms_rounds": prof["rounds"],
         "step_ms_note": "device time per step over the rounds right after the timed regions, launched kernel by kernel "
                         "with CUDA events between steps and a plain draw; the timed regions replay captured launch "
-                        "sequences, in which (dense) the draw of the next round runs beside the Gram on a second stream",
-        "sampling_ahead": p.layout == wl.DENSE and p.n_keep <= 4096,
+                        "sequences, in which the draw of the next round runs beside the Gram on a second stream (dense), or "
+                        "run whole rounds in one launch, with the draw of the next in their shadow (CSC)",
+        "sampling_ahead": p.n_keep <= 4096,
         "clocks": clk,
     }
     rec.update(rooflines(p, workload, step_ms, kept_per_round, examined_per_round, moving_per_round, ms_local / args.steps,

@@ -168,16 +168,20 @@ int strads_round(strads_handle_t h, const strads_round_out_t* out);
  * Each scheduler has its own slice of the workspace.  On return every piece of work has been enqueued and
  * the configured stream waits for all of it.
  *
- * One scheduler, dense X, n_keep <= 4096: the candidates of round t + 1 (Algorithm 1's draw) depend on
+ * One scheduler, n_keep <= 4096, dense X or CSC: the candidates of round t + 1 (Algorithm 1's draw) depend on
  * round t only through the at most P priorities its update changes, so strads_run draws the P' + P best of
- * round t + 1 during round t, on a stream of its own beside the Gram and the walk, from the priorities of
- * round t's start, and round t + 1 starts from that list corrected for the coefficients round t updated
- * (they are struck and entered again with their new keys; the P' smallest remain).  The candidates are
- * exactly those of a draw made at the round's start; the state after strads_run equals that of the same
- * rounds run with strads_round, bit for bit.  Eight rounds are replayed per captured launch sequence, and what is
- * left over of a run as sequences of four, two and one round (with any layout and number of schedulers the rounds
- * of a run are replayed from captured sequences; with several schedulers 16 turns of each per sequence); the
- * streams and events this needs belong to the handle (no device memory is allocated). */
+ * round t + 1 during round t, from the priorities of round t's start, and round t + 1 starts from that list
+ * corrected for the coefficients round t updated (they are struck and entered again with their new keys; the P'
+ * smallest remain).  The candidates are exactly those of a draw made at the round's start; the state after
+ * strads_run equals that of the same rounds run with strads_round, bit for bit.  The list drawn for the round
+ * behind the last one stays: whoever writes delta (or beta, or resid) between two runs calls strads_set_round.
+ *
+ * CSC with one scheduler, and dense X with short columns (N rho^2 <= 9, N <= 2,048), run up to 32 whole rounds per
+ * cooperative launch.  Otherwise the rounds are replayed from captured launch sequences: with one scheduler eight
+ * rounds each (the draw on a stream of its own beside the Gram and the walk), and what is left over of a run as
+ * sequences of four, two and one round, each captured when its length comes up for the third time and
+ * enqueued directly until then; with several schedulers 16 turns of each per sequence.  The streams, events and
+ * executable graphs this needs outlive the handle (strads_release_cached); no device memory is allocated. */
 int strads_run(strads_handle_t h, int64_t n_rounds);
 
 /* The same round as strads_round for callers whose state lives in HOST memory: copies
@@ -230,7 +234,7 @@ int strads_status(strads_handle_t h, uint32_t* bits_host_out);
 
 /* The error contract of the bounded waits ("nothing waits without a bound").  Every device-side wait of the
  * round -- the mbarrier waits of the dense Gram's TMA / tensor-core pipeline (SAP step 2) and the grid-wide
- * barrier of the CSC on-demand walk -- counts its iterations; past the limit the CTA raises
+ * barriers of the CSC on-demand walk and of whole rounds in one launch -- counts its iterations; past the limit the CTA raises
  * STRADS_STATUS_WAIT_EXPIRED, stops issuing work, releases its tensor memory and returns, so the launch ends and
  * strads_status reports STRADS_ERR_TIMEOUT.  From then on the round's outputs and beta / resid / delta are
  * undefined, and the CSC walk does nothing on this handle, until strads_recover has been called:

@@ -225,8 +225,10 @@ bool engine_possible(const strads_lasso_config_t* c) {
 // Whether the rounds go through it: one scheduler, and for dense X columns so short that independent ones correlate
 // beyond rho by chance (their correlations scatter with N^-1/2; the line is three of those).  There the launch chain's
 // screen leaves percents of all pairs open and its window fails round after round (463 x 508,999: 888 us per round as
-// launches, 65 here); with longer columns the captured chain of kernels, each with a whole GPU's worth of loads under way,
-// is the faster one (c1 36.3 us against 39.0, c2 42 against 60).
+// launches, 56 here).  J = 50,000, rho = 0.1, P' = 8 P, us per round here / as launches for P = 16, 128, 512: 464 rows 28 / 96,
+// 53 / 367, 161 / 668; 880 rows 28 / 36, 32 / 48, 100 / 193; 1,060 rows 28 / 30, 33 / 37, 95 / 77; 1,200 rows 28 / 28, 33 / 32,
+// 50 / 40; 2,048 rows 28 / 23, 32 / 28, 46 / 37.  So below the line this is never the slower side; above it the launches are at
+// first up to a seventh slower while few are kept, and faster where many are.
 bool engine_chosen(const strads_lasso_config_t* c) {
   if (!engine_possible(c) || n_sched_of(c) > 1) return false;
   return c->layout == STRADS_CSC || (double)c->n_rows * (double)c->rho * (double)c->rho <= 9.0;

@@ -13,7 +13,7 @@
 //   2  (all CTAs)  Gram tiles on the tensor cores                 inner products from the buckets, x_c^T r and would-be
 //                                                                 changes; keys of round t + 1 below the boundary collected
 //  (2b)            exact products of pairs left open
-//   3              greedy walk (CTA 0); keys of round t + 1       greedy walk (CTA 0); buckets emptied (the others)
+//   3              greedy walk (last CTA); keys of round t + 1    greedy walk (last CTA); buckets emptied (the others)
 //                  below the boundary collected (the others)
 //  (3b)            all candidates instead of the window           walk over all candidates with conflict rows on demand
 //   4  (all CTAs)  residual, beta, delta; the winners of the draw ranked, corrected for this round's changes
@@ -747,9 +747,9 @@ __device__ void commit_changes(const Problem& p, const Engine& e, int nk, int n_
 // that a product's bits do not depend on the number of candidates).
 //
 // The candidates are scattered over X (a page each), so what counts is how much is under way per SM: the columns come
-// into shared memory by bulk copies, several whole columns ahead, where a loop of register loads had 41 KB in flight and
-// waited for each trip (384 columns of 40 KB: 13.8 us, 640 of 80 KB: 31 us).  Every thread holds its rows of r in
-// registers for the whole step.
+// into shared memory by bulk copies, up to four whole columns of a group ahead, instead of through registers trip by trip.
+// Every thread holds its rows of r in registers for the whole step.  1,024 candidates of 463 rows: 3.6 us (their columns
+// were prefetched into L2 when they were ranked).
 // ------------------------------------------------------------------------------------------------
 struct TurnShared { double dot[kTurn][kWarps]; };
 struct PackBars { unsigned long long full[kWarps]; unsigned int uses[kWarps]; };
@@ -1304,64 +1304,62 @@ __device__ __forceinline__ void dense_walk(const Problem& p, const Engine& e, un
 }
 
 // ------------------------------------------------------------------------------------------------
-// Dense, step 4: r <- r - sum_a x_a dbeta_a.  The rows are dealt out evenly, a stretch of 16-byte groups per CTA; a thread
-// takes one group of one column at a time (the moving columns dealt out over kT / groups teams), six loads under way,
-// and the teams' FP64 sums are added in a fixed order.  (Blocks of 32 rows left a CTA three of them in turn at N = 10,000,
-// each with its own reduction: 10.7 us.)
+// Dense, step 4: r <- r - sum_a x_a dbeta_a.  The rows are dealt out evenly, a stretch of 16-byte groups per CTA (four of
+// them at 2,048 rows on 148 CTAs); a thread takes one group of one column at a time (the moving columns dealt out over
+// kT / groups teams), six loads under way, and the teams' FP64 sums are added in a fixed order.  Few rows, few columns that
+// move: 0.8 us at 463 rows, latency.
 // ------------------------------------------------------------------------------------------------
 __device__ void dense_apply(const Problem& p, const Moving& mv, double* part, int nk, int n_moving) {
   const int tid = threadIdx.x;
   const int n4 = (int)((p.N + 3) >> 2), per = (n4 + (int)gridDim.x - 1) / (int)gridDim.x;
   const int g_lo = (int)blockIdx.x * per, g_hi = min(n4, g_lo + per);
   if (g_lo >= n4 || n_moving == 0) return;
-  for (int g0 = g_lo; g0 < g_hi; g0 += kT) {             // (one turn up to 4 * 512 rows per CTA)
-    const int width = min(kT, g_hi - g0), teams = kT / width;
-    const int team = tid / width, q = tid - team * width;
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-    const float* x0 = p.xv + ((long long)(g0 + q) << 2);
-    constexpr int kU = 6;
-    auto add = [&](const float4& x, double d) { s0 += (double)x.x * d; s1 += (double)x.y * d; s2 += (double)x.z * d; s3 += (double)x.w * d; };
-    if (team < teams) {
-      const int here = min(n_moving, kStage);
-      for (int a0 = team; a0 < here; a0 += teams * kU) {
-        float4 x[kU];
-        double d[kU];
+  const int g0 = g_lo, width = g_hi - g_lo, teams = kT / width;          // (at most 2,048 rows: width <= kT)
+  const int team = tid / width, q = tid - team * width;
+  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+  const float* x0 = p.xv + ((long long)(g0 + q) << 2);
+  constexpr int kU = 6;
+  auto add = [&](const float4& x, double d) { s0 += (double)x.x * d; s1 += (double)x.y * d; s2 += (double)x.z * d; s3 += (double)x.w * d; };
+  if (team < teams) {
+    const int here = min(n_moving, kStage);
+    for (int a0 = team; a0 < here; a0 += teams * kU) {
+      float4 x[kU];
+      double d[kU];
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-          const int a = a0 + u * teams;
-          d[u] = a < here ? mv.d[a] : 0.0;
-          x[u] = a < here ? __ldg(reinterpret_cast<const float4*>(x0 + mv.off[a])) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+      for (int u = 0; u < kU; ++u) {
+        const int a = a0 + u * teams;
+        d[u] = a < here ? mv.d[a] : 0.0;
+        x[u] = a < here ? __ldg(reinterpret_cast<const float4*>(x0 + mv.off[a])) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
 #pragma unroll
-        for (int u = 0; u < kU; ++u) add(x[u], d[u]);
-      }
-      if (n_moving > kStage) {                           // beyond what was staged: found again in the kept list
-        int seen = 0;
-        for (int a = 0; a < nk; ++a) {
-          const double d = p.cand_dbeta64[p.kept_pos[a]];
-          if (d == 0.0) continue;
-          if (seen >= kStage && seen % teams == team) add(__ldg(reinterpret_cast<const float4*>(x0 + (long long)p.kept[a] * p.ld)), d);
-          ++seen;
-        }
-      }
-      double* at = part + ((size_t)team * width + q) * 4;
-      at[0] = s0; at[1] = s1; at[2] = s2; at[3] = s3;
+      for (int u = 0; u < kU; ++u) add(x[u], d[u]);
     }
-    __syncthreads();
-    const int rows = width * 4;
-    int tpr = 1;                                         // threads per row
-    while (tpr < 32 && tpr * 2 * rows <= kT) tpr *= 2;
-    for (int r0 = 0; r0 < rows; r0 += kT / tpr) {
-      const int r = r0 + tid / tpr, sub = tid & (tpr - 1);
-      double s = 0.0;
-      if (r < rows)
-        for (int t = sub; t < teams; t += tpr) s += part[(size_t)t * rows + r];
-      for (int o = tpr >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-      const long long row = ((long long)g0 << 2) + r;
-      if (sub == 0 && r < rows && row < p.N && s != 0.0) apply_row(p, row, s);
+    if (n_moving > kStage) {                           // beyond what was staged: found again in the kept list
+      int seen = 0;
+      for (int a = 0; a < nk; ++a) {
+        const double d = p.cand_dbeta64[p.kept_pos[a]];
+        if (d == 0.0) continue;
+        if (seen >= kStage && seen % teams == team) add(__ldg(reinterpret_cast<const float4*>(x0 + (long long)p.kept[a] * p.ld)), d);
+        ++seen;
+      }
     }
-    __syncthreads();
+    double* at = part + ((size_t)team * width + q) * 4;
+    at[0] = s0; at[1] = s1; at[2] = s2; at[3] = s3;
   }
+  __syncthreads();
+  const int rows = width * 4;
+  int tpr = 1;                                         // threads per row
+  while (tpr < 32 && tpr * 2 * rows <= kT) tpr *= 2;
+  for (int r0 = 0; r0 < rows; r0 += kT / tpr) {
+    const int r = r0 + tid / tpr, sub = tid & (tpr - 1);
+    double s = 0.0;
+    if (r < rows)
+      for (int t = sub; t < teams; t += tpr) s += part[(size_t)t * rows + r];
+    for (int o = tpr >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+    const long long row = ((long long)g0 << 2) + r;
+    if (sub == 0 && r < rows && row < p.N && s != 0.0) apply_row(p, row, s);
+  }
+  __syncthreads();
 }
 
 constexpr unsigned int kFewOpen = 48;                    // open pairs the walking CTA decides itself

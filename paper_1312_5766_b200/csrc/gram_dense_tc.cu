@@ -145,7 +145,7 @@ __device__ __forceinline__ float tf32_lo(float x) {
 // at 5,000 rows and 15 at 20,000, where 80 CTAs then bring in 5 TB/s.  What overflows costs a whole list some 75 us more at
 // 20,000 rows (the kernels behind the screen), a window a round of the whole list (400 to 700 us).  With 36 or 48 instead of
 // 24 a whole list of 512 candidates of 20,000 rows with some 25 open pairs a CTA takes 162 and 153 instead of 190 us per
-// round, with more open pairs 218 and 209 instead of 198 or 267 and 291 instead of 267.
+// round, but with some 35 it takes 218 and 209 instead of 198.
 constexpr unsigned int kOwnOpen = 24;
 struct OwnOpen { unsigned int n, pair[kOwnOpen]; };
 // A row's conflicts (bit j: with b0 + j; those above the diagonal are listed for the walk) and the pairs left open.  Few rows
