@@ -43,9 +43,9 @@ NCU_TRAFFIC = {
     # profiles/ncu_k_gram_dense_tc_window_c3_J20000.md: 25.75 MB read + 0 written per launch (captured with J cut to 20,000;
     # the kernel reads the window's BF16 copies only, so its traffic does not depend on J) = the algorithmic 2 N W
     ("c3", "k_gram_dense_tc<screen>"): 25.75e6,
-    # profiles/k_engine.md: one-pass captures of whole launches (32 rounds)
-    ("c4", "k_engine<csc>"): 66.3e6,
-    ("c5", "k_engine<csc>"): 402.9e6,
+    # profiles/k_engine.md: one-pass captures of whole launches of 32 rounds; per round
+    ("c4", "k_engine<csc>"): 66.3e6 / 32,
+    ("c5", "k_engine<csc>"): 402.9e6 / 32,
 }
 ENGINE_ROUNDS = 32                         # CSC: whole rounds in one launch, that many at most
 
@@ -206,7 +206,7 @@ def window_of(p: wl.LassoProblem) -> int:
 
 
 def rooflines(p: wl.LassoProblem, workload: str, step_ms: dict, kept_per_round: float, examined_per_round: float,
-              moving_per_round: float, ms_per_step: float, peaks: dict) -> dict:
+              moving_per_round: float, ms_per_step: float, steps: int, peaks: dict) -> dict:
     """Roofline of the dominant kernel plus the streaming kernels against the measured HBM bandwidth."""
     window = window_of(p)
     out = {}
@@ -239,16 +239,18 @@ def rooflines(p: wl.LassoProblem, workload: str, step_ms: dict, kept_per_round: 
             ops = 0.5 * window * (window - 1) * (nnz_col * nnz_col / p.n_rows) * (2.0 * nnz_col - 1.0)
         # whole rounds in one launch: the kernel of the timed regions, all its steps in its time
         kernel = "k_engine<csc>"
-        ms = ENGINE_ROUNDS * ms_per_step
-        ops *= ENGINE_ROUNDS
+        rounds = min(steps, ENGINE_ROUNDS)
+        ms = rounds * ms_per_step
+        ops *= rounds
+        traffic = NCU_TRAFFIC.get((workload, kernel))
         peak = 148 * 128 * peaks["sm_max_mhz"] * 1e6 / 1e12        # integer / FP32 lanes x clock, T op/s
         achieved = ops / (ms * 1e-3) / 1e12
         out["roofline"] = {
             "kernel": kernel, "bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tcompare/s",
-            "frac": achieved / peak, "traffic": NCU_TRAFFIC.get((workload, kernel)), "window": window, "launch_ms": ms,
-            "algorithmic_ops_per_launch": ops,
+            "frac": achieved / peak, "traffic": traffic and traffic * rounds, "window": window, "launch_ms": ms,
+            "rounds_per_launch": rounds, "algorithmic_ops_per_launch": ops,
             "peak_source": "148 SMs x 128 lanes x max SM clock: one merge step (compare + advance) per lane per cycle",
-            "note": f"a launch is {ENGINE_ROUNDS} whole rounds; of their steps only the inner products of sparse columns are "
+            "note": f"a launch is {rounds} whole rounds; of their steps only the inner products of sparse columns are "
                     "counted, as sorted-list merge steps, over a few MB of columns: bound by dependent loads and barriers, "
                     "not by HBM"}
         upd_bytes = 8.0 * nnz_col * kept_per_round + 8.0 * p.n_rows
@@ -354,7 +356,7 @@ def measure(workload: str, args, device, rank: int, world: int, dist_ok: bool, p
         "sampling_ahead": p.n_keep <= 4096,
         "clocks": clk,
     }
-    rec.update(rooflines(p, workload, step_ms, kept_per_round, examined_per_round, moving_per_round, ms_local / args.steps,
+    rec.update(rooflines(p, workload, step_ms, kept_per_round, examined_per_round, moving_per_round, ms_local / args.steps, args.steps,
                          peaks))
 
     # ---- the same workload with S round-robin scheduler threads (blocks of later rounds prepared during updates) ----
