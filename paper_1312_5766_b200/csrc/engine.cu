@@ -53,52 +53,41 @@ struct Grid {
   unsigned int* status;
 };
 
+// Arrives and waits (one thread; what its CTA wrote is ordered by a barrier before).  False: it gave up.
+__device__ __forceinline__ bool grid_wait(const Grid& g, bool withhold = false) {
+  if (!withhold) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(g.count) : "memory");
+  unsigned int v, it = 0;
+  bool ok;
+  do {
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(g.count) : "memory");
+    ok = v - g.target < g.n;
+  } while (!ok && ++it < g.limit);
+  if (!ok) atomicOr(g.status, STRADS_STATUS_WAIT_EXPIRED);
+  return ok;
+}
+
 // withhold: this CTA does not arrive (an injected stall: everybody's wait runs out).
 __device__ bool grid_sync(Grid& g, bool withhold = false) {
   __shared__ int s_ok;
   g.target += g.n;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    if (!withhold) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(g.count) : "memory");
-    unsigned int v, it = 0;
-    bool ok;
-    do {
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(g.count) : "memory");
-      ok = v - g.target < g.n;
-    } while (!ok && ++it < g.limit);
-    if (!ok) atomicOr(g.status, STRADS_STATUS_WAIT_EXPIRED);
-    s_ok = ok;
-  }
+  if (threadIdx.x == 0) s_ok = grid_wait(g, withhold);
   __syncthreads();
   return s_ok != 0;
 }
 
-// The same, with work for the other warps while the first one waits: step() until it has nothing left or the wait is over.
-template <typename Step>
-__device__ __forceinline__ bool grid_sync_busy(Grid& g, Step&& step) {
-  __shared__ int s_ok;
-  __shared__ volatile int s_over;
-  g.target += g.n;
-  if (threadIdx.x == 0) s_over = 0;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(g.count) : "memory");
-    unsigned int v, it = 0;
-    bool ok;
-    do {
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(g.count) : "memory");
-      ok = v - g.target < g.n;
-    } while (!ok && ++it < g.limit);
-    if (!ok) atomicOr(g.status, STRADS_STATUS_WAIT_EXPIRED);
-    s_ok = ok;
-    s_over = 1;
-  } else if (threadIdx.x >= 32) {
-#pragma unroll 1
-    while (!s_over && step()) {}
-  }
-  __syncthreads();
-  return s_ok != 0;
-}
+// The threads of a CTA that do a step together: all of them, or those that do not walk while the others do (below).
+constexpr int kWalkT = 256;                // threads that walk
+struct AllThreads {
+  static constexpr int kN = kT;
+  static __device__ __forceinline__ int tid() { return threadIdx.x; }
+  static __device__ __forceinline__ void sync() { __syncthreads(); }
+};
+struct OtherThreads {
+  static constexpr int kN = kT - kWalkT;
+  static __device__ __forceinline__ int tid() { return (int)threadIdx.x - kWalkT; }
+  static __device__ __forceinline__ void sync() { asm volatile("bar.sync 2, %0;" ::"n"(kN) : "memory"); }
+};
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -271,11 +260,12 @@ __device__ __forceinline__ void scan_found(const Engine& e, DrawShared& ds, unsi
     if (at < e.cap_surv) e.surv[(size_t)blockIdx.x * e.cap_surv + at] = key;
   }
 }
+template <typename Team>
 __device__ __forceinline__ void scan_close(const Engine& e, const DrawShared& ds, unsigned char* sm) {
   const unsigned int* sh = reinterpret_cast<const unsigned int*>(sm);
-  __syncthreads();
-  if (threadIdx.x == 0) e.saved[blockIdx.x] = ds.saved;
-  for (int b = threadIdx.x; b < kHistBins; b += kT) {
+  Team::sync();
+  if (Team::tid() == 0) e.saved[blockIdx.x] = ds.saved;
+  for (int b = Team::tid(); b < kHistBins; b += Team::kN) {
     const unsigned int v = sh[b];
     if (v) atomicAdd(&e.hist[b], v);
   }
@@ -291,17 +281,21 @@ __device__ __forceinline__ void draw_scan(const Problem& p, const Engine& e, Dra
   const Binning bins = binning_of(cut);
   scan_keys(p, t, cut, scan_queue(sm), (int)(threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x, kWarps * (int)gridDim.x,
             [&](unsigned long long key, bool on) { scan_found(e, ds, sh, bins, key, on); });
-  scan_close(e, ds, sm);
+  scan_close<AllThreads>(e, ds, sm);
 }
 
 // The bin b with before(b) < k <= before(b) + count(b), and the winners before every bin (ds.total < k: there is none).
-__device__ void draw_select(const Engine& e, DrawShared& ds, unsigned int k) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int kPer = kHistBins / kT;
-  static_assert(kPer == 8, "two 16-byte loads per thread");
-  const uint4 a = __ldcg(reinterpret_cast<const uint4*>(e.hist) + 2 * tid), b = __ldcg(reinterpret_cast<const uint4*>(e.hist) + 2 * tid + 1);
-  const unsigned int c[kPer] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-  unsigned int mine = 0u;
+template <typename Team>
+__device__ __forceinline__ void draw_select(const Engine& e, DrawShared& ds, unsigned int k) {
+  const int tid = Team::tid(), lane = tid & 31, warp = tid >> 5;
+  constexpr int kPer = kHistBins / Team::kN, kTeamWarps = Team::kN / 32;
+  static_assert(kPer % 4 == 0, "16-byte loads");
+  unsigned int c[kPer], mine = 0u;
+#pragma unroll
+  for (int u = 0; u < kPer / 4; ++u) {
+    const uint4 v = __ldcg(reinterpret_cast<const uint4*>(e.hist) + tid * (kPer / 4) + u);
+    c[4 * u] = v.x; c[4 * u + 1] = v.y; c[4 * u + 2] = v.z; c[4 * u + 3] = v.w;
+  }
 #pragma unroll
   for (int u = 0; u < kPer; ++u) mine += c[u];
   unsigned int incl = mine;
@@ -310,13 +304,13 @@ __device__ void draw_select(const Engine& e, DrawShared& ds, unsigned int k) {
     const unsigned int v = __shfl_up_sync(kFull, incl, o);
     if (lane >= o) incl += v;
   }
-  __syncthreads();
+  Team::sync();
   if (lane == 31) ds.wsum[warp] = incl;
   if (tid == 0) ds.refined = 0;
-  __syncthreads();
+  Team::sync();
   unsigned int before = 0u, total = 0u;
 #pragma unroll
-  for (int w = 0; w < kWarps; ++w) { const unsigned int v = ds.wsum[w]; if (w < warp) before += v; total += v; }
+  for (int w = 0; w < kTeamWarps; ++w) { const unsigned int v = ds.wsum[w]; if (w < warp) before += v; total += v; }
   unsigned int run = before + incl - mine;
 #pragma unroll
   for (int u = 0; u < kPer; ++u) {
@@ -325,8 +319,10 @@ __device__ void draw_select(const Engine& e, DrawShared& ds, unsigned int k) {
     run += c[u];
   }
   if (tid == 0) { ds.off[pad(kHistBins)] = total; ds.total = total; }
-  __syncthreads();
+  Team::sync();
 }
+// (for the cold paths)
+__device__ __noinline__ void draw_select_all(const Engine& e, DrawShared& ds, unsigned int k) { draw_select<AllThreads>(e, ds, k); }
 
 // Upper edge of the boundary bin, as the bits of a binary32 time.
 __device__ __forceinline__ unsigned int boundary_edge(const DrawShared& ds) {
@@ -358,15 +354,16 @@ __device__ __noinline__ void draw_collect_all(const Problem& p, const Engine& e,
 }
 
 // ... from the keys the scan saved: every CTA its own, and a share of the last one's where that has other work.
+template <typename Team>
 __device__ __forceinline__ void draw_collect(const Engine& e, const DrawShared& ds, bool spare_last) {
   const Binning bins = binning_of(ds.cut);
   const unsigned int own = ds.saved, more = spare_last ? __ldcg(e.saved + gridDim.x - 1u) : 0u;
   const unsigned long long* mine = e.surv + (size_t)blockIdx.x * e.cap_surv;
   const unsigned long long* its = e.surv + (size_t)(gridDim.x - 1u) * e.cap_surv;
 #pragma unroll 1
-  for (unsigned int i = threadIdx.x; i < own; i += kT) take_winner(e, ds, bins, __ldcg(mine + i));
+  for (unsigned int i = Team::tid(); i < own; i += Team::kN) take_winner(e, ds, bins, __ldcg(mine + i));
 #pragma unroll 1
-  for (unsigned int i = threadIdx.x * (gridDim.x - 1u) + blockIdx.x; i < more; i += kT * (gridDim.x - 1u)) take_winner(e, ds, bins, __ldcg(its + i));
+  for (unsigned int i = Team::tid() * (gridDim.x - 1u) + blockIdx.x; i < more; i += Team::kN * (gridDim.x - 1u)) take_winner(e, ds, bins, __ldcg(its + i));
 }
 
 // Rare: more keys share the boundary bin than there is room for (thousands of tied times).  The grid cuts the bin
@@ -429,21 +426,22 @@ __device__ __noinline__ bool draw_refine(const Problem& p, const Engine& e, Draw
 
 // Selection and collection.  Where the selection needs mending (fewer keys than wanted, or too many that tie) the CTAs
 // that see it say so, and all of them meet in draw_mend behind the next barrier.
-__device__ __forceinline__ void draw_gather(const Problem& p, const Engine& e, DrawShared& ds, unsigned long long t, unsigned int k, bool spare_last) {
+template <typename Team>
+__device__ __forceinline__ void draw_gather(const Problem& p, const Engine& e, DrawShared& ds, unsigned int k, bool spare_last) {
   if (spare_last && gridDim.x > 1 && blockIdx.x == gridDim.x - 1) return;
-  draw_select(e, ds, k);
+  draw_select<Team>(e, ds, k);
   // (a stretch that overflowed is seen by its owner alone: the others' winners are collected all the same, and again)
   const bool too_many = ds.saved > e.cap_surv || (spare_last && blockIdx.x == 0 && __ldcg(e.saved + gridDim.x - 1u) > e.cap_surv);
   if (ds.total < k || ds.bnd_count > (unsigned)e.cap_boundary || ds.cut == 0.f || too_many) {
-    if (threadIdx.x == 0 && (blockIdx.x == 0 || too_many)) e.es->mend = 1;
+    if (Team::tid() == 0 && (blockIdx.x == 0 || too_many)) e.es->mend = 1;
     return;
   }
-  draw_collect(e, ds, spare_last);
+  draw_collect<Team>(e, ds, spare_last);
 }
 
 // (cold) by all CTAs.  False: a barrier gave up.
 __device__ __noinline__ bool draw_mend(const Problem& p, const Engine& e, DrawShared& ds, unsigned char* sm, unsigned long long t, unsigned int k, Grid& g) {
-  draw_select(e, ds, k);
+  draw_select_all(e, ds, k);
   if (!grid_sync(g)) return false;                       // everybody has read the counts and the flag
   if (blockIdx.x == 0 && threadIdx.x == 0) e.es->mend = 0;
   if (ds.total < k) {
@@ -452,7 +450,7 @@ __device__ __noinline__ bool draw_mend(const Problem& p, const Engine& e, DrawSh
     if (!grid_sync(g)) return false;
     draw_scan(p, e, ds, sm, t, false);
     if (!grid_sync(g)) return false;
-    draw_select(e, ds, k);
+    draw_select_all(e, ds, k);
   }
   if (ds.bnd_count > (unsigned)e.cap_boundary && !draw_refine(p, e, ds, sm, t, k, g)) return false;
   for (int b = (int)blockIdx.x * kT + (int)threadIdx.x; b < kHistBins; b += (int)gridDim.x * kT) e.bin_cur[b] = 0u;
@@ -1707,36 +1705,134 @@ __device__ void csc_apply(const Problem& p, int nk, int n_moving, int shift) {
 
 // ------------------------------------------------------------------------------------------------
 // CSC, step 3b: the walk over all candidates with conflict rows on demand (see walk_csc.cu for the scheme: batches of 32
-// unblocked candidates, picked, merged among themselves and decided by every CTA alike; then the kept members against
-// all later unblocked candidates over the grid; one barrier per batch).  Here candidate a belongs to CTA a mod ctas, which
-// brings its candidates' columns into shared memory once per walk: the grid-wide merges then touch no global memory
-// but the mask, where a lane used to fetch a column (two dependent far accesses) per merge -- 18 us in the first batch.
+// unblocked candidates, picked, multiplied with one another and decided by every CTA alike; then the kept members against
+// all later unblocked candidates over the grid; one barrier per batch).  Here 32 consecutive candidates -- a word of the mask
+// -- belong to CTA word mod ctas, which brings their columns into shared memory once per walk and publishes the whole word
+// after every batch: no atomics, and nothing to clear.
+//
+// What bounds a batch is its chain of short steps, so products are not merges of two sorted lists (2 nnz dependent steps each)
+// but look-ups: the rows of the batch's columns go into a hash table in shared memory, each with the mask of the members
+// that have an entry there and their values side by side; a thread that has a pair goes through one column's
+// entries, none of which waits for the one before.  Same products, added in the same order of rows.
+//
+// Once few survive, a batch each for the next 32 of them costs more than all their products: every CTA multiplies its share of
+// the survivors with all of them, and behind one more barrier every CTA settles the rest from the bits.
+//
+// The chain leaves most of the SM's issue slots idle whatever the number of its warps, and the next draw up to the collection of
+// its winners needs nothing else: half the warps walk, the other half draw, with barriers of their own.
+//
+// 10^7 columns of 20 entries, 16,384 candidates of which ~64 are kept: 66 us per round.  With merges, batches of 32 to the end
+// (5.1 of them at 9.7 us) and all warps in both, the scan in the walk's waits and behind it, 101.
 // ------------------------------------------------------------------------------------------------
+constexpr int kWalkWarps = kWalkT / 32;
 constexpr int kBatch = 32;
-constexpr int kColCap = 64;                              // entries of a batch member's column in shared memory (longer: global)
-constexpr int kOwn = 128;                                // candidates a CTA can own (more: their columns stay in global memory)
-constexpr int kHeldEntries = 24;                         // entries of a candidate's column held in registers (longer: merged)
-constexpr int kOwnEntries = 12288;                       // entries of their columns (96 KB)
-static_assert(kMaxWords <= kT && kOwn * 4 <= kT, "a mask word per thread, four threads per own candidate");
+constexpr int kColCap = 64;                              // entries of a batch member's column that the table takes
+constexpr int kRowBits = 12, kRowSlots = 1 << kRowBits;  // of the table: at most half full
+constexpr int kFreeRow = -1;
+constexpr unsigned int kNoSlot = 0xffff;
+constexpr int kOwn = 256;                                // candidates a CTA can hold (more: their columns stay in global memory)
+constexpr int kOwnEntries = 5120;                        // entries of their columns
+constexpr int kRestEntries = kOwnEntries * 3 / 2;
+constexpr int kLast = 512;                               // survivors that are settled at once
+constexpr int kPerMember = kWalkT / kBatch, kEach = kColCap / kPerMember;      // threads of a batch member; its entries per thread
+static_assert(kMaxWords <= 2 * kWalkT && kOwn == kT - kWalkT && kBatch == 4 * kWalkWarps && kBatch * kColCap * 2 <= kRowSlots,
+              "two mask words per walking thread, a held candidate per other thread, four members per warp");
 
 struct DemandShared {
-  unsigned int blocked[kMaxWords];
-  int brow[kBatch][kColCap + 1];
-  float bval[kBatch][kColCap + 1];
-  int pos[kBatch], col[kBatch], len[kBatch];
+  int pos[kBatch], col[kBatch], len[kBatch];             // the batch: position in the list, coefficient, entries
   long long ptr[kBatch];
   double n2[kBatch];
-  unsigned int conf[kBatch];
+  float limit[kBatch];                                   // rho^2 n2
+  unsigned int conf[kBatch];                             // conflicts with earlier members
+  int kept_q[kBatch];                                    // members kept, in order
+  int n_shared[kBatch];                                  // a member's entries in rows of later members
   int wsum[kWarps];
-  unsigned int keep;
-  int m, cursor, kept, examined, done;
-  int batch, mask_at;                                    // batches decided; where the conflicts of the last one go in walk_blocked
-  int own_at[kOwn + 1], own_free[kOwn], n_free;
-  double own_n2[kOwn];
+  int longest, n_vals, n_free;
+  int kept, ok, drawn;                                   // results
+  unsigned int target, draw_target;
+  // rows of the batch's columns
+  __align__(16) int row_key[kRowSlots];
+  __align__(16) uint2 row_rec[kRowSlots];                              // members with an entry in the row (0: slot free), and where their values start
+  float row_val[kBatch * kColCap];
+  __align__(16) uint4 ent[kBatch][kColCap];              // ... those: members of the row, where their values start, the entry's value
+  int survivor[kLast];
+  __align__(16) unsigned int state[2][2][kLast / 32];    // the survivors undecided and kept, in turns
+  // the CTA's words and candidates
+  unsigned int own_word[kMaxWords], own_hit[kMaxWords];
+  int own_at[kOwn + 1], own_free[kOwn], n_met[kOwn];
   long long own_q0[kOwn];
-  int orow[kOwnEntries];
-  float oval[kOwnEntries];
+  double own_n2[kOwn];
+  union {
+    struct {
+      int orow[kOwnEntries];
+      float oval[kOwnEntries];
+      unsigned int omet[kOwnEntries];                    // a candidate's entries in rows of kept members: slot, and entry << 16
+    };
+    struct { int rrow[kRestEntries]; float rval[kRestEntries]; };      // survivors' columns
+  };
 };
+
+__device__ __forceinline__ unsigned int row_hash(int row) { return ((unsigned int)row * 2654435761u) >> (32 - kRowBits); }
+// Slots of rows of the batch's columns; kNoSlot: none of the members in `want` has an entry there (kFreeRow: no row).  Their first
+// places are looked at together.
+template <int kU>
+__device__ __forceinline__ void find_rows(const DemandShared& s, const int (&row)[kU], unsigned int want, unsigned int (&slot)[kU]) {
+  int key[kU];
+#pragma unroll
+  for (int u = 0; u < kU; ++u) { slot[u] = row_hash(row[u]); key[u] = s.row_key[slot[u]]; }
+  bool more;
+  do {                                                   // (other rows in their places)
+    more = false;
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      if (key[u] != row[u] && key[u] != kFreeRow) { slot[u] = (slot[u] + 1u) & (kRowSlots - 1); key[u] = s.row_key[slot[u]]; more = true; }
+  } while (more);
+#pragma unroll
+  for (int u = 0; u < kU; ++u) {
+    const unsigned int members = s.row_rec[slot[u]].x;
+    if (row[u] == kFreeRow || key[u] == kFreeRow || !(members & want)) slot[u] = kNoSlot;
+  }
+}
+// dot + the products of member q's entries with values v of a column in rows of the table (rec: their members, where the members'
+// values start), one after the other.  Each is as many accesses deep whether q has an entry or not, so that they go out together.
+template <int kU>
+__device__ __forceinline__ float add_products(const DemandShared& s, int q, const uint2 (&rec)[kU], const float (&v)[kU], float dot) {
+  float x[kU];
+#pragma unroll
+  for (int u = 0; u < kU; ++u) x[u] = s.row_val[(rec[u].x >> q) & 1u ? rec[u].y + (unsigned)__popc(rec[u].x & ((1u << q) - 1u)) : 0u];
+#pragma unroll
+  for (int u = 0; u < kU; ++u) dot = (rec[u].x >> q) & 1u ? fmaf(x[u], v[u], dot) : dot;
+  return dot;
+}
+// The same over n rows; at(i, &rec, &value) for i < n.  most: the largest n of the warp.
+template <typename At>
+__device__ __forceinline__ float row_products(const DemandShared& s, int q, int n, int most, At&& at) {
+  constexpr int kU = 8;
+  float dot = 0.f;
+#pragma unroll 1
+  for (int i0 = 0; i0 < most; i0 += kU) {
+    uint2 rec[kU];
+    float v[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      rec[u] = make_uint2(0u, 0u); v[u] = 0.f;
+      if (i0 + u < n) at(i0 + u, rec[u], v[u]);
+    }
+    dot = add_products<kU>(s, q, rec, v, dot);
+  }
+  return dot;
+}
+// |x_a^T x_b| >= rho ||x_a|| ||x_b||; FP64 only where the product is near the threshold, or where binary32 does not reach.
+// limit_a: rho^2 ||x_a||^2.
+__device__ __forceinline__ bool in_conflict(float dot, float limit_a, double n2a, double n2b, double rho) {
+  const float y = (float)n2b, limit = limit_a * y, d2 = dot * dot;
+  if (fminf(fminf(limit_a, y), limit) > 1e-30f && limit < 1e37f) {
+    if (d2 < 0.9999f * limit) return false;
+    if (d2 > 1.0001f * limit) return true;
+  }
+  const double den = sqrt(n2a * n2b);
+  return den > 0.0 && fabs((double)dot) >= rho * den;
+}
 
 // x_a^T x_b of two ascending row lists, products added in row order; no branch depends on the data.
 __device__ __forceinline__ float merge_dot(const int* ar, const float* av, int na, const int* br, const float* bv, int nb) {
@@ -1751,218 +1847,503 @@ __device__ __forceinline__ float merge_dot(const int* ar, const float* av, int n
   return dot;
 }
 
-// The columns of all candidates lie where p.walk_cols says (written behind the last barrier's far side).  step(): work for
-// the warps that wait at its barriers.  False: a barrier gave up.
-template <typename Step>
-__device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, const Engine& e, unsigned char* sm, Grid& g, Step&& step) {
+// (cold) A batch with a column longer than the table takes: its pairs, and its kept members against a candidate, by merges.
+__device__ __noinline__ void merge_batch(const Problem& p, DemandShared& s, int m) {
+  const double rho = (double)p.rho;
+  for (int i = threadIdx.x; i < m * m; i += kWalkT) {
+    const int qa = i / m, qb = i - qa * m;
+    if (qa >= qb) continue;
+    const float dot = merge_dot(p.xrow + s.ptr[qa], p.xv + s.ptr[qa], s.len[qa], p.xrow + s.ptr[qb], p.xv + s.ptr[qb], s.len[qb]);
+    if (in_conflict(dot, s.limit[qa], s.n2[qa], s.n2[qb], rho)) atomicOr(&s.conf[qb], 1u << qa);
+  }
+}
+__device__ __noinline__ float merge_columns(const Problem& p, long long qa, int na, long long qb, int nb) {
+  return merge_dot(p.xrow + qa, p.xv + qa, na, p.xrow + qb, p.xv + qb, nb);
+}
+
+__device__ __forceinline__ void walk_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kWalkT) : "memory"); }
+
+// Grid barrier of the walking threads.
+__device__ __forceinline__ bool walk_barrier(DemandShared& s, Grid& g) {
+  g.target += g.n;
+  walk_sync();
+  if (threadIdx.x == 0) s.ok = grid_wait(g);
+  walk_sync();
+  return s.ok != 0;
+}
+
+// The columns of `count` candidates (thread i of kOwn has the i-th) into row / val, one behind the other, as far as there is room.
+// Bound by the lines a load touches, so several threads share a column.  Bar: the threads' barrier.
+template <int kBar>
+__device__ __forceinline__ void hold_columns(const Problem& p, DemandShared& s, int i, int count, const WalkColumn& col, int* row, float* val, int room) {
+  const int lane = threadIdx.x & 31, warp = i >> 5;
+  int* wsum = s.wsum + (kBar == 1 ? 0 : kWalkWarps);
+  int incl = col.n;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) wsum[warp] = incl;
+  asm volatile("bar.sync %0, %1;" ::"n"(kBar), "n"(kOwn) : "memory");
+  int before = 0;
+#pragma unroll
+  for (int k = 0; k < kOwn / 32; ++k) if (k < warp) before += wsum[k];
+  if (i == 0) s.own_at[0] = 0;
+  s.own_at[i + 1] = before + incl;
+  s.own_q0[i] = col.q0; s.own_n2[i] = col.n2;
+  asm volatile("bar.sync %0, %1;" ::"n"(kBar), "n"(kOwn) : "memory");
+#pragma unroll 2
+  for (int k = i >> 3; k < count; k += kOwn / 8) {
+    const int at = s.own_at[k], m = s.own_at[k + 1] - at;
+    const long long from = s.own_q0[k];
+    if (at + m <= room)
+#pragma unroll 4
+      for (int q = i & 7; q < m; q += 8) { row[at + q] = __ldg(p.xrow + from + q); val[at + q] = __ldg(p.xv + from + q); }
+  }
+}
+
+// The rest of a walk: the batch's m members are this CTA's share (cta, cta + ctas, ...) of the `total` candidates that are left
+// (s.survivor, in list order); their conflicts with all earlier ones go to global memory, a row of bits per survivor, and
+// behind a barrier every CTA settles them all: a survivor with a kept earlier neighbour is out, one whose earlier neighbours
+// are all out is kept; a thread holds the rows of two survivors, and the passes are as many as the longest chain of such
+// dependencies.  False: the barrier gave up.
+__device__ __forceinline__ bool settle_rest(const Problem& p, const Problem& sp, DemandShared& s, Grid& g, int total, int m, bool table, int& kept,
+                                            int& examined) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cta = (int)blockIdx.x, n_ctas = (int)gridDim.x;
+  const int W = (total + 31) >> 5, pitch = (W + 3) & ~3;
+  const double rho = (double)p.rho;
+  constexpr int kTogether = 4;                           // members at a time
+  constexpr int kU = 8;                                  // entries of a candidate's column at a time
+  const int behind = cta + (m - 1) * n_ctas;             // candidates before the last member
+  for (int c0 = 0, here; c0 < behind; c0 += here) {      // as many at a time as there is room for
+    const int count = min(behind - c0, kOwn);
+    WalkColumn col = {};
+    if (tid < count) col = p.walk_cols[s.survivor[c0 + tid]];
+    hold_columns<1>(p, s, tid, count, col, s.rrow, s.rval, kRestEntries);
+    walk_sync();
+    here = kOwn;                                         // whole words; of the first one whatever does not fit is read where it is
+    while (here > 32 && s.own_at[here] > kRestEntries) here -= 32;
+    const int c = c0 + tid, at = s.own_at[tid], n = tid < here ? s.own_at[tid + 1] - at : 0, most = __reduce_max_sync(kFull, n);
+    const bool held = at + n <= kRestEntries;
+    if (tid < here) {
+#pragma unroll 1
+      for (int g0 = 0; g0 < m; g0 += kTogether) {
+        float dot[kTogether] = {};
+        if (table) {
+#pragma unroll 1
+          for (int x0 = 0; x0 < most; x0 += kU) {
+            int row[kU];
+            float v[kU];
+            unsigned int sl[kU];
+            uint2 rec[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+              row[u] = kFreeRow; v[u] = 0.f;
+              if (x0 + u < n) {
+                row[u] = held ? s.rrow[at + x0 + u] : __ldg(p.xrow + col.q0 + x0 + u);
+                v[u] = held ? s.rval[at + x0 + u] : __ldg(p.xv + col.q0 + x0 + u);
+              }
+            }
+            find_rows<kU>(s, row, ((1u << kTogether) - 1u) << g0, sl);
+#pragma unroll
+            for (int u = 0; u < kU; ++u) rec[u] = sl[u] != kNoSlot ? s.row_rec[sl[u]] : make_uint2(0u, 0u);
+#pragma unroll
+            for (int y = 0; y < kTogether; ++y)
+              if (g0 + y < m) dot[y] = add_products<kU>(s, g0 + y, rec, v, dot[y]);
+          }
+        } else {
+#pragma unroll
+          for (int y = 0; y < kTogether; ++y)
+            if (g0 + y < m) dot[y] = merge_columns(sp, s.ptr[g0 + y], s.len[g0 + y], col.q0, col.n);
+        }
+#pragma unroll
+        for (int y = 0; y < kTogether; ++y) {
+          const int q = g0 + y, i = cta + q * n_ctas;    // the member's place among the survivors
+          if (q >= m) break;
+          const unsigned int word = __ballot_sync(kFull, c < i && in_conflict(dot[y], s.limit[q], s.n2[q], col.n2, rho));
+          if (lane == 0 && (c >> 5) < W) __stcg(p.conflict + i * pitch + (c >> 5), word);
+        }
+      }
+    }
+    walk_sync();
+  }
+  if (tid < 2 * kLast / 32) {                            // undecided, kept
+    const int w = tid % (kLast / 32), here = total - w * 32;
+    s.state[0][tid / (kLast / 32)][w] = tid >= kLast / 32 || here <= 0 ? 0u : (here >= 32 ? kFull : (1u << here) - 1u);
+  }
+  if (!walk_barrier(s, g)) return false;
+  static_assert(kLast == 2 * kWalkT && kLast / 32 == 2 * kWalkWarps, "two survivors per thread, two words per warp");
+  uint4 row[2][kLast / 128];
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int w = 0; w < kLast / 128; ++w) {
+      const int i = tid + h * kWalkT;
+      row[h][w] = make_uint4(0u, 0u, 0u, 0u);            // (nothing was written behind the survivor's own place)
+      if (i < total && 128 * w < i) {
+        const uint4 r = __ldcg(reinterpret_cast<const uint4*>(p.conflict + i * pitch) + w);
+        auto before = [&](int word) { const int k = i - 128 * w - 32 * word; return k >= 32 ? kFull : (k <= 0 ? 0u : (1u << k) - 1u); };
+        row[h][w] = make_uint4(r.x & before(0), r.y & before(1), r.z & before(2), r.w & before(3));
+      }
+    }
+  unsigned int here = 1u;
+#pragma unroll 1
+  for (int pass = 0; here != 0u; ++pass) {
+    const uint4* und = reinterpret_cast<const uint4*>(s.state[pass & 1][0]);
+    const uint4* kep = reinterpret_cast<const uint4*>(s.state[pass & 1][1]);
+    unsigned int wait[2] = {0u, 0u}, out[2] = {0u, 0u}, left = 0u;
+#pragma unroll
+    for (int w = 0; w < kLast / 128; ++w) {
+      if (4 * w >= W) break;
+      const uint4 u = und[w], k = kep[w];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint4 r = row[h][w];
+        wait[h] |= (r.x & u.x) | (r.y & u.y) | (r.z & u.z) | (r.w & u.w);
+        out[h] |= (r.x & k.x) | (r.y & k.y) | (r.z & k.z) | (r.w & k.w);
+      }
+      left |= u.x | u.y | u.z | u.w;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int w = warp + h * kWalkWarps;
+      const unsigned int mine = s.state[pass & 1][0][w];
+      const unsigned int gone = __ballot_sync(kFull, out[h] != 0u) & mine, fresh = __ballot_sync(kFull, out[h] == 0u && wait[h] == 0u) & mine;
+      if (lane == 0) {
+        s.state[(pass + 1) & 1][0][w] = mine & ~(gone | fresh);
+        s.state[(pass + 1) & 1][1][w] = s.state[pass & 1][1][w] | fresh;
+      }
+    }
+    here = left;
+    walk_sync();
+  }
+  // (the last pass changed nothing: both copies hold the kept ones)
+  const int room = p.n_keep - kept;
+  int before[2] = {0, 0}, all = 0;
+#pragma unroll
+  for (int w = 0; w < kLast / 32; ++w) {
+    const int c = __popc(s.state[0][1][w]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) if (w < warp + h * kWalkWarps) before[h] += c;
+    all += c;
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const unsigned int word = s.state[0][1][warp + h * kWalkWarps];
+    const int r = before[h] + __popc(word & ((1u << lane) - 1u));
+    if (((word >> lane) & 1u) && r < room) {             // stop exactly at P
+      const int at = s.survivor[tid + h * kWalkT];
+      if (r == room - 1) s.n_free = at;
+      if ((kept + r) % n_ctas == cta) { p.kept[kept + r] = p.cand[at]; p.kept_pos[kept + r] = at; }
+    }
+  }
+  walk_sync();
+  if (all >= room) examined = s.n_free + 1;
+  kept += min(all, room);
+  return true;
+}
+
+// The columns of all candidates lie where p.walk_cols says (written behind the last barrier's far side).  draw(): what the other
+// threads do meanwhile, with the grid barrier g_draw; false: it gave up.  Every CTA leaves the places of the kept list that it
+// owns (a mod ctas) and, in *n_kept, their number.  False: a barrier gave up.
+template <typename Draw>
+__device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, const Problem& sp, const Engine& e, unsigned char* sm, Grid& g, Grid& g_draw, int* n_kept,
+                                                   Draw&& draw) {
   DemandShared& s = *reinterpret_cast<DemandShared*>(sm);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int cta = (int)blockIdx.x, n_ctas = (int)gridDim.x, n = p.n_cand, W = (n + 31) >> 5;
-  const double rho = (double)p.rho;
+  // this CTA's words of the mask: cta, cta + n_ctas, ...; its k-th candidate is bit k & 31 of the (k / 32)-th of them
+  const int own_words = W > cta ? (W - cta + n_ctas - 1) / n_ctas : 0, n_own = own_words * 32, n_here = min(n_own, kOwn);
+  auto own_index = [&](int k) { return ((cta + (k >> 5) * n_ctas) << 5) | (k & 31); };
   __syncthreads();
-  for (int w = tid; w < W; w += kT) s.blocked[w] = 0u;
-  if (cta == 0) for (int w = tid; w < kWalkMasks * p.mask_words; w += kT) p.walk_blocked[w] = 0u;
-  if (tid == 0) { s.cursor = 0; s.kept = 0; s.examined = n; s.done = 0; s.batch = 0; }
-  // this CTA's candidates: cta, cta + n_ctas, ...; own_at: where their entries start in orow / oval
-  const int n_own = n > cta ? (n - cta + n_ctas - 1) / n_ctas : 0;
-  const int n_here = min(n_own, kOwn);
-  // (kOwn threads find the columns, then four threads per candidate bring the entries: two far accesses in all)
-  {
-    long long q0 = 0;
-    int cnt = 0;
-    if (tid < n_here) {
-      const WalkColumn col = p.walk_cols[cta + tid * n_ctas];
-      q0 = col.q0; cnt = col.n;
-      s.own_n2[tid] = col.n2;
-    }
-    int incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(kFull, incl, o);
-      if (lane >= o) incl += v;
-    }
-    if (lane == 31) s.wsum[warp] = incl;
-    __syncthreads();
-    int before = 0;
-    for (int k = 0; k < warp; ++k) before += s.wsum[k];
-    if (tid == 0) s.own_at[0] = 0;
-    if (tid < n_here) { s.own_at[tid + 1] = before + incl; s.own_q0[tid] = q0; }
-    __syncthreads();
-    const int k = tid >> 2;
-    if (k < n_here) {
-      const int at = s.own_at[k], m = s.own_at[k + 1] - at;
-      const long long from = s.own_q0[k];
-      if (at + m <= kOwnEntries)
-#pragma unroll 4
-        for (int q = tid & 3; q < m; q += 4) { s.orow[at + q] = __ldg(p.xrow + from + q); s.oval[at + q] = __ldg(p.xv + from + q); }
-    }
-  }
-  if (!grid_sync_busy(g, step)) return false;            // the masks in global memory are clear
-
-  while (true) {
-    // ---- A: the next <= 32 unblocked candidates at or after the cursor ----
+  if (warp >= kWalkWarps) {
+    for (int w = tid - kWalkT; w < own_words; w += kT - kWalkT) s.own_word[w] = s.own_hit[w] = 0u;
     {
-      const int cur = s.cursor, first = tid << 5;
-      unsigned int f = 0u;
-      if (tid < W && first + 32 > cur) {
-        f = ~s.blocked[tid];
-        if (first < cur) f &= kFull << (cur - first);
-        if (first + 32 > n) f &= kFull >> (first + 32 - n);
-      }
-      const int c = __popc(f);
-      int incl = c;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(kFull, incl, o);
-        if (lane >= o) incl += v;
-      }
-      if (lane == 31) s.wsum[warp] = incl;
-      __syncthreads();
-      int before = 0, total = 0;
-#pragma unroll
-      for (int k = 0; k < kWarps; ++k) { const int v = s.wsum[k]; if (k < warp) before += v; total += v; }
-      for (int idx = before + incl - c; f != 0u && idx < kBatch; f &= f - 1u, ++idx) s.pos[idx] = first + __ffs((int)f) - 1;
-      if (tid == 0) s.m = min(kBatch, total);
-      if (tid < kBatch) s.conf[tid] = 0u;
+      const int i = tid - kWalkT;
+      WalkColumn col = {};
+      if (i < n_here && own_index(i) < n) col = p.walk_cols[own_index(i)];
+      hold_columns<2>(p, s, i, n_here, col, s.orow, s.oval, kOwnEntries);
     }
-    __syncthreads();
-    const int m = s.m;
-    if (m == 0) break;                                   // list exhausted (the same in every CTA)
-    // ---- B: the members' columns, sixteen threads each, then the pairs among them, one per thread ----
-    {
-      const int q = tid >> 4, l = tid & 15;
-      if (q < m) {
-        const WalkColumn col = p.walk_cols[s.pos[q]];
-        if (l == 0) { s.col[q] = col.j; s.ptr[q] = col.q0; s.len[q] = col.n; s.n2[q] = col.n2; }
-        if (col.n <= kColCap)
-          for (int i = l; i < col.n; i += 16) { s.brow[q][i] = __ldg(p.xrow + col.q0 + i); s.bval[q][i] = __ldg(p.xv + col.q0 + i); }
-      }
-    }
-    __syncthreads();
-    if (tid < m * (m - 1) / 2) {                         // pair number -> (qa, qb), qa < qb
-      int qb = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)tid)) * 0.5f);
-      while (qb * (qb - 1) / 2 > tid) --qb;
-      while ((qb + 1) * qb / 2 <= tid) ++qb;
-      const int qa = tid - qb * (qb - 1) / 2;
-      const int na = s.len[qa], nb = s.len[qb];
-      float dot;
-      if (na <= kColCap && nb <= kColCap) {
-        dot = merge_dot(s.brow[qa], s.bval[qa], na, s.brow[qb], s.bval[qb], nb);
-      } else {
-        const int* ar = na <= kColCap ? s.brow[qa] : p.xrow + s.ptr[qa];
-        const float* av = na <= kColCap ? s.bval[qa] : p.xv + s.ptr[qa];
-        const int* br = nb <= kColCap ? s.brow[qb] : p.xrow + s.ptr[qb];
-        const float* bv = nb <= kColCap ? s.bval[qb] : p.xv + s.ptr[qb];
-        dot = merge_dot(ar, av, na, br, bv, nb);
-      }
-      const double den = sqrt(s.n2[qa] * s.n2[qb]);
-      if (den > 0.0 && fabs((double)dot) >= rho * den) atomicOr(&s.conf[qa], 1u << qb);
-    }
-    __syncthreads();
-    // ---- C: decide the batch (warp 0, lane = member; the same in every CTA) ----
-    if (warp == 0) {
-      const unsigned int mine = s.conf[lane];            // conflicts with later members only
-      unsigned int und = m >= 32 ? kFull : ((1u << m) - 1u), keep = 0u, fresh = 0u;
-      for (int pass = 0; pass < kBatch && und != 0u; ++pass) {
-        if (pass > 0) und &= ~__reduce_or_sync(kFull, ((fresh >> lane) & 1u) ? mine : 0u);
-        fresh = und & ~__reduce_or_sync(kFull, ((und >> lane) & 1u) ? mine : 0u);
-        keep |= fresh;
-        und &= ~fresh;
-      }
-      const int nk = s.kept, room = p.n_keep - nk;
-      bool done = false;
-      if (__popc(keep) >= room) {                        // stop exactly at P: drop the surplus from the back
-        while (__popc(keep) > room) keep &= ~(1u << (31 - __clz((int)keep)));
-        done = true;
-      }
-      if (cta == 0 && ((keep >> lane) & 1u)) {
-        const int r = nk + __popc(keep & ((1u << lane) - 1u));
-        p.kept[r] = s.col[lane];
-        p.kept_pos[r] = s.pos[lane];
-      }
-      if (lane == 0) {
-        s.keep = keep;
-        s.kept = nk + __popc(keep);
-        s.cursor = s.pos[m - 1] + 1;
-        s.mask_at = walk_mask_at((unsigned)s.batch, p.mask_words);
-        s.batch += 1;
-        s.n_free = 0;
-        if (done) { s.examined = s.pos[31 - __clz((int)keep)] + 1; s.done = 1; }
-      }
-    }
-    __syncthreads();
-    if (s.done) break;                                   // P kept: what they block no longer matters
-    // ---- D: the kept members against this CTA's later unblocked candidates ----
-    {
-      const unsigned int keep = s.keep;
-      const int n_new = __popc(keep), first_pos = s.pos[__ffs((int)keep) - 1];
-      for (int k0 = 0; k0 < n_own; k0 += kOwn) {         // (a turn of at most kOwn candidates; one turn as a rule)
-        if (k0 > 0) { __syncthreads(); if (tid == 0) s.n_free = 0; __syncthreads(); }
-        if (tid < kOwn && k0 + tid < n_own) {
-          const int b = cta + (k0 + tid) * n_ctas;
-          if (b > first_pos && !((s.blocked[b >> 5] >> (b & 31)) & 1u)) s.own_free[atomicAdd(&s.n_free, 1)] = k0 + tid;
-        }
-        __syncthreads();
-        // A team of threads per candidate, each with a share of the members.  A thread holds its candidate's column in
-        // registers and compares every entry of a member's with all of it: no step waits for the one before, where a merge
-        // of two sorted lists is 2 nnz dependent steps.
-        const int n_free = s.n_free, teams = n_free > 0 ? max(1, min(n_new, kT / n_free)) : 1;
-        const int c = tid / teams;
-        if (c < n_free) {
-          const int k = s.own_free[c], b = cta + k * n_ctas;
-          const bool here = k < n_here && s.own_at[k + 1] <= kOwnEntries;
-          const int at = here ? s.own_at[k] : 0, nb = here ? s.own_at[k + 1] - at : 0;
-          const bool held = here && nb <= kHeldEntries;
-          int rb[kHeldEntries];
-          float vb[kHeldEntries];
-          if (held) {
-#pragma unroll
-            for (int i = 0; i < kHeldEntries; ++i) { rb[i] = i < nb ? s.orow[at + i] : 0x7fffffff; vb[i] = i < nb ? s.oval[at + i] : 0.f; }
-          }
-          for (int y = tid - c * teams; y < n_new; y += teams) {
-            unsigned int rest = keep;
-            for (int z = y; z > 0; --z) rest &= rest - 1u;
-            const int q = __ffs((int)rest) - 1;
-            if (s.pos[q] >= b) continue;                 // the member comes later in the list: it cannot block b
-            const int na = s.len[q];
-            float dot = 0.f;
-            double n2b;
-            if (held && na <= kColCap) {
-              n2b = s.own_n2[k];
+    asm volatile("bar.arrive 3, %0;" ::"n"(kT) : "memory");
+    const bool drawn = draw();
+    if (tid == kWalkT) { s.drawn = drawn; s.draw_target = g_draw.target; }
+  } else {
+    const double rho = (double)p.rho;
+    for (int i = tid; i < kRowSlots / 4; i += kWalkT) reinterpret_cast<int4*>(s.row_key)[i] = make_int4(kFreeRow, kFreeRow, kFreeRow, kFreeRow);
+    for (int i = tid; i < kRowSlots / 2; i += kWalkT) reinterpret_cast<uint4*>(s.row_rec)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid == 0) { s.longest = 0; s.n_vals = 0; s.n_free = 0; }
+    int cursor = 0, kept = 0, examined = n, mask_at = 0;
+    bool ok = true, held = false;
 #pragma unroll 1
-              for (int i = 0; i < na; ++i) {
-                const int ra = s.brow[q][i];
-                const float va = s.bval[q][i];
+    for (unsigned int batch = 0u;; ++batch) {
+      // ---- A: the next <= 32 unblocked candidates at or after the cursor ----
+      int total = n;
+      bool last = false;
+      if (batch == 0u) {
+        if (tid < kBatch) s.pos[tid] = tid;
+      } else {
+        const int first = tid << 6;
+        unsigned int f[2] = {0u, 0u};
+        if (first + 64 > cursor && first < n) {
+          const uint2 b = __ldcg(reinterpret_cast<const uint2*>(p.walk_blocked + mask_at) + tid);
+          f[0] = ~b.x; f[1] = ~b.y;
 #pragma unroll
-                for (int j = 0; j < kHeldEntries; ++j) dot = rb[j] == ra ? fmaf(va, vb[j], dot) : dot;
-              }
-            } else if (here && na <= kColCap) {
-              n2b = s.own_n2[k];
-              dot = merge_dot(s.brow[q], s.bval[q], na, s.orow + at, s.oval + at, nb);
-            } else {
-              const WalkColumn cb = p.walk_cols[b];
-              n2b = cb.n2;
-              const int* ar = na <= kColCap ? s.brow[q] : p.xrow + s.ptr[q];
-              const float* av = na <= kColCap ? s.bval[q] : p.xv + s.ptr[q];
-              dot = merge_dot(ar, av, na, p.xrow + cb.q0, p.xv + cb.q0, cb.n);
+          for (int u = 0; u < 2; ++u) {
+            const int at = first + 32 * u;
+            if (at + 32 <= cursor || at >= n) f[u] = 0u;
+            else {
+              if (at < cursor) f[u] &= kFull << (cursor - at);
+              if (at + 32 > n) f[u] &= kFull >> (at + 32 - n);
             }
-            const double den = sqrt(s.n2[q] * n2b);
-            if (den > 0.0 && fabs((double)dot) >= rho * den) { atomicOr(p.walk_blocked + s.mask_at + (b >> 5), 1u << (b & 31)); break; }
           }
         }
+        const int c = __popc(f[0]) + __popc(f[1]);
+        int incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_up_sync(kFull, incl, o);
+          if (lane >= o) incl += v;
+        }
+        if (lane == 31) s.wsum[warp] = incl;
+        walk_sync();
+        int idx = incl - c;
+        total = 0;
+#pragma unroll
+        for (int k = 0; k < kWalkWarps; ++k) { const int v = s.wsum[k]; if (k < warp) idx += v; total += v; }
+        if (total == 0) break;                           // list exhausted (the same in every CTA)
+        last = total > kBatch && total <= kLast && total <= n_ctas * kBatch;
+        int* list = last ? s.survivor : s.pos;
+        const int most = last ? kLast : kBatch;
+#pragma unroll 1
+        for (; (f[0] | f[1]) != 0u && idx < most; ++idx) {
+          const int u = f[0] != 0u ? 0 : 1;
+          const unsigned int x = u ? f[1] : f[0];
+          list[idx] = first + 32 * u + __ffs((int)x) - 1;
+          if (u) f[1] &= f[1] - 1u; else f[0] &= f[0] - 1u;
+        }
+      }
+      // (last: the members are this CTA's share of the survivors)
+      const int m = !last ? min(kBatch, total) : (total > cta ? (total - cta + n_ctas - 1) / n_ctas : 0);
+      walk_sync();
+      // ---- B: the members' rows into the table, kPerMember threads each ----
+      const int q = tid / kPerMember, l = tid % kPerMember;
+      unsigned int slot[kEach];
+      float val[kEach];
+      {
+        WalkColumn col = {};
+        if (q < m) col = p.walk_cols[last ? s.survivor[cta + q * n_ctas] : s.pos[q]];
+        if (l == 0) {
+          s.col[q] = col.j; s.ptr[q] = col.q0; s.n2[q] = col.n2; s.limit[q] = (float)(rho * rho * col.n2); s.len[q] = col.n; s.conf[q] = 0u;
+          if (col.n > kColCap) s.longest = col.n;        // (any of them will do)
+        }
+        const int len = min(col.n, kColCap), turns = (__reduce_max_sync(kFull, len) + kPerMember - 1) / kPerMember;
+        int row[kEach], key[kEach];
+#pragma unroll
+        for (int u = 0; u < kEach; ++u) {
+          row[u] = kFreeRow; val[u] = 0.f; slot[u] = kNoSlot;
+          if (l + kPerMember * u < len) { row[u] = __ldg(p.xrow + col.q0 + l + kPerMember * u); val[u] = __ldg(p.xv + col.q0 + l + kPerMember * u); }
+        }
+#pragma unroll
+        for (int u = 0; u < kEach; ++u) {                // (all of them under way together; another row in the place is rare)
+          if (u >= turns) break;
+          if (row[u] != kFreeRow) { slot[u] = row_hash(row[u]); key[u] = atomicCAS(&s.row_key[slot[u]], kFreeRow, row[u]); }
+        }
+#pragma unroll
+        for (int u = 0; u < kEach; ++u) {
+          if (u >= turns) break;
+          if (row[u] == kFreeRow) continue;
+#pragma unroll 1
+          while (key[u] != kFreeRow && key[u] != row[u]) {
+            slot[u] = (slot[u] + 1u) & (kRowSlots - 1);
+            key[u] = atomicCAS(&s.row_key[slot[u]], kFreeRow, row[u]);
+          }
+          atomicOr(&s.row_rec[slot[u]].x, 1u << q);
+        }
+      }
+      walk_sync();
+      const bool table = s.longest == 0;                 // (the same in every CTA)
+      if (table) {
+        // the values of a row side by side, in the order of the members: its first member takes the places
+        unsigned int members[kEach];
+        int want = 0;
+#pragma unroll
+        for (int u = 0; u < kEach; ++u) {
+          members[u] = slot[u] != kNoSlot ? s.row_rec[slot[u]].x : 0u;
+          if ((members[u] & ((1u << q) - 1u)) == 0u) want += __popc(members[u]);
+        }
+        int incl = want;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_up_sync(kFull, incl, o);
+          if (lane >= o) incl += v;
+        }
+        int at = 0;
+        if (lane == 31) at = atomicAdd(&s.n_vals, incl);
+        at = __shfl_sync(kFull, at, 31) + incl - want;
+#pragma unroll
+        for (int u = 0; u < kEach; ++u)
+          if (members[u] != 0u && (members[u] & ((1u << q) - 1u)) == 0u) { s.row_rec[slot[u]].y = (unsigned)at; at += __popc(members[u]); }
+        walk_sync();
+        int n_shared = 0;
+        const unsigned int group = ((1u << kPerMember) - 1u) << (lane & ~(kPerMember - 1));
+#pragma unroll
+        for (int u = 0; u < kEach; ++u) {
+          if (!__any_sync(kFull, members[u] != 0u)) break;
+          const unsigned int start = members[u] != 0u ? s.row_rec[slot[u]].y : 0u;
+          if (members[u] != 0u) s.row_val[start + (unsigned)__popc(members[u] & ((1u << q) - 1u))] = val[u];
+          const bool later = (members[u] >> q) > 1u;
+          const unsigned int mine = __ballot_sync(kFull, later) & group;
+          if (later) s.ent[q][n_shared + __popc(mine & ((1u << lane) - 1u))] = make_uint4(members[u], start, __float_as_uint(val[u]), 0u);
+          n_shared += __popc(mine);
+        }
+        if (l == 0) s.n_shared[q] = n_shared;
+        walk_sync();
+        // the pairs among them, one per lane: member w with those behind it and member 31 - w likewise
+        if (!last) {
+#pragma unroll 1
+          for (int w = warp; w < kBatch / 2; w += kWalkWarps) {
+            const int a = lane > w ? w : kBatch - 1 - w, b = lane > w ? lane : kBatch - 1 - lane;
+            const float dot = row_products(s, b, lane == w ? 0 : s.n_shared[a], max(s.n_shared[w], s.n_shared[kBatch - 1 - w]),
+                                           [&](int i, uint2& rec, float& v) { const uint4 en = s.ent[a][i]; rec = make_uint2(en.x, en.y); v = __uint_as_float(en.z); });
+            if (lane != w && b < m && in_conflict(dot, s.limit[a], s.n2[a], s.n2[b], rho)) atomicOr(&s.conf[b], 1u << a);
+          }
+        }
+      } else if (!last) {
+        merge_batch(sp, s, m);
+      }
+      if (last) {
+        ok = settle_rest(p, sp, s, g, total, m, table, kept, examined);
+        break;
+      }
+      walk_sync();
+      // ---- C: decide the batch (lane = member; the same in every warp and CTA) ----
+      unsigned int keep = 0u;
+      {
+        const unsigned int earlier = s.conf[lane];
+        unsigned int und = m >= 32 ? kFull : ((1u << m) - 1u);
+#pragma unroll 1
+        while (und != 0u) {                              // (the first undecided one is kept every time)
+          const unsigned int fresh = __ballot_sync(kFull, (earlier & (und | keep)) == 0u) & und;
+          keep |= fresh;
+          und &= ~(fresh | __ballot_sync(kFull, (earlier & fresh) != 0u));
+        }
+      }
+      const int room = p.n_keep - kept;
+      const bool done = __popc(keep) >= room;            // stop exactly at P: drop the surplus from the back
+      while (__popc(keep) > room) keep &= ~(1u << (31 - __clz((int)keep)));
+      if (warp < 2 && ((keep >> lane) & 1u)) {
+        const int r = __popc(keep & ((1u << lane) - 1u));
+        if (warp == 0) {
+          s.kept_q[r] = lane;
+        } else if ((kept + r) % n_ctas == cta) {
+          p.kept[kept + r] = s.col[lane];
+          p.kept_pos[kept + r] = s.pos[lane];
+        }
+      }
+      const int n_new = __popc(keep);
+      kept += n_new;
+      cursor = s.pos[m - 1] + 1;
+      if (done) examined = s.pos[31 - __clz((int)keep)] + 1;
+      if (done || total <= kBatch) break;                // P kept: what they block no longer matters; or nobody comes later
+      // ---- D: the kept members against this CTA's later unblocked candidates ----
+      mask_at = walk_mask_at(batch, p.mask_words);
+      if (!held) { held = true; asm volatile("bar.sync 3, %0;" ::"n"(kT) : "memory"); }        // their columns are there
+      for (int k0 = 0; k0 < n_own; k0 += kOwn) {         // (a turn of at most kOwn candidates; one turn as a rule)
+        if (k0 > 0) { walk_sync(); if (tid == 0) s.n_free = 0; walk_sync(); }
+        for (int k = k0 + tid; k < min(n_own, k0 + kOwn); k += kWalkT) {
+          const int b = own_index(k);
+          if (b < n && b >= cursor && !((s.own_word[k >> 5] >> (k & 31)) & 1u)) s.own_free[atomicAdd(&s.n_free, 1)] = k;
+        }
+        walk_sync();
+        const int n_free = s.n_free;
+        if (table && k0 == 0) {                          // their entries in rows of kept members
+          int share = 5;                                 // threads per candidate
+          while (share > 0 && (n_free << share) > kWalkT) --share;
+          const int c = tid >> share, sub = tid & ((1 << share) - 1);
+          const unsigned int group = (share == 5 ? kFull : ((1u << (1 << share)) - 1u)) << (lane - sub);
+          int k = 0, from = 0, end = 0, met = 0;
+          if (c < n_free) {
+            k = s.own_free[c]; from = s.own_at[k]; end = s.own_at[k + 1];
+            if (end > kOwnEntries) end = from;
+          }
+#pragma unroll 1
+          for (int i0 = from + sub; __any_sync(kFull, i0 < end + sub); i0 += 4 << share) {
+            int row[4];
+            unsigned int sl[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) row[u] = i0 + (u << share) < end ? s.orow[i0 + (u << share)] : kFreeRow;
+            find_rows<4>(s, row, keep, sl);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const unsigned int mine = __ballot_sync(kFull, sl[u] != kNoSlot) & group;
+              if (sl[u] != kNoSlot) s.omet[from + met + __popc(mine & ((1u << lane) - 1u))] = sl[u] | (unsigned)(i0 + (u << share) - from) << 16;
+              met += __popc(mine);
+            }
+          }
+          if (c < n_free && sub == 0) s.n_met[k] = met;
+          walk_sync();
+        }
+        const unsigned int per = ((1u << 20) + (unsigned)n_new - 1u) / (unsigned)n_new;        // i / n_new = i per >> 20 (i < 2^13, n_new <= 32)
+        for (int i = tid; i < n_free * n_new; i += kWalkT) {
+          const int c = (int)((unsigned)i * per >> 20), qk = s.kept_q[i - c * n_new], k = s.own_free[c];
+          float dot = 0.f;
+          double n2b;
+          if (table && k < kOwn && s.own_at[k + 1] <= kOwnEntries) {
+            n2b = s.own_n2[k];
+            const int met = s.n_met[k], from = s.own_at[k];
+            dot = row_products(s, qk, met, met, [&](int x, uint2& rec, float& v) {
+              const unsigned int en = s.omet[from + x];
+              rec = s.row_rec[en & 0xffffu]; v = s.oval[from + (int)(en >> 16)];
+            });
+          } else if (table) {                            // (no room for its column)
+            const WalkColumn cb = p.walk_cols[own_index(k)];
+            n2b = cb.n2;
+            for (int x = 0; x < cb.n; ++x) {
+              const int row[1] = {__ldg(p.xrow + cb.q0 + x)};
+              unsigned int sl[1];
+              find_rows<1>(s, row, 1u << qk, sl);
+              const uint2 rec[1] = {s.row_rec[sl[0] != kNoSlot ? sl[0] : 0u]};
+              const float v[1] = {__ldg(p.xv + cb.q0 + x)};
+              if (sl[0] != kNoSlot) dot = add_products<1>(s, qk, rec, v, dot);
+            }
+          } else {
+            const WalkColumn cb = p.walk_cols[own_index(k)];
+            n2b = cb.n2;
+            dot = merge_columns(sp, s.ptr[qk], s.len[qk], cb.q0, cb.n);
+          }
+          if (in_conflict(dot, s.limit[qk], s.n2[qk], n2b, rho)) atomicOr(&s.own_hit[k >> 5], 1u << (k & 31));
+        }
+      }
+      walk_sync();
+      for (int w = tid; w < own_words; w += kWalkT) {    // the words as they are now
+        const unsigned int v = s.own_word[w] | s.own_hit[w];
+        s.own_word[w] = v;
+        s.own_hit[w] = 0u;
+        p.walk_blocked[mask_at + cta + w * n_ctas] = v;
+      }
+      // the table as the next batch expects it
+#pragma unroll
+      for (int u = 0; u < kEach; ++u)
+        if (slot[u] != kNoSlot) { s.row_key[slot[u]] = kFreeRow; s.row_rec[slot[u]].x = 0u; }
+      if (tid == 0) { s.longest = 0; s.n_vals = 0; s.n_free = 0; }
+      if (!(ok = walk_barrier(s, g))) break;
+    }
+    if (!held) asm volatile("bar.sync 3, %0;" ::"n"(kT) : "memory");
+    if (tid == 0) {
+      s.kept = kept; s.ok = ok; s.target = g.target;
+      if (cta == 0 && ok) {
+        EngineState* es = e.es;
+        es->n_kept = kept; es->n_examined = examined; es->walk_open = 0;
+        if (es->avoid > 0) es->avoid -= 1;
+        if (e.window < n) es->skip_window = kept == p.n_keep && examined <= e.window ? 0 : 1;
       }
     }
-    if (!grid_sync_busy(g, step)) return false;
-    for (int w = tid; w < W; w += kT) s.blocked[w] |= __ldcg(p.walk_blocked + s.mask_at + w);
-    __syncthreads();
   }
-  if (cta == 0 && tid == 0) {
-    EngineState* es = e.es;
-    es->n_kept = s.kept; es->n_examined = s.examined; es->walk_open = 0;
-    if (es->avoid > 0) es->avoid -= 1;
-    if (e.window < n) es->skip_window = s.kept == p.n_keep && s.examined <= e.window ? 0 : 1;
-  }
-  return true;
+  __syncthreads();
+  g.target = s.target; g_draw.target = s.draw_target;
+  *n_kept = s.kept;
+  return s.ok != 0 && s.drawn != 0;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -2016,6 +2397,8 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
   }
   Grid g;
   g.count = &e.es->bar_count; g.target = 0u; g.n = gridDim.x; g.limit = p.wait_limit ? p.wait_limit : kSpinLimit; g.status = &p.st->status;
+  Grid g_draw = g;                                       // (CSC: of the threads that draw while the others walk)
+  g_draw.count = &e.es->draw_bar_count;
   EngineState* es = e.es;
   unsigned long long t = p.st->round;
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(sm);
@@ -2064,7 +2447,8 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
       const bool during_walk = !kDense && real && !window && !scanned;
       if (!scanned && !during_walk) { draw_scan(p, e, ds, sm, td, true); scanned = true; }
       if (kDense) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // (the Gram's operands come in over it)
-      if (!(during_walk && !(p.flags & STRADS_FLAG_DYNAMIC_DEPS)) && !(ok = grid_sync(g))) break;      // (the walk begins with a barrier)
+      // (the walk needs nothing of what is before it but the norms that follow beta and delta)
+      if (!(!kDense && real && !window && !(p.flags & STRADS_FLAG_DYNAMIC_DEPS)) && !(ok = grid_sync(g))) break;
       if (kDense && real && !no_filter) {
         unsigned int* amb = &es->amb_count[attempts & 1u];
         if (cta == 0 && tid == 0) es->amb_count[(attempts + 1u) & 1u] = 0u;
@@ -2094,7 +2478,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
       }
       // the winners of the draw: by every CTA but the one that walks; CSC in step 3 as well, unless there is none
       const bool csc_window = !kDense && real && window && !no_filter;
-      if (!collected && !csc_window && !during_walk) { draw_gather(p, e, ds, td, k, spare); collected = true; }
+      if (!collected && !csc_window && !during_walk) { draw_gather<AllThreads>(p, e, ds, k, spare); collected = true; }
       if (!kDense && real) {
         if (!window) {
           unsigned char* sm_scan = sm + sizeof(DemandShared);
@@ -2102,23 +2486,28 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
           const float cut = during_walk ? scan_open(e, ds, sm_scan, true) : 0.f;
           const Binning bins = binning_of(cut);
           const WeightForm wf = weight_form(p);
-          // (the first warp waits at the barriers: with a share of its own it went through it alone afterwards, 14 us of 10^7
-          // coefficients' 18)
-          WarpScan scan = begin_scan(cut, scan_queue(sm_scan), (warp - 1) * n_ctas + cta, (kWarps - 1) * n_ctas);
-          if (warp == 0) scan.next = LLONG_MAX / 2;
-          auto step = [&]() {
-            return during_walk && scan_step(p, td, wf, scan, [&](unsigned long long key, bool on) { scan_found(e, ds, sh, bins, key, on); });
-          };
-          if (!(ok = csc_walk_on_demand(p, e, sm, g, step))) break;
-          if (during_walk) {
+          auto draw = [&]() {
+            if (!during_walk) return true;
+            WarpScan scan = begin_scan(cut, scan_queue(sm_scan), (warp - kWalkWarps) * n_ctas + cta, (kWarps - kWalkWarps) * n_ctas);
 #pragma unroll 1
-            while (step()) {}
-            scan_close(e, ds, sm_scan);
-          }
-          if (!(ok = grid_sync(g))) break;
-          if (during_walk) { draw_gather(p, e, ds, td, k, false); scanned = collected = true; }
+            while (scan_step(p, td, wf, scan, [&](unsigned long long key, bool on) { scan_found(e, ds, sh, bins, key, on); })) {}
+            scan_close<OtherThreads>(e, ds, sm_scan);
+            __shared__ int s_over;
+            g_draw.target += g_draw.n;
+            OtherThreads::sync();
+            if (OtherThreads::tid() == 0) s_over = grid_wait(g_draw);
+            OtherThreads::sync();
+            if (!s_over) return false;
+            draw_gather<OtherThreads>(p, e, ds, k, false);
+            return true;
+          };
+          int walked = 0;
+          if (!(ok = csc_walk_on_demand(p, sp, e, sm, g, g_draw, &walked, draw))) break;
+          if (during_walk) scanned = collected = true;
+          csc_products(p, e, ts, sm, walked, true, false, t + 1, draws);
+        } else {
+          csc_products(p, e, ts, sm, n, false, csc_window, t + 1, draws);
         }
-        csc_products(p, e, ts, sm, window ? n : es->n_kept, !window, csc_window, t + 1, draws);
       }
       if (!(ok = grid_sync(g))) break;
       if (!real || no_filter) break;
@@ -2143,7 +2532,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
           }
         }
         csc_clear_buckets(p, n);
-        if (!collected) { draw_gather(p, e, ds, td, k, true); collected = true; spare = true; }
+        if (!collected) { draw_gather<AllThreads>(p, e, ds, k, true); collected = true; spare = true; }
         if (!(ok = grid_sync(g))) break;
         if (!es->walk_open) break;
         csc_enter(p, e, n_total, false);
@@ -2186,7 +2575,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
   }
   if (!ok) return;
   if (tid == 0 && atomicInc(&e.es->exit_count, gridDim.x - 1u) == gridDim.x - 1u) {
-    e.es->bar_count = 0u;
+    e.es->bar_count = 0u; e.es->draw_bar_count = 0u;
     if (kDense) { e.es->amb_count[0] = 0u; e.es->amb_count[1] = 0u; }
   }
 }
@@ -2256,7 +2645,7 @@ __device__ __forceinline__ bool draw_alone(const Problem& p, const Engine& e, Dr
   for (int b = tid; b < kHistBins; b += kT)
     if (sh[b]) atomicAdd(&e.hist[b], sh[b]);
   if (!grid_sync(g, stall != 0 && blockIdx.x == 0)) return false;
-  draw_select(e, ds, (unsigned)p.n_cand);
+  draw_select<AllThreads>(e, ds, (unsigned)p.n_cand);
   if (ds.bnd_count > (unsigned)e.cap_boundary && !draw_refine(sp, se, ds, sm, t, (unsigned)p.n_cand, g)) return false;
   if (kept_groups > 0) {
     for (int k = 0; k < turn; ++k)

@@ -7,6 +7,7 @@ namespace strads {
 // Device-resident state of the round engine, in the workspace.  Zero before the first launch.
 struct EngineState {
   unsigned int bar_count;       // grid barrier: arrivals of the launch in flight
+  unsigned int draw_bar_count;  // ... of the threads that draw while others walk
   unsigned int exit_count;      // CTAs of the launch that have left
   float t_cut;                  // draw: cutoff for the next scan (0: none)
   unsigned int amb_count[2];    // dense Gram: pairs the screen left open (two counters, in turns)

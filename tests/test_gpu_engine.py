@@ -25,6 +25,13 @@ CASES = {
     "long_columns": dict(kind="csc_uniform", n_rows=20000, n_cols=2000, n_true=20, n_candidates=300, n_keep=60, rho=0.1, nnz_col=150),
     "no_draw_ahead": dict(kind="csc_uniform", n_rows=60000, n_cols=12000, n_true=50, n_candidates=5000, n_keep=4200, rho=0.1, nnz_col=8),
     "on_demand": dict(kind="csc_zipf", n_rows=20000, n_cols=50000, n_true=50, n_candidates=3000, n_keep=500, rho=0.05, nnz_col=21),
+    # walks on demand that stop at P in a batch, and among the last survivors; with columns longer than the table of rows takes;
+    # with more entries than a CTA holds; with few survivors from the start
+    "demand_stops_early": dict(kind="csc_zipf", n_rows=20000, n_cols=50000, n_true=50, n_candidates=3001, n_keep=9, rho=0.05, nnz_col=21),
+    "demand_stops_late": dict(kind="csc_zipf", n_rows=20000, n_cols=50000, n_true=50, n_candidates=2999, n_keep=33, rho=0.05, nnz_col=21),
+    "demand_long_columns": dict(kind="csc_zipf", n_rows=4000, n_cols=9000, n_true=50, n_candidates=1500, n_keep=300, rho=0.05, nnz_col=90),
+    "demand_many_entries": dict(kind="csc_zipf", n_rows=30000, n_cols=40000, n_true=50, n_candidates=9500, n_keep=900, rho=0.05, nnz_col=63),
+    "demand_few": dict(kind="csc_zipf", n_rows=3000, n_cols=2000, n_true=50, n_candidates=70, n_keep=60, rho=0.05, nnz_col=30),
 }
 
 
