@@ -728,6 +728,7 @@ __device__ __forceinline__ void propose_end(const Problem& p, const Proposal& q,
   }
 }
 
+constexpr int kMaxWords = STRADS_MAX_CANDIDATES / 32;
 constexpr int kTurn = 32;                  // candidates a CTA handles per turn of step 1 (dense) / 2 (CSC)
 
 struct RoundOutputs { int* cand; int* kept; float* dbeta; int* counts; };
@@ -941,7 +942,7 @@ __device__ void dense_pack(const Problem& p, const Engine& e, unsigned char* sm,
 
 // ------------------------------------------------------------------------------------------------
 // Dense, step 2: conflict bits of all candidate pairs on the tensor cores: tiles of 128 rows x 64 or 128 columns of the
-// upper triangle, BF16 operands by TMA (128-byte swizzle) into a ring in shared memory, tcgen05.mma into tensor memory.
+// lower triangle, BF16 operands by TMA (128-byte swizzle) into a ring in shared memory, tcgen05.mma into tensor memory.
 // As in gram_dense_tc.cu the result is a screen: pairs closer to rho than its error bound go to a list and are decided
 // from exact products.  The columns are short, so their correlations scatter widely (standard deviation N^-1/2) and the
 // error band of a product of BF16 roundings (2^-8) would leave percents of all pairs open: three products, hi.hi + hi.lo
@@ -958,15 +959,21 @@ constexpr size_t kGramSmem = (size_t)kRingBytes + 1024;
 constexpr uint32_t kTmemCols = 128;
 
 // A stage holds the high and the low parts of 64 elements of K for both operands.  Its size depends on the tile's width alone, so there is a set of barriers per width.
+constexpr unsigned int kOwnOpen = 64;                    // open pairs of its own that a CTA decides itself (a warp each)
 struct GramShared {
   unsigned long long full[2][kMaxStages], empty[2][kMaxStages], done;
   uint32_t tmem;
   int abort_;
   double norm_a[kRowsT], norm_b[128];
   float norm_af[kRowsT], norm_bf[128];
+  unsigned int n_open, open[kOwnOpen];
 };
 // Phases of the barriers so far (the same in all threads of a CTA).
 struct GramCount { unsigned int stages[2], units; };
+
+// Conflict bits here: a candidate's with all earlier ones, as the walk wants them.  Four words (128 earlier candidates) of
+// consecutive candidates lie side by side, so that a warp whose lanes want a candidate each reads whole lines.
+__device__ __forceinline__ unsigned int* conflict_word(const Problem& p, int a, int w) { return p.conflict + ((size_t)(w >> 2) * p.n_cand + a) * 4 + (w & 3); }
 
 __device__ __forceinline__ double engine_band(long long N) { return 1.0 / 32768.0 + 3.0 * (double)N * (1.0 / 33554432.0); }
 
@@ -992,6 +999,26 @@ __device__ __forceinline__ void tmem_load16(uint32_t addr, uint32_t (&v)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// Exact decision of one pair by a warp.
+__device__ __forceinline__ void decide_exactly(const Problem& p, const Engine& e, int a, int b) {
+  const int lane = threadIdx.x & 31;
+  const float* xa = p.xv + (long long)p.cand[a] * p.ld;
+  const float* xb = p.xv + (long long)p.cand[b] * p.ld;
+  const int n4 = (int)(p.N >> 2);
+  double acc = 0.0;
+  for (int g = lane; g < n4; g += 32) {
+    const float4 u = __ldg(reinterpret_cast<const float4*>(xa) + g), w = __ldg(reinterpret_cast<const float4*>(xb) + g);
+    acc += (double)u.x * w.x + (double)u.y * w.y + (double)u.z * w.z + (double)u.w * w.w;
+  }
+  const long long i = ((long long)n4 << 2) + lane;
+  if (i < p.N) acc += (double)xa[i] * xb[i];
+  acc = warp_sum(acc);
+  if (lane == 0) {
+    const double den = e.norm[a] * e.norm[b];
+    if (den > 0.0 && fabs(acc) >= (double)p.rho * den) atomicOr(conflict_word(p, a, b >> 5), 1u << (b & 31));
+  }
+}
+
 __device__ __forceinline__ void dense_gram(const Problem& p, const Engine& e, const GramPlan& pl, const void* tmap_rows, const void* tmap_cols,
                                            unsigned char* sm, GramShared& gs, GramCount& gc, int n, unsigned int* amb_count,
                                            uint32_t wait_limit) {
@@ -1006,13 +1033,13 @@ __device__ __forceinline__ void dense_gram(const Problem& p, const Engine& e, co
   const double rho = (double)p.rho, band = engine_band(p.N);
   const float quick = (float)((rho - band) * 0.99999);   // |g| below quick ||a|| ||b||: certainly no conflict
   const int cols4 = pl.cols >> 2, cols_log = set ? 7 : 6;
+  if (tid == 0) gs.n_open = 0u;                          // (used behind a barrier of the CTA)
 
   for (int unit = (int)blockIdx.x; unit < units; unit += (int)gridDim.x) {
     const int tile = unit / pl.split, sp = unit - tile * pl.split;
-    int ri = 0, rem = tile, len = pl.col_blocks;
-    const int per_row = kRowsT >> cols_log;
-    while (rem >= len) { rem -= len; len -= per_row; ++ri; }
-    const int row0 = ri * kRowsT, col0 = (ri * per_row + rem) << cols_log;
+    int ri = 0, rem = tile, len = kRowsT >> cols_log;    // row block i meets the column blocks that start before its end
+    while (rem >= min(len, pl.col_blocks)) { rem -= min(len, pl.col_blocks); len += kRowsT >> cols_log; ++ri; }
+    const int row0 = ri * kRowsT, col0 = rem << cols_log;
     const int s0 = min(pl.steps, sp * pl.per), count = min(pl.steps, s0 + pl.per) - s0;
     const unsigned int slot0 = gc.stages[set] % stages, ph0 = (gc.stages[set] / stages) & 1u;
     if (warp == 0) {
@@ -1095,18 +1122,12 @@ __device__ __forceinline__ void dense_gram(const Problem& p, const Engine& e, co
 #pragma unroll
           for (int i = 0; i < 16; ++i) v[i] = 0u;
         }
-        // the tile's place in global memory, or (no split) where the operands were; group q of four columns of row r lies at
-        // q ^ (r & 15) there: no bank conflicts either way
-        if (pl.split > 1) {
-          uint4* dst = reinterpret_cast<uint4*>(e.part + (size_t)unit * (kRowsT * 128) + (row << cols_log) + c);
+        // into shared memory, where the operands were; group q of four columns of row r lies at q ^ (r & 15): no bank conflicts
+        // either way
 #pragma unroll
-          for (int i = 0; i < 4; ++i) __stcg(dst + i, make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
-        } else {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int q = ((c >> 2) + i) ^ (row & 15);
-            *reinterpret_cast<uint4*>(tile_sm + (row << cols_log) + 4 * q) = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-          }
+        for (int i = 0; i < 4; ++i) {
+          const int q = ((c >> 2) + i) ^ (row & 15);
+          *reinterpret_cast<uint4*>(tile_sm + (row << cols_log) + 4 * q) = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
         }
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1114,6 +1135,12 @@ __device__ __forceinline__ void dense_gram(const Problem& p, const Engine& e, co
     int r_lo = 0, r_hi = kRowsT;
     __syncthreads();
     if (pl.split > 1) {
+      // as it lies there to global memory (from the accumulator's registers each thread would touch lines of its own row only:
+      // 4,096 of them, 2 us)
+      uint4* dst = reinterpret_cast<uint4*>(e.part + (size_t)unit * (kRowsT * 128));
+#pragma unroll 4
+      for (int i = tid; i < kRowsT * cols4; i += kT) __stcg(dst + i, *reinterpret_cast<const uint4*>(tile_sm + 4 * i));
+      __syncthreads();
       if (tid == 0) {                                    // wait for the other parts of the tile
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(e.tile_ticket + tile) : "memory");
         unsigned int v = 0u;
@@ -1135,7 +1162,7 @@ __device__ __forceinline__ void dense_gram(const Problem& p, const Engine& e, co
       const int r = r_lo + ((in ? i : 0) >> (cols_log - 2)), q = i & (cols4 - 1);
       float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
       if (pl.split > 1) {
-        const float4* src = reinterpret_cast<const float4*>(e.part + (size_t)tile * pl.split * (kRowsT * 128) + (r << cols_log)) + q;
+        const float4* src = reinterpret_cast<const float4*>(e.part + (size_t)tile * pl.split * (kRowsT * 128) + (r << cols_log)) + (q ^ (r & 15));
         for (int k0 = 0; k0 < pl.split; k0 += 4) {       // in split order
           float4 u[4];
 #pragma unroll
@@ -1158,7 +1185,7 @@ __device__ __forceinline__ void dense_gram(const Problem& p, const Engine& e, co
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           const double den = norm_a * gs.norm_b[4 * q + c], gx = fabs((double)gv[c]);
-          const bool live = den > 0.0 && b0 + c > a;
+          const bool live = den > 0.0 && b0 + c < a;
           if (live && fabs(gx - rho * den) <= band * den) open |= 1u << c;
           else if (live && gx >= rho * den) hits |= 1u << c;
         }
@@ -1167,7 +1194,7 @@ __device__ __forceinline__ void dense_gram(const Problem& p, const Engine& e, co
       word |= __shfl_xor_sync(kFull, word, 1);
       word |= __shfl_xor_sync(kFull, word, 2);
       word |= __shfl_xor_sync(kFull, word, 4);
-      if (in && (lane & 7) == 0 && a < n && (b0 >> 5) < p.mask_words) p.conflict[(size_t)a * p.mask_words + (b0 >> 5)] = word;
+      if (in && (lane & 7) == 0 && a < n && (b0 >> 5) < p.mask_words) *conflict_word(p, a, b0 >> 5) = word;
       if (__any_sync(kFull, open)) {                     // too close to call: listed
         const int cnt = __popc(open);
         int incl = cnt;
@@ -1177,10 +1204,14 @@ __device__ __forceinline__ void dense_gram(const Problem& p, const Engine& e, co
           if (lane >= o) incl += u;
         }
         unsigned int at = 0u;
-        if (lane == 31) at = atomicAdd(amb_count, (unsigned)incl);
+        if (lane == 31) at = atomicAdd(&gs.n_open, (unsigned)incl);
         at = __shfl_sync(kFull, at, 31) + (unsigned)(incl - cnt);
-        for (; open; open &= open - 1u, ++at)
-          if (at < (unsigned)p.cap_amb) p.amb_pairs[at] = ((unsigned)a << 16) | (unsigned)(b0 + __ffs((int)open) - 1);
+        for (; open; open &= open - 1u, ++at) {
+          const unsigned int pair = ((unsigned)a << 16) | (unsigned)(b0 + __ffs((int)open) - 1);
+          if (at < kOwnOpen) { gs.open[at] = pair; continue; }
+          const unsigned int over = atomicAdd(amb_count, 1u);
+          if (over < (unsigned)p.cap_amb) p.amb_pairs[over] = pair;
+        }
       }
     }
     if (unit + (int)gridDim.x < units) {                 // (the tile in shared memory, before the next operands)
@@ -1188,140 +1219,141 @@ __device__ __forceinline__ void dense_gram(const Problem& p, const Engine& e, co
       if (__syncthreads_or(*(volatile int*)&gs.abort_)) return;
     }
   }
-}
-
-// Exact decision of one pair by a warp.
-__device__ __forceinline__ void decide_exactly(const Problem& p, const Engine& e, int a, int b) {
-  const int lane = threadIdx.x & 31;
-  const float* xa = p.xv + (long long)p.cand[a] * p.ld;
-  const float* xb = p.xv + (long long)p.cand[b] * p.ld;
-  const int n4 = (int)(p.N >> 2);
-  double acc = 0.0;
-  for (int g = lane; g < n4; g += 32) {
-    const float4 u = __ldg(reinterpret_cast<const float4*>(xa) + g), w = __ldg(reinterpret_cast<const float4*>(xb) + g);
-    acc += (double)u.x * w.x + (double)u.y * w.y + (double)u.z * w.z + (double)u.w * w.w;
-  }
-  const long long i = ((long long)n4 << 2) + lane;
-  if (i < p.N) acc += (double)xa[i] * xb[i];
-  acc = warp_sum(acc);
-  if (lane == 0) {
-    const double den = e.norm[a] * e.norm[b];
-    if (den > 0.0 && fabs(acc) >= (double)p.rho * den) atomicOr(&p.conflict[(long long)a * p.mask_words + (b >> 5)], 1u << (b & 31));
-  }
+  // the pairs left open, by the CTA that found them; a list and a barrier for all of them took 4.6 us at 463 rows
+  __syncthreads();
+#pragma unroll 1
+  for (unsigned int i = warp; i < min(gs.n_open, kOwnOpen); i += kWarps) decide_exactly(p, e, (int)(gs.open[i] >> 16), (int)(gs.open[i] & 0xffffu));
 }
 
 // ------------------------------------------------------------------------------------------------
-// Dense, step 3: first-fit over the conflict bits, by one CTA.  The rows are brought into shared memory by all its
-// threads (a window's all at once, a long list's in pieces); one warp then takes 32 candidates at a time.  Which of them
-// are blocked is one word of every row kept so far, OR-ed over the lanes; their conflicts among themselves are that word
-// of their own rows, settled one kept member at a time while few are in question, else in passes of warp-wide ORs.  One
-// warp issues an instruction every few cycles, so what counts is their number: keeping a whole mask up to date (a
-// row OR-ed in per kept member) took 1 us per 32 candidates.
+// Dense, step 3: first-fit over the conflict bits, by one CTA, 1,024 candidates at a time.  A thread holds the bits of two
+// candidates with the earlier ones of the piece in registers (those with earlier pieces are looked at once), and a piece is settled in
+// passes: a candidate with no undecided earlier neighbour is kept, and those it conflicts with are out.  The passes are
+// as many as the longest chain of such dependencies, five to six where 1,024 candidates of 463 rows leave 110; bound by the
+// ANDs (half the lanes' rate for logic).  One warp
+// going through the words one after the other took 0.7 us a word of 32 candidates, 21.7 us of 463 x 508,999's 56 per round; this
+// takes 6.2 of 36: 1.7 to bring in the rows, 0.7 a pass.
+// (Passes that OR the rows of undecided candidates in shared memory: 2 us each, bound by reading the rows.)
 // ------------------------------------------------------------------------------------------------
-constexpr size_t kWalkSmem = 190 * 1024;
+constexpr int kPiece = 2 * kT, kPieceWords = kPiece / 32;
+struct WalkShared {
+  __align__(16) unsigned int state[2][kPieceWords];      // of the piece: undecided, kept in this pass
+  __align__(16) unsigned int kept[kMaxWords + kPieceWords];      // of all pieces so far
+  int ex;
+};
+__device__ __forceinline__ unsigned int any_of(const uint4& a, const uint4& b) { return (a.x & b.x) | (a.y & b.y) | (a.z & b.z) | (a.w & b.w); }
+
+// Whether the thread's two candidates (of words `warp` and warp + kWarps) have neighbours among `mask`: what lies before them only.
+__device__ __forceinline__ void touch(const uint4 (&row)[2][kPieceWords / 4], const unsigned int* mask, int warp, unsigned int (&met)[2]) {
+#pragma unroll
+  for (int q = 0; q < kPieceWords / 4; ++q) {
+    if (q > (warp + kWarps) / 4) break;
+    const uint4 m = reinterpret_cast<const uint4*>(mask)[q];
+    if (q <= (kWarps - 1) / 4 && q <= warp / 4) met[0] |= any_of(row[0][q], m);
+    met[1] |= any_of(row[1][q], m);
+  }
+}
 
 __device__ __forceinline__ void dense_walk(const Problem& p, const Engine& e, unsigned char* sm, int n, int n_total) {
+  WalkShared& s = *reinterpret_cast<WalkShared*>(sm);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int words = (n + 31) >> 5, quads = (words + 3) >> 2;
-  const int pitch = quads * 4 + 4;                       // words; rows start four banks apart
-  unsigned int* blocked = reinterpret_cast<unsigned int*>(sm);            // [quads * 4] by the members of earlier pieces
-  unsigned int* rows = blocked + quads * 4;
-  int piece = (int)((kWalkSmem / sizeof(unsigned int) - (size_t)quads * 4) / (size_t)(pitch + 2));
-  piece = min(piece & ~31, words * 32);                  // rows in shared memory at a time (at least 64: 512 words a row)
-  int* s_cand = reinterpret_cast<int*>(rows + (size_t)piece * pitch);     // [piece]
-  int* s_row = s_cand + piece;                           // [piece] where the rows of this piece's kept members start
-  __shared__ int s_nk, s_ex, s_done, s_here;
+  constexpr int kQuads = kPieceWords / 4;
+  const uint4* rows = reinterpret_cast<const uint4*>(p.conflict);
+  int kept = 0, examined = n;
+  bool done = false;
   __syncthreads();
-  for (int w = tid; w < quads * 4; w += kT) blocked[w] = 0u;
-  if (tid == 0) { s_nk = 0; s_ex = n; s_done = 0; }
-  for (int r0 = 0; r0 < n; r0 += piece) {
-    const int nr = min(piece, n - r0);
-    const int q0 = (r0 >> 5) >> 2;                       // earlier words are not looked at again
-    const int nq = quads - q0;
-    // sixteen lanes per row, 16 bytes each
-    for (int c = tid & 15; c < nq; c += 16)
-      for (int r = tid >> 4; r < nr; r += 8 * (kT / 16)) {
-        uint4 v[8];
-        const uint4* src = reinterpret_cast<const uint4*>(p.conflict + (size_t)(r0 + r) * p.mask_words) + q0 + c;
-        unsigned int* dst = rows + r * pitch + 4 * (q0 + c);
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (r + u * (kT / 16) < nr) v[u] = __ldcg(src + (size_t)u * (kT / 16) * (p.mask_words >> 2));
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (r + u * (kT / 16) < nr) *reinterpret_cast<uint4*>(dst + u * (kT / 16) * pitch) = v[u];
-      }
-    for (int i = tid; i < nr; i += kT) s_cand[i] = p.cand[r0 + i];
-    __syncthreads();
-    if (warp == 0) {
-      int nk = s_nk, here = 0;                           // kept so far; of this piece
-      bool done = false;
-      const int w_end = (r0 + nr + 31) >> 5;
 #pragma unroll 1
-      for (int w = r0 >> 5; w < w_end; ++w) {
-        unsigned int hit = lane == 0 ? blocked[w] : 0u;
-        for (int i = lane; i < here; i += 32) hit |= rows[s_row[i] + w];
-        hit = __reduce_or_sync(kFull, hit);
-        const int m = n - w * 32;
-        unsigned int avail = ~hit & (m >= 32 ? kFull : ((1u << m) - 1u));
-        if (avail == 0u) continue;
-        const int at = w * 32 - r0 + lane, row = at * pitch;
-        unsigned int mine = ((avail >> lane) & 1u) ? (rows[row + w] & (lane == 31 ? 0u : (kFull << (lane + 1)))) : 0u;
-        mine &= avail;
-        unsigned int keep = avail;
-        if (__any_sync(kFull, mine != 0u)) {
-          keep = 0u;
-          if (__popc(avail) <= 10) {
-            while (avail) {
-              const int i = __ffs((int)avail) - 1;
-              keep |= 1u << i;
-              avail &= ~((1u << i) | __shfl_sync(kFull, mine, i));
-            }
-          } else {
-            unsigned int fresh = 0u;
-            while (avail) {
-              avail &= ~__reduce_or_sync(kFull, ((fresh >> lane) & 1u) ? mine : 0u);
-              fresh = avail & ~__reduce_or_sync(kFull, ((avail >> lane) & 1u) ? mine : 0u);
-              keep |= fresh;
-              avail &= ~fresh;
-            }
-          }
-        }
-        const int room = p.n_keep - nk;
-        if (__popc(keep) >= room) {                      // stop exactly at P: drop the surplus from the back
-          while (__popc(keep) > room) keep &= ~(1u << (31 - __clz((int)keep)));
-          done = true;
-          if (lane == 0) s_ex = w * 32 + 32 - __clz((int)keep);
-        }
-        if ((keep >> lane) & 1u) {
-          const int r = __popc(keep & ((1u << lane) - 1u));
-          s_row[here + r] = row;
-          p.kept[nk + r] = s_cand[at];
-          p.kept_pos[nk + r] = w * 32 + lane;
-        }
-        nk += __popc(keep); here += __popc(keep);
-        if (done) break;
-        __syncwarp();
+  for (int r0 = 0; r0 < n && !done; r0 += kPiece) {
+    uint4 row[2][kQuads];
+    bool out0[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int a = r0 + tid + h * kT, own = a - r0;
+#pragma unroll
+      for (int q = 0; q < kQuads; ++q)
+        row[h][q] = a < n && 128 * q < own ? __ldcg(rows + (size_t)(r0 / 128 + q) * p.n_cand + a) : make_uint4(0u, 0u, 0u, 0u);
+      out0[h] = a >= n;
+    }
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      const int a = r0 + tid + h * kT;
+      unsigned int hit = 0u;
+      if (a < n) {
+#pragma unroll 4
+        for (int q = 0; q < r0 / 128; ++q) hit |= any_of(__ldcg(rows + (size_t)q * p.n_cand + a), reinterpret_cast<const uint4*>(s.kept)[q]);
       }
-      if (lane == 0) { s_nk = nk; s_done = done; s_here = here; }
+      if (hit) out0[h] = true;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int own = tid + h * kT;
+      // (of the last four words only the bits before the candidate's own place mean anything)
+#pragma unroll
+      for (int q = 0; q < kQuads; ++q)
+        if (128 * q < own && own < 128 * (q + 1)) {
+          auto before = [&](int word) { const int k = own - 128 * q - 32 * word; return k >= 32 ? kFull : (k <= 0 ? 0u : (1u << k) - 1u); };
+          row[h][q].x &= before(0); row[h][q].y &= before(1); row[h][q].z &= before(2); row[h][q].w &= before(3);
+        }
+      const unsigned int und = __ballot_sync(kFull, !out0[h]);
+      if (lane == 0) s.state[0][warp + h * kWarps] = und;
     }
     __syncthreads();
-    if (s_done || r0 + piece >= n) break;
-    // the next pieces' words of this piece's kept members
-    for (int w = ((r0 + nr) >> 5) + tid; w < words; w += kT) {
-      unsigned int acc = blocked[w];
-      for (int i = 0; i < s_here; ++i) acc |= rows[s_row[i] + w];
-      blocked[w] = acc;
+    unsigned int und[2] = {s.state[0][warp], s.state[0][warp + kWarps]}, keep[2] = {0u, 0u};     // (this warp's words)
+#pragma unroll 1
+    for (bool open = true; open;) {
+      // kept: those with no undecided earlier neighbour (decided ones are out of everybody's way: kept or not)
+      unsigned int fresh[2] = {0u, 0u};
+      if (und[0] | und[1]) {
+        unsigned int wait[2] = {0u, 0u};
+        touch(row, s.state[0], warp, wait);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) { fresh[h] = __ballot_sync(kFull, wait[h] == 0u) & und[h]; keep[h] |= fresh[h]; }
+      }
+      if (lane == 0) { s.state[1][warp] = fresh[0]; s.state[1][warp + kWarps] = fresh[1]; }
+      __syncthreads();
+      // out: those with one of them before
+      if (und[0] | und[1]) {
+        unsigned int out[2] = {0u, 0u};
+        touch(row, s.state[1], warp, out);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) und[h] &= ~(fresh[h] | __ballot_sync(kFull, out[h] != 0u));
+        if (lane == 0) { s.state[0][warp] = und[0]; s.state[0][warp + kWarps] = und[1]; }
+      }
+      open = __syncthreads_or((und[0] | und[1]) != 0u) != 0;
+    }
+    if (lane == 0) { s.kept[r0 / 32 + warp] = keep[0]; s.kept[r0 / 32 + warp + kWarps] = keep[1]; }
+    __syncthreads();
+    // numbered, up to P
+    const int c = __popc(s.kept[r0 / 32 + lane]);
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += v;
+    }
+    const int total = __shfl_sync(kFull, incl, 31), room = p.n_keep - kept;
+    static_assert(kPieceWords == 32, "a word per lane");
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const unsigned int word = keep[h];
+      const int r = __shfl_sync(kFull, incl - c, warp + h * kWarps) + __popc(word & ((1u << lane) - 1u)), a = r0 + tid + h * kT;
+      if (((word >> lane) & 1u) && r < room) {           // stop exactly at P
+        p.kept[kept + r] = p.cand[a];
+        p.kept_pos[kept + r] = a;
+        if (r == room - 1) s.ex = a + 1;
+      }
     }
     __syncthreads();
+    done = total >= room;
+    if (done) examined = s.ex;
+    kept += min(total, room);
   }
   if (tid == 0) {
-    const int nk = s_nk;
     EngineState* es = e.es;
-    es->n_kept = nk; es->n_examined = s_ex;
-    es->walk_open = nk < p.n_keep && n < n_total ? 1 : 0;
+    es->n_kept = kept; es->n_examined = examined;
+    es->walk_open = kept < p.n_keep && n < n_total ? 1 : 0;
     // would the window have done?  (the next round goes straight to the whole list if not)
-    if (n == n_total && e.window < n_total) es->skip_window = nk == p.n_keep && s_ex <= e.window ? 0 : 1;
+    if (n == n_total && e.window < n_total) es->skip_window = kept == p.n_keep && examined <= e.window ? 0 : 1;
   }
 }
 
@@ -1387,7 +1419,7 @@ __device__ void dense_apply(const Problem& p, const Moving& mv, double* part, in
 constexpr unsigned int kFewOpen = 48;                    // open pairs the walking CTA decides itself
 
 // (cold) Data whose products cluster at rho leave more pairs open than the list holds: all pairs of the first n candidates
-// exactly, tiles of 32 x 128 of the upper triangle.  32 rows of the tile's columns at a time lie in shared memory as
+// exactly, tiles of 32 x 128 of the lower triangle.  32 rows of the tile's columns at a time lie in shared memory as
 // binary64, and a thread adds up 2 x 4 products: bound by reading the operands there (a warp's step takes 9 cycles of shared
 // memory and 4 of the FP64 pipe).  A warp per pair, both columns read again for every pair and the lower triangle stepped
 // through as well, took 9.7 ms per round at 4,096 candidates of 900 rows, this takes 2.2 (the launch chain's 3xTF32 pass, list
@@ -1402,10 +1434,10 @@ __device__ __noinline__ void decide_all(const Problem& p, const Engine& e, int n
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   static_assert(kWarps * 2 == kExactRows && 32 * 4 == kExactCols, "2 x 4 products a thread");
   constexpr int kBoth = kExactRows + kExactCols, kStaged = (kBoth * (kExactK / 4) + kT - 1) / kT;         // columns; groups of four rows a thread brings in
-  const int n4 = (int)((p.N + 3) >> 2), row_tiles = (n + kExactRows - 1) / kExactRows, col_tiles = (n + kExactCols - 1) / kExactCols;
+  const int n4 = (int)((p.N + 3) >> 2), row_tiles = (n + kExactRows - 1) / kExactRows;
   unsigned int tile = 0u;
   for (int r = 0; r < row_tiles; ++r) {
-    for (int c = r * kExactRows / kExactCols; c < col_tiles; ++c) {
+    for (int c = 0; c <= r * kExactRows / kExactCols; ++c) {
       if (tile++ % gridDim.x != blockIdx.x) continue;
       const int row0 = r * kExactRows, col0 = c * kExactCols;
       __syncthreads();                                   // (the tile before)
@@ -1452,8 +1484,8 @@ __device__ __noinline__ void decide_all(const Problem& p, const Engine& e, int n
 #pragma unroll
         for (int y = 0; y < 4; ++y) {
           const double den = s.norm[warp * 2 + x] * s.norm[kExactRows + lane + 32 * y];
-          const unsigned int word = __ballot_sync(kFull, col0 + lane + 32 * y > a && den > 0.0 && fabs(acc[x][y]) >= (double)p.rho * den);
-          if (lane == 0 && a < n && (col0 >> 5) + y < p.mask_words) p.conflict[(size_t)a * p.mask_words + (col0 >> 5) + y] = word;
+          const unsigned int word = __ballot_sync(kFull, col0 + lane + 32 * y < a && den > 0.0 && fabs(acc[x][y]) >= (double)p.rho * den);
+          if (lane == 0 && a < n && (col0 >> 5) + y < p.mask_words) *conflict_word(p, a, (col0 >> 5) + y) = word;
         }
       }
     }
@@ -1465,7 +1497,6 @@ __device__ __noinline__ void decide_all(const Problem& p, const Engine& e, int n
 // (its terms in a list of the warp's own in shared memory: no barrier), no conflict bits (the walk works from the list
 // of conflicting pairs or forms rows on demand), and x_c^T r with the same visit to the column.
 // ------------------------------------------------------------------------------------------------
-constexpr int kMaxWords = STRADS_MAX_CANDIDATES / 32;
 constexpr int kMet = 512;                                // candidates one candidate may meet (of kReach)
 constexpr int kRing = 4;                                 // steps of terms under way, and the one at hand
 constexpr int kReach = 1664;                             // candidates a warp has a place for at a time: a window of 1,024 kept
@@ -2811,7 +2842,7 @@ size_t smem_of(bool dense, int n_keep, bool ahead, int n_cand) {
   if (dense) {
     at_least(kPackSmem);
     at_least(kGramSmem);
-    at_least(kWalkSmem);
+    at_least(sizeof(WalkShared));
     at_least(keys + sizeof(Moving) + sizeof(double) * 4 * kT + (ahead ? sizeof(ChangedByBin) : 0));
   } else {
     at_least(kTermsSmem);

@@ -35,8 +35,9 @@ __host__ __device__ inline GramPlan gram_plan(long long N, int n, int n_ctas) {
     const int per_row = kGramRows / cols;
     pl.cols = cols;
     pl.col_blocks = (n + cols - 1) / cols;
-    // row block i meets the column blocks from i * per_row on
-    pl.tiles = row_blocks * pl.col_blocks - per_row * row_blocks * (row_blocks - 1) / 2;
+    // row block i meets the column blocks that start before its end
+    pl.tiles = 0;
+    for (int i = 1; i <= row_blocks; ++i) pl.tiles += i * per_row < pl.col_blocks ? i * per_row : pl.col_blocks;
     pl.steps = steps;
     pl.split = n_ctas / pl.tiles;
     if (pl.split > 16) pl.split = 16;
