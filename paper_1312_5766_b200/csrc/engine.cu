@@ -2194,7 +2194,7 @@ __device__ __forceinline__ bool settle_rest(const Problem& p, const Problem& sp,
 // threads do meanwhile, with the grid barrier g_draw; false: it gave up.  Every CTA leaves the places of the kept list that it
 // owns (a mod ctas) and, in *n_kept, their number.  False: a barrier gave up.
 template <typename Draw>
-__device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, const Problem& sp, const Engine& e, unsigned char* sm, Grid& g, Grid& g_draw, int* n_kept,
+__device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, Problem& sp, const Engine& e, unsigned char* sm, Grid& g, Grid& g_draw, int* n_kept,
                                                    Draw&& draw) {
   DemandShared& s = *reinterpret_cast<DemandShared*>(sm);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -2308,7 +2308,11 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, const Probl
         }
       }
       walk_sync();
-      const bool table = s.longest == 0;                 // (the same in every CTA)
+      const bool table = s.longest == 0;                 // (the same in every CTA, but for the last batch)
+      if (!table) {
+        if (tid == 0) sp = p;                            // (for the functions that merge)
+        walk_sync();
+      }
       if (table) {
         // the values of a row side by side, in the order of the members: its first member takes the places
         unsigned int members[kEach];
@@ -2511,7 +2515,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
   __shared__ __align__(8) PackBars pb;
   __shared__ __align__(16) GramShared gs;
   __shared__ int s_kept, s_examined;
-  // Copies for the functions that are called rarely and not inlined: a reference to the parameters themselves would make
+  // Copies for the functions that are called rarely and not inlined, made when they are: a reference to the parameters themselves would make
   // every access to them, in the hot code too, a load from memory.
   __shared__ Problem sp;
   __shared__ Engine se;
@@ -2519,8 +2523,11 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
   // meet a barrier that gives up)
   if (p.st->status & STRADS_STATUS_WAIT_EXPIRED) return;
   const int tid = threadIdx.x, warp = tid >> 5, cta = (int)blockIdx.x, n_ctas = (int)gridDim.x;
-  if (tid == 0) { sp = p; se = e; }
-  __syncthreads();
+  auto keep_parameters = [&]() {                         // (where one of those functions is called: one thread takes 2.7 us for it)
+    __syncthreads();
+    if (tid == 0) { sp = p; se = e; }
+    __syncthreads();
+  };
   const bool walker = cta == n_ctas - 1;                 // the CTA that walks
   const uint32_t limit = p.wait_limit ? p.wait_limit : 1u << 24;
   GramCount gc = {};
@@ -2614,6 +2621,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
         const bool listed = open <= (unsigned)p.cap_amb;
         if (!listed) {
           if (cta == 0 && tid == 0) atomicOr(&p.st->status, STRADS_STATUS_GRAM_FALLBACK);
+          keep_parameters();
           decide_all(sp, se, n);
         }
         if (listed && open > 0u && (open > kFewOpen || walker)) {
@@ -2699,7 +2707,10 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
       }
     }
     if (!ok) break;
-    if (draws && es->mend && !(ok = draw_mend(sp, se, ds, sm, td, k, g))) break;
+    if (draws && es->mend) {
+      keep_parameters();
+      if (!(ok = draw_mend(sp, se, ds, sm, td, k, g))) break;
+    }
     // ---- step 4 ----
     int n_changed = 0, nk = 0;
     const int n_next = no_filter ? p.n_keep : (e.window < n_total && es->skip_window ? n_total : e.window);   // looked at first
@@ -2770,8 +2781,15 @@ __device__ __forceinline__ bool draw_alone(const Problem& p, const Engine& e, Dr
     if (b < p.n_cand) p.cand[b] = -1;
   }
   const int dirty = e.es->dirty;
-  if (tid == 0) { sp = p; se = e; ds.cut = 0.f; }
+  if (tid == 0) ds.cut = 0.f;
   __syncthreads();
+  // (for the functions that are called rarely; made where they are: one thread takes 2.7 us for it, before the first key 16.5 -> 15.1 us
+  // per call at J = 100,000)
+  auto keep_parameters = [&]() {
+    __syncthreads();
+    if (tid == 0) { sp = p; se = e; }
+    __syncthreads();
+  };
   Grid g;
   g.count = &e.es->bar_count; g.target = 0u; g.n = gridDim.x; g.limit = p.wait_limit ? p.wait_limit : kSpinLimit; g.status = &p.st->status;
   int turn = 0;
@@ -2797,12 +2815,18 @@ __device__ __forceinline__ bool draw_alone(const Problem& p, const Engine& e, Dr
     }
   }
   __syncthreads();
-  if (dirty && !clear_histogram(se, g)) return false;    // (the same in every CTA: it changes when the last one leaves)
+  if (dirty) {                                           // (the same in every CTA: it changes when the last one leaves)
+    keep_parameters();
+    if (!clear_histogram(se, g)) return false;
+  }
   for (int b = tid; b < kHistBins; b += kT)
     if (sh[b]) atomicAdd(&e.hist[b], sh[b]);
   if (!grid_sync(g, stall != 0 && blockIdx.x == 0)) return false;
   draw_select<AllThreads>(e, ds, (unsigned)p.n_cand);
-  if (ds.bnd_count > (unsigned)e.cap_boundary && !draw_refine(sp, se, ds, sm, t, (unsigned)p.n_cand, g)) return false;
+  if (ds.bnd_count > (unsigned)e.cap_boundary) {
+    keep_parameters();
+    if (!draw_refine(sp, se, ds, sm, t, (unsigned)p.n_cand, g)) return false;
+  }
   if (kept_groups > 0) {
     for (int k = 0; k < turn; ++k)
 #pragma unroll
@@ -2811,6 +2835,7 @@ __device__ __forceinline__ bool draw_alone(const Problem& p, const Engine& e, Dr
         if (key != ~0ull) take_winner(e, ds, bins, key);
       }
   } else {
+    keep_parameters();
     draw_collect_all(sp, se, ds, sm, t);
   }
   if (!grid_sync(g)) return false;
