@@ -1891,7 +1891,8 @@ constexpr unsigned int kNoSlot = 0xffff;
 constexpr int kOwn = 256;                                // candidates a CTA can hold (more: their columns stay in global memory)
 constexpr int kOwnEntries = 5120;                        // entries of their columns
 constexpr int kRestEntries = kOwnEntries * 3 / 2;
-constexpr int kLast = 512;                               // survivors that are settled at once
+constexpr int kLast = 512;                               // survivors that are settled at once,
+constexpr long long kLastEntries = 12288;                // while a CTA's share of their products, bound by going through all their entries, is no more than a batch
 constexpr int kPerMember = kWalkT / kBatch, kEach = kColCap / kPerMember;      // threads of a batch member; its entries per thread
 static_assert(kMaxWords <= 2 * kWalkT && kOwn == kT - kWalkT && kBatch == 4 * kWalkWarps && kBatch * kColCap * 2 <= kRowSlots,
               "two mask words per walking thread, a held candidate per other thread, four members per warp");
@@ -2070,33 +2071,64 @@ __device__ __forceinline__ bool settle_rest(const Problem& p, const Problem& sp,
     walk_sync();
     here = kOwn;                                         // whole words; of the first one whatever does not fit is read where it is
     while (here > 32 && s.own_at[here] > kRestEntries) here -= 32;
-    const int c = c0 + tid, at = s.own_at[tid], n = tid < here ? s.own_at[tid + 1] - at : 0, most = __reduce_max_sync(kFull, n);
+    const int c = c0 + tid, at = s.own_at[tid], n = tid < here ? s.own_at[tid + 1] - at : 0;
     const bool held = at + n <= kRestEntries;
+    int met = 0;
     if (tid < here) {
+      // the entries in rows of members move to the front of the candidate's stretch (its thread has read what lay there), each
+      // with its row's slot: most rows are no member's, and products are four times the instructions of a look-up
+      if (table) {
+#pragma unroll 1
+        for (int x0 = 0; x0 < (held ? n : 0); x0 += kU) {
+          int row[kU];
+          float v[kU];
+          unsigned int sl[kU];
+#pragma unroll
+          for (int u = 0; u < kU; ++u) {
+            const bool on = x0 + u < n;
+            row[u] = on ? s.rrow[at + x0 + u] : kFreeRow;
+            v[u] = on ? s.rval[at + x0 + u] : 0.f;
+          }
+          find_rows<kU>(s, row, kFull, sl);
+#pragma unroll
+          for (int u = 0; u < kU; ++u)
+            if (sl[u] != kNoSlot) { s.rrow[at + met] = (int)sl[u]; s.rval[at + met] = v[u]; ++met; }
+        }
+        __syncwarp();
+      }
+      const int most = __reduce_max_sync(kFull, met);
 #pragma unroll 1
       for (int g0 = 0; g0 < m; g0 += kTogether) {
         float dot[kTogether] = {};
         if (table) {
 #pragma unroll 1
           for (int x0 = 0; x0 < most; x0 += kU) {
-            int row[kU];
             float v[kU];
-            unsigned int sl[kU];
             uint2 rec[kU];
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
-              row[u] = kFreeRow; v[u] = 0.f;
-              if (x0 + u < n) {
-                row[u] = held ? s.rrow[at + x0 + u] : __ldg(p.xrow + col.q0 + x0 + u);
-                v[u] = held ? s.rval[at + x0 + u] : __ldg(p.xv + col.q0 + x0 + u);
-              }
+              const bool on = x0 + u < met;
+              rec[u] = on ? s.row_rec[s.rrow[at + x0 + u]] : make_uint2(0u, 0u);
+              v[u] = on ? s.rval[at + x0 + u] : 0.f;
             }
-            find_rows<kU>(s, row, ((1u << kTogether) - 1u) << g0, sl);
-#pragma unroll
-            for (int u = 0; u < kU; ++u) rec[u] = sl[u] != kNoSlot ? s.row_rec[sl[u]] : make_uint2(0u, 0u);
 #pragma unroll
             for (int y = 0; y < kTogether; ++y)
               if (g0 + y < m) dot[y] = add_products<kU>(s, g0 + y, rec, v, dot[y]);
+          }
+          if (!held) {                                   // (no room for its column: one entry after the other)
+            const unsigned int want = ((1u << kTogether) - 1u) << g0;
+#pragma unroll 1
+            for (int x = 0; x < n; ++x) {
+              const int row[1] = {__ldg(p.xrow + col.q0 + x)};
+              unsigned int sl[1];
+              find_rows<1>(s, row, want, sl);
+              if (sl[0] == kNoSlot) continue;
+              const uint2 rec[1] = {s.row_rec[sl[0]]};
+              const float v[1] = {__ldg(p.xv + col.q0 + x)};
+#pragma unroll
+              for (int y = 0; y < kTogether; ++y)
+                if (g0 + y < m) dot[y] = add_products<1>(s, g0 + y, rec, v, dot[y]);
+            }
           }
         } else {
 #pragma unroll
@@ -2258,7 +2290,7 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Problem& p, Problem& sp
 #pragma unroll
         for (int k = 0; k < kWalkWarps; ++k) { const int v = s.wsum[k]; if (k < warp) idx += v; total += v; }
         if (total == 0) break;                           // list exhausted (the same in every CTA)
-        last = total > kBatch && total <= kLast && total <= n_ctas * kBatch;
+        last = total > kBatch && total <= kLast && total <= n_ctas * kBatch && (long long)total * p.nnz <= kLastEntries * p.J;
         int* list = last ? s.survivor : s.pos;
         const int most = last ? kLast : kBatch;
 #pragma unroll 1
