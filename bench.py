@@ -231,8 +231,8 @@ def rooflines(p: wl.LassoProblem, workload: str, step_ms: dict, kept_per_round: 
     else:
         nnz_col = p.nnz / p.n_cols
         if step_ms["walk_ms"] >= step_ms["gram_ms"]:
-            # its longest step is the walk on demand: every kept candidate's column is merged with every later candidate
-            # not yet blocked (at most all examined ones): <= 2 nnz_col - 1 compare steps per merge
+            # its longest step is the walk on demand: every kept candidate's column against every later candidate not yet
+            # blocked (at most all examined ones), counted as merges of <= 2 nnz_col - 1 compare steps (the kernel looks rows up)
             ops = kept_per_round * examined_per_round * (2.0 * nnz_col - 1.0)
         else:
             # its longest step is the inner products of the window's pairs that share a row
@@ -251,7 +251,7 @@ def rooflines(p: wl.LassoProblem, workload: str, step_ms: dict, kept_per_round: 
             "rounds_per_launch": rounds, "algorithmic_ops_per_launch": ops,
             "peak_source": "148 SMs x 128 lanes x max SM clock: one merge step (compare + advance) per lane per cycle",
             "note": f"a launch is {rounds} whole rounds; of their steps only the inner products of sparse columns are "
-                    "counted, as sorted-list merge steps, over a few MB of columns: bound by dependent loads and barriers, "
+                    "counted, as the sorted-list merge steps they stand for, over a few MB of columns: bound by dependent loads and barriers, "
                     "not by HBM"}
         upd_bytes = 8.0 * nnz_col * kept_per_round + 8.0 * p.n_rows
         pack_bytes = 0.0

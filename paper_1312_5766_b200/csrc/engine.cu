@@ -10,12 +10,13 @@
 //   1  (all CTAs)  BF16 copies of the candidates' columns,        last round's residual applied; candidates entered
 //                  x_c^T r and would-be changes; scan of the      into the row buckets; scan of the keys of round t + 1
 //                  keys of round t + 1
-//   2  (all CTAs)  Gram tiles on the tensor cores                 inner products from the buckets, x_c^T r and would-be
-//                                                                 changes; keys of round t + 1 below the boundary collected
-//  (2b)            exact products of pairs left open
-//   3              greedy walk (last CTA); keys of round t + 1    greedy walk (last CTA); buckets emptied (the others)
+//   2  (all CTAs)  Gram tiles on the tensor cores, then the      inner products from the buckets, x_c^T r and would-be
+//                  pairs they leave open                          changes
+//  (2b)            open pairs that their CTA had no room for
+//   3              greedy walk (last CTA); keys of round t + 1    the same; buckets emptied (the others)
 //                  below the boundary collected (the others)
-//  (3b)            all candidates instead of the window           walk over all candidates with conflict rows on demand
+//  (3b)            all candidates instead of the window           walk over all candidates with conflict rows on demand by half the
+//                                                                 warps, the draw of round t + 1 by the others
 //   4  (all CTAs)  residual, beta, delta; the winners of the draw ranked, corrected for this round's changes
 //
 // Drawing ahead is exact: the draw of round t + 1 collects the P' + P smallest keys by the priorities of round t's
@@ -1879,7 +1880,7 @@ __device__ void csc_apply(const Problem& p, int nk, int n_moving, int shift) {
 // The chain leaves most of the SM's issue slots idle whatever the number of its warps, and the next draw up to the collection of
 // its winners needs nothing else: half the warps walk, the other half draw, with barriers of their own.
 //
-// 10^7 columns of 20 entries, 16,384 candidates of which ~64 are kept: 66 us per round.  With merges, batches of 32 to the end
+// 10^7 columns of 20 entries, 16,384 candidates of which ~64 are kept: 65 us per round.  With merges, batches of 32 to the end
 // (5.1 of them at 9.7 us) and all warps in both, the scan in the walk's waits and behind it, 101.
 // ------------------------------------------------------------------------------------------------
 constexpr int kWalkWarps = kWalkT / 32;
@@ -1891,8 +1892,11 @@ constexpr unsigned int kNoSlot = 0xffff;
 constexpr int kOwn = 256;                                // candidates a CTA can hold (more: their columns stay in global memory)
 constexpr int kOwnEntries = 5120;                        // entries of their columns
 constexpr int kRestEntries = kOwnEntries * 3 / 2;
-constexpr int kLast = 512;                               // survivors that are settled at once,
-constexpr long long kLastEntries = 12288;                // while a CTA's share of their products, bound by going through all their entries, is no more than a batch
+// Survivors that are settled at once: as many as a thread pair of bits per walking thread holds, and while their entries, all of
+// which every CTA goes through, are no more than these (us per round for 1,500 / 2,600 / 4,096 / 7,000 / 12,288: 10^7 columns of 20
+// entries 65.8 / 65.5 / 64.8 / 65.3 / 66.3, 300,000 of 30 34.9 / 35.5 / 37.0 / 39.8 / 41.1, 3,000,000 of 12 47.0 / 44.9 / 45.1 / 48.2 / 48.1).
+constexpr int kLast = 512;
+constexpr long long kLastEntries = 3072;
 constexpr int kPerMember = kWalkT / kBatch, kEach = kColCap / kPerMember;      // threads of a batch member; its entries per thread
 static_assert(kMaxWords <= 2 * kWalkT && kOwn == kT - kWalkT && kBatch == 4 * kWalkWarps && kBatch * kColCap * 2 <= kRowSlots,
               "two mask words per walking thread, a held candidate per other thread, four members per warp");
