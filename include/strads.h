@@ -133,8 +133,10 @@ typedef struct {
                          SIMT Gram kernel, which is the one that can export its values)      */
 } strads_round_out_t;
 
-/* Bytes of device workspace that `cfg` needs (pointer fields of cfg are not read).  Whether whole rounds go in one
- * launch depends on rho, and with it the size; with rho left at 0 the answer covers any. */
+/* Bytes of device workspace that `cfg` needs (pointer fields of cfg are not read).  Dense X: whether whole rounds go in one
+ * launch depends on rho, and they need buffers of their own (13 MB and up).  With rho set the answer includes them for
+ * N rho^2 <= 9 only; with rho left at 0 it includes them wherever they could be used, which is up to N rho^2 = 18: at 9 to 18 rounds in
+ * one launch are up to a quarter faster (strads_run) or a third (strads_round).  A workspace of either size is accepted. */
 int strads_workspace_bytes(const strads_lasso_config_t* cfg, size_t* out_bytes);
 
 /* Algorithm 1's initialisation: n_j = ||x_j||^2 for all j, resid = y - X beta, delta_j = C,
@@ -176,8 +178,8 @@ int strads_round(strads_handle_t h, const strads_round_out_t* out);
  * strads_run equals that of the same rounds run with strads_round, bit for bit.  The list drawn for the round
  * behind the last one stays: whoever writes delta (or beta, or resid) between two runs calls strads_set_round.
  *
- * CSC with one scheduler, and dense X with short columns (N rho^2 <= 9, N <= 2,048), run up to 32 whole rounds per
- * cooperative launch.  Otherwise the rounds are replayed from captured launch sequences: with one scheduler eight
+ * CSC with one scheduler, and dense X with short columns (N rho^2 <= 18, N <= 2,048, and a workspace that provides for
+ * it), run up to 32 whole rounds per cooperative launch.  Otherwise the rounds are replayed from captured launch sequences: with one scheduler eight
  * rounds each (the draw on a stream of its own beside the Gram and the walk), and what is left over of a run as
  * sequences of four, two and one round, each captured when its length comes up for the third time and
  * enqueued directly until then; with several schedulers 16 turns of each per sequence.  The streams, events and

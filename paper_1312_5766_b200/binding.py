@@ -176,7 +176,7 @@ class StradsLasso:
         cfg.layout, cfg.n_rows, cfg.n_cols, cfg.nnz, cfg.ld = self.layout, self.N, self.J, nnz, ld
         cfg.n_candidates, cfg.n_keep = self.n_candidates, self.n_keep
         self.n_schedulers = cfg.n_schedulers = int(n_schedulers)
-        cfg.flags, cfg.rho = flags, rho        # (the logistic loss adds the margin to the workspace; rho decides how rounds run)
+        cfg.flags = flags                      # (the logistic loss adds the margin to the workspace; rho left open: buffers for rounds in one launch)
         need = C.c_size_t(0)
         _check(lib.strads_workspace_bytes(C.byref(cfg), C.byref(need)), "strads_workspace_bytes")
         self.workspace = torch.empty(int(need.value), dtype=torch.uint8, device=dev)

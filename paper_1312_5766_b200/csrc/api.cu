@@ -217,25 +217,28 @@ int check_sizes(const strads_lasso_config_t* c) {
   return STRADS_OK;
 }
 
-// Whether the engine can take the rounds of one scheduler: CSC always; dense X with short columns and the default Gram.
+// Whether the engine can take the rounds: one scheduler; CSC always, dense X with short columns and the default Gram.
 bool engine_possible(const strads_lasso_config_t* c) {
-  if (c->flags & (STRADS_FLAG_SIMT_GRAM | STRADS_FLAG_GRAM_3XTF32)) return false;
+  if (n_sched_of(c) > 1 || (c->flags & (STRADS_FLAG_SIMT_GRAM | STRADS_FLAG_GRAM_3XTF32))) return false;
   return c->layout == STRADS_CSC || c->n_rows <= kEngineDenseRows;
 }
-// Whether the rounds go through it: one scheduler, and for dense X columns so short that independent ones correlate
-// beyond rho by chance (their correlations scatter with N^-1/2; the line is three of those).  There the launch chain's
-// screen leaves percents of all pairs open and its window fails round after round (463 x 508,999: 888 us per round as
-// launches, 56 here).  J = 50,000, rho = 0.1, P' = 8 P, us per round here / as launches for P = 16, 128, 512: 464 rows 28 / 96,
-// 53 / 367, 161 / 668; 880 rows 28 / 36, 32 / 48, 100 / 193; 1,060 rows 28 / 30, 33 / 37, 95 / 77; 1,200 rows 28 / 28, 33 / 32,
-// 50 / 40; 2,048 rows 28 / 23, 32 / 28, 46 / 37.  So below the line this is never the slower side; above it the launches are at
-// first up to a seventh slower while few are kept, and faster where many are.
+bool correlates_by_chance(const strads_lasso_config_t* c, double most) { return (double)c->n_rows * (double)c->rho * (double)c->rho <= most; }
+// Whether they go through it (where the workspace holds its buffers).  For dense X the correlations of independent columns scatter
+// with N^-1/2: with N rho^2 = 9 three of those reach rho, and below that the launch chain's screen leaves percents of all pairs open and
+// its window fails round after round (463 x 508,999: 888 us per round as launches, 36 here).  Above, both are chains of short steps: us
+// per round here / as launches at rho = 0.1, J = 50,000, strads_run with P = 16, 128 (P' = 8 P), then strads_round: 1,000 rows 26 / 31, 27 / 36,
+// 36 / 49, 40 / 57; 1,200 rows 26 / 28, 28 / 33, 36 / 46, 39 / 53; 1,752 rows 26 / 25, 28 / 32, 37 / 43, 38 / 51; 2,048 rows 26 / 23, 29 / 28,
+// 37 / 41, 39 / 47; P = 512 at 1,452 rows 34 / 39, 45 / 58.  The launches gain on it as fewer pairs are left open, so the line is in N rho^2:
+// at 17.5 neither is ahead by more than 2 % in strads_run and this by 8 to 25 % in strads_round, at 20.5 the launches by up to 14 %
+// (rho = 0.2: 880 rows, 35, 25 / 25; 1,452 rows, 58, 25 / 23).
 bool engine_chosen(const strads_lasso_config_t* c) {
-  if (!engine_possible(c) || n_sched_of(c) > 1) return false;
-  return c->layout == STRADS_CSC || (double)c->n_rows * (double)c->rho * (double)c->rho <= 9.0;
+  return engine_possible(c) && (c->layout == STRADS_CSC || correlates_by_chance(c, 18.0));
 }
-// Whether the workspace provides for it (1,000 x 10,000, P' = 200: 13.6 of 15.3 MB): where it is chosen.  A query of the size need not have
-// set rho; it is then answered for any.
-bool engine_provided(const strads_lasso_config_t* c) { return c->rho > 0.f ? engine_chosen(c) : engine_possible(c); }
+// Whether a query of the size asks for its buffers (1,000 x 10,000, P' = 200: 13.6 of 15.3 MB): with rho set, only below the first of those
+// lines, where the launches are two to twenty times slower; with rho left open, wherever it may be chosen.
+bool engine_provided(const strads_lasso_config_t* c) {
+  return engine_possible(c) && (c->layout == STRADS_CSC || !(c->rho > 0.f) || correlates_by_chance(c, 9.0));
+}
 // Keys each CTA can save of a scan that finds a few times `winners` of them in all.
 unsigned int engine_saved(size_t winners) { return (unsigned int)(winners / 16 + 64); }
 size_t engine_boundary(size_t winners) { return winners / 2 > 2048 ? winners / 2 : 2048; }
@@ -712,8 +715,8 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
   const int S = n_sched_of(c);
   const Layout Lrest = carve(c, false, false);
   const size_t rest = (size_t)(S - 1) * Lrest.total;
-  Layout L = carve(c, true, engine_provided(c));
-  // (a workspace sized for a larger rho, with which the engine would not be chosen, still does: without the engine)
+  Layout L = carve(c, true, engine_chosen(c));
+  // (dense X: a workspace without room for the engine's buffers does too, the rounds then go through the launch chain)
   if (L.engine && c->workspace_bytes < L.total + rest) L = carve(c, true, false);
   if (c->workspace_bytes < L.total + rest) return STRADS_ERR_WORKSPACE_TOO_SMALL;
 

@@ -25,10 +25,11 @@ def _fit(b, p, rounds, **kw):
     return out
 
 
-@pytest.mark.parametrize("kw", [dict(), dict(n_schedulers=4)])
-def test_handles_in_turn_and_side_by_side(kw):
+# (more rows: columns too long for rounds in one launch)
+@pytest.mark.parametrize("kw,more_rows", [(dict(), 0), (dict(), 1200), (dict(n_schedulers=4), 0)])
+def test_handles_in_turn_and_side_by_side(kw, more_rows):
     from paper_1312_5766_b200 import binding as b
-    problems = [wl.make_problem(SHAPES[name], seed=seed, device="cuda") for name in SHAPES for seed in (1, 2)]
+    problems = [wl.make_problem(dict(SHAPES[name], n_rows=SHAPES[name]["n_rows"] + more_rows), seed=seed, device="cuda") for name in SHAPES for seed in (1, 2)]
     rounds = (23, 23, 23, 70)                              # every length of captured sequence, left-overs launched one by one first
     b.load().strads_release_cached()
     want = []
@@ -63,6 +64,35 @@ def test_handles_in_turn_and_side_by_side(kw):
             for x, y in zip(out, want[i % 4]):
                 assert torch.equal(x, y), i
     assert b.load().strads_release_cached() == 0
+
+
+def test_dense_rounds_in_one_launch_beyond_the_first_line():
+    """1,200 rows, rho = 0.1 (N rho^2 = 12): with room for its buffers rounds go in one launch, without it by the launch chain; the
+    same blocks, and the same state up to the order of the dense products (each good to 2^-44 of its terms, then rounded to binary32)."""
+    import ctypes as C
+    from paper_1312_5766_b200 import binding as b
+    p = wl.make_problem(SHAPES["window"], seed=7, device="cuda")
+    s = b.StradsLasso.from_problem(p, device="cuda")
+    lib, cfg = b.load(), b.Config()
+    C.memmove(C.byref(cfg), C.byref(s._cfg), C.sizeof(cfg))
+    need = C.c_size_t(0)
+    assert lib.strads_workspace_bytes(C.byref(cfg), C.byref(need)) == 0 and need.value + (12 << 20) < s.workspace.numel()
+    ws = torch.empty(need.value, dtype=torch.uint8, device="cuda")
+    beta, resid, delta = torch.zeros_like(s.beta), torch.empty_like(s.resid), torch.empty_like(s.delta)
+    cfg.workspace, cfg.workspace_bytes = ws.data_ptr(), need.value
+    cfg.beta, cfg.resid, cfg.delta = beta.data_ptr(), resid.data_ptr(), delta.data_ptr()
+    h = C.c_void_p(None)
+    assert lib.strads_lasso_init(C.byref(cfg), C.byref(h)) == 0
+    cand, kept = torch.empty(p.n_candidates, dtype=torch.int32, device="cuda"), torch.empty(p.n_keep, dtype=torch.int32, device="cuda")
+    out = b.RoundOut()
+    out.cand, out.kept = cand.data_ptr(), kept.data_ptr()
+    for t in range(200):
+        assert lib.strads_round(h, C.byref(out)) == 0
+        mine = s.round()
+        assert torch.equal(mine[0], cand) and torch.equal(mine[1], kept), t
+    for x, y in ((s.beta, beta), (s.resid, resid), (s.delta, delta)):
+        assert float((x - y).norm()) <= 1e-5 * float(x.norm())
+    assert lib.strads_destroy(h) == 0
 
 
 def test_a_workspace_sized_for_another_rho():
