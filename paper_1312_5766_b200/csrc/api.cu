@@ -63,6 +63,10 @@ struct strads_lasso_s {
   bool engine_ok;
   Engine engine;
   alignas(64) unsigned char engine_maps[256];
+  // CSC with several schedulers, or with the static schedule: rounds by squads of CTAs (squads.cu)
+  bool squads_ok;
+  SquadSet squads;
+  long long lists_round;     // the round from which on every squad's list for its next one is in place (-1: none)
 };
 
 // The driver objects of a handle.  Making and destroying them costs far more than many a run (a captured sequence about
@@ -167,9 +171,15 @@ constexpr int kEdgeCap = 8192;        // conflicting pairs the Gram kernels can 
 constexpr int kEngineRounds = 32;     // rounds per launch of the engine: a launch every few hundred microseconds, so that other streams get their turn
 constexpr int kEngineDenseRows = 2048;
 constexpr int kEngineMaxCtas = 192;   // CTAs the engine's scratch provides for
+constexpr int kSquadRounds = 64;      // rounds per launch of the squads (the first block and the last update of a launch overlap with nothing)
+constexpr int kStaticSquads = 4;      // blocks under way with the static schedule
+constexpr int kSquadMinCtas = 8;      // CTAs of a squad at least
 constexpr int kAheadMaxKeep = 4096;   // sampling ahead: the patch kernel holds 2 P keys in shared memory
 
 Scheduler& on_turn(strads_lasso_s* h) { return h->sch[h->round_host % h->n_sched]; }
+
+// Lists of candidates drawn for rounds to come are not to be used: the priorities, or what the lists came with, change.
+void forget_lists(strads_lasso_s* h) { h->ahead_round = -1; h->lists_round = -1; }
 
 thread_local char g_cuda_err[256] = "";
 
@@ -193,6 +203,7 @@ struct Layout {
       off_ahead_state, off_ahead_hist, off_ahead_sure, off_ahead_boundary, off_ahead_keys, off_ahead_idx,
       off_eng_state, off_eng_hist, off_eng_cur, off_eng_win, off_eng_surv, off_eng_saved, off_eng_xb, off_eng_norm, off_eng_part, off_eng_tickets, total;
   long long eng_pitch, eng_lo;
+  long long eng_saved;
   int eng_list, eng_tiles;
   bool engine;
   int cap_sure, cap_boundary, mask_words, dot_parts, cap_amb, n_ahead, cap_ahead_boundary, cap_survivors;
@@ -217,9 +228,9 @@ int check_sizes(const strads_lasso_config_t* c) {
   return STRADS_OK;
 }
 
-// Whether the engine can take the rounds: one scheduler; CSC always, dense X with short columns and the default Gram.
+// Whether the engine can take the rounds of one scheduler: CSC always; dense X with short columns and the default Gram.
 bool engine_possible(const strads_lasso_config_t* c) {
-  if (n_sched_of(c) > 1 || (c->flags & (STRADS_FLAG_SIMT_GRAM | STRADS_FLAG_GRAM_3XTF32))) return false;
+  if (c->flags & (STRADS_FLAG_SIMT_GRAM | STRADS_FLAG_GRAM_3XTF32)) return false;
   return c->layout == STRADS_CSC || c->n_rows <= kEngineDenseRows;
 }
 bool correlates_by_chance(const strads_lasso_config_t* c, double most) { return (double)c->n_rows * (double)c->rho * (double)c->rho <= most; }
@@ -232,19 +243,25 @@ bool correlates_by_chance(const strads_lasso_config_t* c, double most) { return 
 // at 17.5 neither is ahead by more than 2 % in strads_run and this by 8 to 25 % in strads_round, at 20.5 the launches by up to 14 %
 // (rho = 0.2: 880 rows, 35, 25 / 25; 1,452 rows, 58, 25 / 23).
 bool engine_chosen(const strads_lasso_config_t* c) {
-  return engine_possible(c) && (c->layout == STRADS_CSC || correlates_by_chance(c, 18.0));
+  return engine_possible(c) && n_sched_of(c) == 1 && (c->layout == STRADS_CSC || correlates_by_chance(c, 18.0));
 }
 // Whether a query of the size asks for its buffers (1,000 x 10,000, P' = 200: 13.6 of 15.3 MB): with rho set, only below the first of those
 // lines, where the launches are two to twenty times slower; with rho left open, wherever it may be chosen.
 bool engine_provided(const strads_lasso_config_t* c) {
-  return engine_possible(c) && (c->layout == STRADS_CSC || !(c->rho > 0.f) || correlates_by_chance(c, 9.0));
+  return c->rho > 0.f ? engine_chosen(c) && (c->layout == STRADS_CSC || correlates_by_chance(c, 9.0)) : engine_possible(c);
+}
+// CSC rounds by squads of CTAs: how many blocks can be under way (1: blocks depend on the updates of the round before).
+int squads_of(const strads_lasso_config_t* c) {
+  if (c->layout != STRADS_CSC) return 1;
+  if (n_sched_of(c) > 1) return n_sched_of(c);
+  return (c->flags & STRADS_FLAG_UNIFORM_DRAW) && !(c->flags & STRADS_FLAG_DYNAMIC_DEPS) ? kStaticSquads : 1;
 }
 // Keys each CTA can save of a scan that finds a few times `winners` of them in all.
 unsigned int engine_saved(size_t winners) { return (unsigned int)(winners / 16 + 64); }
 size_t engine_boundary(size_t winners) { return winners / 2 > 2048 ? winners / 2 : 2048; }
 
-// Slice of the workspace of one scheduler; the first one (`first`) also holds what all share
-// (column norms, the objective's partial sums) and, with `engine`, the round engine's buffers.
+// Slice of the workspace of one scheduler or squad; the first one (`first`) also holds what all share
+// (column norms, the objective's partial sums).  `engine`: with the buffers of rounds in one launch.
 Layout carve(const strads_lasso_config_t* c, bool first, bool engine) {
   Layout L;
   L.cap_sure = c->n_candidates;
@@ -270,7 +287,7 @@ Layout carve(const strads_lasso_config_t* c, bool first, bool engine) {
   L.off_dbeta64 = take(sizeof(double) * (size_t)c->n_keep);
   L.off_conflict = take(sizeof(unsigned int) * (size_t)c->n_candidates * L.mask_words);
   const bool dense = c->layout == STRADS_DENSE_COLMAJOR;
-  L.engine = first && engine;
+  L.engine = engine;
   const bool proposals = dense || L.engine;
   L.off_cand_dbeta64 = take(proposals ? sizeof(double) * (size_t)c->n_candidates : 0);
   L.off_cand_bnew = take(proposals ? sizeof(float) * (size_t)c->n_candidates : 0);
@@ -328,7 +345,10 @@ Layout carve(const strads_lasso_config_t* c, bool first, bool engine) {
   L.off_eng_hist = take(en ? sizeof(unsigned int) * kHistBins : 0);
   L.off_eng_cur = take(en ? sizeof(unsigned int) * kHistBins : 0);
   L.off_eng_win = take(en ? sizeof(unsigned long long) * (most + engine_boundary(most)) : 0);
-  L.off_eng_surv = take(en ? sizeof(unsigned long long) * kEngineMaxCtas * (size_t)engine_saved(most) : 0);
+  // (a squad has half the CTAs at most, so that less is lost where they find unevenly many)
+  const bool whole = first && n_sched_of(c) == 1;
+  L.eng_saved = en ? (whole ? (long long)kEngineMaxCtas * engine_saved(most) : 10 * (long long)most + 64 * kEngineMaxCtas / 2) : 0;
+  L.off_eng_surv = take(sizeof(unsigned long long) * (size_t)L.eng_saved);
   L.off_eng_saved = take(en ? sizeof(unsigned int) * kEngineMaxCtas : 0);
   L.eng_lo = (c->n_rows + 127) / 128 * 128;
   L.eng_pitch = 2 * L.eng_lo;
@@ -418,7 +438,7 @@ bool update_after_pack(const Problem& p, bool gram_exported) {
 // One round, every step on the caller's stream, by the scheduler whose turn it is.
 // before_gram: an event steps 2 and 3 have to wait for (state still on its way from the host; the draw needs only delta).
 int one_round(strads_lasso_s* h, const strads_round_out_t* out, cudaEvent_t before_gram = nullptr) {
-  h->ahead_round = -1;                                 // delta changes without a new early list
+  forget_lists(h);                                     // delta changes without a new early list
   const Scheduler& sc = on_turn(h);
   const Problem& p = sc.p;
   cudaEvent_t* ev = (h->prof_events != nullptr && h->prof_rounds < h->prof_cap) ? h->prof_events + kProfEvents * h->prof_rounds : nullptr;
@@ -638,7 +658,8 @@ void fill_ahead(Problem& a, const Problem& p0, const Layout& L, char* ws) {
   a.survivors = nullptr; a.cap_survivors = 0;         // (the early draw is off the round's path: it keeps to the plain passes)
 }
 
-void fill_engine(Engine& en, const Problem& p, const Layout& L, char* ws) {
+// For n_ctas CTAs; whole: all of them, one round after the other.
+void fill_engine(Engine& en, const Problem& p, const Layout& L, char* ws, int n_ctas, bool whole) {
   en.es = reinterpret_cast<EngineState*>(ws + L.off_eng_state);
   en.hist = reinterpret_cast<unsigned int*>(ws + L.off_eng_hist);
   en.bin_cur = reinterpret_cast<unsigned int*>(ws + L.off_eng_cur);
@@ -648,8 +669,8 @@ void fill_engine(Engine& en, const Problem& p, const Layout& L, char* ws) {
   en.cap_win = (int)most + en.cap_boundary;
   en.surv = reinterpret_cast<unsigned long long*>(ws + L.off_eng_surv);
   en.saved = reinterpret_cast<unsigned int*>(ws + L.off_eng_saved);
-  en.cap_surv = engine_saved(most);
-  en.n_list = L.eng_list;
+  en.cap_surv = whole ? engine_saved(most) : (unsigned int)(L.eng_saved / n_ctas);
+  en.n_list = L.eng_list < owned_count(p) ? L.eng_list : (int)owned_count(p);
   en.window = window_of(p, p.n_cand);
   en.xb = reinterpret_cast<unsigned short*>(ws + L.off_eng_xb);
   en.xb_pitch = L.eng_pitch; en.lo_off = L.eng_lo;
@@ -659,21 +680,27 @@ void fill_engine(Engine& en, const Problem& p, const Layout& L, char* ws) {
   en.tile_ticket = reinterpret_cast<unsigned int*>(ws + L.off_eng_tickets);
 }
 
-// What must be zero before a launch of the engine (it leaves it so, unless a wait expired).
-cudaError_t clear_engine(const strads_lasso_s* h) {
-  const Engine& en = h->engine;
-  const Problem& p = h->sch[0].p;
+// What must be zero before a launch of the engine or the squads (they leave it so, unless a wait expired).
+cudaError_t clear_engine(const Problem& p, const Engine& en, cudaStream_t s) {
   cudaError_t e;
-  if ((e = cudaMemsetAsync(en.es, 0, sizeof(EngineState), h->stream)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(en.hist, 0, sizeof(unsigned int) * kHistBins, h->stream)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(en.es, 0, sizeof(EngineState), s)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(en.hist, 0, sizeof(unsigned int) * kHistBins, s)) != cudaSuccess) return e;
   if (p.layout == STRADS_DENSE_COLMAJOR) {
     const long long side = (p.n_cand + 63) / 64;
-    return cudaMemsetAsync(en.tile_ticket, 0, sizeof(unsigned int) * (size_t)(side * (side + 1) / 2), h->stream);
+    return cudaMemsetAsync(en.tile_ticket, 0, sizeof(unsigned int) * (size_t)(side * (side + 1) / 2), s);
   }
   if (p.bucket_count != nullptr &&
-      (e = cudaMemsetAsync(p.bucket_count, 0, sizeof(unsigned int) * (size_t)p.N, h->stream)) != cudaSuccess) return e;
-  return cudaMemsetAsync(p.resid_acc, 0, sizeof(long long) * (size_t)p.N, h->stream);
+      (e = cudaMemsetAsync(p.bucket_count, 0, sizeof(unsigned int) * (size_t)p.N, s)) != cudaSuccess) return e;
+  return cudaMemsetAsync(p.resid_acc, 0, sizeof(long long) * (size_t)p.N, s);
 }
+cudaError_t clear_engines(const strads_lasso_s* h) {
+  cudaError_t e = cudaSuccess;
+  if (h->engine_ok && (e = clear_engine(h->sch[0].p, h->engine, h->stream)) != cudaSuccess) return e;
+  for (int i = 0; h->squads_ok && i < h->squads.n; ++i)
+    if ((e = clear_engine(h->squads.p[i], h->squads.e[i], h->stream)) != cudaSuccess) return e;
+  return e;
+}
+
 
 // The engine takes a round unless the steps are timed one by one or the Gram matrix itself is asked for.
 bool engine_runs(const strads_lasso_s* h, const strads_round_out_t* out) {
@@ -693,7 +720,8 @@ int strads_workspace_bytes(const strads_lasso_config_t* cfg, size_t* out_bytes) 
   if (out_bytes == nullptr) return STRADS_ERR_INVALID_ARG;
   const int rc = check_sizes(cfg);
   if (rc) return rc;
-  *out_bytes = carve(cfg, true, engine_provided(cfg)).total + (size_t)(n_sched_of(cfg) - 1) * carve(cfg, false, false).total;
+  const int n = squads_of(cfg) > n_sched_of(cfg) ? squads_of(cfg) : n_sched_of(cfg);
+  *out_bytes = carve(cfg, true, engine_provided(cfg) || squads_of(cfg) > 1).total + (size_t)(n - 1) * carve(cfg, false, squads_of(cfg) > 1).total;
   return STRADS_OK;
 }
 
@@ -713,12 +741,13 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
   // first phase turns from a randomised sweep into one in index order
   if (c->c_init > STRADS_MAX_C_INIT) return STRADS_ERR_INVALID_ARG;
   const int S = n_sched_of(c);
-  const Layout Lrest = carve(c, false, false);
-  const size_t rest = (size_t)(S - 1) * Lrest.total;
-  Layout L = carve(c, true, engine_chosen(c));
-  // (dense X: a workspace without room for the engine's buffers does too, the rounds then go through the launch chain)
-  if (L.engine && c->workspace_bytes < L.total + rest) L = carve(c, true, false);
-  if (c->workspace_bytes < L.total + rest) return STRADS_ERR_WORKSPACE_TOO_SMALL;
+  int Q = squads_of(c);
+  Layout L = carve(c, true, engine_chosen(c) || Q > 1), Lrest = carve(c, false, Q > 1);
+  auto need = [&]() { return L.total + (size_t)((Q > S ? Q : S) - 1) * Lrest.total; };
+  // (a workspace without room for the squads or the engine does too, the rounds then go without them)
+  if (Q > 1 && c->workspace_bytes < need()) { Q = 1; L = carve(c, true, engine_chosen(c)); Lrest = carve(c, false, false); }
+  if (L.engine && c->workspace_bytes < need()) L = carve(c, true, false);
+  if (c->workspace_bytes < need()) return STRADS_ERR_WORKSPACE_TOO_SMALL;
 
   strads_lasso_s* h = new (std::nothrow) strads_lasso_s();     // value-initialised: every pointer null
   if (h == nullptr) return STRADS_ERR_INVALID_ARG;
@@ -754,10 +783,10 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
       (e = want_event(&kit.copy_done)) != cudaSuccess)
     return fail(cuda_fail(e, "copy stream"));
   h->copy_stream = kit.copy; h->copy_fork = kit.copy_fork; h->copy_done = kit.copy_done;
-  h->ahead_round = -1;
-  h->engine_ok = L.engine && sm_count <= kEngineMaxCtas;
+  forget_lists(h);
+  h->engine_ok = S == 1 && L.engine && sm_count <= kEngineMaxCtas;
   if (h->engine_ok) {
-    fill_engine(h->engine, p0, L, ws);
+    fill_engine(h->engine, p0, L, ws, sm_count, true);
     if ((e = prepare_engine(p0, h->engine)) != cudaSuccess) return fail(cuda_fail(e, "prepare_engine"));
     if (p0.layout == STRADS_DENSE_COLMAJOR && (e = encode_engine_maps(p0, h->engine, h->engine_maps)) != cudaSuccess)
       return fail(cuda_fail(e, "encode_engine_maps"));
@@ -802,7 +831,25 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
       sc.stream = kit.sched[s]; sc.block_ready = kit.ready[s]; sc.updated = kit.updated[s];
     }
   }
-  if (h->engine_ok && (e = clear_engine(h)) != cudaSuccess) return fail(cuda_fail(e, "clear_engine"));
+  h->squads_ok = Q > 1 && sm_count <= kEngineMaxCtas && sm_count / Q >= kSquadMinCtas;
+  if (h->squads_ok) {
+    SquadSet& set = h->squads;
+    set.n = Q; set.size = sm_count / Q;
+    for (int i = 0; i < Q; ++i) {
+      const Layout& Li = i == 0 ? L : Lrest;
+      char* at = i == 0 ? ws : ws + L.total + (size_t)(i - 1) * Lrest.total;
+      if (S > 1) {
+        set.p[i] = h->sch[i].p;
+      } else {                                           // one scheduler's blocks: everything of a slice but the state
+        fill_problem(set.p[i], c, Li, at, 0, 1, i == 0 ? nullptr : &p0);
+        set.p[i].st = p0.st; set.p[i].round_ptr = p0.round_ptr;
+      }
+      fill_engine(set.e[i], set.p[i], Li, at, set.size, false);
+      set.e[i].grid = set.size;
+    }
+    if ((e = prepare_squads()) != cudaSuccess) return fail(cuda_fail(e, "prepare_squads"));
+  }
+  if ((e = clear_engines(h)) != cudaSuccess) return fail(cuda_fail(e, "clear_engines"));
   if (S > 1 && (e = want_event(&kit.fork)) != cudaSuccess) return fail(cuda_fail(e, "cudaEventCreate"));
   h->fork = kit.fork;
   *out_handle = h;
@@ -812,7 +859,7 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
 int strads_round(strads_handle_t h, const strads_round_out_t* out) {
   if (h == nullptr) return STRADS_ERR_INVALID_ARG;
   if (engine_runs(h, out)) {
-    h->ahead_round = -1;
+    forget_lists(h);
     CK(launch_engine(h->sch[0].p, h->engine, h->engine_maps, 1, false, false, out, h->stream));
     h->round_host += 1;
     return STRADS_OK;
@@ -886,7 +933,20 @@ static int build_round_graph(strads_lasso_s* h, int tail_kind = -1) {
 
 int strads_run(strads_handle_t h, int64_t n_rounds) {
   if (h == nullptr || n_rounds < 0) return STRADS_ERR_INVALID_ARG;
+  // (with one scheduler a run too short for every squad to have a round or two goes one round after the other)
+  if (h->squads_ok && h->prof_events == nullptr && (h->n_sched > 1 || n_rounds >= 2 * h->squads.n)) {
+    h->ahead_round = -1;
+    while (n_rounds > 0) {
+      const int n = n_rounds < kSquadRounds ? (int)n_rounds : kSquadRounds;
+      CK(launch_squads(h->squads, n, h->lists_round == h->round_host, true, h->stream));
+      h->round_host += n;
+      h->lists_round = h->squads.e[0].n_list > 0 ? h->round_host : -1;
+      n_rounds -= n;
+    }
+    return STRADS_OK;
+  }
   if (engine_runs(h, nullptr)) {
+    h->lists_round = -1;
     while (n_rounds > 0) {
       const int n = n_rounds < kEngineRounds ? (int)n_rounds : kEngineRounds;
       const bool ahead = h->engine.n_list > 0;
@@ -1028,7 +1088,7 @@ int strads_filter(strads_handle_t h, const int32_t* cand_dev, int32_t n_cand, in
   if (h == nullptr || cand_dev == nullptr || kept_dev == nullptr) return STRADS_ERR_INVALID_ARG;
   const Scheduler& sc = on_turn(h);
   if (n_cand < 0 || n_cand > sc.p.n_cand) return STRADS_ERR_INVALID_ARG;
-  h->ahead_round = -1;                                 // (the early list is corrected from the last round's kept list)
+  forget_lists(h);                                     // (the early list is corrected from the last round's kept list)
   CK(launch_set_counts(sc.p, n_cand, 0, 0, h->stream));
   const int rc = gram_and_filter(sc, h->stream, cand_dev, n_cand, gram_dev_or_null);
   if (rc) return rc;
@@ -1040,7 +1100,7 @@ int strads_update(strads_handle_t h, const int32_t* kept_dev, int32_t n_kept, fl
   if (h == nullptr) return STRADS_ERR_INVALID_ARG;
   const Problem& p = on_turn(h).p;
   if (n_kept < 0 || n_kept > p.n_keep || (n_kept > 0 && kept_dev == nullptr)) return STRADS_ERR_INVALID_ARG;
-  h->ahead_round = -1;
+  forget_lists(h);
   CK(launch_set_counts(p, n_kept, n_kept, n_kept, h->stream));
   if (n_kept > 0)
     CK(cudaMemcpyAsync(p.kept, kept_dev, sizeof(int) * n_kept, cudaMemcpyDeviceToDevice, h->stream));
@@ -1058,7 +1118,7 @@ int strads_get_round(strads_handle_t h, int64_t* t) {
 int strads_set_round(strads_handle_t h, int64_t t) {
   if (h == nullptr || t < 0) return STRADS_ERR_INVALID_ARG;
   h->round_host = t;
-  h->ahead_round = -1;
+  forget_lists(h);
   unsigned long long next[STRADS_MAX_SCHEDULERS];          // every scheduler's next turn at or after t
   for (int s = 0; s < h->n_sched; ++s) {
     next[s] = (unsigned long long)t + (unsigned long long)(((s - t % h->n_sched) + h->n_sched) % h->n_sched);
@@ -1104,6 +1164,7 @@ int strads_set_wait_limit(strads_handle_t h, uint32_t iterations) {
   CK(cudaStreamSynchronize(h->stream));
   for (int s = 0; s < h->n_sched; ++s) h->sch[s].p.wait_limit = iterations;
   h->ahead.wait_limit = iterations;
+  for (Problem& p : h->squads.p) p.wait_limit = iterations;
   drop_round_graph(h);
   return STRADS_OK;
 }
@@ -1118,6 +1179,7 @@ int strads_inject_stall(strads_handle_t h, int32_t which) {
     // an arrival count no barrier of the walk can complete from
     CK(cudaMemsetAsync(&sc.p.walk_ctl->bar_count, 0x40, sizeof(unsigned int), h->stream));
     if (h->engine_ok) CK(cudaMemsetAsync(&h->engine.es->bar_count, 0x40, sizeof(unsigned int), h->stream));
+    if (h->squads_ok) CK(cudaMemsetAsync(&h->squads.e[h->round_host % h->squads.n].es->bar_count, 0x40, sizeof(unsigned int), h->stream));
   } else if (which == STRADS_STALL_GRAM_LOADS) {
     if (sc.p.layout != STRADS_DENSE_COLMAJOR) return STRADS_ERR_INVALID_ARG;
     sc.p.stall = 1;
@@ -1139,9 +1201,9 @@ int strads_recover(strads_handle_t h) {
     CK(cudaMemsetAsync(&p.st->status, 0, sizeof(unsigned int), h->stream));
     if (p.layout == STRADS_CSC) CK(cudaMemsetAsync(p.walk_ctl, 0, sizeof(WalkControl), h->stream));
   }
-  if (h->engine_ok) CK(clear_engine(h));
+  CK(clear_engines(h));
   if (had_stall) drop_round_graph(h);
-  h->ahead_round = -1;                                   // (whatever was drawn ahead belongs to the abandoned rounds)
+  forget_lists(h);                                       // (whatever was drawn ahead belongs to the abandoned rounds)
   CK(cudaStreamSynchronize(h->stream));
   return STRADS_OK;
 }

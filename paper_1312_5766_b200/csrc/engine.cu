@@ -812,7 +812,6 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
   __shared__ ChangeShared cs;
   __shared__ __align__(8) PackBars pb;
   __shared__ __align__(16) GramShared gs;
-  __shared__ int s_kept, s_examined;
   // Copies for the functions that are called rarely and not inlined, made when they are: a reference to the parameters themselves would make
   // every access to them, in the hot code too, a load from memory.
   __shared__ Problem sp;
@@ -942,56 +941,19 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
       if (!collected && !csc_window && !during_walk) { draw_gather<AllThreads>(WholeGrid(), p, e, ds, k, spare); collected = true; }
       if (!kDense && real) {
         if (!window) {
-          unsigned char* sm_scan = sm + sizeof(DemandShared);
-          unsigned int* sh = reinterpret_cast<unsigned int*>(sm_scan);
-          const float cut = during_walk ? scan_open(WholeGrid(), e, ds, sm_scan, true) : 0.f;
-          const Binning bins = binning_of(cut);
-          const WeightForm wf = weight_form(p);
-          auto draw = [&]() {
-            if (!during_walk) return true;
-            WarpScan scan = begin_scan(cut, scan_queue(sm_scan), (warp - kWalkWarps) * n_ctas + cta, (kWarps - kWalkWarps) * n_ctas);
-#pragma unroll 1
-            while (scan_step(p, td, wf, scan, [&](unsigned long long key, bool on) { scan_found(WholeGrid(), e, ds, sh, bins, key, on); })) {}
-            scan_close<OtherThreads>(WholeGrid(), e, ds, sm_scan);
-            __shared__ int s_over;
-            g_draw.target += g_draw.n;
-            OtherThreads::sync();
-            if (OtherThreads::tid() == 0) s_over = grid_wait(g_draw);
-            OtherThreads::sync();
-            if (!s_over) return false;
-            draw_gather<OtherThreads>(WholeGrid(), p, e, ds, k, false);
-            return true;
-          };
           int walked = 0;
-          if (!(ok = csc_walk_on_demand(WholeGrid(), p, sp, e, sm, g, g_draw, &walked, draw))) break;
+          if (!(ok = csc_walk_and_draw(WholeGrid(), p, sp, e, ds, sm, g, g_draw, during_walk, td, k, &walked))) break;
           if (during_walk) scanned = collected = true;
-          csc_products(WholeGrid(), p, e, ts, sm, walked, true, false, t + 1, draws);
+          csc_products<true>(WholeGrid(), p, e, ts, sm, walked, true, false, t + 1, draws);
         } else {
-          csc_products(WholeGrid(), p, e, ts, sm, n, false, csc_window, t + 1, draws);
+          csc_products<true>(WholeGrid(), p, e, ts, sm, n, false, csc_window, t + 1, draws);
         }
       }
       if (!(ok = grid_sync(g))) break;
       if (!real || no_filter) break;
       if (!kDense) {
         if (!window) break;
-        if (walker) {
-          const unsigned int edges = es->edge_count;
-          const int failed = es->bucket_failed;
-          if (tid == 0) { s_kept = 0; s_examined = n; }
-          __syncthreads();
-          bool settled = !failed && edges <= (unsigned)p.cap_edges;
-          if (settled) settled = walk_from_pair_list<kT>(p, p.cand, n, edges, sm, p.kept, &s_kept, &s_examined);
-          __syncthreads();
-          if (tid == 0) {
-            es->n_kept = s_kept; es->n_examined = s_examined;
-            es->walk_open = !settled || (s_kept < p.n_keep && n < n_total) ? 1 : 0;
-            // after an overflow the buckets are left alone: for a round, then twice as long after every further one, to 64
-            // (a count of rounds, not the round to wait for: strads_set_round may go back); this round's walk counts too
-            if (!settled) es->avoid = 1 + (1 << es->streak);
-            es->streak = settled ? 0 : min(es->streak + 1, 6);
-            es->bucket_failed = 0; es->edge_count = 0u;
-          }
-        }
+        if (walker) csc_walk_window(p, e, sm, n);
         const ClearAhead rows = csc_clear_begin(WholeGrid(), p, n);
         if (!collected) { draw_gather<AllThreads>(WholeGrid(), p, e, ds, k, true); collected = true; spare = true; }
         csc_clear_end(p, rows);
@@ -1019,7 +981,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
       commit_changes(p, e, nk, n_moving, out, final_round);
       last.nk = nk; last.n_moving = n_moving;
       if (!kDense) {
-        last.shift = csc_shift(p, cs.dmax, nk);
+        last.shift = csc_shift(p.st->x_abs_max, cs.dmax, nk);
         csc_scatter(WholeGrid(), p, nk, last.shift);
       }
       --left;

@@ -19,8 +19,16 @@ struct EngineState {
   int mend;                     // a draw's selection has to be mended
   int streak;                   // CSC: attempts with the row buckets in a row that overflowed (or left the walk open)
   int avoid;                    // CSC: rounds until they are tried again
+  // rounds prepared by squads of CTAs (squads.cu): the round whose turn it is, and (in the first squad's) the turns
+  unsigned int turn_moving;     // kept coefficients that move
+  unsigned long long turn_dmax; // bits of the largest |change|
+  unsigned int turn_count;      // arrivals: one per CTA of the launch at its start, then one per CTA of a squad whose turn is over
+  unsigned int turn_exit;       // CTAs of the launch that have left
   int dirty;                    // strads_sample_static: the last call gave up and left the histogram as it was
 };
+
+// The coefficients that a scheduler draws from.
+__host__ __device__ inline long long owned_count(const Problem& p) { return (p.J - p.part_index + p.part_count - 1) / p.part_count; }
 
 // How the pairs of a list are cut into tiles of the dense Gram: kGramRows x cols, K in stages of 64 elements, `split` CTAs sharing a tile with `per` stages each.
 constexpr int kGramRows = 128;
@@ -85,6 +93,18 @@ size_t engine_smem(const Problem& p, bool ahead);
 cudaError_t encode_engine_maps(const Problem& p, const Engine& e, void* out_256_bytes);
 cudaError_t launch_engine(const Problem& p, const Engine& e, const void* maps, int n_rounds, bool have_list, bool draw_next,
                           const strads_round_out_t* out, cudaStream_t s);
+
+// CSC rounds whose blocks do not wait for one another's updates: several schedulers, or the static schedule.  As many squads of CTAs as
+// there are blocks under way; problem i / engine i: the i-th squad's, which takes the rounds t with t mod n == i.
+constexpr int kMaxSquads = STRADS_MAX_SCHEDULERS;
+struct SquadSet {
+  Problem p[kMaxSquads];
+  Engine e[kMaxSquads];
+  int n, size;                  // squads, CTAs of each
+};
+cudaError_t prepare_squads();
+// have_list: every squad's list for its next round is in place; draw_next: leave them so.
+cudaError_t launch_squads(const SquadSet& set, int n_rounds, bool have_list, bool draw_next, cudaStream_t s);
 
 // The draw alone: p.cand[0 .. p.n_cand) for round t from p.delta (e: es, hist, bin_cur and win).  The barrier in es is zero before
 // and after, and hist unless es->dirty says otherwise.

@@ -105,7 +105,7 @@ __device__ __forceinline__ bool in_conflict(float dot, float limit_a, double n2a
   return conflict_exactly(dot, n2a, b->n2, rho);
 }
 
-// x_c^T r and the would-be changes of candidates [0, count) (kept: of the kept ones), and with `pairs` their inner
+// x_c^T r and the would-be changes (kDots) of candidates [0, count) (kept: of the kept ones), and with `pairs` their inner
 // products with the later candidates that share a row with them.  The CTA's k-th entry is cta + k * ctas; a warp per entry.
 // What bounds it is the chain of dependent far accesses -- column, row, bucket -- so each link's loads go out together,
 // and then the number of instructions per term.  The terms of 64 positions are laid out in the order of positions and dealt to
@@ -127,7 +127,7 @@ __device__ __forceinline__ void csc_products_begin(const Problem& p, const Engin
     for (int i = threadIdx.x & 31; i < kReach / 4; i += 32) reinterpret_cast<float4*>(wt.dot)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   if (!(p.flags & STRADS_FLAG_DYNAMIC_DEPS)) csc_norms(p, e, sm, count);
 }
-template <typename Crew>
+template <bool kDots, typename Crew>
 __device__ __forceinline__ void csc_products(const Crew& crew, const Problem& p, const Engine& e, TurnShared& ts, unsigned char* sm, int count, bool kept, bool pairs,
                                              unsigned long long t_next, bool want_keys) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -146,6 +146,7 @@ __device__ __forceinline__ void csc_products(const Crew& crew, const Problem& p,
     const int turn = min(kTurn, mine - k0);
     if (k0 > 0) __syncthreads();
     if (warp == kWorkers) {
+      if (!kDots) continue;
       int j_own = 0, pos_own = 0;
       float E = 0.f;
       Proposal prop = {};
@@ -162,13 +163,14 @@ __device__ __forceinline__ void csc_products(const Crew& crew, const Problem& p,
       if (lane < turn) propose_end(p, prop, pos_own, j_own, ts.dot[lane][0], E, want_keys);
       continue;
     }
-    if (warp >= turn) asm volatile("bar.arrive 4, %0;" ::"n"(kT) : "memory");
+    if (kDots && warp >= turn) asm volatile("bar.arrive 4, %0;" ::"n"(kT) : "memory");
 #pragma unroll 1
     for (int k = warp; k < turn; k += kWorkers) {
       const int a = cta + n_ctas * (k0 + k);
       const WalkColumn col = p.walk_cols[kept ? p.kept_pos[a] : a];
       double acc = 0.0;
       auto tell = [&]() {                                // this candidate's x_c^T r; the last one of the warp's: all of them
+        if (!kDots) return;
         acc = warp_sum(acc);
         if (lane == 0) ts.dot[k][0] = acc;
         if (k + kWorkers >= turn) {
@@ -197,13 +199,13 @@ __device__ __forceinline__ void csc_products(const Crew& crew, const Problem& p,
           float x[2];
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            x[h] = r[h] >= 0 && reach == reach0 ? p.resid[r[h]] : 0.f;
+            x[h] = kDots && r[h] >= 0 && reach == reach0 ? p.resid[r[h]] : 0.f;
             cnt[h] = pairs && r[h] >= 0 ? p.bucket_count[r[h]] : 0u;
           }
           if (reach == reach0) {
 #pragma unroll
             for (int h = 0; h < 2; ++h)
-              if (r[h] >= 0) acc += (double)v[h] * (double)x[h];
+              if (kDots && r[h] >= 0) acc += (double)v[h] * (double)x[h];
             if (q0 + kPart >= col.n) tell();
           }
           if (!pairs) continue;
@@ -330,11 +332,11 @@ __device__ __forceinline__ void csc_products(const Crew& crew, const Problem& p,
 // CSC, step 4 and the next step 1: the residual.  Contributions are added as 64-bit fixed-point integers (unit 2^-shift, the
 // same bits in any order) and every row with a non-zero accumulator is updated once behind the next barrier.
 // ------------------------------------------------------------------------------------------------
-__device__ __forceinline__ int csc_shift(const Problem& p, unsigned long long dmax_bits, int nk) {
+__device__ __forceinline__ int csc_shift(float x_abs_max, unsigned long long dmax_bits, int nk) {
   const double m = __longlong_as_double((long long)dmax_bits);
   if (!(m > 0.0) || !isfinite(m)) return INT_MIN;
   int x = 0;
-  frexp(m * (double)p.st->x_abs_max * (double)max(nk, 1), &x);
+  frexp(m * (double)x_abs_max * (double)max(nk, 1), &x);
   return 61 - x;
 }
 
@@ -360,6 +362,16 @@ __device__ void csc_scatter(const Crew& crew, const Problem& p, int nk, int shif
 }
 
 template <typename Crew>
+__device__ __forceinline__ void csc_apply_rows(const Crew& crew, const Problem& p, int shift) {
+  for (long long r = (long long)crew.rank() * kT + threadIdx.x; r < p.N; r += (long long)crew.size() * kT) {
+    const long long v = p.resid_acc[r];
+    if (v != 0) {
+      apply_row(p, r, ldexp((double)v, -shift));
+      p.resid_acc[r] = 0;
+    }
+  }
+}
+template <typename Crew>
 __device__ void csc_apply(const Crew& crew, const Problem& p, int nk, int n_moving, int shift) {
   if (shift == INT_MIN) return;
   // few moving entries against the rows: visit the entries' rows (the first visitor of a row takes its sum), else all rows
@@ -371,13 +383,7 @@ __device__ void csc_apply(const Crew& crew, const Problem& p, int nk, int n_movi
     });
     return;
   }
-  for (long long r = (long long)crew.rank() * kT + threadIdx.x; r < p.N; r += (long long)crew.size() * kT) {
-    const long long v = p.resid_acc[r];
-    if (v != 0) {
-      apply_row(p, r, ldexp((double)v, -shift));
-      p.resid_acc[r] = 0;
-    }
-  }
+  csc_apply_rows(crew, p, shift);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1049,6 +1055,57 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Crew& crew, const Probl
   g.target = s.target; g_draw.target = s.draw_target;
   *n_kept = s.kept;
   return s.ok != 0 && s.drawn != 0;
+}
+
+// The walk from the list of the window's conflicting pairs, by one CTA.
+__device__ __forceinline__ void csc_walk_window(const Problem& p, const Engine& e, unsigned char* sm, int n) {
+  __shared__ int s_kept, s_examined;
+  EngineState* es = e.es;
+  const unsigned int edges = es->edge_count;
+  const int failed = es->bucket_failed, tid = threadIdx.x;
+  if (tid == 0) { s_kept = 0; s_examined = n; }
+  __syncthreads();
+  bool settled = !failed && edges <= (unsigned)p.cap_edges;
+  if (settled) settled = walk_from_pair_list<kT>(p, p.cand, n, edges, sm, p.kept, &s_kept, &s_examined);
+  __syncthreads();
+  if (tid == 0) {
+    es->n_kept = s_kept; es->n_examined = s_examined;
+    es->walk_open = !settled || (s_kept < p.n_keep && n < p.n_cand) ? 1 : 0;
+    // after an overflow the buckets are left alone: for a round, then twice as long after every further one, to 64
+    // (a count of rounds, not the round to wait for: strads_set_round may go back); this round's walk counts too
+    if (!settled) es->avoid = 1 + (1 << es->streak);
+    es->streak = settled ? 0 : min(es->streak + 1, 6);
+    es->bucket_failed = 0; es->edge_count = 0u;
+  }
+}
+
+// The walk over all candidates by half the warps, with `draws` the draw of round td up to the collection of its k winners by the
+// others.  False: a barrier gave up.
+template <typename Crew>
+__device__ __forceinline__ bool csc_walk_and_draw(const Crew& crew, const Problem& p, Problem& sp, const Engine& e, DrawShared& ds, unsigned char* sm, Grid& g,
+                                                  Grid& g_draw, bool draws, unsigned long long td, unsigned int k, int* n_kept) {
+  const int warp = (int)threadIdx.x >> 5;
+  unsigned char* sm_scan = sm + sizeof(DemandShared);
+  unsigned int* sh = reinterpret_cast<unsigned int*>(sm_scan);
+  const float cut = draws ? scan_open(crew, e, ds, sm_scan, true) : 0.f;
+  const Binning bins = binning_of(cut);
+  const WeightForm wf = weight_form(p);
+  auto draw = [&]() {
+    if (!draws) return true;
+    WarpScan scan = begin_scan(cut, scan_queue(sm_scan), (warp - kWalkWarps) * crew.size() + crew.rank(), (kWarps - kWalkWarps) * crew.size());
+#pragma unroll 1
+    while (scan_step<Crew::kParts>(p, td, wf, scan, [&](unsigned long long key, bool on) { scan_found(crew, e, ds, sh, bins, key, on); })) {}
+    scan_close<OtherThreads>(crew, e, ds, sm_scan);
+    __shared__ int s_over;
+    g_draw.target += g_draw.n;
+    OtherThreads::sync();
+    if (OtherThreads::tid() == 0) s_over = grid_wait(g_draw);
+    OtherThreads::sync();
+    if (!s_over) return false;
+    draw_gather<OtherThreads>(crew, p, e, ds, k, false);
+    return true;
+  };
+  return csc_walk_on_demand(crew, p, sp, e, sm, g, g_draw, n_kept, draw);
 }
 
 }  // namespace

@@ -61,10 +61,12 @@ __device__ bool grid_complete(const Grid& g) {
 
 // The CTAs that make a round together: all of them, or as many of them as prepare the rounds whose turn is theirs (squads.cu).
 struct WholeGrid {
+  static constexpr bool kParts = false;    // all coefficients
   __device__ __forceinline__ int rank() const { return (int)blockIdx.x; }
   __device__ __forceinline__ int size() const { return (int)gridDim.x; }
 };
 struct Squad {
+  static constexpr bool kParts = true;     // a scheduler's
   int r, n;
   __device__ __forceinline__ int rank() const { return r; }
   __device__ __forceinline__ int size() const { return n; }
@@ -176,7 +178,7 @@ __device__ __forceinline__ WarpScan begin_scan(float cut, uint2* queue, int warp
   return s;
 }
 // One step; past the end it only empties the queue.  Whether there was anything to do.
-template <typename F>
+template <bool kParts, typename F>
 __device__ __forceinline__ bool scan_step(const Problem& p, unsigned long long t, const WeightForm& wf, WarpScan& s, F&& f) {
   const int lane = threadIdx.x & 31;
   const long long groups = (p.J + 3) >> 2, whole = p.J >> 2, g = s.next + lane;
@@ -202,6 +204,16 @@ __device__ __forceinline__ bool scan_step(const Problem& p, unsigned long long t
 #pragma unroll
       for (int i = 0; i < 4; ++i) in[i] = in[i] && (g << 2) + i < p.J;
     }
+    if (kParts && p.part_count > 1) {                    // (S >= 2: at most two S below 4)
+      const unsigned int S = (unsigned)p.part_count, m = (uint32_t)(g << 2) % S;
+#pragma unroll
+      for (unsigned int i = 0; i < 4; ++i) {
+        unsigned int r = m + i;
+        if (r >= S) r -= S;
+        if (r >= S) r -= S;
+        in[i] = in[i] && r == (unsigned)p.part_index;
+      }
+    }
     s.next += s.step;
     if (!__any_sync(kFull, in[0] | in[1] | in[2] | in[3])) return true;
 #pragma unroll
@@ -224,12 +236,12 @@ __device__ __forceinline__ bool scan_step(const Problem& p, unsigned long long t
   }
   return true;
 }
-template <typename F>
+template <bool kParts, typename F>
 __device__ __forceinline__ void scan_keys(const Problem& p, unsigned long long t, float cut, uint2* queue, int warp0, int n_warps, F&& f) {
   const WeightForm wf = weight_form(p);
   WarpScan s = begin_scan(cut, queue, warp0, n_warps);
 #pragma unroll 1
-  while (scan_step(p, t, wf, s, f)) {}
+  while (scan_step<kParts>(p, t, wf, s, f)) {}
 }
 
 // Shared memory of a scan: the CTA's histogram, then a queue per warp.
@@ -278,7 +290,7 @@ __device__ __forceinline__ void draw_scan(const Crew& crew, const Problem& p, co
   unsigned int* sh = reinterpret_cast<unsigned int*>(sm);
   const float cut = scan_open(crew, e, ds, sm, guided);
   const Binning bins = binning_of(cut);
-  scan_keys(p, t, cut, scan_queue(sm), (int)(threadIdx.x >> 5) * crew.size() + crew.rank(), kWarps * crew.size(),
+  scan_keys<Crew::kParts>(p, t, cut, scan_queue(sm), (int)(threadIdx.x >> 5) * crew.size() + crew.rank(), kWarps * crew.size(),
             [&](unsigned long long key, bool on) { scan_found(crew, e, ds, sh, bins, key, on); });
   scan_close<AllThreads>(crew, e, ds, sm);
 }
@@ -349,7 +361,7 @@ __device__ __noinline__ void draw_collect_all(const Crew& crew, const Problem& p
   const unsigned int edge = boundary_edge(ds);
   uint2* queue = reinterpret_cast<uint2*>(sm + sizeof(unsigned int) * kHistBins) + warp * kQueue;
   __syncthreads();
-  scan_keys(p, t, edge < 0x7f800000u ? __uint_as_float(edge) : 0.f, queue, warp * crew.size() + crew.rank(), kWarps * crew.size(),
+  scan_keys<Crew::kParts>(p, t, edge < 0x7f800000u ? __uint_as_float(edge) : 0.f, queue, warp * crew.size() + crew.rank(), kWarps * crew.size(),
             [&](unsigned long long key, bool on) { if (on) take_winner(e, ds, bins, key); });
 }
 
@@ -393,7 +405,7 @@ __device__ __noinline__ bool draw_refine(const Crew& crew, const Problem& p, con
     for (int b = tid; b < kHistBins; b += kT) sh[b] = 0u;
     if (!grid_sync(g)) return false;
     const int up = 64 - bits - width;
-    scan_keys(p, t, 0.f, queue, warp * crew.size() + crew.rank(), kWarps * crew.size(), [&](unsigned long long key, bool on) {
+    scan_keys<Crew::kParts>(p, t, 0.f, queue, warp * crew.size() + crew.rank(), kWarps * crew.size(), [&](unsigned long long key, bool on) {
       if (on && bin_of(bins, (unsigned int)(key >> 32)) == bnd && (bits == 0 || (key >> (64 - bits)) == prefix))
         atomicAdd(&sh[(key >> up) & ((1u << width) - 1u)], 1u);
     });
@@ -620,7 +632,7 @@ __device__ __forceinline__ void draw_rank(const Crew& crew, const Problem& p, co
     // (a new key behind the boundary ranks behind all candidates: the winners before it are more than P')
     // -- unless the winners are all there are
     const bool behind = fresh && (bin > bnd || (bin == bnd && ds.refined && (key >> shift) > ds.prefix));
-    if (behind && total < (unsigned long long)p.J) on = false;
+    if (behind && total < (unsigned long long)(Crew::kParts ? owned_count(p) : p.J)) on = false;
     unsigned int first = 0u, count = 0u;
     if (on) { first = behind ? total : ds.off[pad((int)bin)]; count = behind ? 0u : (bin < bnd ? ds.off[pad((int)bin + 1)] : total) - first; }
     int below = 0, struck = 0;
@@ -702,7 +714,8 @@ __device__ __forceinline__ Proposal propose_begin(const Problem& p, int j, doubl
   q.old_key = want_keys ? race_key_from(E, d_old, p.eta, (uint32_t)j, weight_mode_of(p.flags)) : 0ull;
   return q;
 }
-__device__ __forceinline__ void propose_end(const Problem& p, const Proposal& q, int pos, int j, double g, float E, bool want_keys) {
+struct Change { double d; float b_new; };
+__device__ __forceinline__ Change propose_end(const Problem& p, const Proposal& q, int pos, int j, double g, float E, bool want_keys) {
   float b_new = q.b_old;
   if (q.n > 0.0) {
     const double z = (double)q.b_old + step_scale(p) * g / q.n;
@@ -716,6 +729,7 @@ __device__ __forceinline__ void propose_end(const Problem& p, const Proposal& q,
     p.cand_keys[pos] = q.old_key;
     p.cand_keys[p.n_cand + pos] = race_key_from(E, (float)fabs(d), p.eta, (uint32_t)j, weight_mode_of(p.flags));
   }
+  return {d, b_new};
 }
 
 constexpr int kMaxWords = STRADS_MAX_CANDIDATES / 32;
