@@ -250,11 +250,19 @@ bool engine_chosen(const strads_lasso_config_t* c) {
 bool engine_provided(const strads_lasso_config_t* c) {
   return c->rho > 0.f ? engine_chosen(c) && (c->layout == STRADS_CSC || correlates_by_chance(c, 9.0)) : engine_possible(c);
 }
-// CSC rounds by squads of CTAs: how many blocks can be under way (1: blocks depend on the updates of the round before).
-int squads_of(const strads_lasso_config_t* c) {
+// CSC rounds by squads of CTAs on a GPU of n_ctas: how many blocks can be under way (1: one round after the other).  Updates come one after
+// the other, each by one squad, and every entry of a kept column costs a CTA some 10 ns there; so the squads are taken while a CTA has up to 3,400
+// (mean) entries of them.  us per round, squads / launches, uniform rows, P' = 16,384 (4,096 for P = 1,024 and less): 10^6 rows, 60 entries, P = 2,048,
+// S = 2, 4, 8 (1,660, 3,320, 6,830 entries): 57 / 71, 51 / 58, 68 / 59; P = 1,024: 33 / 48, 28 / 43, 40 / 46; 200 entries, P = 512: 41 / 61, 38 / 49, 61 / 52 (5,690).
+// With P beyond 2,048 the window is gone through in several passes by the few CTAs of a squad: P = 4,096, S = 2: 105 / 99, P = 8,192 of 20 entries 164 / 142.
+// (The static schedule, squads / one launch round after round: 52 / 60, 28 / 39, 38 / 56 for the same; without the rho test 31 / 34, 19 / 25,
+// 29 / 33, but 72 / 39 with 11,000 entries.)
+int squads_of(const strads_lasso_config_t* c, int n_ctas) {
   if (c->layout != STRADS_CSC) return 1;
-  if (n_sched_of(c) > 1) return n_sched_of(c);
-  return (c->flags & STRADS_FLAG_UNIFORM_DRAW) && !(c->flags & STRADS_FLAG_DYNAMIC_DEPS) ? kStaticSquads : 1;
+  int n = n_sched_of(c);
+  if (n == 1 && (c->flags & STRADS_FLAG_UNIFORM_DRAW) && !(c->flags & STRADS_FLAG_DYNAMIC_DEPS)) n = kStaticSquads;
+  const int size = n_ctas / n;
+  return c->n_keep <= 2048 && (double)c->n_keep * (double)c->nnz <= 3400.0 * (double)size * (double)c->n_cols ? n : 1;
 }
 // Keys each CTA can save of a scan that finds a few times `winners` of them in all.
 unsigned int engine_saved(size_t winners) { return (unsigned int)(winners / 16 + 64); }
@@ -720,8 +728,8 @@ int strads_workspace_bytes(const strads_lasso_config_t* cfg, size_t* out_bytes) 
   if (out_bytes == nullptr) return STRADS_ERR_INVALID_ARG;
   const int rc = check_sizes(cfg);
   if (rc) return rc;
-  const int n = squads_of(cfg) > n_sched_of(cfg) ? squads_of(cfg) : n_sched_of(cfg);
-  *out_bytes = carve(cfg, true, engine_provided(cfg) || squads_of(cfg) > 1).total + (size_t)(n - 1) * carve(cfg, false, squads_of(cfg) > 1).total;
+  const int squads = squads_of(cfg, kEngineMaxCtas), n = squads > n_sched_of(cfg) ? squads : n_sched_of(cfg);
+  *out_bytes = carve(cfg, true, engine_provided(cfg) || squads > 1).total + (size_t)(n - 1) * carve(cfg, false, squads > 1).total;
   return STRADS_OK;
 }
 
@@ -741,7 +749,7 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
   // first phase turns from a randomised sweep into one in index order
   if (c->c_init > STRADS_MAX_C_INIT) return STRADS_ERR_INVALID_ARG;
   const int S = n_sched_of(c);
-  int Q = squads_of(c);
+  int Q = squads_of(c, kEngineMaxCtas);
   Layout L = carve(c, true, engine_chosen(c) || Q > 1), Lrest = carve(c, false, Q > 1);
   auto need = [&]() { return L.total + (size_t)((Q > S ? Q : S) - 1) * Lrest.total; };
   // (a workspace without room for the squads or the engine does too, the rounds then go without them)
@@ -831,7 +839,7 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
       sc.stream = kit.sched[s]; sc.block_ready = kit.ready[s]; sc.updated = kit.updated[s];
     }
   }
-  h->squads_ok = Q > 1 && sm_count <= kEngineMaxCtas && sm_count / Q >= kSquadMinCtas;
+  h->squads_ok = Q > 1 && sm_count <= kEngineMaxCtas && sm_count / Q >= kSquadMinCtas && squads_of(c, sm_count) == Q;
   if (h->squads_ok) {
     SquadSet& set = h->squads;
     set.n = Q; set.size = sm_count / Q;

@@ -36,20 +36,44 @@ __device__ __forceinline__ void csc_enter(const Crew& crew, const Problem& p, co
   const int lane = threadIdx.x & 31;
   const bool dynamic = (p.flags & STRADS_FLAG_DYNAMIC_DEPS) != 0;
   if (!buckets && !dynamic) return;
+  constexpr int kU = Crew::kTogether;                    // candidates at a time: their chains of far accesses side by side
 #pragma unroll 1
-  for (int a = ((int)threadIdx.x >> 5) * crew.size() + crew.rank(); a < n; a += kWarps * crew.size()) {
-    const WalkColumn col = p.walk_cols[a];
-    if (dynamic && lane == 0) {
-      const double n2 = coupling_n2(p, col.j);
-      p.walk_cols[a].n2 = n2;
-      e.norm_f[a] = (float)n2;
+  for (int a0 = ((int)threadIdx.x >> 5) * crew.size() + crew.rank(); a0 < n; a0 += kU * kWarps * crew.size()) {
+    WalkColumn col[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int a = a0 + u * kWarps * crew.size();
+      col[u] = {};
+      if (a < n) col[u] = p.walk_cols[a];
+    }
+    int most = 0;
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int a = a0 + u * kWarps * crew.size();
+      if (dynamic && lane == 0 && a < n) {
+        const double n2 = coupling_n2(p, col[u].j);
+        p.walk_cols[a].n2 = n2;
+        e.norm_f[a] = (float)n2;
+      }
+      most = max(most, col[u].n);
     }
     if (!buckets) continue;
-    for (int q = lane; q < col.n; q += 32) {
-      const int r = __ldg(p.xrow + col.q0 + q);
-      const float v = __ldg(p.xv + col.q0 + q);
-      const unsigned int slot = atomicAdd(&p.bucket_count[r], 1u);
-      if (slot < (unsigned)kBucketSlots) p.bucket_pairs[(size_t)r * kBucketSlots + slot] = make_int2(a, __float_as_int(v));
+#pragma unroll 1
+    for (int q = lane; q - lane < most; q += 32) {
+      int r[kU];
+      float v[kU];
+      unsigned int slot[kU];
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        r[u] = q < col[u].n ? __ldg(p.xrow + col[u].q0 + q) : -1;
+        v[u] = q < col[u].n ? __ldg(p.xv + col[u].q0 + q) : 0.f;
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) slot[u] = r[u] >= 0 ? atomicAdd(&p.bucket_count[r[u]], 1u) : (unsigned)kBucketSlots;
+#pragma unroll
+      for (int u = 0; u < kU; ++u)
+        if (slot[u] < (unsigned)kBucketSlots)
+          p.bucket_pairs[(size_t)r[u] * kBucketSlots + slot[u]] = make_int2(a0 + u * kWarps * crew.size(), __float_as_int(v[u]));
     }
   }
 }
@@ -361,6 +385,18 @@ __device__ void csc_scatter(const Crew& crew, const Problem& p, int nk, int shif
   });
 }
 
+// Rows r[] by the sums in v[] (0: nothing to do), with what they are now under way together.
+template <int kU>
+__device__ __forceinline__ void apply_sums(const Problem& p, const long long (&r)[kU], const long long (&v)[kU], int shift) {
+  const bool logistic = (p.flags & STRADS_FLAG_LOGISTIC) != 0;
+  const float* now = logistic ? p.margin : p.resid;
+  float x[kU];
+#pragma unroll
+  for (int u = 0; u < kU; ++u) x[u] = v[u] != 0 ? now[r[u]] : 0.f;
+#pragma unroll
+  for (int u = 0; u < kU; ++u)
+    if (v[u] != 0) apply_row(p, r[u], x[u], ldexp((double)v[u], -shift));
+}
 template <typename Crew>
 __device__ __forceinline__ void csc_apply_rows(const Crew& crew, const Problem& p, int shift) {
   for (long long r = (long long)crew.rank() * kT + threadIdx.x; r < p.N; r += (long long)crew.size() * kT) {
@@ -1093,8 +1129,7 @@ __device__ __forceinline__ bool csc_walk_and_draw(const Crew& crew, const Proble
   auto draw = [&]() {
     if (!draws) return true;
     WarpScan scan = begin_scan(cut, scan_queue(sm_scan), (warp - kWalkWarps) * crew.size() + crew.rank(), (kWarps - kWalkWarps) * crew.size());
-#pragma unroll 1
-    while (scan_step<Crew::kParts>(p, td, wf, scan, [&](unsigned long long key, bool on) { scan_found(crew, e, ds, sh, bins, key, on); })) {}
+    scan_all<Crew::kParts>(p, td, wf, scan, [&](unsigned long long key, bool on) { scan_found(crew, e, ds, sh, bins, key, on); });
     scan_close<OtherThreads>(crew, e, ds, sm_scan);
     __shared__ int s_over;
     g_draw.target += g_draw.n;

@@ -62,11 +62,13 @@ __device__ bool grid_complete(const Grid& g) {
 // The CTAs that make a round together: all of them, or as many of them as prepare the rounds whose turn is theirs (squads.cu).
 struct WholeGrid {
   static constexpr bool kParts = false;    // all coefficients
+  static constexpr int kTogether = 1;      // entries of a list that a warp goes through side by side: it has one as a rule
   __device__ __forceinline__ int rank() const { return (int)blockIdx.x; }
   __device__ __forceinline__ int size() const { return (int)gridDim.x; }
 };
 struct Squad {
   static constexpr bool kParts = true;     // a scheduler's
+  static constexpr int kTogether = 4;
   int r, n;
   __device__ __forceinline__ int rank() const { return r; }
   __device__ __forceinline__ int size() const { return n; }
@@ -177,8 +179,72 @@ __device__ __forceinline__ WarpScan begin_scan(float cut, uint2* queue, int warp
   s.k = cut > 0.f ? __fmul_rn(cut, 1.02f * 4294967296.0f) : __uint_as_float(0x7f800000u);
   return s;
 }
+// The keys of the coefficients in the queue, computed by all lanes together.
+template <typename F>
+__device__ __forceinline__ void scan_flush(const Problem& p, const WeightForm& wf, WarpScan& s, F&& f) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+#pragma unroll 1
+  for (int i = 0; i < s.n; i += 32) {
+    const bool on = i + lane < s.n;
+    const uint2 e = on ? s.queue[i + lane] : make_uint2(0u, 0u);
+    f(on ? key_of(wf, p.delta[e.x], e.y, e.x) : ~0ull, on);
+  }
+  __syncwarp();
+  s.n = 0;
+}
+// A step over a scheduler's coefficients, 64 of them or 32 groups of four.  With four schedulers or more a group has one coefficient of
+// each at most, so that the coefficients are enumerated (a Philox block each, 1 / S of them all); with two or three a group has two at most.
+template <typename F>
+__device__ __forceinline__ bool scan_step_part(const Problem& p, unsigned long long t, const WeightForm& wf, WarpScan& s, F&& f) {
+  const int lane = threadIdx.x & 31;
+  const unsigned int S = (unsigned)p.part_count, idx = (unsigned)p.part_index;
+  const bool each = S >= 4u;
+  const long long units = each ? (owned_count(p) + 1) >> 1 : (p.J + 3) >> 2;
+  const bool more = s.next < units;
+  if (!more && s.n == 0) return false;
+  if (more) {
+    long long j[2];
+    uint32_t word[2];
+    if (each) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        j[u] = idx + (long long)S * (2 * s.next + 32 * u + lane);
+        uint32_t w[4];
+        philox4x32_10((uint32_t)(j[u] >> 2), (uint32_t)t, (uint32_t)(t >> 32), 0u, (uint32_t)p.seed, (uint32_t)(p.seed >> 32), w);
+        word[u] = (j[u] & 2) ? ((j[u] & 1) ? w[3] : w[2]) : ((j[u] & 1) ? w[1] : w[0]);
+      }
+    } else {
+      const long long g = s.next + lane;
+      uint32_t w[4];
+      philox4x32_10((uint32_t)g, (uint32_t)t, (uint32_t)(t >> 32), 0u, (uint32_t)p.seed, (uint32_t)(p.seed >> 32), w);
+      const unsigned int m = S == 3u ? (uint32_t)g % 3u : 0u;            // 4 g mod S
+      const unsigned int i = idx >= m ? idx - m : idx + S - m;
+      j[0] = (g << 2) + i;
+      word[0] = i == 0u ? w[0] : (i == 1u ? w[1] : w[2]);
+      j[1] = i + S < 4u ? j[0] + S : p.J;
+      word[1] = i + S == 2u ? w[2] : w[3];
+    }
+    s.next += s.step;
+    bool in[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const float d = j[u] < p.J ? __ldcg(p.delta + j[u]) : 0.f;
+      in[u] = j[u] < p.J && !(__uint2float_rn(word[u]) > __fmul_rn(s.k, weight_of(wf, d)));
+    }
+    if (!__any_sync(kFull, in[0] | in[1])) return true;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const unsigned int m = __ballot_sync(kFull, in[u]);
+      if (in[u]) s.queue[s.n + __popc(m & ((1u << lane) - 1u))] = make_uint2((uint32_t)j[u], word[u]);
+      s.n += __popc(m);
+    }
+  }
+  if (s.n > kQueue - 128 || !more) scan_flush(p, wf, s, f);
+  return true;
+}
 // One step; past the end it only empties the queue.  Whether there was anything to do.
-template <bool kParts, typename F>
+template <typename F>
 __device__ __forceinline__ bool scan_step(const Problem& p, unsigned long long t, const WeightForm& wf, WarpScan& s, F&& f) {
   const int lane = threadIdx.x & 31;
   const long long groups = (p.J + 3) >> 2, whole = p.J >> 2, g = s.next + lane;
@@ -204,16 +270,6 @@ __device__ __forceinline__ bool scan_step(const Problem& p, unsigned long long t
 #pragma unroll
       for (int i = 0; i < 4; ++i) in[i] = in[i] && (g << 2) + i < p.J;
     }
-    if (kParts && p.part_count > 1) {                    // (S >= 2: at most two S below 4)
-      const unsigned int S = (unsigned)p.part_count, m = (uint32_t)(g << 2) % S;
-#pragma unroll
-      for (unsigned int i = 0; i < 4; ++i) {
-        unsigned int r = m + i;
-        if (r >= S) r -= S;
-        if (r >= S) r -= S;
-        in[i] = in[i] && r == (unsigned)p.part_index;
-      }
-    }
     s.next += s.step;
     if (!__any_sync(kFull, in[0] | in[1] | in[2] | in[3])) return true;
 #pragma unroll
@@ -223,25 +279,24 @@ __device__ __forceinline__ bool scan_step(const Problem& p, unsigned long long t
       s.n += __popc(m);
     }
   }
-  if (s.n > kQueue - 128 || !more) {                     // the keys of the survivors, computed by all lanes together
-    __syncwarp();
-#pragma unroll 1
-    for (int i = 0; i < s.n; i += 32) {
-      const bool on = i + lane < s.n;
-      const uint2 e = on ? s.queue[i + lane] : make_uint2(0u, 0u);
-      f(on ? key_of(wf, p.delta[e.x], e.y, e.x) : ~0ull, on);
-    }
-    __syncwarp();
-    s.n = 0;
-  }
+  if (s.n > kQueue - 128 || !more) scan_flush(p, wf, s, f);
   return true;
+}
+template <bool kParts, typename F>
+__device__ __forceinline__ void scan_all(const Problem& p, unsigned long long t, const WeightForm& wf, WarpScan& s, F&& f) {
+  if (kParts && p.part_count > 1) {
+#pragma unroll 1
+    while (scan_step_part(p, t, wf, s, f)) {}
+  } else {
+#pragma unroll 1
+    while (scan_step(p, t, wf, s, f)) {}
+  }
 }
 template <bool kParts, typename F>
 __device__ __forceinline__ void scan_keys(const Problem& p, unsigned long long t, float cut, uint2* queue, int warp0, int n_warps, F&& f) {
   const WeightForm wf = weight_form(p);
   WarpScan s = begin_scan(cut, queue, warp0, n_warps);
-#pragma unroll 1
-  while (scan_step<kParts>(p, t, wf, s, f)) {}
+  scan_all<kParts>(p, t, wf, s, f);
 }
 
 // Shared memory of a scan: the CTA's histogram, then a queue per warp.

@@ -17,10 +17,10 @@ namespace {
 
 // The update of a squad's round in its turn: x_a^T r of the kept coefficients, their changes, beta, delta and the residual.
 // A warp has the kept coefficients warp * size + rank + k * (warps of the squad), 32 of them at a time; the columns of the first 32
-// wait in shared memory as far as there is room (`entry`, kHeldEntries per warp).
+// wait in shared memory as far as there is room.
 constexpr int kHeldEntries = 512;
-struct HeldEntry { int row; float val; };
-constexpr size_t kHeldSmem = sizeof(HeldEntry) * kHeldEntries * kWarps;
+struct HeldEntries { int row[kHeldEntries]; float val[kHeldEntries]; };      // a warp's
+constexpr size_t kHeldSmem = sizeof(HeldEntries) * kWarps;
 
 struct Turn {
   unsigned int* count;
@@ -49,7 +49,7 @@ struct Held {
   int a, pos, j, len, at;                  // place in the kept list and among the candidates, coefficient, entries, where they wait (-1: in X)
   long long q0;
 };
-__device__ __forceinline__ Held hold(const Squad& crew, const Problem& p, int nk, int chunk, HeldEntry* entry) {
+__device__ __forceinline__ Held hold(const Squad& crew, const Problem& p, int nk, int chunk, HeldEntries* entry) {
   const int lane = threadIdx.x & 31, warp = (int)threadIdx.x >> 5;
   const int first = warp * crew.size() + crew.rank(), step = kWarps * crew.size();
   Held h;
@@ -79,17 +79,15 @@ __device__ __forceinline__ Held hold(const Squad& crew, const Problem& p, int nk
     const long long q0 = __shfl_sync(kFull, h.q0, k);
     if (at < 0) continue;
     for (int q = lane; q < len; q += 32) {
-      HeldEntry v;
-      v.row = __ldg(p.xrow + q0 + q); v.val = __ldg(p.xv + q0 + q);
-      entry[at + q] = v;
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(&entry->row[at + q])), "l"(p.xrow + q0 + q) : "memory");
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(&entry->val[at + q])), "l"(p.xv + q0 + q) : "memory");
     }
   }
-  __syncwarp();
   return h;
 }
 // f(k, row, value) for the entries of the warp's columns for which want(k): whole warps, lanes side by side.
 template <typename W, typename F>
-__device__ __forceinline__ void for_held(const Problem& p, const Held& h, int chunk, const HeldEntry* entry, W&& want, F&& f) {
+__device__ __forceinline__ void for_held(const Problem& p, const Held& h, int chunk, const HeldEntries* entry, W&& want, F&& f) {
   const int lane = threadIdx.x & 31, m = min(32, h.n - chunk * 32);
 #pragma unroll 1
   for (int k = 0; k < m; ++k) {
@@ -97,7 +95,7 @@ __device__ __forceinline__ void for_held(const Problem& p, const Held& h, int ch
     const long long q0 = __shfl_sync(kFull, h.q0, k);
     if (!want(k)) continue;
     for (int q = lane; q < len; q += 32) {
-      if (at >= 0) { const HeldEntry v = entry[at + q]; f(k, v.row, v.val); }
+      if (at >= 0) f(k, entry->row[at + q], entry->val[at + q]);
       else f(k, __ldg(p.xrow + q0 + q), __ldg(p.xv + q0 + q));
     }
   }
@@ -107,7 +105,7 @@ __device__ __forceinline__ void for_held(const Problem& p, const Held& h, int ch
 __device__ __forceinline__ bool squad_update(const Squad& crew, const Problem& p, const Engine& e, unsigned char* sm, Grid& g, const Turn& turn, int nk,
                                              unsigned long long t_next, bool want_keys) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  HeldEntry* entry = reinterpret_cast<HeldEntry*>(sm) + warp * kHeldEntries;
+  HeldEntries* entry = reinterpret_cast<HeldEntries*>(sm) + warp;
   EngineState* es = e.es;
   __syncthreads();                                       // (what lay there before)
   Held h = hold(crew, p, nk, 0, entry);
@@ -120,7 +118,8 @@ __device__ __forceinline__ bool squad_update(const Squad& crew, const Problem& p
   }
   const int examined = es->n_examined;
   const float x_max = p.st->x_abs_max;
-  if (!await_turn(turn)) return false;
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (!await_turn(turn)) return false;                   // (a barrier of the CTA in it)
   // ---- x_a^T r and the changes ----
   double d0 = 0.0;                                       // of the lane's kept coefficient (the first 32 of the warp)
   unsigned long long dmax = 0ull;
@@ -162,9 +161,9 @@ __device__ __forceinline__ bool squad_update(const Squad& crew, const Problem& p
           for (int y = 0; y < 2; ++y) {
             v[u][y] = 0.f; r[u][y] = 0.f;
             if (q + 32 * y < len[u]) {
-              const HeldEntry en = at[u] >= 0 ? entry[at[u] + q + 32 * y] : HeldEntry{__ldg(p.xrow + q0[u] + q + 32 * y), __ldg(p.xv + q0[u] + q + 32 * y)};
-              v[u][y] = en.val;
-              r[u][y] = p.resid[en.row];
+              const int i = q + 32 * y;
+              v[u][y] = at[u] >= 0 ? entry->val[at[u] + i] : __ldg(p.xv + q0[u] + i);
+              r[u][y] = p.resid[at[u] >= 0 ? entry->row[at[u] + i] : __ldg(p.xrow + q0[u] + i)];
             }
           }
 #pragma unroll
@@ -230,10 +229,31 @@ __device__ __forceinline__ bool squad_update(const Squad& crew, const Problem& p
         Held c = h;
         if (chunk > 0) c = hold(crew, p, nk, chunk, nullptr);
         const double d_lane = change_of(c, chunk);
-        for_held(p, c, chunk, entry, [&](int k) { return __shfl_sync(kFull, d_lane, k) != 0.0; }, [&](int, int row, float) {
-          const long long v = (long long)atomicExch(reinterpret_cast<unsigned long long*>(p.resid_acc + row), 0ull);
-          if (v != 0) apply_row(p, row, ldexp((double)v, -shift));
-        });
+        const int m = min(32, h.n - chunk * 32);
+        constexpr int kU = 4;                            // columns at a time
+#pragma unroll 1
+        for (int k0 = 0; k0 < m; k0 += kU) {
+          int at[kU], len[kU], most = 0;
+          long long q0[kU];
+#pragma unroll
+          for (int u = 0; u < kU; ++u) {
+            const int k = (k0 + u) & 31;
+            at[u] = __shfl_sync(kFull, c.at, k); q0[u] = __shfl_sync(kFull, c.q0, k);
+            len[u] = k0 + u < m && __shfl_sync(kFull, d_lane, k) != 0.0 ? __shfl_sync(kFull, c.len, k) : 0;
+            most = max(most, len[u]);
+          }
+#pragma unroll 1
+          for (int q = lane; q - lane < most; q += 32) {
+            long long row[kU], v[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+              row[u] = 0; v[u] = 0;
+              if (q < len[u]) row[u] = at[u] >= 0 ? entry->row[at[u] + q] : __ldg(p.xrow + q0[u] + q);
+              if (q < len[u]) v[u] = (long long)atomicExch(reinterpret_cast<unsigned long long*>(p.resid_acc + row[u]), 0ull);
+            }
+            apply_sums<kU>(p, row, v, shift);
+          }
+        }
       }
     } else {
       csc_apply_rows(crew, p, shift);

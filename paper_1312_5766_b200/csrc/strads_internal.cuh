@@ -283,15 +283,18 @@ __device__ __forceinline__ double coupling_n2(const Problem& p, int j) {
 // threshold by 4 (Shotgun's step for this loss).
 __device__ __forceinline__ double step_scale(const Problem& p) { return (p.flags & STRADS_FLAG_LOGISTIC) ? 4.0 : 1.0; }
 __device__ __forceinline__ double sigmoid64(double m) { return m >= 0.0 ? 1.0 / (1.0 + exp(-m)) : exp(m) / (1.0 + exp(m)); }
-// Row i after the kept coefficients have moved the linear predictor x_i^T beta by s.
-__device__ __forceinline__ void apply_row(const Problem& p, long long i, double s) {
+// Row i after the kept coefficients have moved the linear predictor x_i^T beta by s (now: its margin, or its residual).
+__device__ __forceinline__ void apply_row(const Problem& p, long long i, float now, double s) {
   if (p.flags & STRADS_FLAG_LOGISTIC) {
-    const float m = (float)((double)p.margin[i] + s);
+    const float m = (float)((double)now + s);
     p.margin[i] = m;
     p.resid[i] = (float)((double)p.y[i] - sigmoid64((double)m));
   } else {
-    p.resid[i] = (float)((double)p.resid[i] - s);
+    p.resid[i] = (float)((double)now - s);
   }
+}
+__device__ __forceinline__ void apply_row(const Problem& p, long long i, double s) {
+  apply_row(p, i, (p.flags & STRADS_FLAG_LOGISTIC) ? p.margin[i] : p.resid[i], s);
 }
 
 // x_a^T x_b of two CSC columns (ascending rows): a given as arrays (possibly staged in shared memory), b read
