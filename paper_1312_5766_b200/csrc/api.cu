@@ -199,7 +199,7 @@ int pow2_ceil(int n) { int v = 1; while (v < n) v <<= 1; return v; }
 struct Layout {
   size_t off_state, off_n2, off_hist, off_sure, off_boundary, off_cand, off_kept, off_kept_pos, off_dbeta, off_dbeta64,
       off_conflict, off_cand_dbeta64, off_cand_bnew, off_dot_partial, off_dot_ticket, off_margin, off_obj, off_amb, off_xcb, off_walk_blocked, off_walk_ctl, off_walk_cols,
-      off_bucket_count, off_bucket_items, off_bucket_vals, off_bucket_cols, off_resid_acc, off_delta_prev, off_edges, off_patch_keys, off_cand_keys, off_survivors, off_bin_off, off_bin_cur, off_ahead_bin_off, off_ahead_bin_cur,
+      off_bucket_count, off_bucket_items, off_bucket_vals, off_bucket_cols, off_bucket_own, off_resid_acc, off_delta_prev, off_edges, off_patch_keys, off_cand_keys, off_survivors, off_bin_off, off_bin_cur, off_ahead_bin_off, off_ahead_bin_cur,
       off_ahead_state, off_ahead_hist, off_ahead_sure, off_ahead_boundary, off_ahead_keys, off_ahead_idx,
       off_eng_state, off_eng_hist, off_eng_cur, off_eng_win, off_eng_surv, off_eng_saved, off_eng_xb, off_eng_norm, off_eng_part, off_eng_tickets, total;
   long long eng_pitch, eng_lo;
@@ -317,6 +317,7 @@ Layout carve(const strads_lasso_config_t* c, bool first, bool engine) {
   L.off_bucket_count = take(L.buckets ? sizeof(unsigned int) * (size_t)c->n_rows : 0);
   L.off_bucket_items = take(L.buckets ? sizeof(int) * (size_t)c->n_rows * kBucketSlots : 0);
   L.off_bucket_vals = take(L.buckets ? sizeof(float) * (size_t)c->n_rows * kBucketSlots : 0);   // (directly behind: the engine keeps pairs there)
+  L.off_bucket_own = take(L.buckets && L.engine ? 64 * (size_t)c->n_candidates : 0);
   L.off_bucket_cols = take(L.buckets ? sizeof(BucketColumn) * (size_t)c->n_candidates : 0);
   L.off_resid_acc = take(csc ? sizeof(long long) * (size_t)c->n_rows : 0);
   L.off_delta_prev = take(sizeof(float) * (size_t)c->n_keep);
@@ -629,6 +630,7 @@ void fill_problem(Problem& p, const strads_lasso_config_t* c, const Layout& L, c
   p.bucket_items = L.buckets ? reinterpret_cast<int*>(ws + L.off_bucket_items) : nullptr;
   p.bucket_vals = L.buckets ? reinterpret_cast<float*>(ws + L.off_bucket_vals) : nullptr;
   p.bucket_pairs = L.buckets ? reinterpret_cast<int2*>(ws + L.off_bucket_items) : nullptr;
+  p.bucket_own = L.buckets && L.engine ? reinterpret_cast<unsigned char*>(ws + L.off_bucket_own) : nullptr;
   p.bucket_cols = L.buckets ? reinterpret_cast<BucketColumn*>(ws + L.off_bucket_cols) : nullptr;
   p.part_count = S; p.part_index = s;
   p.sm_count = first ? first->sm_count : 0;

@@ -131,6 +131,7 @@ struct Problem {
   int* bucket_items;            // [N][kBucketSlots] their positions in the list
   float* bucket_vals;           // [N][kBucketSlots] their values in row i
   int2* bucket_pairs;           // [N][kBucketSlots] position and value side by side (the round engine; same memory as the two above)
+  unsigned char* bucket_own;    // [P'][64] (rounds in one launch) the places that a candidate's first entries have in their rows' buckets
   BucketColumn* bucket_cols;    // [P'] where each candidate's column lies, as the bucket kernels need it
   int sm_count;
   // sampling ahead (one scheduler): the draw of round t + 1 is made during round t from the priorities of its start
