@@ -170,6 +170,7 @@ constexpr int kLeftoverUses = 3;      // a left-over sequence is captured when o
 constexpr int kEdgeCap = 8192;        // conflicting pairs the Gram kernels can list for the walk (32 KB)
 constexpr int kEngineRounds = 32;     // rounds per launch of the engine: a launch every few hundred microseconds, so that other streams get their turn
 constexpr int kEngineDenseRows = 2048;
+constexpr int kEngineMinCtas = 32;    // a lane per kept column of a warp
 constexpr int kEngineMaxCtas = 192;   // CTAs the engine's scratch provides for
 constexpr int kSquadRounds = 64;      // rounds per launch of the squads (the first block and the last update of a launch overlap with nothing)
 constexpr int kStaticSquads = 4;      // blocks under way with the static schedule
@@ -794,7 +795,7 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
     return fail(cuda_fail(e, "copy stream"));
   h->copy_stream = kit.copy; h->copy_fork = kit.copy_fork; h->copy_done = kit.copy_done;
   forget_lists(h);
-  h->engine_ok = S == 1 && L.engine && sm_count <= kEngineMaxCtas;
+  h->engine_ok = S == 1 && L.engine && sm_count >= kEngineMinCtas && sm_count <= kEngineMaxCtas;
   if (h->engine_ok) {
     fill_engine(h->engine, p0, L, ws, sm_count, true);
     if ((e = prepare_engine(p0, h->engine)) != cudaSuccess) return fail(cuda_fail(e, "prepare_engine"));

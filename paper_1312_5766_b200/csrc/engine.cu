@@ -37,7 +37,7 @@ namespace {
 
 struct RoundOutputs { int* cand; int* kept; float* dbeta; int* counts; };
 
-__device__ void commit_changes(const Problem& p, const Engine& e, int nk, int n_moving, const RoundOutputs& out, bool last) {
+__device__ void commit_changes(const Problem& p, int examined, int nk, int n_moving, const RoundOutputs& out, bool last) {
   const int tid = threadIdx.x;
   DeviceState* st = p.st;
   for (int a = tid * (int)gridDim.x + (int)blockIdx.x; a < p.n_keep; a += kT * (int)gridDim.x) {
@@ -60,7 +60,6 @@ __device__ void commit_changes(const Problem& p, const Engine& e, int nk, int n_
   if (last && out.cand != nullptr)                       // (the candidates of this round; the draw ahead would overwrite them)
     for (int i = tid * (int)gridDim.x + (int)blockIdx.x; i < p.n_cand; i += kT * (int)gridDim.x) out.cand[i] = p.cand[i];
   if (blockIdx.x == 0 && tid == 0) {
-    const int examined = e.es->n_examined;
     st->counts[0] = p.n_cand; st->counts[1] = examined; st->counts[2] = nk; st->counts[3] = n_moving;
     if (last && out.counts != nullptr) { out.counts[0] = p.n_cand; out.counts[1] = examined; out.counts[2] = nk; out.counts[3] = n_moving; }
     st->totals[0] += 1; st->totals[1] += (unsigned)examined; st->totals[2] += (unsigned)nk; st->totals[3] += (unsigned)n_moving;
@@ -812,6 +811,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
   __shared__ ChangeShared cs;
   __shared__ __align__(8) PackBars pb;
   __shared__ __align__(16) GramShared gs;
+  __shared__ Settled walk;
   // Copies for the functions that are called rarely and not inlined, made when they are: a reference to the parameters themselves would make
   // every access to them, in the hot code too, a load from memory.
   __shared__ Problem sp;
@@ -856,6 +856,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
   Moving* mv = reinterpret_cast<Moving*>(behind_keys);
   double* part = reinterpret_cast<double*>(behind_keys + sizeof(Moving));
   ChangedByBin* cb = reinterpret_cast<ChangedByBin*>(behind_keys + (kDense ? sizeof(Moving) + sizeof(double) * 4 * kT : 0));
+  unsigned short* kept_at = reinterpret_cast<unsigned short*>(sm + kept_at_offset(p, (size_t)(behind_keys - sm) + sizeof(ChangedByBin)));
   const bool no_filter = (p.flags & STRADS_FLAG_NO_FILTER) != 0;
   const int n_total = p.n_cand;
   Pending last;
@@ -878,7 +879,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
     bool scanned = !draws, collected = !draws;
     bool spare = kDense && real && !no_filter;           // the last CTA leaves the draw's winners to the others
     int n = no_filter ? p.n_keep : e.window, packed = 0;
-    bool window = true;
+    bool window = true, pending = false;                   // pending: a barrier to be met, and the kept list is this CTA's own
     if (kDense) {
       if (n < n_total && es->skip_window && !no_filter) n = n_total;
     } else {
@@ -953,12 +954,15 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
       if (!real || no_filter) break;
       if (!kDense) {
         if (!window) break;
-        if (walker) csc_walk_window(p, e, sm, n);
-        const ClearAhead rows = csc_clear_begin(WholeGrid(), p, n);
-        if (!collected) { draw_gather<AllThreads>(WholeGrid(), p, e, ds, k, true); collected = true; spare = true; }
-        csc_clear_end(p, rows);
+        csc_settle(WholeGrid(), p, e, sm, kept_at, walk, n, [&]() {
+          const ClearAhead rows = csc_clear_begin(WholeGrid(), p, n);
+          if (!collected) draw_gather<OtherThreads>(WholeGrid(), p, e, ds, k, false);
+          csc_clear_end(p, rows);
+        });
+        collected = true;
+        if (!walk_is_open(p, walk, n)) { pending = true; break; }
         if (!(ok = grid_sync(g))) break;
-        if (!es->walk_open) break;
+        if (cta == 0 && tid == 0) settle_note(e, walk);
         csc_enter(WholeGrid(), p, e, n_total, false);
         window = false;
       } else {
@@ -967,27 +971,38 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
       }
     }
     if (!ok) break;
-    if (draws && es->mend) {
-      keep_parameters();
-      if (!(ok = draw_mend(WholeGrid(), sp, se, ds, sm, td, k, g))) break;
-    }
     // ---- step 4 ----
-    int n_changed = 0, nk = 0;
+    int n_moving = 0, nk = 0, examined = 0;
     const int n_next = no_filter ? p.n_keep : (e.window < n_total && es->skip_window ? n_total : e.window);   // looked at first
     if (real) {
-      nk = es->n_kept;
-      const int n_moving = gather_changes<kDense>(p, binning_of(ds.cut), nk, draws, keys, cb, mv, cs);
-      n_changed = cs.n_changed;
-      commit_changes(p, e, nk, n_moving, out, final_round);
+      nk = pending ? walk.kept : es->n_kept;
+      examined = pending ? walk.examined : es->n_examined;
+      KeptColumns kept;
+      if (!kDense) kept = kept_columns(WholeGrid(), p, nk, pending ? kept_at : nullptr);
+      if (pending) grid_arrive(g);
+      n_moving = gather_changes<kDense>(p, binning_of(ds.cut), nk, pending ? kept_at : nullptr, draws, keys, cb, mv, cs);
       last.nk = nk; last.n_moving = n_moving;
       if (!kDense) {
         last.shift = csc_shift(p.st->x_abs_max, cs.dmax, nk);
-        csc_scatter(WholeGrid(), p, nk, last.shift);
+        csc_scatter(p, kept, last.shift);
       }
+    }
+    if (pending) {
+      if (!(ok = grid_complete(g))) break;
+      if (cta == 0 && tid == 0) settle_note(e, walk);
+    }
+    // (the priorities as they were, and nothing of this round's changes in shared memory)
+    if (draws && es->mend) {
+      keep_parameters();
+      if (!(ok = draw_mend(WholeGrid(), sp, se, ds, sm, td, k, g))) break;
+      if (real) gather_again<kDense>(sp, binning_of(ds.cut), nk, keys, cb, mv, cs);
+    }
+    if (real) {
+      commit_changes(p, examined, nk, n_moving, out, final_round);
       --left;
       ++t;
     }
-    if (draws) draw_rank<kDense>(WholeGrid(), p, e, ds, keys, cb, n_changed, nk, cs.rank_wsum, spare ? max(1, n_ctas - 1) : n_ctas, n_next);
+    if (draws) draw_rank<kDense>(WholeGrid(), p, e, ds, keys, cb, real ? cs.n_changed : 0, nk, cs.rank_wsum, spare ? max(1, n_ctas - 1) : n_ctas, n_next);
     if (kDense && real) dense_apply(p, *mv, part, nk, last.n_moving);
     have = draws;
     if (left == 0 && kDense) break;
@@ -1119,7 +1134,9 @@ __global__ void __launch_bounds__(kT, 1) k_draw(const __grid_constant__ Problem 
   e.es->dirty = !ok || left >= kGaveUp ? 1 : 0;
 }
 
-size_t smem_of(bool dense, int n_keep, bool ahead, int n_cand) {
+size_t smem_of(const Problem& p, bool ahead) {
+  const bool dense = p.layout == STRADS_DENSE_COLMAJOR;
+  const int n_keep = p.n_keep;
   size_t need = kScanSmem;
   const size_t keys = ahead ? 2 * sizeof(unsigned long long) * (size_t)n_keep : 0;
   auto at_least = [&](size_t v) { if (need < v) need = v; };
@@ -1132,15 +1149,14 @@ size_t smem_of(bool dense, int n_keep, bool ahead, int n_cand) {
   } else {
     at_least(kTermsSmem);
     at_least(sizeof(DemandShared) + kScanSmem);
-    at_least(walk_pairs_smem(n_cand, 8192));
-    if (ahead) at_least(keys + sizeof(ChangedByBin));
+    at_least(kept_at_offset(p, keys + sizeof(ChangedByBin)) + sizeof(unsigned short) * (size_t)n_keep);
   }
   return need;
 }
 
 }  // namespace
 
-size_t engine_smem(const Problem& p, bool ahead) { return smem_of(p.layout == STRADS_DENSE_COLMAJOR, p.n_keep, ahead, p.n_cand); }
+size_t engine_smem(const Problem& p, bool ahead) { return smem_of(p, ahead); }
 
 // The grid: one CTA per SM.  (A single thread-block cluster of 16 CTAs for small problems, whose barriers cost a fifth, was
 // slower all the same: c1 41.6 us per round instead of 36.6, every CTA having nine times the candidates to go through.)

@@ -81,29 +81,38 @@ __device__ __forceinline__ void csc_enter(const Crew& crew, const Problem& p, co
   }
 }
 
-// Emptied again by all CTAs but the last, which walks meanwhile.  In two parts, so that what there is to fetch is under way while
-// the winners are collected: the rows of a warp's first candidate, two per lane; the others at once.
-struct ClearAhead { int row[2]; };
+// Emptied again by the threads that do not walk meanwhile.  In two parts, so that what there is to fetch is under way while
+// the winners are collected: the rows of a warp's first candidates, two per lane; the others at once.
+constexpr int kClearAhead = 2;
+struct ClearAhead { int row[kClearAhead][2]; };
 template <typename Crew>
 __device__ __forceinline__ ClearAhead csc_clear_begin(const Crew& crew, const Problem& p, int n) {
-  const int cta = crew.rank(), n_ctas = max(1, crew.size() - 1), lane = threadIdx.x & 31;
-  ClearAhead c = {{-1, -1}};
-  if (cta >= n_ctas) return c;
-  const int first = ((int)threadIdx.x >> 5) * n_ctas + cta;
-  for (int a = first; a < n; a += kWarps * n_ctas) {
-    const WalkColumn col = p.walk_cols[a];
-    if (a == first) {
+  constexpr int kClearing = OtherThreads::kN / 32;
+  const int lane = threadIdx.x & 31, step = kClearing * crew.size();
+  ClearAhead c;
+  int a = (OtherThreads::tid() >> 5) * crew.size() + crew.rank();
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-        if (lane + 32 * h < col.n) c.row[h] = __ldg(p.xrow + col.q0 + lane + 32 * h);
-    }
-    for (int q = lane + (a == first ? 64 : 0); q < col.n; q += 32) p.bucket_count[__ldg(p.xrow + col.q0 + q)] = 0u;
+  for (int k = 0; k < kClearAhead; ++k, a += step) {
+    c.row[k][0] = c.row[k][1] = -1;
+    if (a >= n) continue;
+    const WalkColumn col = p.walk_cols[a];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (lane + 32 * h < col.n) c.row[k][h] = __ldg(p.xrow + col.q0 + lane + 32 * h);
+    for (int q = lane + 64; q < col.n; q += 32) p.bucket_count[__ldg(p.xrow + col.q0 + q)] = 0u;
+  }
+#pragma unroll 1
+  for (; a < n; a += step) {
+    const WalkColumn col = p.walk_cols[a];
+    for (int q = lane; q < col.n; q += 32) p.bucket_count[__ldg(p.xrow + col.q0 + q)] = 0u;
   }
   return c;
 }
 __device__ __forceinline__ void csc_clear_end(const Problem& p, const ClearAhead& c) {
 #pragma unroll
-  for (int h = 0; h < 2; ++h) if (c.row[h] >= 0) p.bucket_count[c.row[h]] = 0u;
+  for (int k = 0; k < kClearAhead; ++k)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) if (c.row[k][h] >= 0) p.bucket_count[c.row[k][h]] = 0u;
 }
 
 // |x_a^T x_b| >= rho ||x_a|| ||x_b||, with limit_a = rho^2 ||x_a||^2 and n2b = ||x_b||^2 in binary32: for certain not (may_conflict), for
@@ -387,14 +396,42 @@ __device__ __forceinline__ void for_moving_entries(const Crew& crew, const Probl
   }
 }
 
+// A warp's kept columns (a mod warps of the crew): lane k has the k-th.  kept_at: positions of the kept candidates in shared memory, read
+// before anybody can rank the next candidates over these; null: the lists in global memory.
+struct KeptColumns { int m, len; long long q0; double d; };
 template <typename Crew>
-__device__ void csc_scatter(const Crew& crew, const Problem& p, int nk, int shift) {
-  if (shift == INT_MIN) return;
-  for_moving_entries(crew, p, nk, [&](long long q, double d) {
-    const long long fx = __double2ll_rn(ldexp((double)__ldg(p.xv + q) * d, shift));
-    atomicAdd(reinterpret_cast<unsigned long long*>(p.resid_acc + __ldg(p.xrow + q)), (unsigned long long)fx);
-  });
+__device__ __forceinline__ KeptColumns kept_columns(const Crew& crew, const Problem& p, int nk, const unsigned short* kept_at) {
+  const int first = ((int)threadIdx.x >> 5) * crew.size() + crew.rank(), step = kWarps * crew.size();
+  const int a = first + ((int)threadIdx.x & 31) * step;
+  KeptColumns c;
+  c.m = nk > first ? (nk - first + step - 1) / step : 0; c.len = 0; c.q0 = 0; c.d = 0.0;
+  if (a >= nk) return c;
+  if (kept_at != nullptr) {
+    const int pos = kept_at[a];
+    const WalkColumn col = p.walk_cols[pos];
+    c.d = p.cand_dbeta64[pos]; c.q0 = col.q0; c.len = col.n;
+  } else {
+    const int j = p.kept[a];
+    c.d = p.cand_dbeta64[p.kept_pos[a]]; c.q0 = p.xptr[j]; c.len = (int)(p.xptr[j + 1] - c.q0);
+  }
+  return c;
 }
+__device__ __forceinline__ void csc_scatter(const Problem& p, const KeptColumns& c, int shift) {
+  if (shift == INT_MIN) return;
+  const int lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int k = 0; k < c.m; ++k) {
+    const double d = __shfl_sync(kFull, c.d, k);
+    const long long q0 = __shfl_sync(kFull, c.q0, k);
+    const int len = __shfl_sync(kFull, c.len, k);
+    if (d == 0.0) continue;
+    for (int q = lane; q < len; q += 32) {
+      const long long fx = __double2ll_rn(ldexp((double)__ldg(p.xv + q0 + q) * d, shift));
+      atomicAdd(reinterpret_cast<unsigned long long*>(p.resid_acc + __ldg(p.xrow + q0 + q)), (unsigned long long)fx);
+    }
+  }
+}
+static_assert(STRADS_MAX_CANDIDATES <= 32 * kWarps * 32, "a lane per kept column of a warp with 32 CTAs or more");
 
 // Rows r[] by the sums in v[] (0: nothing to do), with what they are now under way together.
 template <int kU>
@@ -1104,26 +1141,57 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Crew& crew, const Probl
   return s.ok != 0 && s.drawn != 0;
 }
 
-// The walk from the list of the window's conflicting pairs, by one CTA.
-__device__ __forceinline__ void csc_walk_window(const Problem& p, const Engine& e, unsigned char* sm, int n) {
-  __shared__ int s_kept, s_examined;
-  EngineState* es = e.es;
-  const unsigned int edges = es->edge_count;
-  const int failed = es->bucket_failed, tid = threadIdx.x;
-  if (tid == 0) { s_kept = 0; s_examined = n; }
-  __syncthreads();
-  bool settled = !failed && edges <= (unsigned)p.cap_edges;
-  if (settled) settled = walk_from_pair_list<kT>(p, p.cand, n, edges, sm, p.kept, &s_kept, &s_examined);
-  __syncthreads();
-  if (tid == 0) {
-    es->n_kept = s_kept; es->n_examined = s_examined;
-    es->walk_open = !settled || (s_kept < p.n_keep && n < p.n_cand) ? 1 : 0;
-    // after an overflow the buckets are left alone: for a round, then twice as long after every further one, to 64
-    // (a count of rounds, not the round to wait for: strads_set_round may go back); this round's walk counts too
-    if (!settled) es->avoid = 1 + (1 << es->streak);
-    es->streak = settled ? 0 : min(es->streak + 1, 6);
-    es->bucket_failed = 0; es->edge_count = 0u;
+// The walk from the list of the window's conflicting pairs, by every CTA for itself with half its threads -- what it needs is in L2 for all of
+// them behind the barrier, and nobody then waits for one of them -- while the others do what else there is (`meanwhile`).  The kept
+// candidates' positions go to kept_at (shared memory, not among the walk's own); the last CTA leaves the lists in global memory as well.
+// All threads of the CTA; settle_note makes the notes behind a barrier.
+struct WalkThreads {
+  static constexpr int kN = kWalkT;
+  static __device__ __forceinline__ void sync() { asm volatile("bar.sync 1, %0;" ::"n"(kN) : "memory"); }
+  static __device__ __forceinline__ bool any(int x) {
+    int r;
+    asm volatile("{ .reg .pred p, q; setp.ne.s32 p, %1, 0; bar.red.or.pred q, 1, %2, p; selp.s32 %0, 1, 0, q; }" : "=r"(r) : "r"(x), "n"(kN) : "memory");
+    return r != 0;
   }
+};
+struct Settled { int kept, examined, settled; };
+// Where kept_at can lie: behind the walk's own, and behind step 4's (`changes` bytes).
+__host__ __device__ inline size_t kept_at_offset(const Problem& p, size_t changes) {
+  const size_t walk = walk_pairs_smem(p.n_cand, (unsigned)p.cap_edges);
+  return ((walk > changes ? walk : changes) + 15) & ~(size_t)15;
+}
+template <typename Crew, typename F>
+__device__ __forceinline__ void csc_settle(const Crew& crew, const Problem& p, const Engine& e, unsigned char* sm, unsigned short* kept_at, Settled& out, int n,
+                                           F&& meanwhile) {
+  const int tid = threadIdx.x;
+  __syncthreads();                                       // (what lay there before)
+  if (tid >= kWalkT) {
+    meanwhile();
+  } else {
+    const unsigned int edges = e.es->edge_count;
+    const int failed = e.es->bucket_failed;
+    if (tid == 0) { out.kept = 0; out.examined = n; }
+    WalkThreads::sync();
+    const bool last = crew.rank() == crew.size() - 1;
+    bool settled = !failed && edges <= (unsigned)p.cap_edges;
+    if (settled)
+      settled = walk_pairs<WalkThreads>(p, p.cand, n, edges, sm, &out.kept, &out.examined, [&](int a, int i, int c) {
+        kept_at[a] = (unsigned short)i;
+        if (last) { p.kept[a] = c; p.kept_pos[a] = i; }
+      });
+    if (tid == 0) out.settled = settled;
+  }
+  __syncthreads();
+}
+__device__ __forceinline__ bool walk_is_open(const Problem& p, const Settled& w, int n) { return !w.settled || (w.kept < p.n_keep && n < p.n_cand); }
+// One thread, when everybody has read what it changes.
+__device__ __forceinline__ void settle_note(const Engine& e, const Settled& w) {
+  EngineState* es = e.es;
+  // after an overflow the buckets are left alone: for a round, then twice as long after every further one, to 64
+  // (a count of rounds, not the round to wait for: strads_set_round may go back); this round's walk counts too
+  if (!w.settled) es->avoid = 1 + (1 << es->streak);
+  es->streak = w.settled ? 0 : min(es->streak + 1, 6);
+  es->bucket_failed = 0; es->edge_count = 0u;
 }
 
 // The walk over all candidates by half the warps, with `draws` the draw of round td up to the collection of its k winners by the

@@ -553,9 +553,10 @@ struct ChangedByBin { int before[kHistBins + (kHistBins >> 5)]; int head[kHistBi
 // The kept coefficients' changes: how many move, the largest, the keys that change (in any order), and for dense X the
 // moving columns in list order.  Returns the number that move.
 constexpr int kFewChanged = 48;            // kept coefficients up to which draw_rank counts through all changed keys
+// kept_at: the positions of the kept candidates, where they are in shared memory (else null).
 template <bool kDense>
-__device__ int gather_changes(const Problem& p, const Binning& bins, int nk, bool want_keys, unsigned long long* keys, ChangedByBin* cb, Moving* mv,
-                              ChangeShared& cs) {
+__device__ __forceinline__ int gather_changes(const Problem& p, const Binning& bins, int nk, const unsigned short* kept_at, bool want_keys, unsigned long long* keys,
+                                              ChangedByBin* cb, Moving* mv, ChangeShared& cs) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool indexed = want_keys && nk > kFewChanged;
   __syncthreads();
@@ -571,7 +572,7 @@ __device__ int gather_changes(const Problem& p, const Binning& bins, int nk, boo
   double d_first = 0.0;
   int moving = 0;
   for (int a = a_lo; a < a_hi; ++a) {
-    const int pos = p.kept_pos[a];
+    const int pos = !kDense && kept_at != nullptr ? (int)kept_at[a] : p.kept_pos[a];
     const double d = p.cand_dbeta64[pos];
     unsigned long long o = 0ull, w = 0ull;
     if (want_keys) { o = p.cand_keys[pos]; w = p.cand_keys[p.n_cand + pos]; }
@@ -625,6 +626,12 @@ __device__ int gather_changes(const Problem& p, const Binning& bins, int nk, boo
 __device__ __forceinline__ void prefetch_l2(const void* from, const void* to) {
   const unsigned long long lo = (unsigned long long)from & ~15ull, hi = ((unsigned long long)to + 15ull) & ~15ull;
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(lo), "r"((unsigned)(hi - lo)) : "memory");
+}
+
+// (cold)
+template <bool kDense>
+__device__ __noinline__ int gather_again(const Problem& p, const Binning& bins, int nk, unsigned long long* keys, ChangedByBin* cb, Moving* mv, ChangeShared& cs) {
+  return gather_changes<kDense>(p, bins, nk, nullptr, true, keys, cb, mv, cs);
 }
 
 // Winners ranked; with changes, corrected for the kept coefficients' changed priorities (keys[0 .. n_changed) old,

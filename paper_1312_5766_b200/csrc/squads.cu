@@ -21,6 +21,11 @@ namespace {
 constexpr int kHeldEntries = 512;
 struct HeldEntries { int row[kHeldEntries]; float val[kHeldEntries]; };      // a warp's
 constexpr size_t kHeldSmem = sizeof(HeldEntries) * kWarps;
+// Shared memory of a round's update and of what follows it.
+__host__ __device__ inline size_t squad_smem(const Problem& p, bool ahead) {
+  const size_t changes = (ahead ? 2 * sizeof(unsigned long long) * (size_t)p.n_keep : 0) + sizeof(ChangedByBin);
+  return changes > kHeldSmem ? changes : kHeldSmem;
+}
 
 struct Turn {
   unsigned int* count;
@@ -49,22 +54,24 @@ struct Held {
   int a, pos, j, len, at;                  // place in the kept list and among the candidates, coefficient, entries, where they wait (-1: in X)
   long long q0;
 };
-__device__ __forceinline__ Held hold(const Squad& crew, const Problem& p, int nk, int chunk, HeldEntries* entry) {
+// kept_at: their positions where they are in shared memory (else null).  ranked: the next candidates may be in the place of these.
+__device__ __forceinline__ Held hold(const Squad& crew, const Problem& p, int nk, const unsigned short* kept_at, int chunk, HeldEntries* entry, bool ranked) {
   const int lane = threadIdx.x & 31, warp = (int)threadIdx.x >> 5;
   const int first = warp * crew.size() + crew.rank(), step = kWarps * crew.size();
   Held h;
   h.n = nk > first ? (nk - first + step - 1) / step : 0;
   const bool on = chunk * 32 + lane < h.n;
   h.a = first + (chunk * 32 + lane) * step; h.pos = 0; h.j = 0; h.len = 0; h.q0 = 0; h.at = -1;
-  if (on) h.pos = p.kept_pos[h.a];
-  if (entry == nullptr) {                                // (not p.walk_cols: behind the last barrier others rank the next candidates)
-    if (on) { h.j = p.kept[h.a]; h.q0 = p.xptr[h.j]; h.len = (int)(p.xptr[h.j + 1] - h.q0); }
-    return h;
-  }
   if (on) {
-    const WalkColumn col = p.walk_cols[h.pos];
-    h.j = col.j; h.len = max(col.n, 0); h.q0 = col.q0;
+    h.pos = kept_at != nullptr ? (int)kept_at[h.a] : p.kept_pos[h.a];
+    if (ranked) {
+      h.j = p.kept[h.a]; h.q0 = p.xptr[h.j]; h.len = (int)(p.xptr[h.j + 1] - h.q0);
+    } else {
+      const WalkColumn col = p.walk_cols[h.pos];
+      h.j = col.j; h.len = max(col.n, 0); h.q0 = col.q0;
+    }
   }
+  if (entry == nullptr) return h;
   int incl = h.len;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -102,13 +109,15 @@ __device__ __forceinline__ void for_held(const Problem& p, const Held& h, int ch
 }
 
 // False: a wait gave up.
-__device__ __forceinline__ bool squad_update(const Squad& crew, const Problem& p, const Engine& e, unsigned char* sm, Grid& g, const Turn& turn, int nk,
-                                             unsigned long long t_next, bool want_keys) {
+// own: the walk was this CTA's own (kept_at, and notes to be made), else null.
+__device__ __forceinline__ bool squad_update(const Squad& crew, const Problem& p, const Engine& e, unsigned char* sm, Grid& g, const Turn& turn, const Settled* own,
+                                             const unsigned short* kept_at, unsigned long long t_next, bool want_keys) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   HeldEntries* entry = reinterpret_cast<HeldEntries*>(sm) + warp;
   EngineState* es = e.es;
   __syncthreads();                                       // (what lay there before)
-  Held h = hold(crew, p, nk, 0, entry);
+  const int nk = own != nullptr ? own->kept : es->n_kept, examined = own != nullptr ? own->examined : es->n_examined;
+  const Held h = hold(crew, p, nk, kept_at, 0, entry, false);
   double n2 = 0.0;
   float E = 0.f;
   const bool on0 = lane < h.n;
@@ -116,7 +125,6 @@ __device__ __forceinline__ bool squad_update(const Squad& crew, const Problem& p
     n2 = p.n2[h.j];
     if (want_keys) E = exponential_of(p, t_next, (uint32_t)h.j);
   }
-  const int examined = es->n_examined;
   const float x_max = p.st->x_abs_max;
   asm volatile("cp.async.wait_all;" ::: "memory");
   if (!await_turn(turn)) return false;                   // (a barrier of the CTA in it)
@@ -127,7 +135,7 @@ __device__ __forceinline__ bool squad_update(const Squad& crew, const Problem& p
 #pragma unroll 1
   for (int chunk = 0; chunk * 32 < h.n; ++chunk) {
     Held c = h;
-    if (chunk > 0) c = hold(crew, p, nk, chunk, nullptr);
+    if (chunk > 0) c = hold(crew, p, nk, kept_at, chunk, nullptr, false);
     const bool on = chunk * 32 + lane < h.n;
     const int m = min(32, h.n - chunk * 32);
     float b_old = 0.f, d_old = 0.f;
@@ -183,7 +191,7 @@ __device__ __forceinline__ bool squad_update(const Squad& crew, const Problem& p
       const Proposal q = propose_begin(p, c.j, n2, b_old, d_old, E, want_keys);
       const Change ch = propose_end(p, q, c.pos, c.j, dot, E, want_keys);
       p.beta[c.j] = ch.b_new;
-      p.delta[c.j] = (float)fabs(ch.d);
+      if (!want_keys) p.delta[c.j] = (float)fabs(ch.d);  // (else the draw may want it as it was: commit_deltas)
       p.dbeta[c.a] = (float)ch.d;
       if (!isfinite(ch.d)) atomicOr(&p.st->status, STRADS_STATUS_NONFINITE);
       moving += ch.d != 0.0;
@@ -202,6 +210,7 @@ __device__ __forceinline__ bool squad_update(const Squad& crew, const Problem& p
     }
   }
   if (!grid_sync(g)) return false;
+  if (own != nullptr && crew.rank() == 0 && tid == 0) settle_note(e, *own);
   // ---- the residual: sums in fixed point (engine_csc.cuh), then every row once ----
   const unsigned long long largest = __ldcg(&es->turn_dmax);
   const int n_moving = (int)__ldcg(&es->turn_moving);
@@ -211,7 +220,7 @@ __device__ __forceinline__ bool squad_update(const Squad& crew, const Problem& p
 #pragma unroll 1
     for (int chunk = 0; chunk * 32 < h.n; ++chunk) {
       Held c = h;
-      if (chunk > 0) c = hold(crew, p, nk, chunk, nullptr);
+      if (chunk > 0) c = hold(crew, p, nk, kept_at, chunk, nullptr, false);
       const double d_lane = change_of(c, chunk);
       double d = 0.0;
       for_held(p, c, chunk, entry, [&](int k) { d = __shfl_sync(kFull, d_lane, k); return d != 0.0; }, [&](int, int row, float v) {
@@ -227,7 +236,7 @@ __device__ __forceinline__ bool squad_update(const Squad& crew, const Problem& p
 #pragma unroll 1
       for (int chunk = 0; chunk * 32 < h.n; ++chunk) {
         Held c = h;
-        if (chunk > 0) c = hold(crew, p, nk, chunk, nullptr);
+        if (chunk > 0) c = hold(crew, p, nk, kept_at, chunk, nullptr, true);
         const double d_lane = change_of(c, chunk);
         const int m = min(32, h.n - chunk * 32);
         constexpr int kU = 4;                            // columns at a time
@@ -270,12 +279,17 @@ __device__ __forceinline__ bool squad_update(const Squad& crew, const Problem& p
   for (int a = nk + tid * crew.size() + crew.rank(); a < p.n_keep; a += kT * crew.size()) { p.kept[a] = -1; p.dbeta[a] = 0.f; }
   return true;
 }
+__device__ __forceinline__ void commit_deltas(const Squad& crew, const Problem& p, int nk, const unsigned short* kept_at) {
+  for (int a = (int)threadIdx.x * crew.size() + crew.rank(); a < nk; a += kT * crew.size())
+    p.delta[p.kept[a]] = (float)fabs(p.cand_dbeta64[kept_at != nullptr ? (int)kept_at[a] : p.kept_pos[a]]);
+}
 
 __global__ void __launch_bounds__(kT, 1) k_squads(const __grid_constant__ SquadSet set, int n_rounds, int have_list, int draw_next) {
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ DrawShared ds;
   __shared__ TurnShared ts;
   __shared__ ChangeShared cs;
+  __shared__ Settled walk;
   __shared__ Problem sp;                                 // copies for the functions that are called rarely and not inlined
   __shared__ Engine se;
   const int tid = threadIdx.x, squad = (int)blockIdx.x / set.size, n_squads = set.n;
@@ -307,6 +321,7 @@ __global__ void __launch_bounds__(kT, 1) k_squads(const __grid_constant__ SquadS
   unsigned long long t = t0 + (unsigned long long)((squad - (int)(t0 % (unsigned)n_squads) + n_squads) % n_squads);
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(sm);
   ChangedByBin* cb = reinterpret_cast<ChangedByBin*>(sm + (e.n_list > 0 ? 2 * sizeof(unsigned long long) * (size_t)p.n_keep : 0));
+  unsigned short* kept_at = reinterpret_cast<unsigned short*>(sm + kept_at_offset(p, squad_smem(p, e.n_list > 0)));
   const bool no_filter = (p.flags & STRADS_FLAG_NO_FILTER) != 0, uniform = (p.flags & STRADS_FLAG_UNIFORM_DRAW) != 0;
   const int n_total = p.n_cand;
   bool have = have_list != 0, ok = true;
@@ -317,7 +332,7 @@ __global__ void __launch_bounds__(kT, 1) k_squads(const __grid_constant__ SquadS
     const bool draws = !real || (e.n_list > 0 && (t + (unsigned)n_squads < t_end || draw_next));
     const unsigned long long td = real ? t + (unsigned)n_squads : t;             // the round drawn for
     const unsigned int k = real ? (unsigned)e.n_list : (unsigned)n_total;
-    bool scanned = !draws, collected = !draws, spare = false;
+    bool scanned = !draws, collected = !draws, own = false;                // own: the kept list is this CTA's own
     const int n = no_filter ? p.n_keep : e.window;
     bool window = no_filter || (p.bucket_count != nullptr && !(n < n_total && es->skip_window) && es->avoid == 0);
     if (real) csc_enter(crew, p, e, window ? n : n_total, window && !no_filter);
@@ -336,7 +351,7 @@ __global__ void __launch_bounds__(kT, 1) k_squads(const __grid_constant__ SquadS
         for (int i = tid; i < p.n_keep; i += kT) { p.kept[i] = p.cand[i]; p.kept_pos[i] = i; }
         if (tid == 0) { es->n_kept = p.n_keep; es->n_examined = p.n_keep; es->walk_open = 0; }
       }
-      if (!collected && !ahead && !during_walk) { draw_gather<AllThreads>(crew, p, e, ds, k, spare); collected = true; }
+      if (!collected && !ahead && !during_walk) { draw_gather<AllThreads>(crew, p, e, ds, k, false); collected = true; }
       if (real && !window) {
         int walked = 0;
         if (!(ok = csc_walk_and_draw(crew, p, sp, e, ds, sm, g, g_draw, during_walk, td, k, &walked))) break;
@@ -346,34 +361,39 @@ __global__ void __launch_bounds__(kT, 1) k_squads(const __grid_constant__ SquadS
       }
       if (!(ok = grid_sync(g))) break;
       if (!ahead) break;
-      if (walker) csc_walk_window(p, e, sm, n);
-      const ClearAhead rows = csc_clear_begin(crew, p, n);
-      if (!collected) { draw_gather<AllThreads>(crew, p, e, ds, k, true); collected = true; spare = true; }
-      csc_clear_end(p, rows);
+      csc_settle(crew, p, e, sm, kept_at, walk, n, [&]() {
+        const ClearAhead rows = csc_clear_begin(crew, p, n);
+        if (!collected) draw_gather<OtherThreads>(crew, p, e, ds, k, false);
+        csc_clear_end(p, rows);
+      });
+      collected = true;
+      if (!walk_is_open(p, walk, n)) { own = true; break; }              // (the update's barriers stand for one here)
       if (!(ok = grid_sync(g))) break;
-      if (!es->walk_open) break;
+      if (crew.r == 0 && tid == 0) settle_note(e, walk);
       csc_enter(crew, p, e, n_total, false);
       window = false;
     }
     if (!ok) break;
+    // ---- the update in its turn, then the list of this squad's next round ----
+    const int n_next = no_filter ? p.n_keep : (e.window < n_total && es->skip_window ? n_total : e.window);   // looked at first
+    const unsigned short* at = own ? kept_at : nullptr;
+    const int nk = own ? walk.kept : es->n_kept;
+    if (real) {
+      turn.target = gridDim.x + (unsigned)(t - t0) * (unsigned)crew.n;
+      if (!(ok = squad_update(crew, p, e, sm, g, turn, own ? &walk : nullptr, at, td, draws && !uniform))) break;
+      t += (unsigned)n_squads;
+    }
     if (draws && es->mend) {
       keep_parameters();
       if (!(ok = draw_mend(crew, sp, se, ds, sm, td, k, g))) break;
     }
-    // ---- the update in its turn, then the list of this squad's next round ----
-    int n_changed = 0, nk = 0;
-    const int n_next = no_filter ? p.n_keep : (e.window < n_total && es->skip_window ? n_total : e.window);   // looked at first
-    if (real) {
-      nk = es->n_kept;
-      turn.target = gridDim.x + (unsigned)(t - t0) * (unsigned)crew.n;
-      if (!(ok = squad_update(crew, p, e, sm, g, turn, nk, td, draws && !uniform))) break;
-      if (draws && !uniform) {                           // (equal weights: no key changes)
-        gather_changes<false>(p, binning_of(ds.cut), nk, true, keys, cb, nullptr, cs);
-        n_changed = cs.n_changed;
-      }
-      t += (unsigned)n_squads;
+    int n_changed = 0;
+    if (real && draws && !uniform) {                     // (equal weights: no key changes)
+      gather_changes<false>(p, binning_of(ds.cut), nk, at, true, keys, cb, nullptr, cs);
+      n_changed = cs.n_changed;
+      commit_deltas(crew, p, nk, at);
     }
-    if (draws) draw_rank<false>(crew, p, e, ds, keys, cb, n_changed, n_changed > 0 ? nk : 0, cs.rank_wsum, spare ? max(1, crew.n - 1) : crew.n, n_next);
+    if (draws) draw_rank<false>(crew, p, e, ds, keys, cb, n_changed, n_changed > 0 ? nk : 0, cs.rank_wsum, crew.n, n_next);
     have = draws;
     if (!(ok = grid_sync(g))) break;
   }
@@ -397,7 +417,8 @@ cudaError_t prepare_squads() {
 
 cudaError_t launch_squads(const SquadSet& set, int n_rounds, bool have_list, bool draw_next, cudaStream_t s) {
   size_t smem = engine_smem(set.p[0], set.e[0].n_list > 0);
-  if (smem < kHeldSmem) smem = kHeldSmem;
+  const size_t update = kept_at_offset(set.p[0], squad_smem(set.p[0], set.e[0].n_list > 0)) + sizeof(unsigned short) * (size_t)set.p[0].n_keep;
+  if (smem < update) smem = update;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;

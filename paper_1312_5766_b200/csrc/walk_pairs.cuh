@@ -27,12 +27,20 @@ __host__ __device__ inline size_t walk_pairs_smem(int n_cand, unsigned int n_edg
   return 3 * bytes + 2 * sizeof(unsigned int) * words + sizeof(unsigned int) * (size_t)n_edges;
 }
 
-// Returns whether the walk was settled (uniform over the CTA).  If so, kept_out[0 .. *n_kept) and
-// p.kept_pos[0 .. *n_kept) hold the kept coefficients and their positions in the list, and *n_examined the
-// position after the P-th kept one (left alone when fewer than P are kept).  n_kept / n_examined: shared memory.
+// The threads that walk: the kNT of a CTA, or (a type of the same form) its first kN with a barrier of their own.
 template <int kNT>
-__device__ bool walk_from_pair_list(const Problem& p, const int* cand, int n_cand, unsigned int n_edges,
-                                    unsigned char* sm, int* kept_out, int* n_kept, int* n_examined) {
+struct WalkByCta {
+  static constexpr int kN = kNT;
+  static __device__ __forceinline__ void sync() { __syncthreads(); }
+  static __device__ __forceinline__ bool any(int x) { return __syncthreads_or(x) != 0; }
+};
+
+// Returns whether the walk was settled (uniform over the walking threads).  If so, put(a, i, cand[i]) has been called for the a-th
+// kept candidate, at position i of the list, a < *n_kept, and *n_examined is the position after the P-th kept one (left alone when
+// fewer than P are kept).  n_kept / n_examined: shared memory.
+template <typename Walkers, typename Put>
+__device__ bool walk_pairs(const Problem& p, const int* cand, int n_cand, unsigned int n_edges, unsigned char* sm, int* n_kept, int* n_examined, Put&& put) {
+  constexpr int kNT = Walkers::kN;
   const int tid = threadIdx.x, lane = tid & 31;
   const size_t bytes = ((size_t)n_cand + 15) & ~(size_t)15;
   const int n_words = (n_cand + 31) / 32;
@@ -51,14 +59,14 @@ __device__ bool walk_from_pair_list(const Problem& p, const int* cand, int n_can
   for (int i = tid; i < n_cand; i += kNT) state[i] = 1;                    // kept unless a listed pair says otherwise
 #pragma unroll 1
   for (unsigned int k = tid; k < n_edges; k += kNT) e[k] = __ldcg(p.edges + k);
-  __syncthreads();
+  Walkers::sync();
   if (n_edges > 0) {
 #pragma unroll 1
     for (unsigned int k = tid; k < n_edges; k += kNT) {                   // (several threads may store the same values: benign)
       const int b = (int)(e[k] & 0xffffu);
       state[b] = 0; hit[b] = 0; pend[b] = 0;
     }
-    __syncthreads();
+    Walkers::sync();
     bool settled = false;
 #pragma unroll 1
     for (int pass = 0; pass < kSparsePasses && !settled; ++pass) {
@@ -72,7 +80,7 @@ __device__ bool walk_from_pair_list(const Problem& p, const int* cand, int n_can
           else if (sa == 0) pend[b] = mark;
         }
       }
-      __syncthreads();
+      Walkers::sync();
       int open = 0;
 #pragma unroll 1
       for (unsigned int k = tid; k < n_edges; k += kNT) {                 // every thread that shares b reads the same and stores the same
@@ -83,7 +91,7 @@ __device__ bool walk_from_pair_list(const Problem& p, const int* cand, int n_can
           else open = 1;
         }
       }
-      settled = __syncthreads_or(open) == 0;
+      settled = !Walkers::any(open);
     }
     if (!settled) return false;
   }
@@ -95,7 +103,7 @@ __device__ bool walk_from_pair_list(const Problem& p, const int* cand, int n_can
     const unsigned int word = __ballot_sync(0xffffffffu, i < n_cand && state[i] == 1);
     if (lane == 0) wbits[i0 >> 5] = word;
   }
-  __syncthreads();
+  Walkers::sync();
   if (tid < 32) {
     unsigned int carry = 0u;
 #pragma unroll 1
@@ -113,7 +121,7 @@ __device__ bool walk_from_pair_list(const Problem& p, const int* cand, int n_can
     }
     if (lane == 0) wpre[n_words] = carry;
   }
-  __syncthreads();
+  Walkers::sync();
   int u = 0;
 #pragma unroll 1
   for (int i = tid; i < n_cand; i += kNT, ++u) {
@@ -123,15 +131,22 @@ __device__ bool walk_from_pair_list(const Problem& p, const int* cand, int n_can
       if (rank < p.n_keep) {
         int c;
         switch (u) { case 0: c = cv[0]; break; case 1: c = cv[1]; break; case 2: c = cv[2]; break; case 3: c = cv[3]; break; default: c = cand[i]; }
-        kept_out[rank] = c;
-        p.kept_pos[rank] = i;
+        put(rank, i, c);
         if (rank == p.n_keep - 1) *n_examined = i + 1;     // the walk stops here
       }
     }
   }
   if (tid == 0) *n_kept = min((int)wpre[n_words], p.n_keep);
-  __syncthreads();
+  Walkers::sync();
   return true;
+}
+
+// By a whole CTA, into kept_out and p.kept_pos.
+template <int kNT>
+__device__ __forceinline__ bool walk_from_pair_list(const Problem& p, const int* cand, int n_cand, unsigned int n_edges,
+                                                    unsigned char* sm, int* kept_out, int* n_kept, int* n_examined) {
+  return walk_pairs<WalkByCta<kNT>>(p, cand, n_cand, n_edges, sm, n_kept, n_examined,
+                                    [&](int rank, int i, int c) { kept_out[rank] = c; p.kept_pos[rank] = i; });
 }
 
 }  // namespace strads
