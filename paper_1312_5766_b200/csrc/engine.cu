@@ -884,6 +884,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
       if (n < n_total && es->skip_window && !no_filter) n = n_total;
     } else {
       window = no_filter || (p.bucket_count != nullptr && !(n < n_total && es->skip_window) && es->avoid == 0);
+      if (real && window && !no_filter) csc_norms_begin(p, e, sm, n);
       if (real) csc_enter(WholeGrid(), p, e, window ? n : n_total, window && !no_filter);
     }
     // ---- steps 1 to 3, once more over all candidates where a window does not do ----
@@ -904,7 +905,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
       if (kDense) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // (the Gram's operands come in over it)
       // (the walk needs nothing of what is before it but the norms that follow beta and delta)
       if (ahead) {
-        if (!kDense) csc_products_begin(p, e, sm, n);
+        if (!kDense) csc_products_begin(sm);
         if (!(ok = grid_complete(g))) break;
       } else if (!(!kDense && real && !window && !(p.flags & STRADS_FLAG_DYNAMIC_DEPS)) && !(ok = grid_sync(g))) {
         break;
@@ -954,7 +955,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
       if (!real || no_filter) break;
       if (!kDense) {
         if (!window) break;
-        csc_settle(WholeGrid(), p, e, sm, kept_at, walk, n, [&]() {
+        csc_settle(p, e, sm, kept_at, walk, n, [&]() {
           const ClearAhead rows = csc_clear_begin(WholeGrid(), p, n);
           if (!collected) draw_gather<OtherThreads>(WholeGrid(), p, e, ds, k, false);
           csc_clear_end(p, rows);
@@ -980,7 +981,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
       KeptColumns kept;
       if (!kDense) kept = kept_columns(WholeGrid(), p, nk, pending ? kept_at : nullptr);
       if (pending) grid_arrive(g);
-      n_moving = gather_changes<kDense>(p, binning_of(ds.cut), nk, pending ? kept_at : nullptr, draws, keys, cb, mv, cs);
+      n_moving = gather_changes<kDense>(p, ds, nk, pending ? kept_at : nullptr, draws, keys, cb, mv, cs);
       last.nk = nk; last.n_moving = n_moving;
       if (!kDense) {
         last.shift = csc_shift(p.st->x_abs_max, cs.dmax, nk);
@@ -995,7 +996,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
     if (draws && es->mend) {
       keep_parameters();
       if (!(ok = draw_mend(WholeGrid(), sp, se, ds, sm, td, k, g))) break;
-      if (real) gather_again<kDense>(sp, binning_of(ds.cut), nk, keys, cb, mv, cs);
+      if (real) gather_again<kDense>(sp, ds, nk, keys, cb, mv, cs);
     }
     if (real) {
       commit_changes(p, examined, nk, n_moving, out, final_round);

@@ -158,12 +158,20 @@ __device__ __forceinline__ void csc_norms(const Problem& p, const Engine& e, uns
   float* norm_f = reinterpret_cast<float*>(sm + sizeof(MetTable) * kWorkers);
   for (int i = threadIdx.x; i < min(count, kNear); i += kT) norm_f[i] = __ldcg(e.norm_f + i);
 }
-__device__ __forceinline__ void csc_products_begin(const Problem& p, const Engine& e, unsigned char* sm, int count) {
+// (behind the scan's shared memory and that of what comes before it, so that they come in beside both)
+__device__ __forceinline__ void csc_norms_begin(const Problem& p, const Engine& e, unsigned char* sm, int count) {
+  static_assert(sizeof(MetTable) * kWorkers >= kScanSmem, "the norms lie behind the scan's shared memory");
+  if (p.flags & STRADS_FLAG_DYNAMIC_DEPS) return;
+  const uint32_t norm_f = smem_u32(sm + sizeof(MetTable) * kWorkers);
+  for (int i = threadIdx.x; i < min(count, kNear); i += kT)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(norm_f + 4u * (unsigned)i), "l"(e.norm_f + i) : "memory");
+}
+__device__ __forceinline__ void csc_products_begin(unsigned char* sm) {
   MetTable& wt = reinterpret_cast<MetTable*>(sm)[threadIdx.x >> 5];
+  asm volatile("cp.async.wait_all;" ::: "memory");       // (the norms)
   __syncthreads();                                       // (what lay there before)
   if (threadIdx.x < 32 * kWorkers)
     for (int i = threadIdx.x & 31; i < kReach / 4; i += 32) reinterpret_cast<float4*>(wt.dot)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (!(p.flags & STRADS_FLAG_DYNAMIC_DEPS)) csc_norms(p, e, sm, count);
 }
 template <bool kDots, typename Crew>
 __device__ __forceinline__ void csc_products(const Crew& crew, const Problem& p, const Engine& e, TurnShared& ts, unsigned char* sm, int count, bool kept, bool pairs,
@@ -397,7 +405,7 @@ __device__ __forceinline__ void for_moving_entries(const Crew& crew, const Probl
 }
 
 // A warp's kept columns (a mod warps of the crew): lane k has the k-th.  kept_at: positions of the kept candidates in shared memory, read
-// before anybody can rank the next candidates over these; null: the lists in global memory.
+// before anybody can rank the next candidates over these, and entered into the lists in global memory; null: from there.
 struct KeptColumns { int m, len; long long q0; double d; };
 template <typename Crew>
 __device__ __forceinline__ KeptColumns kept_columns(const Crew& crew, const Problem& p, int nk, const unsigned short* kept_at) {
@@ -410,6 +418,7 @@ __device__ __forceinline__ KeptColumns kept_columns(const Crew& crew, const Prob
     const int pos = kept_at[a];
     const WalkColumn col = p.walk_cols[pos];
     c.d = p.cand_dbeta64[pos]; c.q0 = col.q0; c.len = col.n;
+    p.kept[a] = col.j; p.kept_pos[a] = pos;
   } else {
     const int j = p.kept[a];
     c.d = p.cand_dbeta64[p.kept_pos[a]]; c.q0 = p.xptr[j]; c.len = (int)(p.xptr[j + 1] - c.q0);
@@ -1143,7 +1152,7 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Crew& crew, const Probl
 
 // The walk from the list of the window's conflicting pairs, by every CTA for itself with half its threads -- what it needs is in L2 for all of
 // them behind the barrier, and nobody then waits for one of them -- while the others do what else there is (`meanwhile`).  The kept
-// candidates' positions go to kept_at (shared memory, not among the walk's own); the last CTA leaves the lists in global memory as well.
+// candidates' positions go to kept_at (shared memory, not among the walk's own); whoever fetches their columns leaves the lists in global memory.
 // All threads of the CTA; settle_note makes the notes behind a barrier.
 struct WalkThreads {
   static constexpr int kN = kWalkT;
@@ -1160,8 +1169,8 @@ __host__ __device__ inline size_t kept_at_offset(const Problem& p, size_t change
   const size_t walk = walk_pairs_smem(p.n_cand, (unsigned)p.cap_edges);
   return ((walk > changes ? walk : changes) + 15) & ~(size_t)15;
 }
-template <typename Crew, typename F>
-__device__ __forceinline__ void csc_settle(const Crew& crew, const Problem& p, const Engine& e, unsigned char* sm, unsigned short* kept_at, Settled& out, int n,
+template <typename F>
+__device__ __forceinline__ void csc_settle(const Problem& p, const Engine& e, unsigned char* sm, unsigned short* kept_at, Settled& out, int n,
                                            F&& meanwhile) {
   const int tid = threadIdx.x;
   __syncthreads();                                       // (what lay there before)
@@ -1172,13 +1181,9 @@ __device__ __forceinline__ void csc_settle(const Crew& crew, const Problem& p, c
     const int failed = e.es->bucket_failed;
     if (tid == 0) { out.kept = 0; out.examined = n; }
     WalkThreads::sync();
-    const bool last = crew.rank() == crew.size() - 1;
     bool settled = !failed && edges <= (unsigned)p.cap_edges;
     if (settled)
-      settled = walk_pairs<WalkThreads>(p, p.cand, n, edges, sm, &out.kept, &out.examined, [&](int a, int i, int c) {
-        kept_at[a] = (unsigned short)i;
-        if (last) { p.kept[a] = c; p.kept_pos[a] = i; }
-      });
+      settled = walk_pairs<WalkThreads>(p, nullptr, n, edges, sm, &out.kept, &out.examined, [&](int a, int i, int) { kept_at[a] = (unsigned short)i; });
     if (tid == 0) out.settled = settled;
   }
   __syncthreads();

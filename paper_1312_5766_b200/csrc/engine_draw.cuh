@@ -555,10 +555,14 @@ struct ChangedByBin { int before[kHistBins + (kHistBins >> 5)]; int head[kHistBi
 constexpr int kFewChanged = 48;            // kept coefficients up to which draw_rank counts through all changed keys
 // kept_at: the positions of the kept candidates, where they are in shared memory (else null).
 template <bool kDense>
-__device__ __forceinline__ int gather_changes(const Problem& p, const Binning& bins, int nk, const unsigned short* kept_at, bool want_keys, unsigned long long* keys,
+__device__ __forceinline__ int gather_changes(const Problem& p, const DrawShared& ds, int nk, const unsigned short* kept_at, bool want_keys, unsigned long long* keys,
                                               ChangedByBin* cb, Moving* mv, ChangeShared& cs) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool indexed = want_keys && nk > kFewChanged;
+  const Binning bins = binning_of(ds.cut);
+  // Keys behind the boundary's bin concern no rank -- unless the winners are all there are -- and are not entered: most new keys are
+  // there, those beyond the cutoff all in one bin, one after the other (50,000 x 1,000,000: a step of 3 us of 34).
+  const int last_bin = (long long)ds.total >= (p.part_count > 1 ? owned_count(p) : p.J) ? kHistBins : ds.bnd;
   __syncthreads();
   if (tid == 0) { cs.n_changed = 0; cs.dmax = 0ull; }
   if (indexed) {
@@ -571,24 +575,44 @@ __device__ __forceinline__ int gather_changes(const Problem& p, const Binning& b
   unsigned long long dmax = 0ull;
   double d_first = 0.0;
   int moving = 0;
-  for (int a = a_lo; a < a_hi; ++a) {
-    const int pos = !kDense && kept_at != nullptr ? (int)kept_at[a] : p.kept_pos[a];
-    const double d = p.cand_dbeta64[pos];
-    unsigned long long o = 0ull, w = 0ull;
-    if (want_keys) { o = p.cand_keys[pos]; w = p.cand_keys[p.n_cand + pos]; }
-    if (a == a_lo) d_first = d;
-    moving += d != 0.0;
-    dmax = max(dmax, (unsigned long long)__double_as_longlong(fabs(d)));
-    if (o != w) {
-      const int at = atomicAdd(&cs.n_changed, 1);
-      keys[at] = o;
-      keys[p.n_keep + at] = w;
+  constexpr int kU = kDense ? 1 : 2;                     // entries of a thread at a time (dense: rarely more than one)
+#pragma unroll 1
+  for (int i0 = 0; i0 < per; i0 += kU) {
+    double d[kU];
+    unsigned long long o[kU], w[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int a = a_lo + i0 + u;
+      d[u] = 0.0; o[u] = w[u] = 0ull;
+      if (i0 + u < per && a < a_hi) {
+        const int pos = !kDense && kept_at != nullptr ? (int)kept_at[a] : p.kept_pos[a];
+        d[u] = p.cand_dbeta64[pos];
+        if (want_keys) { o[u] = p.cand_keys[pos]; w[u] = p.cand_keys[p.n_cand + pos]; }
+      }
+    }
+    if (i0 == 0) d_first = d[0];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      moving += d[u] != 0.0;
+      dmax = max(dmax, (unsigned long long)__double_as_longlong(fabs(d[u])));
+      const unsigned int changed = __ballot_sync(kFull, o[u] != w[u]);
+      if (changed == 0u) continue;
+      int at = 0;                                        // (one addition per warp: they all go to one address)
+      if (lane == 0) at = atomicAdd(&cs.n_changed, __popc(changed));
+      at = __shfl_sync(kFull, at, 0) + __popc(changed & ((1u << lane) - 1u));
+      if (o[u] == w[u]) continue;
+      keys[at] = o[u];
+      keys[p.n_keep + at] = w[u];
       if (indexed) {                                     // by bin: a count for the prefix sum, and a list
-        const unsigned int bo = bin_of(bins, (unsigned int)(o >> 32)), bw = bin_of(bins, (unsigned int)(w >> 32));
-        atomicAdd(&cb->before[pad((int)bo)], -1);
-        atomicAdd(&cb->before[pad((int)bw)], 1);
-        cb->next[2 * at] = (unsigned short)atomicExch(&cb->head[bo], 2 * at);
-        cb->next[2 * at + 1] = (unsigned short)atomicExch(&cb->head[bw], 2 * at + 1);
+        const int bo = (int)bin_of(bins, (unsigned int)(o[u] >> 32)), bw = (int)bin_of(bins, (unsigned int)(w[u] >> 32));
+        if (bo <= last_bin) {
+          atomicAdd(&cb->before[pad(bo)], -1);
+          cb->next[2 * at] = (unsigned short)atomicExch(&cb->head[bo], 2 * at);
+        }
+        if (bw <= last_bin) {
+          atomicAdd(&cb->before[pad(bw)], 1);
+          cb->next[2 * at + 1] = (unsigned short)atomicExch(&cb->head[bw], 2 * at + 1);
+        }
       }
     }
   }
@@ -630,8 +654,8 @@ __device__ __forceinline__ void prefetch_l2(const void* from, const void* to) {
 
 // (cold)
 template <bool kDense>
-__device__ __noinline__ int gather_again(const Problem& p, const Binning& bins, int nk, unsigned long long* keys, ChangedByBin* cb, Moving* mv, ChangeShared& cs) {
-  return gather_changes<kDense>(p, bins, nk, nullptr, true, keys, cb, mv, cs);
+__device__ __noinline__ int gather_again(const Problem& p, const DrawShared& ds, int nk, unsigned long long* keys, ChangedByBin* cb, Moving* mv, ChangeShared& cs) {
+  return gather_changes<kDense>(p, ds, nk, nullptr, true, keys, cb, mv, cs);
 }
 
 // Winners ranked; with changes, corrected for the kept coefficients' changed priorities (keys[0 .. n_changed) old,

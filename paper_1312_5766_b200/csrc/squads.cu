@@ -69,6 +69,7 @@ __device__ __forceinline__ Held hold(const Squad& crew, const Problem& p, int nk
     } else {
       const WalkColumn col = p.walk_cols[h.pos];
       h.j = col.j; h.len = max(col.n, 0); h.q0 = col.q0;
+      if (kept_at != nullptr) { p.kept[h.a] = h.j; p.kept_pos[h.a] = h.pos; }
     }
   }
   if (entry == nullptr) return h;
@@ -335,6 +336,7 @@ __global__ void __launch_bounds__(kT, 1) k_squads(const __grid_constant__ SquadS
     bool scanned = !draws, collected = !draws, own = false;                // own: the kept list is this CTA's own
     const int n = no_filter ? p.n_keep : e.window;
     bool window = no_filter || (p.bucket_count != nullptr && !(n < n_total && es->skip_window) && es->avoid == 0);
+    if (real && window && !no_filter) csc_norms_begin(p, e, sm, n);
     if (real) csc_enter(crew, p, e, window ? n : n_total, window && !no_filter);
     // ---- the block; once more over all candidates where a window does not do ----
     while (true) {
@@ -342,7 +344,7 @@ __global__ void __launch_bounds__(kT, 1) k_squads(const __grid_constant__ SquadS
       if (ahead) grid_arrive(g);
       if (!scanned && !during_walk) { draw_scan(crew, p, e, ds, sm, td, true); scanned = true; }
       if (ahead) {
-        csc_products_begin(p, e, sm, n);
+        csc_products_begin(sm);
         if (!(ok = grid_complete(g))) break;
       } else if (!(real && !window && !(p.flags & STRADS_FLAG_DYNAMIC_DEPS)) && !(ok = grid_sync(g))) {
         break;
@@ -361,7 +363,7 @@ __global__ void __launch_bounds__(kT, 1) k_squads(const __grid_constant__ SquadS
       }
       if (!(ok = grid_sync(g))) break;
       if (!ahead) break;
-      csc_settle(crew, p, e, sm, kept_at, walk, n, [&]() {
+      csc_settle(p, e, sm, kept_at, walk, n, [&]() {
         const ClearAhead rows = csc_clear_begin(crew, p, n);
         if (!collected) draw_gather<OtherThreads>(crew, p, e, ds, k, false);
         csc_clear_end(p, rows);
@@ -389,7 +391,7 @@ __global__ void __launch_bounds__(kT, 1) k_squads(const __grid_constant__ SquadS
     }
     int n_changed = 0;
     if (real && draws && !uniform) {                     // (equal weights: no key changes)
-      gather_changes<false>(p, binning_of(ds.cut), nk, at, true, keys, cb, nullptr, cs);
+      gather_changes<false>(p, ds, nk, at, true, keys, cb, nullptr, cs);
       n_changed = cs.n_changed;
       commit_deltas(crew, p, nk, at);
     }

@@ -35,8 +35,8 @@ struct WalkByCta {
   static __device__ __forceinline__ bool any(int x) { return __syncthreads_or(x) != 0; }
 };
 
-// Returns whether the walk was settled (uniform over the walking threads).  If so, put(a, i, cand[i]) has been called for the a-th
-// kept candidate, at position i of the list, a < *n_kept, and *n_examined is the position after the P-th kept one (left alone when
+// Returns whether the walk was settled (uniform over the walking threads).  If so, put(a, i, c) has been called for the a-th
+// kept candidate, at position i of the list, a < *n_kept (c = cand[i]; cand may be null), and *n_examined is the position after the P-th kept one (left alone when
 // fewer than P are kept).  n_kept / n_examined: shared memory.
 template <typename Walkers, typename Put>
 __device__ bool walk_pairs(const Problem& p, const int* cand, int n_cand, unsigned int n_edges, unsigned char* sm, int* n_kept, int* n_examined, Put&& put) {
@@ -54,9 +54,9 @@ __device__ bool walk_pairs(const Problem& p, const int* cand, int n_cand, unsign
   constexpr int kAhead = 4;
   int cv[kAhead];
 #pragma unroll
-  for (int u = 0; u < kAhead; ++u) cv[u] = tid + u * kNT < n_cand ? cand[tid + u * kNT] : 0;
+  for (int u = 0; u < kAhead; ++u) cv[u] = cand != nullptr && tid + u * kNT < n_cand ? cand[tid + u * kNT] : 0;
 #pragma unroll 1
-  for (int i = tid; i < n_cand; i += kNT) state[i] = 1;                    // kept unless a listed pair says otherwise
+  for (int i = tid; i < (int)(bytes / 16); i += kNT) reinterpret_cast<uint4*>(state)[i] = make_uint4(0x01010101u, 0x01010101u, 0x01010101u, 0x01010101u);   // kept unless a listed pair says otherwise
 #pragma unroll 1
   for (unsigned int k = tid; k < n_edges; k += kNT) e[k] = __ldcg(p.edges + k);
   Walkers::sync();
@@ -130,7 +130,7 @@ __device__ bool walk_pairs(const Problem& p, const int* cand, int n_cand, unsign
       const int rank = (int)wpre[i >> 5] + __popc(word & ((1u << lane) - 1u));
       if (rank < p.n_keep) {
         int c;
-        switch (u) { case 0: c = cv[0]; break; case 1: c = cv[1]; break; case 2: c = cv[2]; break; case 3: c = cv[3]; break; default: c = cand[i]; }
+        switch (u) { case 0: c = cv[0]; break; case 1: c = cv[1]; break; case 2: c = cv[2]; break; case 3: c = cv[3]; break; default: c = cand != nullptr ? cand[i] : 0; }
         put(rank, i, c);
         if (rank == p.n_keep - 1) *n_examined = i + 1;     // the walk stops here
       }
