@@ -17,6 +17,7 @@ using namespace strads;
 struct Scheduler {
   alignas(64) unsigned char gram_tmap[128];   // tensor map over the BF16 copies of its candidates (dense layouts)
   Problem p;
+  Engine draw;               // buffers of its draws made launch by launch
   int walk_grid;             // CTAs of the cooperative on-demand walk (CSC)
   cudaStream_t stream;       // S > 1: steps 1 and 2 of its rounds are enqueued here
   cudaEvent_t block_ready;   // its block (the kept list) is complete
@@ -43,6 +44,7 @@ struct strads_lasso_s {
   // Sampling ahead (one scheduler; strads_run only): the draw of round t + 1 runs on its own stream beside the Gram
   // and walk of round t, and the round then starts from that list corrected for round t's update.
   bool ahead_ok;             // the configuration allows it
+  Engine ahead_draw;
   Problem ahead;             // the early draw's view of the problem: own sampler state and buffers, P' + P winners
   cudaStream_t ahead_stream;
   cudaEvent_t ahead_fork, ahead_done;
@@ -172,6 +174,7 @@ constexpr int kEngineRounds = 32;     // rounds per launch of the engine: a laun
 constexpr int kEngineDenseRows = 2048;
 constexpr int kEngineMinCtas = 32;    // a lane per kept column of a warp
 constexpr int kEngineMaxCtas = 192;   // CTAs the engine's scratch provides for
+constexpr int kDrawCtas = 16;         // CTAs a draw's scratch provides for
 constexpr int kSquadRounds = 64;      // rounds per launch of the squads (the first block and the last update of a launch overlap with nothing)
 constexpr int kStaticSquads = 4;      // blocks under way with the static schedule
 constexpr int kSquadMinCtas = 8;      // CTAs of a squad at least
@@ -202,7 +205,7 @@ struct Layout {
       off_conflict, off_cand_dbeta64, off_cand_bnew, off_dot_partial, off_dot_ticket, off_margin, off_obj, off_amb, off_xcb, off_walk_blocked, off_walk_ctl, off_walk_cols,
       off_bucket_count, off_bucket_items, off_bucket_vals, off_bucket_cols, off_bucket_own, off_resid_acc, off_delta_prev, off_edges, off_patch_keys, off_cand_keys, off_survivors, off_bin_off, off_bin_cur, off_ahead_bin_off, off_ahead_bin_cur,
       off_ahead_state, off_ahead_hist, off_ahead_sure, off_ahead_boundary, off_ahead_keys, off_ahead_idx,
-      off_eng_state, off_eng_hist, off_eng_cur, off_eng_win, off_eng_surv, off_eng_saved, off_eng_xb, off_eng_norm, off_eng_part, off_eng_tickets, total;
+      off_eng_state, off_eng_hist, off_eng_cur, off_eng_win, off_eng_surv, off_eng_saved, off_eng_xb, off_eng_norm, off_eng_part, off_eng_tickets, off_draw[2], total;
   long long eng_pitch, eng_lo;
   long long eng_saved;
   int eng_list, eng_tiles;
@@ -269,6 +272,13 @@ int squads_of(const strads_lasso_config_t* c, int n_ctas) {
 unsigned int engine_saved(size_t winners) { return (unsigned int)(winners / 16 + 64); }
 size_t engine_boundary(size_t winners) { return winners / 2 > 2048 ? winners / 2 : 2048; }
 
+// Draws launch by launch go in one launch of a cluster up to so many coefficients.
+constexpr long long kClusterDrawCols = 1 << 19;
+// Its scratch for n winners: state, histogram, cursors, counts, keys below the cutoff (a few times n).
+size_t draw_bytes(int n) {
+  return align_up(sizeof(EngineState)) + 2 * sizeof(unsigned int) * kHistBins + align_up(sizeof(unsigned int) * kDrawCtas) +
+         sizeof(unsigned long long) * (6 * (size_t)n + 256 * kDrawCtas);
+}
 // Slice of the workspace of one scheduler or squad; the first one (`first`) also holds what all share
 // (column norms, the objective's partial sums).  `engine`: with the buffers of rounds in one launch.
 Layout carve(const strads_lasso_config_t* c, bool first, bool engine) {
@@ -368,6 +378,10 @@ Layout carve(const strads_lasso_config_t* c, bool first, bool engine) {
   L.off_eng_norm = take(en ? sizeof(double) * (size_t)c->n_candidates : 0);
   L.off_eng_part = take(en && dense ? sizeof(float) * 128 * 128 * (size_t)kEngineMaxCtas : 0);
   L.off_eng_tickets = take(sizeof(unsigned int) * (size_t)L.eng_tiles);
+  for (int i = 0; i < 2; ++i) {
+    const int n = i == 0 ? c->n_candidates : L.n_ahead;
+    L.off_draw[i] = take(c->n_cols <= kClusterDrawCols && n > 0 ? draw_bytes(n) : 0);
+  }
   L.total = o;
   return L;
 }
@@ -669,6 +683,24 @@ void fill_ahead(Problem& a, const Problem& p0, const Layout& L, char* ws) {
   a.survivors = nullptr; a.cap_survivors = 0;         // (the early draw is off the round's path: it keeps to the plain passes)
 }
 
+// The draw of p in one launch of a cluster: its scratch, the winners where the three launches have theirs.
+bool fill_draw(Engine& en, const Problem& p, const Layout& L, char* ws, int i, int n_ctas) {
+  if (p.J > kClusterDrawCols || n_ctas == 0) return false;
+  char* at = ws + L.off_draw[i];
+  en = Engine();
+  en.es = reinterpret_cast<EngineState*>(at); at += align_up(sizeof(EngineState));
+  en.hist = reinterpret_cast<unsigned int*>(at); at += sizeof(unsigned int) * kHistBins;
+  en.bin_cur = reinterpret_cast<unsigned int*>(at); at += sizeof(unsigned int) * kHistBins;
+  en.saved = reinterpret_cast<unsigned int*>(at); at += align_up(sizeof(unsigned int) * kDrawCtas);
+  en.surv = reinterpret_cast<unsigned long long*>(at);
+  en.grid = n_ctas;
+  en.cap_surv = (unsigned int)((6 * (size_t)p.n_cand + 256 * kDrawCtas) / n_ctas);
+  en.win = p.sure;                                       // (the boundary's keys lie behind them)
+  en.cap_boundary = p.cap_boundary;
+  en.cap_win = (int)(p.boundary - p.sure) + p.cap_boundary;
+  return true;
+}
+
 // For n_ctas CTAs; whole: all of them, one round after the other.
 void fill_engine(Engine& en, const Problem& p, const Layout& L, char* ws, int n_ctas, bool whole) {
   en.es = reinterpret_cast<EngineState*>(ws + L.off_eng_state);
@@ -689,6 +721,12 @@ void fill_engine(Engine& en, const Problem& p, const Layout& L, char* ws, int n_
   en.norm_f = reinterpret_cast<float*>(ws + L.off_eng_norm);
   en.part = reinterpret_cast<float*>(ws + L.off_eng_part);
   en.tile_ticket = reinterpret_cast<unsigned int*>(ws + L.off_eng_tickets);
+}
+
+// Whether the Gram of the window leaves the SMs of a few clusters free for a draw beside it.
+bool draw_beside_gram(const Problem& p) {
+  const long long side = (window_of(p, p.n_cand) + 127) / 128;
+  return side * (side + 1) / 2 * 8 * 2 <= p.sm_count;
 }
 
 // What must be zero before a launch of the engine or the squads (they leave it so, unless a wait expired).
@@ -788,6 +826,16 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
   if ((e = prepare_sample(p0)) != cudaSuccess) return fail(cuda_fail(e, "prepare_sample"));
   if ((e = prepare_filter(p0)) != cudaSuccess) return fail(cuda_fail(e, "prepare_filter"));
   if ((e = prepare_gram_dense_tc()) != cudaSuccess) return fail(cuda_fail(e, "prepare_gram_dense_tc"));
+  int draw_ctas = 0;
+  if ((e = prepare_draw_cluster(&draw_ctas)) != cudaSuccess) return fail(cuda_fail(e, "prepare_draw_cluster"));
+  for (int s = 0; s < S; ++s) {
+    Scheduler& sc = h->sch[s];
+    if (!fill_draw(sc.draw, sc.p, s == 0 ? L : Lrest, s == 0 ? ws : ws + L.total + (size_t)(s - 1) * Lrest.total, 0, draw_ctas)) continue;
+    sc.p.draw = &sc.draw;
+    if ((e = cudaMemsetAsync(sc.draw.es, 0, sizeof(EngineState), h->stream)) != cudaSuccess ||
+        (e = cudaMemsetAsync(sc.draw.hist, 0, sizeof(unsigned int) * kHistBins, h->stream)) != cudaSuccess)
+      return fail(cuda_fail(e, "cudaMemsetAsync"));
+  }
   if ((e = launch_init(p0, h->stream)) != cudaSuccess) return fail(cuda_fail(e, "launch_init"));
   if ((e = launch_resid_from_beta(p0, h->stream)) != cudaSuccess) return fail(cuda_fail(e, "launch_resid_from_beta"));
   if ((e = want_stream(&kit.copy, 0)) != cudaSuccess || (e = want_event(&kit.copy_fork)) != cudaSuccess ||
@@ -808,6 +856,13 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
   h->ahead_ok = S == 1 && L.n_ahead > 0;
   if (h->ahead_ok) {
     fill_ahead(h->ahead, p0, L, ws);
+    h->ahead.draw = nullptr;
+    if (draw_beside_gram(p0) && fill_draw(h->ahead_draw, h->ahead, L, ws, 1, draw_ctas)) {
+      h->ahead.draw = &h->ahead_draw;
+      if ((e = cudaMemsetAsync(h->ahead_draw.es, 0, sizeof(EngineState), h->stream)) != cudaSuccess ||
+          (e = cudaMemsetAsync(h->ahead_draw.hist, 0, sizeof(unsigned int) * kHistBins, h->stream)) != cudaSuccess)
+        return fail(cuda_fail(e, "cudaMemsetAsync"));
+    }
     if ((e = launch_init_scheduler(h->ahead, p0, h->stream)) != cudaSuccess) return fail(cuda_fail(e, "launch_init_scheduler"));
     if ((e = want_stream(&kit.ahead, prio_least)) != cudaSuccess || (e = want_event(&kit.ahead_fork)) != cudaSuccess ||
         (e = want_event(&kit.ahead_done)) != cudaSuccess || (e = want_stream(&kit.retry, prio_least)) != cudaSuccess ||

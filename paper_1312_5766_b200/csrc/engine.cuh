@@ -94,6 +94,11 @@ cudaError_t encode_engine_maps(const Problem& p, const Engine& e, void* out_256_
 cudaError_t launch_engine(const Problem& p, const Engine& e, const void* maps, int n_rounds, bool have_list, bool draw_next,
                           const strads_round_out_t* out, cudaStream_t s);
 
+// The draw of p (as launch_sample's) in one launch of a thread-block cluster of e.grid CTAs; e: es, hist (zero before and after), bin_cur, win,
+// surv, saved.  *ctas: its size on the current device (0: none).
+cudaError_t prepare_draw_cluster(int* ctas);
+cudaError_t launch_draw_cluster(const Problem& p, const Engine& e, int* cand_out, cudaStream_t s);
+
 // CSC rounds whose blocks do not wait for one another's updates: several schedulers, or the static schedule.  As many squads of CTAs as
 // there are blocks under way; problem i / engine i: the i-th squad's, which takes the rounds t with t mod n == i.
 constexpr int kMaxSquads = STRADS_MAX_SCHEDULERS;

@@ -62,17 +62,32 @@ __device__ bool grid_complete(const Grid& g) {
 // The CTAs that make a round together: all of them, or as many of them as prepare the rounds whose turn is theirs (squads.cu).
 struct WholeGrid {
   static constexpr bool kParts = false;    // all coefficients
+  static constexpr bool kKeys = false;     // the winners' keys are not wanted beside the list
   static constexpr int kTogether = 1;      // entries of a list that a warp goes through side by side: it has one as a rule
   __device__ __forceinline__ int rank() const { return (int)blockIdx.x; }
   __device__ __forceinline__ int size() const { return (int)gridDim.x; }
 };
 struct Squad {
   static constexpr bool kParts = true;     // a scheduler's
+  static constexpr bool kKeys = false;
   static constexpr int kTogether = 4;
   int r, n;
   __device__ __forceinline__ int rank() const { return r; }
   __device__ __forceinline__ int size() const { return n; }
 };
+
+// The CTAs of a launch of one thread-block cluster (draw_cluster.cu), and their barrier.
+struct ClusterCrew {
+  static constexpr bool kParts = true, kKeys = true;
+  static constexpr int kTogether = 1;
+  __device__ __forceinline__ int rank() const { return (int)blockIdx.x; }
+  __device__ __forceinline__ int size() const { return (int)gridDim.x; }
+};
+struct ClusterGrid {};
+__device__ __forceinline__ bool grid_sync(ClusterGrid&) {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  return true;
+}
 
 // The threads of a CTA that do a step together: all of them, or those that do not walk while the others do (below).
 constexpr int kWalkT = 256;                // threads that walk
@@ -440,8 +455,8 @@ __device__ __forceinline__ void draw_collect(const Crew& crew, const Engine& e, 
 
 // Rare: more keys share the boundary bin than there is room for (thousands of tied times).  The grid cuts the bin
 // further, digit by digit, over all J keys.  False: a barrier gave up.
-template <typename Crew>
-__device__ __noinline__ bool draw_refine(const Crew& crew, const Problem& p, const Engine& e, DrawShared& ds, unsigned char* sm, unsigned long long t, unsigned int k, Grid& g) {
+template <typename Crew, typename G>
+__device__ __noinline__ bool draw_refine(const Crew& crew, const Problem& p, const Engine& e, DrawShared& ds, unsigned char* sm, unsigned long long t, unsigned int k, G& g) {
   const int tid = threadIdx.x, warp = tid >> 5;
   unsigned int* sh = reinterpret_cast<unsigned int*>(sm);
   uint2* queue = reinterpret_cast<uint2*>(sm + sizeof(unsigned int) * kHistBins) + warp * kQueue;
@@ -515,8 +530,8 @@ __device__ __forceinline__ void draw_gather(const Crew& crew, const Problem& p, 
 }
 
 // (cold) by all CTAs.  False: a barrier gave up.
-template <typename Crew>
-__device__ __noinline__ bool draw_mend(const Crew& crew, const Problem& p, const Engine& e, DrawShared& ds, unsigned char* sm, unsigned long long t, unsigned int k, Grid& g) {
+template <typename Crew, typename G>
+__device__ __noinline__ bool draw_mend(const Crew& crew, const Problem& p, const Engine& e, DrawShared& ds, unsigned char* sm, unsigned long long t, unsigned int k, G& g) {
   draw_select_all(e, ds, k);
   if (!grid_sync(g)) return false;                       // everybody has read the counts and the flag
   if (crew.rank() == 0 && threadIdx.x == 0) e.es->mend = 0;
@@ -758,6 +773,7 @@ __device__ __forceinline__ void draw_rank(const Crew& crew, const Problem& p, co
     const int rank = (int)first + below;
     if (on && slice == 0 && (fresh || !struck) && (unsigned)rank < (unsigned)p.n_cand) {
       p.cand[rank] = j;
+      if (Crew::kKeys && p.keys_out != nullptr) p.keys_out[rank] = key;
       // the columns of the next round's window start towards L2 while this round's changes are applied
       if (kDense) {
         if (rank < n_prefetch)

@@ -523,6 +523,7 @@ cudaError_t launch_sample_patch(const Problem& p, const Problem& ahead, int* can
 }
 
 cudaError_t launch_sample(const Problem& p, int* cand_out, cudaStream_t s) {
+  if (p.draw != nullptr) return launch_draw_cluster(p, *p.draw, cand_out, s);
   const long long groups = (p.J + 3) >> 2;
   long long blocks = (groups + kThreads - 1) / kThreads;
   // (an early draw runs beside the round's Gram and walk and leaves them most of every SM)

@@ -77,6 +77,7 @@ static constexpr int kHistBits = 12;
 static constexpr int kHistBins = 1 << kHistBits;
 
 // Everything a launch needs; filled once at init (host copy in the handle).
+struct Engine;
 struct Problem {
   int layout;
   long long N, J, ld;
@@ -150,6 +151,7 @@ struct Problem {
   // pairs (a << 16 | b, a < b, positions in the list) and the walk works from that list when it is complete.
   unsigned int* edges;                   // [cap_edges]
   int cap_edges;
+  const Engine* draw;                    // (host) its draws go in one launch of a cluster, with these buffers (null: three launches)
   // scheduler threads: this Problem is scheduler part_index of part_count and owns { j : j mod part_count == part_index }
   int part_count, part_index;
   // bounded device-side waits: iteration limit of every spin (0: each kernel's own default), and, for exercising the
