@@ -847,6 +847,8 @@ __device__ __forceinline__ bool settle_rest(const Crew& crew, const Problem& p, 
 // The columns of all candidates lie where p.walk_cols says (written behind the last barrier's far side).  draw(): what the other
 // threads do meanwhile, with the grid barrier g_draw; false: it gave up.  Every CTA leaves the places of the kept list that it
 // owns (a mod ctas) and, in *n_kept, their number.  False: a barrier gave up.
+// Nobody need have met before: others may still be applying the last round's changes to the residual, or reading how this round is to be
+// made, which CTA 0 decides anew at the end.  A walk without a barrier -- its first batch was the last one -- has one there.
 template <typename Draw, typename Crew>
 __device__ __forceinline__ bool csc_walk_on_demand(const Crew& crew, const Problem& p, Problem& sp, const Engine& e, unsigned char* sm, Grid& g, Grid& g_draw, int* n_kept,
                                                    Draw&& draw) {
@@ -856,6 +858,7 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Crew& crew, const Probl
   // this CTA's words of the mask: cta, cta + n_ctas, ...; its k-th candidate is bit k & 31 of the (k / 32)-th of them
   const int own_words = W > cta ? (W - cta + n_ctas - 1) / n_ctas : 0, n_own = own_words * 32, n_here = min(n_own, kOwn);
   auto own_index = [&](int k) { return ((cta + (k >> 5) * n_ctas) << 5) | (k & 31); };
+  const unsigned int begun = g.target;
   __syncthreads();
   if (warp >= kWalkWarps) {
     for (int w = tid - kWalkT; w < own_words; w += kT - kWalkT) s.own_word[w] = s.own_hit[w] = 0u;
@@ -1134,6 +1137,7 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Crew& crew, const Probl
       if (!(ok = walk_barrier(s, g))) break;
     }
     if (!held) asm volatile("bar.sync 3, %0;" ::"n"(kT) : "memory");
+    if (ok && walk_to_meet(begun, g.target)) ok = walk_barrier(s, g);
     if (tid == 0) {
       s.kept = kept; s.ok = ok; s.target = g.target;
       if (cta == 0 && ok) {
