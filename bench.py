@@ -231,12 +231,12 @@ def rooflines(p: wl.LassoProblem, workload: str, step_ms: dict, kept_per_round: 
     else:
         nnz_col = p.nnz / p.n_cols
         if step_ms["walk_ms"] >= step_ms["gram_ms"]:
-            # its longest step is the walk on demand: every kept candidate's column against every later candidate not yet
-            # blocked (at most all examined ones), counted as merges of <= 2 nnz_col - 1 compare steps (the kernel looks rows up)
-            ops = kept_per_round * examined_per_round * (2.0 * nnz_col - 1.0)
+            # its longest step is the walk on demand: whichever way it goes, every entry of an examined candidate has to be looked up once
+            # among the rows of those before it
+            ops = examined_per_round * nnz_col
         else:
-            # its longest step is the inner products of the window's pairs that share a row
-            ops = 0.5 * window * (window - 1) * (nnz_col * nnz_col / p.n_rows) * (2.0 * nnz_col - 1.0)
+            # its longest step is the inner products of the window's pairs that share a row: a multiplication per pair and row
+            ops = 0.5 * window * (window - 1) * nnz_col * nnz_col / p.n_rows
         # whole rounds in one launch: the kernel of the timed regions, all its steps in its time
         kernel = "k_engine<csc>"
         rounds = min(steps, ENGINE_ROUNDS)
@@ -246,13 +246,13 @@ def rooflines(p: wl.LassoProblem, workload: str, step_ms: dict, kept_per_round: 
         peak = 148 * 128 * peaks["sm_max_mhz"] * 1e6 / 1e12        # integer / FP32 lanes x clock, T op/s
         achieved = ops / (ms * 1e-3) / 1e12
         out["roofline"] = {
-            "kernel": kernel, "bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tcompare/s",
+            "kernel": kernel, "bound": "alu", "achieved": achieved, "peak": peak, "unit": "Top/s",
             "frac": achieved / peak, "traffic": traffic and traffic * rounds, "window": window, "launch_ms": ms,
             "rounds_per_launch": rounds, "algorithmic_ops_per_launch": ops,
-            "peak_source": "148 SMs x 128 lanes x max SM clock: one merge step (compare + advance) per lane per cycle",
-            "note": f"a launch is {rounds} whole rounds; of their steps only the inner products of sparse columns are "
-                    "counted, as the sorted-list merge steps they stand for, over a few MB of columns: bound by dependent loads and barriers, "
-                    "not by HBM"}
+            "peak_source": "148 SMs x 128 lanes x max SM clock: one operation per lane per cycle",
+            "note": f"a launch is {rounds} whole rounds; of their steps only the inner products of sparse columns are counted, by what they "
+                    "cannot do without (a look-up per entry examined, or a multiplication per row that two candidates share): the round is "
+                    "bound by dependent loads and barriers, so the fraction says how little of it is arithmetic"}
         upd_bytes = 8.0 * nnz_col * kept_per_round + 8.0 * p.n_rows
         pack_bytes = 0.0
         ns_bytes = 8.0 * nnz_col * (p.n_candidates + kept_per_round) + 8.0 * p.n_rows
