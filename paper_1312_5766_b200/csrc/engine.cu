@@ -905,7 +905,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
       if (kDense) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // (the Gram's operands come in over it)
       // (the walk needs nothing of what is before it but the norms that follow beta and delta)
       if (ahead) {
-        if (!kDense) csc_products_begin(sm);
+        if (!kDense) csc_products_begin(sm, n);
         if (!(ok = grid_complete(g))) break;
       } else if (!(!kDense && real && !window && !(p.flags & STRADS_FLAG_DYNAMIC_DEPS)) && !(ok = grid_sync(g))) {
         break;

@@ -11,14 +11,19 @@ namespace {
 // (its terms in a list of the warp's own in shared memory: no barrier), no conflict bits (the walk works from the list
 // of conflicting pairs or forms rows on demand), and x_c^T r with the same visit to the column.
 // ------------------------------------------------------------------------------------------------
-constexpr int kMet = 512;                                // candidates one candidate may meet (of kReach)
+constexpr int kMet = 512;                                // candidates one candidate may meet
 constexpr int kRing = 4;                                 // steps of terms under way, and the one at hand
-constexpr int kReach = 1664;                             // candidates a warp has a place for at a time: a window of 1,024 kept
+constexpr int kReach = 1664;                             // candidates of a window for each of which a warp has a place: 1,024 kept
+constexpr int kPlaces = 1024;                            // ... places where there are more: at most half of them in use
+constexpr unsigned short kNobody = 0xffff;
 constexpr int kPart = 64;                                // positions of a column at a time
 constexpr int kWorkers = kWarps - 1;                     // warps that form products; the last one makes the would-be changes
 struct __align__(16) MetTable {
   int4 entry[kPart];                     // of a position of the column: row, terms before it, value, its own place in the row's bucket
-  float dot[kReach];                     // by candidate; zero between candidates
+  union {
+    float dot[kReach];                   // by candidate; zero between candidates
+    struct { float of_place[kPlaces]; unsigned short who[kPlaces]; };    // more candidates than that: by place (the same dot[]), and whose it is
+  };
   unsigned short met[kMet];              // the places in use
   unsigned char lane[kReach];            // that had a term of the candidate last
   unsigned char pos[kPart * kBucketSlots];   // position of a term
@@ -28,6 +33,26 @@ struct __align__(16) MetTable {
 constexpr int kNear = 2048;                              // candidates whose norms a CTA keeps in shared memory
 constexpr size_t kTermsSmem = sizeof(MetTable) * kWorkers + sizeof(float) * kNear;
 static_assert(STRADS_MAX_CANDIDATES < 0xffff && kPart <= 256, "16 bits per candidate, 8 per position");
+static_assert(kPlaces + kPlaces / 2 <= kReach && kMet + 32 < kPlaces, "in the same memory; a search ends");
+
+// The place of candidate b among more than kReach, taken if it has none: the next free one from its own number on.  Lanes that want the same
+// free place all write to it and read who has it.  (Going through a candidate's terms once for every kReach candidates instead: us per
+// round, 200,000 x 1,000,000 of 50 entries, P = 2,048, window of 6,000 75.4 -> 59.7, of 3,200 43.5 -> 41.6; P = 1,025, of 1,792 36.2 -> 34.1.
+// Places of their own need no search: P = 1,024, of 1,664, 33.3.)
+__device__ __forceinline__ int place_of(MetTable& wt, int b, bool on) {
+  int at = b & (kPlaces - 1);
+  bool open = on;
+#pragma unroll 1
+  while (__any_sync(kFull, open)) {
+    if (open && wt.who[at] == kNobody) wt.who[at] = (unsigned short)b;
+    __syncwarp();
+    if (open) {
+      if (wt.who[at] == (unsigned short)b) open = false;
+      else at = (at + 1) & (kPlaces - 1);
+    }
+  }
+  return at;
+}
 
 // The entries of candidates [0, n) into the buckets of their rows.  Where the columns lie was noted when the candidates
 // were ranked, but for the dependencies dropped at run time (coupling_n2 follows beta and delta).
@@ -166,12 +191,14 @@ __device__ __forceinline__ void csc_norms_begin(const Problem& p, const Engine& 
   for (int i = threadIdx.x; i < min(count, kNear); i += kT)
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(norm_f + 4u * (unsigned)i), "l"(e.norm_f + i) : "memory");
 }
-__device__ __forceinline__ void csc_products_begin(unsigned char* sm) {
+__device__ __forceinline__ void csc_products_begin(unsigned char* sm, int count) {
   MetTable& wt = reinterpret_cast<MetTable*>(sm)[threadIdx.x >> 5];
   asm volatile("cp.async.wait_all;" ::: "memory");       // (the norms)
   __syncthreads();                                       // (what lay there before)
   if (threadIdx.x < 32 * kWorkers)
-    for (int i = threadIdx.x & 31; i < kReach / 4; i += 32) reinterpret_cast<float4*>(wt.dot)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = threadIdx.x & 31; i < kReach / 4; i += 32)
+      reinterpret_cast<float4*>(wt.dot)[i] = count > kReach && i >= kPlaces / 4 ? make_float4(__int_as_float(-1), __int_as_float(-1), __int_as_float(-1), __int_as_float(-1))
+                                                                              : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 template <bool kDots, typename Crew>
 __device__ __forceinline__ void csc_products(const Crew& crew, const Problem& p, const Engine& e, TurnShared& ts, unsigned char* sm, int count, bool kept, bool pairs,
@@ -182,6 +209,7 @@ __device__ __forceinline__ void csc_products(const Crew& crew, const Problem& p,
   MetTable& wt = reinterpret_cast<MetTable*>(sm)[warp];
   float* norm_f = reinterpret_cast<float*>(sm + sizeof(MetTable) * kWorkers);
   const int mine = count > cta ? (count - cta + n_ctas - 1) / n_ctas : 0;
+  const bool direct = count <= kReach;
   if (mine == 0) return;
   if (pairs && (p.flags & STRADS_FLAG_DYNAMIC_DEPS)) {
     csc_norms(p, e, sm, count);
@@ -226,9 +254,7 @@ __device__ __forceinline__ void csc_products(const Crew& crew, const Problem& p,
         }
       };
       if (col.n <= 0) tell();
-      const int reach0 = pairs ? a / kReach * kReach : 0;
-#pragma unroll 1
-      for (int reach = reach0; reach == reach0 || reach < count; reach += kReach) {      // (one trip up to a window of kReach)
+      {
         int n_met = 0;                                   // (the same in all lanes)
         bool failed = false;
 #pragma unroll 1
@@ -247,15 +273,13 @@ __device__ __forceinline__ void csc_products(const Crew& crew, const Problem& p,
           float x[2];
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            x[h] = kDots && r[h] >= 0 && reach == reach0 ? p.resid[r[h]] : 0.f;
+            x[h] = kDots && r[h] >= 0 ? p.resid[r[h]] : 0.f;
             cnt[h] = pairs && r[h] >= 0 ? p.bucket_count[r[h]] : 0u;
           }
-          if (reach == reach0) {
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
-              if (kDots && r[h] >= 0) acc += (double)v[h] * (double)x[h];
-            if (q0 + kPart >= col.n) tell();
-          }
+          for (int h = 0; h < 2; ++h)
+            if (kDots && r[h] >= 0) acc += (double)v[h] * (double)x[h];
+          if (q0 + kPart >= col.n) tell();
           if (!pairs) continue;
 #pragma unroll
           for (int h = 0; h < 2; ++h)
@@ -306,8 +330,8 @@ __device__ __forceinline__ void csc_products(const Crew& crew, const Problem& p,
               const int2 m = wt.term[i % kRing][lane];
               term.b = m.x; term.fb = __int_as_float(m.y); term.fa = wt.value[i % kRing][lane];
             }
-            const bool on = term.b > a && (unsigned)(term.b - reach) < (unsigned)kReach;
-            const int b = on ? term.b - reach : 0;
+            const bool on = term.b > a && (direct || n_met <= kMet);
+            const int b = direct ? (on ? term.b : 0) : place_of(wt, term.b, on);
             if (on) wt.lane[b] = (unsigned char)lane;
             __syncwarp();
             float old = 1.f;
@@ -335,7 +359,7 @@ __device__ __forceinline__ void csc_products(const Crew& crew, const Problem& p,
             __syncwarp();
           }
         }
-        if (!pairs) break;
+        if (!pairs) continue;
         const bool overflow = __any_sync(kFull, failed) || n_met > kMet;
         if (overflow && lane == 0) e.es->bucket_failed = 1;
         // which of them conflict: those that may are gathered first, so that the far accesses are made for all of them at once
@@ -343,11 +367,12 @@ __device__ __forceinline__ void csc_products(const Crew& crew, const Problem& p,
         int n_near = 0;
 #pragma unroll 1
         for (int i0 = 0; i0 < min(n_met, kMet); i0 += 32) {
-          const bool on = i0 + lane < min(n_met, kMet);
-          const int b = on ? wt.met[i0 + lane] : 0;
+          bool on = i0 + lane < min(n_met, kMet);
+          const int b = on ? wt.met[i0 + lane] : 0, c = direct ? b : wt.who[b];
+          on = on && (direct || c != kNobody);           // (listed twice, and settled)
           const float dot = on ? wt.dot[b] : 0.f;
-          const bool near = on && may_conflict(dot, limit_a, b + reach < kNear ? norm_f[b + reach] : __ldcg(e.norm_f + b + reach));
-          if (on && !near) wt.dot[b] = 0.f;
+          const bool near = on && may_conflict(dot, limit_a, c < kNear ? norm_f[c] : __ldcg(e.norm_f + c));
+          if (on && !near) { wt.dot[b] = 0.f; if (!direct) wt.who[b] = kNobody; }
           const unsigned int m = __ballot_sync(kFull, near);
           if (near) wt.met[n_near + __popc(m & ((1u << lane) - 1u))] = (unsigned short)b;      // (places that have been read)
           n_near += __popc(m);
@@ -355,25 +380,29 @@ __device__ __forceinline__ void csc_products(const Crew& crew, const Problem& p,
         }
 #pragma unroll 1
         for (int i0 = 0; i0 < n_near; i0 += 32) {
-          const bool on = i0 + lane < n_near;
-          const int b = on ? wt.met[i0 + lane] : 0;
+          bool on = i0 + lane < n_near;
+          const int b = on ? wt.met[i0 + lane] : 0, c = direct ? b : wt.who[b];
+          on = on && (direct || c != kNobody);
           const float dot = on ? wt.dot[b] : 0.f;
           __syncwarp();
           bool conflict = false;
           if (on) {
             wt.dot[b] = 0.f;
-            conflict = dot != 0.f && in_conflict(dot, limit_a, col.n2, b + reach < kNear ? norm_f[b + reach] : __ldcg(e.norm_f + b + reach), p.walk_cols + b + reach, rho);
+            if (!direct) wt.who[b] = kNobody;
+            conflict = dot != 0.f && in_conflict(dot, limit_a, col.n2, c < kNear ? norm_f[c] : __ldcg(e.norm_f + c), p.walk_cols + c, rho);
           }
           const unsigned int m = __ballot_sync(kFull, conflict);
           if (m == 0u) continue;
           unsigned int at = 0u;
           if (lane == 0) at = atomicAdd(&e.es->edge_count, (unsigned)__popc(m));
           at = __shfl_sync(kFull, at, 0) + (unsigned)__popc(m & ((1u << lane) - 1u));
-          if (conflict && at < (unsigned)p.cap_edges) p.edges[at] = ((unsigned int)a << 16) | (unsigned)(b + reach);
+          if (conflict && at < (unsigned)p.cap_edges) p.edges[at] = ((unsigned int)a << 16) | (unsigned)c;
         }
         __syncwarp();
-        if (n_met > kMet)                                // (places that were not listed)
-          for (int i = lane; i < kReach; i += 32) wt.dot[i] = 0.f;
+        if (n_met > kMet) {                              // (places that were not listed)
+          for (int i = lane; i < (direct ? kReach : kPlaces); i += 32) wt.dot[i] = 0.f;
+          for (int i = lane; i < (direct ? 0 : kPlaces); i += 32) wt.who[i] = kNobody;
+        }
         __syncwarp();
       }
     }

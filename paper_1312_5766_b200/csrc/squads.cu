@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(kT, 1) k_squads(const __grid_constant__ SquadS
       if (ahead) grid_arrive(g);
       if (!scanned && !during_walk) { draw_scan(crew, p, e, ds, sm, td, true); scanned = true; }
       if (ahead) {
-        csc_products_begin(sm);
+        csc_products_begin(sm, n);
         if (!(ok = grid_complete(g))) break;
       } else if (!(real && !window && !(p.flags & STRADS_FLAG_DYNAMIC_DEPS)) && !(ok = grid_sync(g))) {
         break;

@@ -181,3 +181,48 @@ def test_launches_that_end_in_a_mended_draw(name, tied):
     for x, y in ((s.beta, ahead.beta), (s.resid, ahead.resid), (s.delta, ahead.delta)):
         assert torch.equal(x, y)
     assert (s.status()[1] & 1) == (1 if tied else 0)        # ties: the boundary was cut further
+
+
+def _csc(lengths, n_rows, value, seed):
+    """Columns of these lengths, rows uniform; value(generator, n): their entries."""
+    g = torch.Generator().manual_seed(seed)
+    ptr = torch.cat([torch.zeros(1, dtype=torch.int64), torch.cumsum(lengths, 0)])
+    rows = torch.cat([torch.randperm(n_rows, generator=g)[:n].sort().values for n in lengths.tolist()]).to(torch.int32)
+    return value(g, int(ptr[-1])), rows, ptr, torch.randn(n_rows, generator=g)
+
+
+# products that are zero again and again (values of +-1, one in eight of the stored ones 0), by buckets and by the walk over all candidates;
+# columns of 4 to 400 entries: more than the table of rows takes, and other than the mean says of the last survivors; windows with more
+# candidates than a warp has places for, each with few of them and with more than it can list
+@pytest.mark.parametrize("name,n_rows,n_candidates,n_keep,rho", [("cancel", 3000, 900, 130, 0.1), ("cancel", 700, 800, 300, 0.2), ("uneven", 700, 1500, 300, 0.1),
+                                                                 ("uneven", 60000, 1700, 1000, 0.02), ("cancel", 20000, 2000, 1300, 0.1), ("many_met", 70000, 2000, 1300, 0.3)])
+def test_rounds_on_unusual_columns(name, n_rows, n_candidates, n_keep, rho):
+    from paper_1312_5766_b200 import binding as b
+    J = 8000
+    if name == "many_met":
+        lengths, value = torch.full((J,), 150, dtype=torch.int64), lambda g, n: torch.randn(n, generator=g)
+    elif name == "cancel":
+        lengths = torch.full((J,), 33, dtype=torch.int64)
+        value = lambda g, n: ((torch.randint(0, 2, (n,), generator=g) * 2 - 1) * (torch.randint(0, 8, (n,), generator=g) > 0)).float()
+    else:
+        lengths = (400.0 * (torch.arange(J) + 1.0) ** -0.5).long()[torch.randperm(J, generator=torch.Generator().manual_seed(1))]
+        value = lambda g, n: torch.randn(n, generator=g)
+    values, rows, ptr, y = _csc(lengths, n_rows, value, 7)
+    X = oracle.Matrix.csc(n_rows, J, values.numpy(), rows.numpy(), ptr.numpy())
+    n2 = oracle.colnorm2(X)
+    args = (wl.CSC, n_rows, J, values.cuda(), y.cuda(), 0.05, 1e-6, rho, n_candidates, n_keep)
+    kw = dict(seed=2, row_idx=rows.cuda(), col_ptr=ptr.cuda())
+    s, ahead = b.StradsLasso(*args, **kw), b.StradsLasso(*args, **kw)
+    for t in range(10):
+        delta = s.delta.cpu().numpy().astype(np.float64)
+        cand, kept, _, counts = (x.cpu().numpy() for x in s.round())
+        assert np.array_equal(cand, oracle.sample(delta, float(np.float32(1e-6)), 2, t, n_candidates)), t
+        _assert_kept_matches(X, n2, cand, n_keep, float(np.float32(rho)), kept[: int(counts[2])], int(counts[1]))
+    ahead.run(10)
+    four, one = (b.StradsLasso(*args, n_schedulers=4, **kw) for _ in range(2))
+    four.run(10)
+    for _ in range(10):
+        one.round()
+    for u, v in ((s, ahead), (four, one)):
+        assert all(torch.equal(x, y) for x, y in ((u.beta, v.beta), (u.resid, v.resid), (u.delta, v.delta)))
+        assert u.status()[0] == 0 and v.status()[0] == 0
