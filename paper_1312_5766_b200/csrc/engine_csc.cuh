@@ -537,9 +537,14 @@ constexpr int kFreeRow = -1;
 constexpr unsigned int kNoSlot = 0xffff;
 constexpr int kOwn = 256;                                // candidates a CTA can hold (more: their columns stay in global memory)
 constexpr int kOwnEntries = 5120;                        // entries of their columns
+// ... where there are more: without the values, which the few entries in rows of kept members then fetch.  What finds no room at all is read
+// from global memory for every kept member (us per round, 10^6 x 10^6 by Zipf's law, 16,384 candidates of 60 / 50 entries, up to 7,680 / 6,400 to a CTA:
+// 137 / 107 with a third / a fifth of them so, one entry after the other; 131 / 101 with eight at a time; 87 / 77 with all rows held).
+constexpr int kOwnRows = kOwnEntries * 3 / 2;
 constexpr int kRestEntries = kOwnEntries * 3 / 2;
 // Survivors that are settled at once: as many as a thread pair of bits per walking thread holds, and while their entries, all of
-// which every CTA goes through, are no more than these (us per round for 1,500 / 2,600 / 4,096 / 7,000 / 12,288: 10^7 columns of 20
+// which every CTA goes through, are no more than these -- by the mean length of all columns: an estimate, the pieces they are gone through in make up
+// for it -- (us per round for 1,500 / 2,600 / 4,096 / 7,000 / 12,288: 10^7 columns of 20
 // entries 65.8 / 65.5 / 64.8 / 65.3 / 66.3, 300,000 of 30 34.9 / 35.5 / 37.0 / 39.8 / 41.1, 3,000,000 of 12 47.0 / 44.9 / 45.1 / 48.2 / 48.1).
 constexpr int kLast = 512;
 constexpr long long kLastEntries = 3072;
@@ -577,6 +582,7 @@ struct DemandShared {
       float oval[kOwnEntries];
       unsigned int omet[kOwnEntries];                    // a candidate's entries in rows of kept members: slot, and entry << 16
     };
+    struct { int only_row[kOwnRows]; unsigned int only_met[kOwnRows]; };
     struct { int rrow[kRestEntries]; float rval[kRestEntries]; };      // survivors' columns
   };
 };
@@ -631,6 +637,29 @@ __device__ __forceinline__ float row_products(const DemandShared& s, int q, int 
   }
   return dot;
 }
+// The same over a column in global memory, entries side by side.  (Out of line: rare, and the hot code is fetched anew every round.)
+__device__ __noinline__ float column_products(const int* rows, const float* vals, int n, const DemandShared& s, int q) {
+  constexpr int kU = 8;
+  float dot = 0.f;
+#pragma unroll 1
+  for (int x0 = 0; x0 < n; x0 += kU) {
+    int row[kU];
+    float v[kU];
+    unsigned int sl[kU];
+    uint2 rec[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const bool on = x0 + u < n;
+      row[u] = on ? __ldg(rows + x0 + u) : kFreeRow;
+      v[u] = on ? __ldg(vals + x0 + u) : 0.f;
+    }
+    find_rows<kU>(s, row, 1u << q, sl);
+#pragma unroll
+    for (int u = 0; u < kU; ++u) rec[u] = sl[u] != kNoSlot ? s.row_rec[sl[u]] : make_uint2(0u, 0u);
+    dot = add_products<kU>(s, q, rec, v, dot);
+  }
+  return dot;
+}
 // x_a^T x_b of two ascending row lists, products added in row order; no branch depends on the data.
 __device__ __forceinline__ float merge_dot(const int* ar, const float* av, int na, const int* br, const float* bv, int nb) {
   float dot = 0.f;
@@ -669,10 +698,11 @@ __device__ __forceinline__ bool walk_barrier(DemandShared& s, Grid& g) {
   return s.ok != 0;
 }
 
-// The columns of `count` candidates (thread i of kOwn has the i-th) into row / val, one behind the other, as far as there is room.
-// Bound by the lines a load touches, so several threads share a column.  Bar: the threads' barrier.
+// The columns of `count` candidates (thread i of kOwn has the i-th) into row / val, one behind the other, as far as there is room
+// (room_rows > 0: if not for all, as far as there is without the values).  Bound by the lines a load touches, so several threads share a column.  Bar: the threads' barrier.
 template <int kBar>
-__device__ __forceinline__ void hold_columns(const Problem& p, DemandShared& s, int i, int count, const WalkColumn& col, int* row, float* val, int room) {
+__device__ __forceinline__ void hold_columns(const Problem& p, DemandShared& s, int i, int count, const WalkColumn& col, int* row, float* val, int room,
+                                             int room_rows) {
   const int lane = threadIdx.x & 31, warp = i >> 5;
   int* wsum = s.wsum + (kBar == 1 ? 0 : kWalkWarps);
   int incl = col.n;
@@ -690,13 +720,15 @@ __device__ __forceinline__ void hold_columns(const Problem& p, DemandShared& s, 
   s.own_at[i + 1] = before + incl;
   s.own_q0[i] = col.q0; s.own_n2[i] = col.n2;
   asm volatile("bar.sync %0, %1;" ::"n"(kBar), "n"(kOwn) : "memory");
+  const bool values = room_rows == 0 || s.own_at[count] <= room;
+  if (!values) room = room_rows;
 #pragma unroll 2
   for (int k = i >> 3; k < count; k += kOwn / 8) {
     const int at = s.own_at[k], m = s.own_at[k + 1] - at;
     const long long from = s.own_q0[k];
     if (at + m <= room)
 #pragma unroll 4
-      for (int q = i & 7; q < m; q += 8) { row[at + q] = __ldg(p.xrow + from + q); val[at + q] = __ldg(p.xv + from + q); }
+      for (int q = i & 7; q < m; q += 8) { row[at + q] = __ldg(p.xrow + from + q); if (values) val[at + q] = __ldg(p.xv + from + q); }
   }
 }
 
@@ -718,7 +750,7 @@ __device__ __forceinline__ bool settle_rest(const Crew& crew, const Problem& p, 
     const int count = min(behind - c0, kOwn);
     WalkColumn col = {};
     if (tid < count) col = p.walk_cols[s.survivor[c0 + tid]];
-    hold_columns<1>(p, s, tid, count, col, s.rrow, s.rval, kRestEntries);
+    hold_columns<1>(p, s, tid, count, col, s.rrow, s.rval, kRestEntries, 0);
     walk_sync();
     here = kOwn;                                         // whole words; of the first one whatever does not fit is read where it is
     while (here > 32 && s.own_at[here] > kRestEntries) here -= 32;
@@ -895,7 +927,7 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Crew& crew, const Probl
       const int i = tid - kWalkT;
       WalkColumn col = {};
       if (i < n_here && own_index(i) < n) col = p.walk_cols[own_index(i)];
-      hold_columns<2>(p, s, i, n_here, col, s.orow, s.oval, kOwnEntries);
+      hold_columns<2>(p, s, i, n_here, col, s.orow, s.oval, kOwnEntries, kOwnRows);
     }
     asm volatile("bar.arrive 3, %0;" ::"n"(kT) : "memory");
     const bool drawn = draw();
@@ -1065,9 +1097,9 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Crew& crew, const Probl
           und &= ~(fresh | __ballot_sync(kFull, (earlier & fresh) != 0u));
         }
       }
-      const int room = p.n_keep - kept;
-      const bool done = __popc(keep) >= room;            // stop exactly at P: drop the surplus from the back
-      while (__popc(keep) > room) keep &= ~(1u << (31 - __clz((int)keep)));
+      const int open = p.n_keep - kept;
+      const bool done = __popc(keep) >= open;            // stop exactly at P: drop the surplus from the back
+      while (__popc(keep) > open) keep &= ~(1u << (31 - __clz((int)keep)));
       if (warp < 2 && ((keep >> lane) & 1u)) {
         const int r = __popc(keep & ((1u << lane) - 1u));
         if (warp == 0) {
@@ -1085,6 +1117,9 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Crew& crew, const Probl
       // ---- D: the kept members against this CTA's later unblocked candidates ----
       mask_at = walk_mask_at(batch, p.mask_words);
       if (!held) { held = true; asm volatile("bar.sync 3, %0;" ::"n"(kT) : "memory"); }        // their columns are there
+      const bool values = s.own_at[n_here] <= kOwnEntries;
+      const int room = values ? kOwnEntries : kOwnRows;
+      unsigned int* omet = values ? s.omet : s.only_met;
       for (int k0 = 0; k0 < n_own; k0 += kOwn) {         // (a turn of at most kOwn candidates; one turn as a rule)
         if (k0 > 0) { walk_sync(); if (tid == 0) s.n_free = 0; walk_sync(); }
         for (int k = k0 + tid; k < min(n_own, k0 + kOwn); k += kWalkT) {
@@ -1101,7 +1136,7 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Crew& crew, const Probl
           int k = 0, from = 0, end = 0, met = 0;
           if (c < n_free) {
             k = s.own_free[c]; from = s.own_at[k]; end = s.own_at[k + 1];
-            if (end > kOwnEntries) end = from;
+            if (end > room) end = from;
           }
 #pragma unroll 1
           for (int i0 = from + sub; __any_sync(kFull, i0 < end + sub); i0 += 4 << share) {
@@ -1113,7 +1148,7 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Crew& crew, const Probl
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
               const unsigned int mine = __ballot_sync(kFull, sl[u] != kNoSlot) & group;
-              if (sl[u] != kNoSlot) s.omet[from + met + __popc(mine & ((1u << lane) - 1u))] = sl[u] | (unsigned)(i0 + (u << share) - from) << 16;
+              if (sl[u] != kNoSlot) omet[from + met + __popc(mine & ((1u << lane) - 1u))] = sl[u] | (unsigned)(i0 + (u << share) - from) << 16;
               met += __popc(mine);
             }
           }
@@ -1125,24 +1160,17 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Crew& crew, const Probl
           const int c = (int)((unsigned)i * per >> 20), qk = s.kept_q[i - c * n_new], k = s.own_free[c];
           float dot = 0.f;
           double n2b;
-          if (table && k < kOwn && s.own_at[k + 1] <= kOwnEntries) {
+          if (table && k < kOwn && s.own_at[k + 1] <= room) {
             n2b = s.own_n2[k];
             const int met = s.n_met[k], from = s.own_at[k];
             dot = row_products(s, qk, met, met, [&](int x, uint2& rec, float& v) {
-              const unsigned int en = s.omet[from + x];
-              rec = s.row_rec[en & 0xffffu]; v = s.oval[from + (int)(en >> 16)];
+              const unsigned int en = omet[from + x];
+              rec = s.row_rec[en & 0xffffu]; v = values ? s.oval[from + (int)(en >> 16)] : __ldg(p.xv + s.own_q0[k] + (en >> 16));
             });
           } else if (table) {                            // (no room for its column)
             const WalkColumn cb = p.walk_cols[own_index(k)];
             n2b = cb.n2;
-            for (int x = 0; x < cb.n; ++x) {
-              const int row[1] = {__ldg(p.xrow + cb.q0 + x)};
-              unsigned int sl[1];
-              find_rows<1>(s, row, 1u << qk, sl);
-              const uint2 rec[1] = {s.row_rec[sl[0] != kNoSlot ? sl[0] : 0u]};
-              const float v[1] = {__ldg(p.xv + cb.q0 + x)};
-              if (sl[0] != kNoSlot) dot = add_products<1>(s, qk, rec, v, dot);
-            }
+            dot = column_products(p.xrow + cb.q0, p.xv + cb.q0, cb.n, s, qk);
           } else {
             const WalkColumn cb = p.walk_cols[own_index(k)];
             n2b = cb.n2;
