@@ -539,7 +539,7 @@ constexpr int kOwn = 256;                                // candidates a CTA can
 constexpr int kOwnEntries = 5120;                        // entries of their columns
 // ... where there are more: without the values, which the few entries in rows of kept members then fetch.  What finds no room at all is read
 // from global memory for every kept member (us per round, 10^6 x 10^6 by Zipf's law, 16,384 candidates of 60 / 50 entries, up to 7,680 / 6,400 to a CTA:
-// 137 / 107 with a third / a fifth of them so, one entry after the other; 131 / 101 with eight at a time; 87 / 77 with all rows held).
+// 137 / 107 with a third / a fifth of them so, one entry after the other; 131 / 101 with eight at a time; 86 / 76 with all rows held).
 constexpr int kOwnRows = kOwnEntries * 3 / 2;
 constexpr int kRestEntries = kOwnEntries * 3 / 2;
 // Survivors that are settled at once: as many as a thread pair of bits per walking thread holds, and while their entries, all of
@@ -660,6 +660,16 @@ __device__ __noinline__ float column_products(const int* rows, const float* vals
   }
   return dot;
 }
+// The same over the entries of held candidate k in rows of kept members, their values fetched.  (Out of line like that: as a branch in the
+// loop where the values are held it cost rounds whose columns all fit 7 %, 10^6 x 10^7 with 20 entries 61.9 -> 66.4 us, like this under 1 %.)
+__device__ __noinline__ float fetched_products(const DemandShared& s, const float* vals, int k, int q) {
+  const int met = s.n_met[k], from = s.own_at[k];
+  vals += s.own_q0[k];
+  return row_products(s, q, met, met, [&](int x, uint2& rec, float& v) {
+    const unsigned int en = s.only_met[from + x];
+    rec = s.row_rec[en & 0xffffu]; v = __ldg(vals + (en >> 16));
+  });
+}
 // x_a^T x_b of two ascending row lists, products added in row order; no branch depends on the data.
 __device__ __forceinline__ float merge_dot(const int* ar, const float* av, int na, const int* br, const float* bv, int nb) {
   float dot = 0.f;
@@ -698,6 +708,15 @@ __device__ __forceinline__ bool walk_barrier(DemandShared& s, Grid& g) {
   return s.ok != 0;
 }
 
+// (cold, see hold_columns)
+__device__ __noinline__ void hold_rows(DemandShared& s, const int* rows, int i, int count, int* row, int room) {
+  for (int k = i >> 3; k < count; k += kOwn / 8) {
+    const int at = s.own_at[k], m = s.own_at[k + 1] - at;
+    if (at + m <= room)
+#pragma unroll 4
+      for (int q = i & 7; q < m; q += 8) row[at + q] = __ldg(rows + s.own_q0[k] + q);
+  }
+}
 // The columns of `count` candidates (thread i of kOwn has the i-th) into row / val, one behind the other, as far as there is room
 // (room_rows > 0: if not for all, as far as there is without the values).  Bound by the lines a load touches, so several threads share a column.  Bar: the threads' barrier.
 template <int kBar>
@@ -720,15 +739,17 @@ __device__ __forceinline__ void hold_columns(const Problem& p, DemandShared& s, 
   s.own_at[i + 1] = before + incl;
   s.own_q0[i] = col.q0; s.own_n2[i] = col.n2;
   asm volatile("bar.sync %0, %1;" ::"n"(kBar), "n"(kOwn) : "memory");
-  const bool values = room_rows == 0 || s.own_at[count] <= room;
-  if (!values) room = room_rows;
+  if (room_rows > 0 && s.own_at[count] > room) {
+    hold_rows(s, p.xrow, i, count, row, room_rows);
+    return;
+  }
 #pragma unroll 2
   for (int k = i >> 3; k < count; k += kOwn / 8) {
     const int at = s.own_at[k], m = s.own_at[k + 1] - at;
     const long long from = s.own_q0[k];
     if (at + m <= room)
 #pragma unroll 4
-      for (int q = i & 7; q < m; q += 8) { row[at + q] = __ldg(p.xrow + from + q); if (values) val[at + q] = __ldg(p.xv + from + q); }
+      for (int q = i & 7; q < m; q += 8) { row[at + q] = __ldg(p.xrow + from + q); val[at + q] = __ldg(p.xv + from + q); }
   }
 }
 
@@ -1162,11 +1183,15 @@ __device__ __forceinline__ bool csc_walk_on_demand(const Crew& crew, const Probl
           double n2b;
           if (table && k < kOwn && s.own_at[k + 1] <= room) {
             n2b = s.own_n2[k];
-            const int met = s.n_met[k], from = s.own_at[k];
-            dot = row_products(s, qk, met, met, [&](int x, uint2& rec, float& v) {
-              const unsigned int en = omet[from + x];
-              rec = s.row_rec[en & 0xffffu]; v = values ? s.oval[from + (int)(en >> 16)] : __ldg(p.xv + s.own_q0[k] + (en >> 16));
-            });
+            if (values) {
+              const int met = s.n_met[k], from = s.own_at[k];
+              dot = row_products(s, qk, met, met, [&](int x, uint2& rec, float& v) {
+                const unsigned int en = s.omet[from + x];
+                rec = s.row_rec[en & 0xffffu]; v = s.oval[from + (int)(en >> 16)];
+              });
+            } else {
+              dot = fetched_products(s, p.xv, k, qk);
+            }
           } else if (table) {                            // (no room for its column)
             const WalkColumn cb = p.walk_cols[own_index(k)];
             n2b = cb.n2;
