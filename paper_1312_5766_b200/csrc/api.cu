@@ -45,6 +45,7 @@ struct strads_lasso_s {
   // and walk of round t, and the round then starts from that list corrected for round t's update.
   bool ahead_ok;             // the configuration allows it
   Engine ahead_draw;
+  bool draw_beside;          // several schedulers: draws beside other blocks' Grams go so too
   Problem ahead;             // the early draw's view of the problem: own sampler state and buffers, P' + P winners
   cudaStream_t ahead_stream;
   cudaEvent_t ahead_fork, ahead_done;
@@ -587,7 +588,9 @@ int pipelined_rounds(strads_lasso_s* h, long long count, cudaStream_t main) {
     const Problem& p = sc.p;
     CK(cudaStreamWaitEvent(sc.stream, joined[s] ? sc.updated : h->fork, 0));
     joined[s] = true;
-    CK(launch_sample(p, p.cand, sc.stream));
+    Problem drawn = p;
+    if (!h->draw_beside) drawn.draw = nullptr;
+    CK(launch_sample(drawn, p.cand, sc.stream));
     const int rc = gram_and_filter(sc, sc.stream, p.cand, p.n_cand, nullptr);
     if (rc) return rc;
     CK(cudaEventRecord(sc.block_ready, sc.stream));
@@ -723,10 +726,19 @@ void fill_engine(Engine& en, const Problem& p, const Layout& L, char* ws, int n_
   en.tile_ticket = reinterpret_cast<unsigned int*>(ws + L.off_eng_tickets);
 }
 
-// Whether the Gram of the window leaves the SMs of a few clusters free for a draw beside it.
-bool draw_beside_gram(const Problem& p) {
-  const long long side = (window_of(p, p.n_cand) + 127) / 128;
-  return side * (side + 1) / 2 * 8 * 2 <= p.sm_count;
+// Whether a draw beside Grams goes in one launch of a cluster: where the Grams under way (one per scheduler, a cluster of eight CTAs per tile of the
+// window) leave the SMs of a few clusters free -- with them taken, a cluster waits for a whole one and the Grams for it: S = 4, P = 240 and more
+// 7 to 10 % slower than three launches -- and, with one scheduler, where three launches would not be over in time anyway.  us per round,
+// three launches / cluster, 2,500 and 8,000 rows: S = 1, P' = 140, J = 200,000 31.8 / 24.2, 30.9 / 26.5; P' = 1,200, J = 72,000 31.1 / 28.9,
+// 34.5 / 33.1; S = 2, P' = 600, J = 20,000 26.0 / 23.2, 28.5 / 25.7; S = 3 19.2 / 17.3, 21.4 / 18.6.  S = 1, 3,836 rows, P' = 140 and 300 (windows of
+// 140 and 128), J = 72,000 (8,000) 23.5 / 23.8, 25.5 / 26.4 (22.2 / 21.8, 25.5 / 25.7), logistic 24.2 / 24.6, 26.4 / 27.4 (23.1 / 23.9, 25.4 / 26.3); J = 130,000
+// 25.8 / 22.6, 27.2 / 26.5; P' = 600 (a window of 256), J = 8,000 27.9 / 27.8, logistic 27.6 / 28.2.
+bool draw_beside_gram(const Problem& p, int n_sched) {
+  if (p.layout != STRADS_DENSE_COLMAJOR) return false;
+  const int window = window_of(p, p.n_cand);
+  const long long side = (window + 127) / 128;
+  if (n_sched == 1 && (window <= 192 ? p.J <= 100000 : window <= 256 && p.J <= 16000)) return false;
+  return n_sched * (side * (side + 1) / 2) * 8 * 2 <= p.sm_count;
 }
 
 // What must be zero before a launch of the engine or the squads (they leave it so, unless a wait expired).
@@ -857,7 +869,7 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
   if (h->ahead_ok) {
     fill_ahead(h->ahead, p0, L, ws);
     h->ahead.draw = nullptr;
-    if (draw_beside_gram(p0) && fill_draw(h->ahead_draw, h->ahead, L, ws, 1, draw_ctas)) {
+    if (draw_beside_gram(p0, 1) && fill_draw(h->ahead_draw, h->ahead, L, ws, 1, draw_ctas)) {
       h->ahead.draw = &h->ahead_draw;
       if ((e = cudaMemsetAsync(h->ahead_draw.es, 0, sizeof(EngineState), h->stream)) != cudaSuccess ||
           (e = cudaMemsetAsync(h->ahead_draw.hist, 0, sizeof(unsigned int) * kHistBins, h->stream)) != cudaSuccess)
@@ -897,6 +909,7 @@ int strads_lasso_init(const strads_lasso_config_t* c, strads_handle_t* out_handl
       sc.stream = kit.sched[s]; sc.block_ready = kit.ready[s]; sc.updated = kit.updated[s];
     }
   }
+  h->draw_beside = draw_beside_gram(h->sch[0].p, S);
   h->squads_ok = Q > 1 && sm_count <= kEngineMaxCtas && sm_count / Q >= kSquadMinCtas && squads_of(c, sm_count) == Q;
   if (h->squads_ok) {
     SquadSet& set = h->squads;
