@@ -259,7 +259,8 @@ bool engine_provided(const strads_lasso_config_t* c) {
 // the other, each by one squad, and every entry of a kept column costs a CTA some 10 ns there; so the squads are taken while a CTA has up to 3,400
 // (mean) entries of them.  us per round, squads / launches, uniform rows, P' = 16,384 (4,096 for P = 1,024 and less): 10^6 rows, 60 entries, P = 2,048,
 // S = 2, 4, 8 (1,660, 3,320, 6,830 entries): 57 / 71, 51 / 58, 68 / 59; P = 1,024: 33 / 48, 28 / 43, 40 / 46; 200 entries, P = 512: 41 / 61, 38 / 49, 61 / 52 (5,690).
-// With P beyond 2,048 the window is gone through in several passes by the few CTAs of a squad: P = 4,096, S = 2: 105 / 99, P = 8,192 of 20 entries 164 / 142.
+// A column counts as one entry more: 10^6 columns of 5 entries, P = 12,000, S = 2, 4, 8 (973, 1,946, 4,000 with it): 67 / 101, 58 / 83, 94 / 87.
+// P = 4,096 of 20 entries, S = 2, 4: 49 / 71, 42 / 57, by Zipf's law 41 / 87, 34 / 79; P = 8,192 of 8 entries 71 / 109, 63 / 86.
 // (The static schedule, squads / one launch round after round: 52 / 60, 28 / 39, 38 / 56 for the same; without the rho test 31 / 34, 19 / 25,
 // 29 / 33, but 72 / 39 with 11,000 entries.)
 int squads_of(const strads_lasso_config_t* c, int n_ctas) {
@@ -267,7 +268,7 @@ int squads_of(const strads_lasso_config_t* c, int n_ctas) {
   int n = n_sched_of(c);
   if (n == 1 && (c->flags & STRADS_FLAG_UNIFORM_DRAW) && !(c->flags & STRADS_FLAG_DYNAMIC_DEPS)) n = kStaticSquads;
   const int size = n_ctas / n;
-  return c->n_keep <= 2048 && (double)c->n_keep * (double)c->nnz <= 3400.0 * (double)size * (double)c->n_cols ? n : 1;
+  return (double)c->n_keep * ((double)c->nnz + (double)c->n_cols) <= 3400.0 * (double)size * (double)c->n_cols ? n : 1;
 }
 // Keys each CTA can save of a scan that finds a few times `winners` of them in all.
 unsigned int engine_saved(size_t winners) { return (unsigned int)(winners / 16 + 64); }

@@ -3,7 +3,7 @@
 //
 // A round is a chain of short dependent steps over a few MB at most, so what bounds it is the number of times the
 // whole grid has to hand over to itself and what every hand-over costs.  As separate launches a round took 11 to 17
-// kernels, each with its launch, its ramp and the drain of the one before; here it takes four barriers of ~1.5 us, and the
+// kernels, each with its launch, its ramp and the drain of the one before; here it takes four barriers of 2 to 3 us, and the
 // draw of the next round runs in the shadow of the steps of this one:
 //
 //   step           dense                                          CSC
@@ -13,8 +13,8 @@
 //   2  (all CTAs)  Gram tiles on the tensor cores, then the      inner products from the buckets, x_c^T r and would-be
 //                  pairs they leave open                          changes
 //  (2b)            open pairs that their CTA had no room for
-//   3              greedy walk (last CTA); keys of round t + 1    the same; buckets emptied (the others)
-//                  below the boundary collected (the others)
+//   3              greedy walk (last CTA); keys of round t + 1    greedy walk by half the threads of every CTA; buckets emptied,
+//                  below the boundary collected (the others)      keys of round t + 1 collected by the others
 //  (3b)            all candidates instead of the window           walk over all candidates with conflict rows on demand by half the
 //                                                                 warps, the draw of round t + 1 by the others
 //   4  (all CTAs)  residual, beta, delta; the winners of the draw ranked, corrected for this round's changes
@@ -1027,7 +1027,7 @@ __global__ void __launch_bounds__(kT, 1) k_engine(const __grid_constant__ Proble
 // The draw alone (strads_sample_static), all of it in one launch: keys computed once and kept in shared memory, histogram,
 // selection, collection and ranking with two grid barriers between them.  Bound by the launch and the barriers: 22.6 us
 // as six launches (clear, round index, two passes, ordering), each waiting for the one before, at J = 100,000, P' = 2,048;
-// one launch and a clear before it still took 16.4, so the kernel leaves its scratch clear instead.
+// one launch 16.4, and 14.3 since its parameters are copied to shared memory only where a rare path wants them.  It leaves its scratch clear.
 // A call whose wait runs out leaves -1 in the places of the list that it did not come to, and says so to the next one
 // (EngineState::dirty), which then clears the histogram behind a barrier of its own: every CTA leaves through the same few
 // lines, and the one that leaves last sets the barrier back and knows from their count whether any of them gave up.

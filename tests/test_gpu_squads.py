@@ -29,6 +29,7 @@ CASES = {
     "held": dict(kind="csc_uniform", n_rows=200000, n_cols=20000, n_candidates=2000, n_keep=1900, rho=0.3, nnz_col=150, S=8),
     "long": dict(kind="csc_uniform", n_rows=50000, n_cols=3000, n_candidates=300, n_keep=200, rho=0.3, nnz_col=600, S=7),
     "many_kept": dict(kind="csc_uniform", n_rows=500000, n_cols=131500, n_candidates=16000, n_keep=15000, rho=0.4, nnz_col=4, S=8),
+    "most_kept": dict(kind="csc_uniform", n_rows=500000, n_cols=100500, n_candidates=12500, n_keep=11900, rho=0.4, nnz_col=4, S=8),
     # the walk over all candidates by few CTAs: more candidates and entries than a CTA holds
     "on_demand_turns": dict(kind="csc_zipf", n_rows=30000, n_cols=140000, n_candidates=16384, n_keep=400, rho=0.05, nnz_col=21, S=8),
     "on_demand_entries": dict(kind="csc_zipf", n_rows=30000, n_cols=40000, n_candidates=9500, n_keep=700, rho=0.05, nnz_col=63, S=4),
