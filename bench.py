@@ -47,7 +47,7 @@ NCU_TRAFFIC = {
     ("c4", "k_engine<csc>"): 66.3e6 / 32,
     ("c5", "k_engine<csc>"): 402.9e6 / 32,
 }
-ENGINE_ROUNDS = 32                         # CSC: whole rounds in one launch, that many at most
+ENGINE_ROUNDS = 32                         # CSC and short dense columns: whole rounds in one launch, that many at most
 
 
 def measured_peaks():
@@ -277,9 +277,11 @@ def rooflines(p: wl.LassoProblem, workload: str, step_ms: dict, kept_per_round: 
 def launches_of_run(p: wl.LassoProblem, steps: int) -> int:
     """Kernels of the library launched by a strads_run of `steps` rounds (dense: a fixed sequence per round; launches of the
     retry branch return at once when the screen's last CTA settled the round)."""
-    if p.layout != wl.DENSE:
+    if p.layout != wl.DENSE or (p.n_rows <= 2048 and p.n_rows * p.rho * p.rho <= 18.0):
         return (steps + ENGINE_ROUNDS - 1) // ENGINE_ROUNDS
-    n = 3                  # the early draw of the next round: histogram pass, collect pass, ordering
+    # the early draw of the next round: one cluster where the Gram's clusters of eight leave it room, else histogram pass, collect pass, ordering
+    side, short = (window_of(p) + 127) // 128, window_of(p) <= 192 and p.n_cols <= 100_000 or window_of(p) <= 256 and p.n_cols <= 16_000
+    n = 1 if p.n_cols <= 1 << 19 and side * (side + 1) // 2 * 16 <= 148 and not short else 3
     n += 1                 # correction of the early list
     n += 2                 # pack, Gram (screen + cluster split-K + recheck + walk)
     n += 1                 # update

@@ -179,7 +179,9 @@ int strads_round(strads_handle_t h, const strads_round_out_t* out);
  * behind the last one stays: whoever writes delta (or beta, or resid) between two runs calls strads_set_round.
  *
  * CSC with one scheduler, and dense X with short columns (N rho^2 <= 18, N <= 2,048, and a workspace that provides for
- * it), run up to 32 whole rounds per cooperative launch.  Otherwise the rounds are replayed from captured launch sequences: with one scheduler eight
+ * it), run up to 32 whole rounds per cooperative launch; CSC with several schedulers, or with the static schedule, up to 64, a squad of
+ * CTAs for every block under way, where the kept columns are not too many for a squad and the workspace provides for it.
+ * Otherwise the rounds are replayed from captured launch sequences: with one scheduler eight
  * rounds each (the draw on a stream of its own beside the Gram and the walk), and what is left over of a run as
  * sequences of four, two and one round, each captured when its length comes up for the third time and
  * enqueued directly until then; with several schedulers 16 turns of each per sequence.  The streams, events and

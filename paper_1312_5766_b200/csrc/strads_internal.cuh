@@ -297,7 +297,13 @@ __device__ __forceinline__ void apply_row(const Problem& p, long long i, float n
   }
 }
 __device__ __forceinline__ void apply_row(const Problem& p, long long i, double s) {
-  apply_row(p, i, (p.flags & STRADS_FLAG_LOGISTIC) ? p.margin[i] : p.resid[i], s);
+  if (p.flags & STRADS_FLAG_LOGISTIC) {
+    const float m = (float)((double)p.margin[i] + s);
+    p.margin[i] = m;
+    p.resid[i] = (float)((double)p.y[i] - sigmoid64((double)m));
+  } else {
+    p.resid[i] = (float)((double)p.resid[i] - s);
+  }
 }
 
 // x_a^T x_b of two CSC columns (ascending rows): a given as arrays (possibly staged in shared memory), b read
